@@ -24,6 +24,7 @@ struct mhd_ctx {
   bool tiled;          // FP32: TMA-fed z-march kernels; otherwise the simple kernel
   bool split;          // FP32 forward: split passes (else the fused z-march kernel)
   bool pair;           // FP32 forward: one-pass f32x2 kernel with TMEM z histories
+  bool rk64;           // FP64 forward: z-march with shared first derivatives (else one thread per cell)
   void* bj;            // split: [6][nz][ny][nx] B, J of the current substep
   void* sw;            // split: [3][nz - ksw][ny][nx] swamp terms
   int ksw;             // first layer with a nonzero swamp weight or slope (nz if none)
@@ -591,6 +592,11 @@ static void launch_rk_any(mhd_ctx* h, const R* fin, R* fout, int sub, const CUte
                     h->st);
     return;
   }
+  if (sizeof(R) == 8 && h->rk64) {
+    launch_rk64(h->L, *(const Phys<double>*)&ph, h->bgd, (const double*)fin, (double*)fout, (double*)h->df,
+                (const double*)h->wtab, (const double*)h->wptab, drv, h->ss, sub, h->st);
+    return;
+  }
   launch_rk<R>(h->L, ph, bgr<R>(h), fin, fout, (R*)h->df, (const R*)h->wtab, (const R*)h->wptab, drv, h->ss, sub,
                h->st);
 }
@@ -826,6 +832,7 @@ extern "C" int mhd_create(const mhd_params* p, void* workspace, size_t ws_bytes,
   {
     const char* v = getenv("MHD_RK_VARIANT");
     h->tiled = p->precision == 32 && !(v && strcmp(v, "simple") == 0);
+    h->rk64 = p->precision == 64 && !(v && strcmp(v, "simple") == 0);
     h->split = h->tiled && !(v && strcmp(v, "fused") == 0);
     h->pair = h->split && !(v && (strcmp(v, "tiled") == 0 || strcmp(v, "split") == 0)) &&
               rk_pair_supported(h->L);
@@ -1483,6 +1490,9 @@ static void adjoint_reverse(mhd_ctx* h, R* const (&S)[3], const CUtensorMap* con
       launch_adj_point_tiled(tms[s], h->L, *(const Phys<float>*)&ph, h->bgf, (const float*)h->dbar,
                              (float*)h->coef, h->thbar, (const float*)h->wtab, (const float*)h->wptab, h->ss, s,
                              h->p.dx, h->p.dy, h->p.dz, h->st);
+    else if (sizeof(R) == 8 && h->adj_tiled)
+      launch_adj_point64(h->L, *(const Phys<double>*)&ph, h->bgd, (const double*)S[s], (const double*)h->dbar,
+                         (double*)h->coef, h->thbar, (const double*)h->wtab, (const double*)h->wptab, h->ss, s, h->st);
     else
       launch_adj_point<R>(h->L, ph, bg, S[s], (const R*)h->dbar, (R*)h->coef, h->thbar, (const R*)h->wtab,
                           (const R*)h->wptab, h->ss, s, h->st);

@@ -102,6 +102,14 @@ template <typename R> void launch_rk(const Layout& L, const Phys<R>& ph, const B
                                      const R* fin, R* fout, R* df,
                                      const R* wtab, const R* wptab, const Driver& drv, const StepState* ss,
                                      int sub, cudaStream_t st);
+// the same in FP64 as a z-march that shares the first derivatives between the
+// mixed ones (mhd_rk64.cu), and the FP64 pointwise adjoint on it
+void launch_rk64(const Layout& L, const Phys<double>& ph, const Background<double>& bg, const double* fin,
+                 double* fout, double* df, const double* wtab, const double* wptab, const Driver& drv,
+                 const StepState* ss, int sub, cudaStream_t st);
+void launch_adj_point64(const Layout& L, const Phys<double>& ph, const Background<double>& bg, const double* g,
+                        const double* dbar, double* coef, double* thbar, const double* wtab, const double* wptab,
+                        const StepState* ss, int sub, cudaStream_t st);
 // FP32 TMA-fed variant of launch_rk (tensor map of the input state set)
 void launch_rk_tiled(const CUtensorMap* tm, const Layout& L, const Phys<float>& ph, const Background<float>& bg,
                      float* fout, float* df, const float* wtab, const float* wptab, const Driver& drv,
