@@ -266,9 +266,8 @@ __global__ void adj_bc_kernel(Layout L, Phys<R> ph, Background<R> bg, const R* _
 // Elementwise adjoint updates over the cells that carry state (interior, and
 // the u_x, u_y ghost layers below the photosphere), 16 bytes per thread and
 // row-contiguous (nx is a multiple of 4):
-//   mode 0, start of a sweep: D = beta_2 F
-//   mode 1, end of substep s: F += G;  D = alpha_s D + beta F, with beta = beta_{s-1},
-//           and for s = 0 (alpha_0 = 0) beta = beta_2: the next step's first update
+// at the end of substep s, F += G and D = alpha_s D + beta F, with beta = beta_{s-1},
+// and for s = 0 (alpha_0 = 0) beta = beta_2: the next step's first update.
 // Interior layers klo <= k < khi are skipped (the tiled gather updates them).
 template <typename R>
 struct Vec16;
@@ -289,7 +288,7 @@ __device__ __forceinline__ R& vat(V& v, int e) {
 
 template <typename R>
 __global__ void __launch_bounds__(256) adj_update_kernel(Layout L, R* __restrict__ fbar, R* __restrict__ dbar,
-                                                         const R* __restrict__ gbar, R alpha, R beta, int mode,
+                                                         const R* __restrict__ gbar, R alpha, R beta,
                                                          int klo, int khi, const StepState* ss) {
   using V = typename Vec16<R>::T;
   constexpr int E = Vec16<R>::N;
@@ -316,20 +315,14 @@ __global__ void __launch_bounds__(256) adj_update_kernel(Layout L, R* __restrict
     }
     const long long p = L.at(f, k, j, (int)(v * E));
     V fv = *reinterpret_cast<const V*>(fbar + p);
-    V dv;
-    if (mode == 0) {
+    const V gv = *reinterpret_cast<const V*>(gbar + p);
+    V dv = *reinterpret_cast<const V*>(dbar + p);
 #pragma unroll
-      for (int e = 0; e < E; ++e) vat<V, R>(dv, e) = beta * vat<V, R>(fv, e);
-    } else {
-      const V gv = *reinterpret_cast<const V*>(gbar + p);
-      dv = *reinterpret_cast<const V*>(dbar + p);
-#pragma unroll
-      for (int e = 0; e < E; ++e) {
-        vat<V, R>(fv, e) += vat<V, R>(const_cast<V&>(gv), e);
-        vat<V, R>(dv, e) = alpha * vat<V, R>(dv, e) + beta * vat<V, R>(fv, e);
-      }
-      *reinterpret_cast<V*>(fbar + p) = fv;
+    for (int e = 0; e < E; ++e) {
+      vat<V, R>(fv, e) += vat<V, R>(const_cast<V&>(gv), e);
+      vat<V, R>(dv, e) = alpha * vat<V, R>(dv, e) + beta * vat<V, R>(fv, e);
     }
+    *reinterpret_cast<V*>(fbar + p) = fv;
     *reinterpret_cast<V*>(dbar + p) = dv;
   }
 }
@@ -370,54 +363,12 @@ __global__ void bz_plane_kernel(int nx, int ny, int nz, int k, R idx, R idy, con
   }
 }
 
-// adjoint state <-> interior layout (no background: these are adjoints);
-// on the way out the stateful u_x, u_y ghost adjoints are folded onto the
-// photospheric layer (the ghosts are initialised from it)
-template <typename R>
-__global__ void adj_pack_kernel(Layout L, int bcz, const R* __restrict__ fbar, R* __restrict__ out) {
-  const long long n2 = (long long)L.nx * L.ny, n3 = n2 * L.nz;
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n3 * NF;
-       q += (long long)gridDim.x * blockDim.x) {
-    const int fl = (int)(q / n3);
-    const long long r = q - (long long)fl * n3;
-    const int k = (int)(r / n2);
-    const long long rem = r - (long long)k * n2;
-    const int j = (int)(rem / L.nx), i = (int)(rem - (long long)j * L.nx);
-    R v = fbar[L.at(fl, k, j, i)];
-    if (bcz == 0 && k == 0 && (fl == UX || fl == UY))
-      for (int m = 1; m <= NG; ++m) v += fbar[L.at(fl, -m, j, i)];
-    out[q] = v;
-  }
-}
-
-template <typename R>
-__global__ void adj_unpack_kernel(Layout L, const R* __restrict__ in, R* __restrict__ fbar) {
-  const long long n2 = (long long)L.nx * L.ny, n3 = n2 * L.nz;
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n3 * NF;
-       q += (long long)gridDim.x * blockDim.x) {
-    const int fl = (int)(q / n3);
-    const long long r = q - (long long)fl * n3;
-    const int k = (int)(r / n2);
-    const long long rem = r - (long long)k * n2;
-    const int j = (int)(rem / L.nx), i = (int)(rem - (long long)j * L.nx);
-    fbar[L.at(fl, k, j, i)] = in[q];
-  }
-}
-
 template <typename R>
 __global__ void d2r_kernel(const double* __restrict__ in, R* __restrict__ out, long long n) {
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x)
     out[q] = (R)in[q];
 }
 
-template <typename R>
-void launch_adj_pack(const Layout& L, int bcz, const R* fbar, R* out, cudaStream_t st) {
-  adj_pack_kernel<R><<<1216, 256, 0, st>>>(L, bcz, fbar, out);
-}
-template <typename R>
-void launch_adj_unpack(const Layout& L, const R* in, R* fbar, cudaStream_t st) {
-  adj_unpack_kernel<R><<<1216, 256, 0, st>>>(L, in, fbar);
-}
 template <typename R>
 void launch_d2r(const double* in, R* out, long long n, cudaStream_t st) {
   d2r_kernel<R><<<304, 256, 0, st>>>(in, out, n);
@@ -451,9 +402,9 @@ void launch_adj_bc(const Layout& L, const Phys<R>& ph, const Background<R>& bg, 
 }
 
 template <typename R>
-void launch_adj_update(const Layout& L, R* fbar, R* dbar, const R* gbar, double alpha, double beta, int mode,
+void launch_adj_update(const Layout& L, R* fbar, R* dbar, const R* gbar, double alpha, double beta,
                        int klo, int khi, const StepState* ss, cudaStream_t st) {
-  adj_update_kernel<R><<<152 * 8, 256, 0, st>>>(L, fbar, dbar, gbar, (R)alpha, (R)beta, mode, klo, khi, ss);
+  adj_update_kernel<R><<<152 * 8, 256, 0, st>>>(L, fbar, dbar, gbar, (R)alpha, (R)beta, klo, khi, ss);
 }
 
 template <typename R>
@@ -471,12 +422,10 @@ void launch_bz_plane(int nx, int ny, int nz, int k, double dx, double dy, const 
                                      cudaStream_t);                                                               \
   template void launch_adj_bc<R>(const Layout&, const Phys<R>&, const Background<R>&, const R*, R*, R,             \
                                  const StepState*, cudaStream_t);                                                 \
-  template void launch_adj_update<R>(const Layout&, R*, R*, const R*, double, double, int, int, int,              \
+  template void launch_adj_update<R>(const Layout&, R*, R*, const R*, double, double, int, int,              \
                                      const StepState*, cudaStream_t);                                             \
   template void launch_bz_plane<R>(int, int, int, int, double, double, const R*, R*, int, const R*, R*,             \
                                    cudaStream_t);                                                                 \
-  template void launch_adj_pack<R>(const Layout&, int, const R*, R*, cudaStream_t);                                \
-  template void launch_adj_unpack<R>(const Layout&, const R*, R*, cudaStream_t);                                   \
   template void launch_d2r<R>(const double*, R*, long long, cudaStream_t);
 INST(float)
 INST(double)

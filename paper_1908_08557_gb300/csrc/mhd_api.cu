@@ -915,6 +915,10 @@ extern "C" int mhd_create(const mhd_params* p, void* workspace, size_t ws_bytes,
     // zero the driver (no nudging target until mhd_set_driver)
     rc = cuda_check(h, cudaMemsetAsync(h->bz, 0, (size_t)(o.red - o.bz), h->st), "zero driver");
   }
+  if (!rc) {
+    // row padding and alignment gaps of the second state set (mhd_write fills the first)
+    rc = cuda_check(h, cudaMemsetAsync(h->f[1], 0, (size_t)NF * h->L.fs * h->esz, h->st), "zero state set");
+  }
   if (!rc && h->abg_mode) {
     // no background until mhd_set_a_background: every table zero
     rc = cuda_check(h, cudaMemsetAsync(h->ws + o.abB, 0, o.at64 - o.abB, h->st), "zero background tables");
@@ -958,26 +962,22 @@ extern "C" int mhd_write(mhd_handle h, const void* src, int mem) {
   if (mem != MHD_MEM_DEVICE && mem != MHD_MEM_HOST) return fail(h, MHD_ERR_ARG, "bad mem flag");
   const Layout& L = h->L;
   size_t bytes = (size_t)NF * L.nx * L.ny * L.nz * h->esz;
-  int rc = cuda_check(h, cudaMemcpyAsync(h->df, src, bytes, kind_in(mem), h->st), "copy state in");
-  if (rc) return rc;
+  int rc = MHD_OK;
+  if (mem == MHD_MEM_HOST) {
+    // a host array is staged in the accumulator buffer; a device array is
+    // read where it lies
+    rc = cuda_check(h, cudaMemcpyAsync(h->df, src, bytes, cudaMemcpyHostToDevice, h->st), "copy state in");
+    if (rc) return rc;
+    src = h->df;
+  }
   // a state written afresh may be stepped again: clear the halt flag
   rc = cuda_check(h, cudaMemsetAsync(&h->ss->nonfinite, 0, sizeof(int), h->st), "clear status");
   if (rc) return rc;
-  for (int s = 0; s < 2; ++s) {
-    if (h->esz == 8) {
-      double* f = (double*)h->f[s];
-      cudaMemsetAsync(f, 0, (size_t)NF * L.fs * 8, h->st);
-      launch_unpack<double>(L, h->bgd, (const double*)h->df, f, h->st);
-      launch_rims<double>(L, f, 0, L.nz, h->st);
-      if (h->p.bc_z == 0) launch_init_u_ghosts<double>(L, f, h->st);
-    } else {
-      float* f = (float*)h->f[s];
-      cudaMemsetAsync(f, 0, (size_t)NF * L.fs * 4, h->st);
-      launch_unpack<float>(L, h->bgf, (const float*)h->df, f, h->st);
-      launch_rims<float>(L, f, 0, L.nz, h->st);
-      if (h->p.bc_z == 0) launch_init_u_ghosts<float>(L, f, h->st);
-    }
-  }
+  // the other state set needs nothing: a substep writes its interior, images
+  // and u ghost rows, and the ghost rules the rest, before anything reads it
+  const bool ug = h->p.bc_z == 0;
+  if (h->esz == 8) launch_unpack<double>(L, h->bgd, (const double*)src, (double*)h->f[0], ug, h->st);
+  else launch_unpack<float>(L, h->bgf, (const float*)src, (float*)h->f[0], ug, h->st);
   h->cur = 0;
   rc = cuda_check(h, cudaSuccess, "state unpack");
   if (rc) return rc;
@@ -1416,24 +1416,20 @@ extern "C" int mhd_adjoint_init(mhd_handle h, const void* lam, int mem) {
   if (!h || !lam) return fail(h, MHD_ERR_ARG, "NULL argument");
   int rc = adjoint_ready(h);
   if (rc) return rc;
-  const size_t set = (size_t)NF * h->L.fs * h->esz;
   const size_t n2 = (size_t)h->p.nx * h->p.ny;
-  rc = cuda_check(h, cudaMemsetAsync(h->fbar, 0, set, h->st), "zero fbar");
-  if (!rc) rc = cuda_check(h, cudaMemsetAsync(h->dbar, 0, set, h->st), "zero dbar");
-  if (!rc) rc = cuda_check(h, cudaMemsetAsync(h->thbar, 0, 6 * n2 * sizeof(double), h->st), "zero thbar");
-  if (!rc) rc = cuda_check(h, cudaMemcpyAsync(h->gbar, lam, (size_t)NF * h->p.nx * h->p.ny * h->p.nz * h->esz,
-                                              kind_in(mem), h->st), "copy lam");
-  if (rc) return rc;
-  if (h->esz == 8) {
-    launch_adj_unpack<double>(h->L, (const double*)h->gbar, (double*)h->fbar, h->st);
-    launch_adj_update<double>(h->L, (double*)h->fbar, (double*)h->dbar, nullptr, 0.0, rk_beta(2), 0, 0, 0, h->ss,
-                              h->st);
-  } else {
-    launch_adj_unpack<float>(h->L, (const float*)h->gbar, (float*)h->fbar, h->st);
-    launch_adj_update<float>(h->L, (float*)h->fbar, (float*)h->dbar, nullptr, 0.0, rk_beta(2), 0, 0, 0, h->ss,
-                             h->st);
+  rc = cuda_check(h, cudaMemsetAsync(h->thbar, 0, 6 * n2 * sizeof(double), h->st), "zero thbar");
+  if (!rc && mem == MHD_MEM_HOST) {
+    rc = cuda_check(h, cudaMemcpyAsync(h->gbar, lam, (size_t)NF * h->p.nx * h->p.ny * h->p.nz * h->esz,
+                                       cudaMemcpyHostToDevice, h->st), "copy lam");
+    lam = h->gbar;
   }
-  h->nlaunch += 2;
+  if (rc) return rc;
+  // F = lam and D = beta_2 F in one pass
+  if (h->esz == 8)
+    launch_adj_unpack<double>(h->L, (const double*)lam, (double*)h->fbar, (double*)h->dbar, rk_beta(2), h->st);
+  else
+    launch_adj_unpack<float>(h->L, (const float*)lam, (float*)h->fbar, (float*)h->dbar, rk_beta(2), h->st);
+  h->nlaunch += 1;
   rc = cuda_check(h, cudaSuccess, "adjoint init");
   if (!rc && mem == MHD_MEM_HOST) rc = cuda_check(h, cudaStreamSynchronize(h->st), "init synchronize");
   return rc;
@@ -1506,7 +1502,7 @@ static void adjoint_reverse(mhd_ctx* h, R* const (&S)[3], const CUtensorMap* con
       launch_adj_gather<R>(h->L, ph, (const R*)h->coef, (const R*)h->dbar, (R*)h->gbar, h->ss, h->st);
     launch_adj_bc<R>(h->L, ph, bg, S[s], (R*)h->gbar, (R)h->p.dz, h->ss, h->st);
     launch_pfe_adjoint<R>(fpa, h->L, (R*)h->gbar, h->ss, h->st);
-    launch_adj_update<R>(h->L, (R*)h->fbar, (R*)h->dbar, (const R*)h->gbar, alpha, beta, 1, klo, khi, h->ss, h->st);
+    launch_adj_update<R>(h->L, (R*)h->fbar, (R*)h->dbar, (const R*)h->gbar, alpha, beta, klo, khi, h->ss, h->st);
     h->nlaunch += (tg && !h->adj_zm) ? 8 : 7;  // point, [fold], gather, bc, 3 FFT, update
   }
 }
@@ -1636,9 +1632,11 @@ extern "C" int mhd_adjoint_read(mhd_handle h, void* lam, void* grad_bz, void* gr
   // results are staged in the coefficient buffer, then copied out
   char* stage = (char*)h->coef;
   if (lam) {
-    if (h->esz == 8) launch_adj_pack<double>(h->L, h->p.bc_z, (const double*)h->fbar, (double*)stage, h->st);
-    else launch_adj_pack<float>(h->L, h->p.bc_z, (const float*)h->fbar, (float*)stage, h->st);
-    rc = cuda_check(h, cudaMemcpyAsync(lam, stage, n3b, kind_out(mem), h->st), "copy lam");
+    // a device array takes the copy directly, a host array through the stage
+    void* to = mem == MHD_MEM_HOST ? (void*)stage : lam;
+    if (h->esz == 8) launch_adj_pack<double>(h->L, h->p.bc_z, (const double*)h->fbar, (double*)to, h->st);
+    else launch_adj_pack<float>(h->L, h->p.bc_z, (const float*)h->fbar, (float*)to, h->st);
+    if (mem == MHD_MEM_HOST) rc = cuda_check(h, cudaMemcpyAsync(lam, stage, n3b, cudaMemcpyDeviceToHost, h->st), "copy lam");
     if (rc) return rc;
   }
   char* stage2 = stage + (n3b + 255) / 256 * 256;

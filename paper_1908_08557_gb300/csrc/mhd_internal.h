@@ -83,8 +83,6 @@ constexpr int RED_BLOCKS_MAX = 4096;   // partial-reduction slots
 constexpr int CFL_SLOTS = 256;         // CFL maxima slot pairs (after the partials)
 
 // ghost fill
-template <typename R> void launch_rims(const Layout& L, R* f, int k0, int k1, cudaStream_t st);
-template <typename R> void launch_init_u_ghosts(const Layout& L, R* f, cudaStream_t st);
 template <typename R> void launch_bc(const Layout& L, const Phys<R>& ph, const Background<R>& bg, R* f,
                                      R dz, const StepState* ss, cudaStream_t st);
 // potential-field ghosts of A (three FFT kernels)
@@ -171,16 +169,20 @@ template <typename R> void launch_adj_gather_zm(const Layout& L, const Phys<R>& 
                                                 cudaStream_t st);
 template <typename R> void launch_adj_bc(const Layout& L, const Phys<R>& ph, const Background<R>& bg, const R* g,
                                          R* gbar, R dz, const StepState* ss, cudaStream_t st);
-// adjoint elementwise updates (mode 0: D = beta F; mode 1: F += G, D = alpha D + beta F),
+// adjoint elementwise update F += G, D = alpha D + beta F,
 // skipping interior layers klo <= k < khi; nx must be a multiple of 4 and
 // NF * (nz + 6) * ny * nx / 4 < 2^31
 template <typename R> void launch_adj_update(const Layout& L, R* fbar, R* dbar, const R* gbar, double alpha,
-                                             double beta, int mode, int klo, int khi, const StepState* ss,
-                                             cudaStream_t st);
+                                             double beta, int klo, int khi, const StepState* ss, cudaStream_t st);
 template <typename R> void launch_bz_plane(int nx, int ny, int nz, int k, double dx, double dy, const R* st_in,
                                            R* out, int adjoint, const R* bbar, R* lam, cudaStream_t st);
+// adjoint state <-> interior layout (no background: these are adjoints); on
+// the way out the stateful u_x, u_y ghost adjoints are folded onto the
+// photospheric layer (the ghosts start as copies of it); on the way in every
+// cell of F and of D = beta F is written, zero outside the interior
 template <typename R> void launch_adj_pack(const Layout& L, int bcz, const R* fbar, R* out, cudaStream_t st);
-template <typename R> void launch_adj_unpack(const Layout& L, const R* in, R* fbar, cudaStream_t st);
+template <typename R> void launch_adj_unpack(const Layout& L, const R* in, R* fbar, R* dbar, double beta,
+                                             cudaStream_t st);
 template <typename R> void launch_d2r(const double* in, R* out, long long n, cudaStream_t st);
 template <typename R> void launch_pfe_adjoint(const FFTPlan& fp_adj, const Layout& L, R* gbar, const StepState* ss,
                                               cudaStream_t st);
@@ -243,7 +245,9 @@ void launch_stats_finalize(const double* partial, int nblk, StepState* ss, doubl
 // (the background is added on the way out and removed on the way in)
 template <typename R> void launch_pack(const Layout& L, const Background<R>& bg, const R* f, R* out, int field,
                                        cudaStream_t st);
-template <typename R> void launch_unpack(const Layout& L, const Background<R>& bg, const R* in, R* f,
+// (the whole padded set is written: interior, x,y images, and with ughost the
+// u_x, u_y layers below the photosphere as copies of it; zero elsewhere)
+template <typename R> void launch_unpack(const Layout& L, const Background<R>& bg, const R* in, R* f, bool ughost,
                                          cudaStream_t st);
 // padded copy with the background added (diagnostics)
 template <typename R> void launch_pack_padded(const Layout& L, const Background<R>& bg, const R* f, R* out,
