@@ -114,12 +114,15 @@ __device__ __forceinline__ FItems make_items(int tid) {
 
 // z-chunking of a persistent grid of `ctas` CTAs over tiles: balance whole
 // waves against the six extra planes each chunk loads before its first
-// centre plane; returns the chunk length
+// centre plane; returns the chunk length.  Chunks go down to one layer: where
+// the tiles are few, the layers of a chunk are a serial chain (about 1.7 us a
+// centre plane) and most SMs would idle (64^3, chunks of 16 -> 4 layers: ten
+// steps 2.88 -> 2.35 ms; 32^3, 16 -> 2: 2.81 -> 2.03 ms); where they are many
+// the whole-wave term keeps the chunks long.
 inline int zchunk(int nz, int tiles, int ctas) {
   int best = 1;
   double best_eff = 0.0;
-  const int maxch = nz / 16 > 1 ? nz / 16 : 1;
-  for (int nch = 1; nch <= maxch; ++nch) {
+  for (int nch = 1; nch <= nz; ++nch) {
     const int kc = (nz + nch - 1) / nch;
     const int nc = (nz + kc - 1) / kc;
     const long long items = (long long)tiles * nc;
