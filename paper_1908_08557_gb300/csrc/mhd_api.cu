@@ -504,7 +504,7 @@ static void ghost_fill(mhd_ctx* h, R* f) {
   Phys<R> ph = make_phys<R>(&h->p);
   {
     ClassTimer ct(h, MHD_KC_GHOST, 1);
-    launch_bc<R>(h->L, ph, bgr<R>(h), f, (R)h->p.dz, h->ss, h->st);
+    launch_bc<R>(h->L, ph, bgr<R>(h), f, h->ss, h->st);
   }
   if (h->p.bc_z == 0) {
     ClassTimer ct(h, MHD_KC_PFE, 3);
@@ -638,7 +638,7 @@ static void run_step(mhd_ctx* h, bool stats) {
       cudaEventRecord(h->evj, h->side);
       {
         ClassTimer ct(h, MHD_KC_GHOST, 1);
-        launch_bc<R>(h->L, ph, bgr<R>(h), fin, (R)h->p.dz, h->ss, h->st);
+        launch_bc<R>(h->L, ph, bgr<R>(h), fin, h->ss, h->st);
       }
       {
         ClassTimer ct(h, MHD_KC_CFL, 1);

@@ -405,24 +405,35 @@ static void set_smem_once() {
 // pairs per block (ppb) so there are enough blocks for every SM; shared
 // memory sized to the batch
 struct FFTLaunch {
-  int nb, ppb, lg;                          // lg: ghost layers per inverse batch in cols
-  size_t smem_rows, smem_cols, smem_cols3;  // cols: one output layer, three
+  int ppb, lg;                   // lg: ghost layers per inverse batch in cols
+  int threads, threads3;         // cols: one output layer, three
+  size_t smem_cols, smem_cols3;
 };
 
-static FFTLaunch fft_launch(const FFTPlan& fp) {
+// one thread per radix-4 butterfly of a stage of `lines` lines of n points
+static int butterfly_threads(int lines, int n) {
+  const int t = (lines * n / 4 + 31) / 32 * 32;
+  return t < 32 ? 32 : (t > 256 ? 256 : t);
+}
+
+static FFTLaunch fft_launch(const FFTPlan& fp, int planes) {
   FFTLaunch l;
-  l.nb = 1024 / fp.nx;
-  if (l.nb < 1) l.nb = 1;
-  if (l.nb > fp.ny) l.nb = fp.ny;
+  // column pairs per block: up to 256 points, but no more than leaves two
+  // blocks for every SM (the FP64 pipes of idle SMs are lost: 64 x 64 planes
+  // with four pairs a block ran on 9 SMs, 22 us a launch)
+  const int npairs = fp.nx / 2 + 1;
   l.ppb = 256 / fp.ny;
+  const int spread = npairs * planes / (2 * sm_count());
+  if (l.ppb > spread) l.ppb = spread;
   if (l.ppb < 1) l.ppb = 1;
-  l.smem_rows = (size_t)2 * l.nb * fp.nx * sizeof(double2);
   l.smem_cols = (size_t)3 * 2 * l.ppb * fp.ny * sizeof(double2);  // also cols_adj_kernel
   // the three ghost layers in one batch while that keeps two column blocks
   // per SM (at most 96 KB), one at a time otherwise (at 1024^2 the batched
   // form, 192 KB and one block per SM, measured 8 % slower)
   l.lg = (size_t)6 * 2 * l.ppb * fp.ny * sizeof(double2) <= (size_t)96 * 1024 ? 3 : 1;
   l.smem_cols3 = (size_t)(l.lg == 3 ? 6 : 3) * 2 * l.ppb * fp.ny * sizeof(double2);
+  l.threads = butterfly_threads(2 * l.ppb, fp.ny);
+  l.threads3 = butterfly_threads(2 * l.ppb * l.lg, fp.ny);
   return l;
 }
 
@@ -462,13 +473,16 @@ template <typename R>
 void launch_pfe(const FFTPlan& fp, const Layout& L, R* f, const StepState* ss, cudaStream_t st,
                 const PlaneStreams* ps) {
   set_smem_once();
-  const FFTLaunch l = fft_launch(fp);
   const int npairs = fp.nx / 2 + 1;
-  if (!ps) {
+  const FFTLaunch l = fft_launch(fp, 3);
+  // small planes are bound by launches and latency, not by the FP64 pipe: the
+  // three planes go as one chain (64 x 64, ten steps: 2.06 -> 1.95 ms; at
+  // 128 x 128 three chains are 2 % faster, at 256 x 256 5 %)
+  if (!ps || fp.nx * fp.ny <= 8192) {
     const RowsCfg rf = rows_cfg(fp, 3), ri = rows_cfg(fp, 9);
     rows_fwd_kernel<R><<<dim3(fp.ny / rf.nb, 3), rf.threads, rf.smem, st>>>(fp, L, f, nullptr, 0, ss, rf.nb,
                                                                             nullptr, nullptr);
-    cols_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 3), 256, l.smem_cols3, st>>>(fp, 0, ss, l.ppb, l.lg);
+    cols_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 3), l.threads3, l.smem_cols3, st>>>(fp, 0, ss, l.ppb, l.lg);
     rows_inv_kernel<R><<<dim3(fp.ny / ri.nb, 3, 3), ri.threads, ri.smem, st>>>(fp, L, f, nullptr, nullptr, 0, ss,
                                                                               ri.nb);
     return;
@@ -485,7 +499,7 @@ void launch_pfe(const FFTPlan& fp, const Layout& L, R* f, const StepState* ss, c
     fq.p0 = p;
     rows_fwd_kernel<R><<<dim3(fp.ny / rf.nb, 1), rf.threads, rf.smem, sp>>>(fq, L, f, nullptr, 0, ss, rf.nb,
                                                                             nullptr, nullptr);
-    cols_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 1), 256, l.smem_cols3, sp>>>(fq, 0, ss, l.ppb, l.lg);
+    cols_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 1), l.threads3, l.smem_cols3, sp>>>(fq, 0, ss, l.ppb, l.lg);
     rows_inv_kernel<R><<<dim3(fp.ny / ri.nb, 1, 3), ri.threads, ri.smem, sp>>>(fq, L, f, nullptr, nullptr, 0, ss,
                                                                               ri.nb);
   }
@@ -499,12 +513,12 @@ template <typename R>
 void launch_atarget(const FFTPlan& fp, const R* bz, R* axt, R* ayt, cudaStream_t st) {
   set_smem_once();
   Layout L{};
-  const FFTLaunch l = fft_launch(fp);
+  const FFTLaunch l = fft_launch(fp, 1);
   const int npairs = fp.nx / 2 + 1;
   const RowsCfg r1 = rows_cfg(fp, 1);
   rows_fwd_kernel<R><<<dim3(fp.ny / r1.nb, 1), r1.threads, r1.smem, st>>>(fp, L, nullptr, bz, 1, nullptr, r1.nb,
                                                                           nullptr, nullptr);
-  cols_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 1), 256, l.smem_cols, st>>>(fp, 1, nullptr, l.ppb, 1);
+  cols_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 1), l.threads, l.smem_cols, st>>>(fp, 1, nullptr, l.ppb, 1);
   rows_inv_kernel<R><<<dim3(fp.ny / r1.nb, 1, 1), r1.threads, r1.smem, st>>>(fp, L, nullptr, axt, ayt, 1, nullptr,
                                                                              r1.nb);
 }
@@ -513,12 +527,12 @@ void launch_rotational(const FFTPlan& fp, const double* vx, const double* vy, do
                        cudaStream_t st) {
   set_smem_once();
   Layout L{};
-  const FFTLaunch l = fft_launch(fp);
+  const FFTLaunch l = fft_launch(fp, 1);
   const int npairs = fp.nx / 2 + 1;
   const RowsCfg r1 = rows_cfg(fp, 1);
   rows_fwd_kernel<double><<<dim3(fp.ny / r1.nb, 1), r1.threads, r1.smem, st>>>(fp, L, nullptr, nullptr, 3, nullptr,
                                                                                r1.nb, vx, vy);
-  cols_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 1), 256, l.smem_cols, st>>>(fp, 4, nullptr, l.ppb, 1);
+  cols_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 1), l.threads, l.smem_cols, st>>>(fp, 4, nullptr, l.ppb, 1);
   rows_inv_kernel<double><<<dim3(fp.ny / r1.nb, 1, 1), r1.threads, r1.smem, st>>>(fp, L, nullptr, rx, ry, 1,
                                                                                  nullptr, r1.nb);
 }
@@ -530,12 +544,12 @@ void launch_rotational(const FFTPlan& fp, const double* vx, const double* vy, do
 template <typename R>
 void launch_pfe_adjoint(const FFTPlan& fp_adj, const Layout& L, R* gbar, const StepState* ss, cudaStream_t st) {
   set_smem_once();
-  const FFTLaunch l = fft_launch(fp_adj);
+  const FFTLaunch l = fft_launch(fp_adj, 3);
   const int npairs = fp_adj.nx / 2 + 1;
   const RowsCfg r9 = rows_cfg(fp_adj, 9), r3 = rows_cfg(fp_adj, 3);
   rows_fwd_kernel<R><<<dim3(fp_adj.ny / r9.nb, 9), r9.threads, r9.smem, st>>>(fp_adj, L, gbar, nullptr, 2, ss, r9.nb,
                                                                               nullptr, nullptr);
-  cols_adj_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 3), 256, l.smem_cols, st>>>(fp_adj, ss, l.ppb);
+  cols_adj_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 3), l.threads, l.smem_cols, st>>>(fp_adj, ss, l.ppb);
   rows_inv_kernel<R><<<dim3(fp_adj.ny / r3.nb, 3, 1), r3.threads, r3.smem, st>>>(fp_adj, L, gbar, nullptr, nullptr, 2,
                                                                                 ss, r3.nb);
 }
@@ -546,13 +560,14 @@ template <typename R>
 void launch_atarget_adjoint(const FFTPlan& fp, const double* abx, const double* aby, R* out, cudaStream_t st) {
   set_smem_once();
   Layout L{};
-  const FFTLaunch l = fft_launch(fp);
+  const FFTLaunch l = fft_launch(fp, 1);
   const int npairs = fp.nx / 2 + 1;
-  rows_fwd_kernel<R><<<dim3(fp.ny / l.nb, 1), 256, l.smem_rows, st>>>(fp, L, nullptr, nullptr, 3, nullptr, l.nb, abx,
-                                                                       aby);
-  cols_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 1), 256, l.smem_cols, st>>>(fp, 2, nullptr, l.ppb, 1);
-  rows_inv_kernel<R><<<dim3(fp.ny / l.nb, 1, 1), 256, l.smem_rows, st>>>(fp, L, nullptr, out, nullptr, 3, nullptr,
-                                                                          l.nb);
+  const RowsCfg r1 = rows_cfg(fp, 1);
+  rows_fwd_kernel<R><<<dim3(fp.ny / r1.nb, 1), r1.threads, r1.smem, st>>>(fp, L, nullptr, nullptr, 3, nullptr, r1.nb,
+                                                                          abx, aby);
+  cols_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 1), l.threads, l.smem_cols, st>>>(fp, 2, nullptr, l.ppb, 1);
+  rows_inv_kernel<R><<<dim3(fp.ny / r1.nb, 1, 1), r1.threads, r1.smem, st>>>(fp, L, nullptr, out, nullptr, 3, nullptr,
+                                                                             r1.nb);
 }
 
 template void launch_pfe_adjoint<float>(const FFTPlan&, const Layout&, float*, const StepState*, cudaStream_t);

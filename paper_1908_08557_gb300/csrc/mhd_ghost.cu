@@ -20,54 +20,73 @@ namespace mhd {
 // background differences enter through the constants cb, ctT, ctL (FP64 on
 // the host), and the background ghost values of ln rho equal the fixed
 // profile, so their perturbation is zero.
+//
+// Bound by latency: each column is a chain of exponentials and divisions (in
+// FP64 some hundred dependent operations), and there are few columns.  The
+// two ends are separate threads and blocks hold 64 of them, so that the
+// chains run side by side over all SMs (32^2 columns in FP64: blocks of 256
+// threads with both ends in a thread took 19 us on 6 SMs).
+constexpr int BC_TH = 64;
 template <typename R>
-__global__ void bc_kernel(Layout L, Phys<R> ph, Background<R> bg, R* __restrict__ f, R dz,
-                          const StepState* ss) {
+__global__ void __launch_bounds__(BC_TH) bc_kernel(Layout L, Phys<R> ph, Background<R> bg, R* __restrict__ f,
+                                                   const StepState* ss) {
   const int pw = L.nx + 2 * NG, phh = L.ny + 2 * NG;
-  int q = blockIdx.x * blockDim.x + threadIdx.x;
+  const int q = blockIdx.x * BC_TH + threadIdx.x;
   if (q >= pw * phh) return;
   if (halted(ss)) return;
   const int i = q % pw - NG, j = q / pw - NG;
   const int nz = L.nz, kt = nz - 1;
+  const bool top = blockIdx.y != 0;
   if (ph.bcz == 1) {
     for (int fl = 0; fl < NF; ++fl)
       for (int m = 1; m <= NG; ++m) {
-        f[L.at(fl, -m, j, i)] = f[L.at(fl, nz - m, j, i)];
-        f[L.at(fl, kt + m, j, i)] = f[L.at(fl, m - 1, j, i)];
+        if (!top) f[L.at(fl, -m, j, i)] = f[L.at(fl, nz - m, j, i)];
+        else f[L.at(fl, kt + m, j, i)] = f[L.at(fl, m - 1, j, i)];
       }
     return;
   }
-  // bottom
   // (layer distances from the vertical grid: bg.dzb[m] = z_{1-m} - z_{-m},
   // bg.dzt[m] = z_{nz-1+m} - z_{nz-1-m}; dz and 2 m dz on the uniform grid)
-  R th1 = f[L.at(LT, 0, j, i)];
-  R l1 = f[L.at(LR, 0, j, i)];
-  for (int m = 1; m <= NG; ++m) {
-    const R T1 = rexp<R>(bg.tbar[NG - m + 1] + th1);
-    const R l0 = R(0);
-    const R th0 = th1 + l1 - l0 + bg.cb[m] - bg.dzb[m] * ph.gz / T1;
-    f[L.at(LR, -m, j, i)] = l0;
-    f[L.at(LT, -m, j, i)] = th0;
-    f[L.at(UZ, -m, j, i)] = -f[L.at(UZ, m, j, i)];
-    th1 = th0;
-    l1 = l0;
+  if (!top) {
+    R th1 = f[L.at(LT, 0, j, i)];
+    R l1 = f[L.at(LR, 0, j, i)];
+    R uz[NG];
+#pragma unroll
+    for (int m = 1; m <= NG; ++m) uz[m - 1] = f[L.at(UZ, m, j, i)];
+#pragma unroll
+    for (int m = 1; m <= NG; ++m) {
+      const R T1 = rexp<R>(bg.tbar[NG - m + 1] + th1);
+      const R l0 = R(0);
+      const R th0 = th1 + l1 - l0 + bg.cb[m] - bg.dzb[m] * ph.gz / T1;
+      f[L.at(LR, -m, j, i)] = l0;
+      f[L.at(LT, -m, j, i)] = th0;
+      f[L.at(UZ, -m, j, i)] = -uz[m - 1];
+      th1 = th0;
+      l1 = l0;
+    }
+    return;
   }
-  // top
+  R v[NG][5];
+#pragma unroll
+  for (int m = 1; m <= NG; ++m)
+#pragma unroll
+    for (int c = 0; c < 5; ++c) v[m - 1][c] = f[L.at(UX + c, kt - m, j, i)];
   const R Ttop = rexp<R>(bg.tbar[NG + kt] + f[L.at(LT, kt, j, i)]);
+#pragma unroll
   for (int m = 1; m <= NG; ++m) {
-    f[L.at(LT, kt + m, j, i)] = f[L.at(LT, kt - m, j, i)] + bg.ctT[m];
-    f[L.at(LR, kt + m, j, i)] = f[L.at(LR, kt - m, j, i)] + bg.ctL[m] + bg.dzt[m] * ph.gz / Ttop;
-    f[L.at(UZ, kt + m, j, i)] = -f[L.at(UZ, kt - m, j, i)];
-    f[L.at(UX, kt + m, j, i)] = f[L.at(UX, kt - m, j, i)];
-    f[L.at(UY, kt + m, j, i)] = f[L.at(UY, kt - m, j, i)];
+    f[L.at(LT, kt + m, j, i)] = v[m - 1][LT - UX] + bg.ctT[m];
+    f[L.at(LR, kt + m, j, i)] = v[m - 1][LR - UX] + bg.ctL[m] + bg.dzt[m] * ph.gz / Ttop;
+    f[L.at(UZ, kt + m, j, i)] = -v[m - 1][UZ - UX];
+    f[L.at(UX, kt + m, j, i)] = v[m - 1][0];
+    f[L.at(UY, kt + m, j, i)] = v[m - 1][1];
   }
 }
 
 template <typename R>
-void launch_bc(const Layout& L, const Phys<R>& ph, const Background<R>& bg, R* f, R dz, const StepState* ss,
+void launch_bc(const Layout& L, const Phys<R>& ph, const Background<R>& bg, R* f, const StepState* ss,
                cudaStream_t st) {
   int n = (L.nx + 2 * NG) * (L.ny + 2 * NG);
-  bc_kernel<R><<<(n + 255) / 256, 256, 0, st>>>(L, ph, bg, f, dz, ss);
+  bc_kernel<R><<<dim3((n + BC_TH - 1) / BC_TH, 2), BC_TH, 0, st>>>(L, ph, bg, f, ss);
 }
 
 // interior [field][nz][ny][nx] <-> padded; the background is added on the
@@ -333,7 +352,7 @@ void launch_layer_mean(const Layout& L, const R* in, int field, double* out, cud
 }
 
 #define INST(R)                                                                               \
-  template void launch_bc<R>(const Layout&, const Phys<R>&, const Background<R>&, R*, R,       \
+  template void launch_bc<R>(const Layout&, const Phys<R>&, const Background<R>&, R*,          \
                              const StepState*, cudaStream_t);                                  \
   template void launch_pack<R>(const Layout&, const Background<R>&, const R*, R*, int, cudaStream_t); \
   template void launch_adj_pack<R>(const Layout&, int, const R*, R*, cudaStream_t);           \

@@ -84,7 +84,7 @@ constexpr int CFL_SLOTS = 256;         // CFL maxima slot pairs (after the parti
 
 // ghost fill
 template <typename R> void launch_bc(const Layout& L, const Phys<R>& ph, const Background<R>& bg, R* f,
-                                     R dz, const StepState* ss, cudaStream_t st);
+                                     const StepState* ss, cudaStream_t st);
 // potential-field ghosts of A (three FFT kernels)
 // (ps: run the three planes on three streams; nullptr: one stream)
 template <typename R> void launch_pfe(const FFTPlan& fp, const Layout& L, R* f, const StepState* ss,
