@@ -1,51 +1,58 @@
 // mhd_rk64.cu -- FP64 right-hand side + RK3 update, and the FP64 pointwise
-// adjoint, as a z-march that forms every first derivative once.
+// adjoint, forming every first derivative once.
 //
 // What bounds it: the FP64 pipe.  An SM retires two FP64 operations per clock
-// (one warp instruction every 16 clocks) while its four schedulers could issue
-// 64 other instructions in that time, so loads, index arithmetic and shared
-// memory are nearly free and only the count of FP64 operations matters.  The
+// (a warp instruction holds its scheduler's share of the pipe for 64 clocks),
+// so loads, index arithmetic and shared memory are nearly free and only the
+// count of FP64 operations matters, and how evenly they lie on the SMs.  The
 // mixed derivatives D1_a D1_b dominate a cell-by-cell evaluation: as product
 // stencils they cost 36 operations each, twelve of them 432 of 1022 per cell.
 // Here a mixed derivative is one more first difference (5 operations) of a
 // first difference that some cell has already taken:
-//  - z mixed: thread (i, j) marches in z and keeps, in shared memory, the x and
-//    y differences of its own column that the grad-div terms need (six sources
-//    of A and u, a ring of six planes; the plane three above the centre is
-//    formed once, as the march reaches it);
-//  - xy mixed: the y differences of A_x, A_y, u_x, u_y of the tile's rows with
-//    an x halo pass through a shared scratch.
+//  - z mixed: the x and y differences that the grad-div terms need (six sources
+//    of A and u) are formed by each cell for its own plane and handed along z
+//    through shared memory; the three planes at each end of the block's layers
+//    are formed once per block;
+//  - xy mixed: the y differences of A_x, A_y, u_x, u_y of the row with an x halo
+//    pass through a scratch of the warp.
 // Weights: the differences are taken in units of their smallest weight,
 //   d f  = (f_3 - f_-3) - 9 (f_2 - f_-2) + 45 (f_1 - f_-1)       (D1 = d / 60 h)
 //   dd f = (f_3 + f_-3) - 13.5 (f_2 + f_-2) + 135 (f_1 + f_-1) - 245 f
 //                                                                (D2 = dd / 90 h^2)
 // which saves a multiplication per difference; the scales enter the
-// multiply-adds that consume them.  About 500 operations per cell in all.
+// multiply-adds that consume them.  About 510 operations per cell in all.
 //
-// Tile 32 x 4 of 128 threads (45 doubles of shared memory per thread for the
-// rings, four CTAs per SM): x rows are whole sectors; four rows, not eight, so
-// that small boxes spread over more SMs.  The z chunk is chosen by zchunk64.
-// The neighbours' values come through L1 from the padded state.
+// A block is one row of 32 cells over KZ = 8 layers, a warp per layer: a single
+// barrier, and work in pieces small enough to spread over the SMs (a z-march
+// of the same arithmetic, a ring of sources per column, leaves one warp per
+// scheduler in small boxes, where dependent FP64 operations take 114 clocks
+// each instead of 64).  Neighbours come through L1 from the padded state.
 //
-// Measured (256^3, one substep): 33.1 ms with one thread per cell and product
-// stencils, see the table of kernels for this form.
 #include "mhd_adjoint_point.cuh"
 #include "mhd_internal.h"
 
 namespace mhd {
 namespace r64 {
 
-constexpr int TX = 32, TY = 4, NT = TX * TY;
+constexpr int TX = 32, KZ = 8, NT = TX * KZ;
 constexpr int NSRC = 6;          // z-mixed sources: dxAz, dyAz, div_h A, dxUz, dyUz, div_h u
-constexpr int NAUX = 3;          // also kept from the front to the centre: dyAy, D1x u_x, D1y u_y
-constexpr int RS = 6, RA = 3;    // ring depths in planes
+constexpr int NAUX = 3;          // kept by the cell itself: dyAy, D1x u_x, D1y u_y
 constexpr int SW = TX + 8;       // scratch row: x0 - 3 .. x0 + TX + 2, padded
 constexpr int NSC = 4;           // scratch fields: dy of A_y, A_x, u_y, u_x
-constexpr int SMEM_D = (RS * NSRC + RA * NAUX) * NT + NSC * TY * SW;
-constexpr size_t SMEM = sizeof(double) * SMEM_D;
+
+// Products of the scheme constants, formed on the host: a uniform product
+// costs every thread an FP64 operation as any other does.  c*: D1 scales
+// 1 / 60 h and their products, e*: D2 scales 1 / 90 h^2, v*: times nu (1, 1/3
+// or 4/3 of it); the z entries are replaced per layer on a non-uniform grid.
+struct Coef64 {
+  double cx, cy, cz, cxy, cxz, cyz, ex, ey, ez;
+  double v1ex, v1ey, v1ez, v4ex, v4ey, v4ez, v3cx, v3cxy, v3cxz, v3cyz, v3cz;
+  double heat, visc, cond;  // (gamma - 1) eta, (gamma - 1) nu, (gamma - 1) kappa0
+};
 
 struct Args {
   Layout L;
+  Coef64 c;
   Phys<double> ph;
   Background<double> bg;
   const double* fin;
@@ -59,7 +66,6 @@ struct Args {
   const double* v1;
   const StepState* ss;
   int sub;
-  int kchunk;
   // adjoint mode
   const double* dbar;
   double* coef;
@@ -107,29 +113,23 @@ __device__ __forceinline__ void put_images(const Layout& L, double* __restrict__
 }
 
 // ADJ = false: right-hand side + RK update of substep `sub` (sub < 0: the
-// right-hand side alone into df); ADJ = true: the pointwise adjoint.
-template <bool ADJ>
-__global__ void __launch_bounds__(NT, 4) rk64_kernel(const __grid_constant__ Args a) {
-  extern __shared__ double sm[];
+// right-hand side alone into df); ADJ = true: the pointwise adjoint.  ZG: a
+// non-uniform vertical grid, D_z f = m1 D_xi f, D_z^2 f = m1^2 D_xi^2 f + r21 D_z f.
+template <bool ADJ, bool ZG>
+__global__ void __launch_bounds__(NT, 2) rk64_kernel(const __grid_constant__ Args a) {
+  __shared__ double src[KZ + 2 * NG][NSRC][TX];
+  __shared__ double scr_all[KZ][NSC][SW];
   if (halted(a.ss)) return;
   const Layout& L = a.L;
   const Phys<double>& ph = a.ph;
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
-  double* ring = sm + tid;                       // [slot * NSRC + q] * NT
-  double* aux = sm + RS * NSRC * NT + tid;       // [slot * NAUX + q] * NT
-  double* scr = sm + (RS * NSRC + RA * NAUX) * NT;
-  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-  const int i = x0 + tx, j = y0 + ty;
-  const int k0 = blockIdx.z * a.kchunk, k1 = min(L.nz, k0 + a.kchunk);
-  const bool row = j < L.ny;
-  const bool live = row && i < L.nx;
-  const bool near = row && i < L.nx + NG;        // its y differences are read by live threads
+  const int tx = threadIdx.x, w_ = threadIdx.y;
+  const int x0 = blockIdx.x * TX;
+  const int i = x0 + tx, j = blockIdx.y, k0 = blockIdx.z * KZ, k = k0 + w_;
+  const bool live = i < L.nx && k < L.nz;
+  const bool near = i < L.nx + NG && k < L.nz;  // its y differences are read by live threads
   const int sy = L.mx, sz = L.mx * L.my;
   const long long fs = L.fs;
-  // a non-uniform vertical grid: D_z f = m1 D_xi f, D_z^2 f = m1^2 D_xi^2 f + r21 D_z f
-  const bool zg = a.bg.zm1 != nullptr;
-  const double cx = ph.idx * (1.0 / 60.0), cy = ph.idy * (1.0 / 60.0);
-  const double ex = ph.idx2 * (1.0 / 90.0), ey = ph.idy2 * (1.0 / 90.0);
+  const Coef64& C = a.c;
 
   const int sub = a.sub;
   const bool eval = sub < 0;
@@ -137,90 +137,76 @@ __global__ void __launch_bounds__(NT, 4) rk64_kernel(const __grid_constant__ Arg
   const double alpha = eval ? 0.0 : rk_alpha(sub);
   const double beta = eval ? 0.0 : rk_beta(sub);
 
-  // scratch halo item of this thread: field hf, row hr, column hc (x0 + hc)
-  const bool hal = tid < NSC * TY * 2 * NG;
-  const int hf = tid / (TY * 2 * NG), hr = (tid / (2 * NG)) % TY, hq = tid % (2 * NG);
-  const int hc = hq < NG ? hq - NG : TX + hq - NG;
-  const bool hlive = hal && y0 + hr < L.ny && x0 + hc < L.nx + NG;
-  const int hfield = hf == 0 ? AY : (hf == 1 ? AX : (hf == 2 ? UY : UX));
-  double* hdst = scr + (hf * TY + hr) * SW + hc + NG;
-
   // sources of plane p at this column, into n (z-mixed) and e (kept for the centre)
   auto front = [&](int p, double (&n)[NSRC], double (&e)[NAUX]) {
     const double* q = a.fin + L.at(0, p, j, i);
     n[0] = dd1(q + AZ * fs, 1);
     n[1] = dd1(q + AZ * fs, sy);
     e[0] = dd1(q + AY * fs, sy);
-    n[2] = fma(cx, dd1(q + AX * fs, 1), cy * e[0]);
+    n[2] = fma(C.cx, dd1(q + AX * fs, 1), C.cy * e[0]);
     n[3] = dd1(q + UZ * fs, 1);
     n[4] = dd1(q + UZ * fs, sy);
-    e[1] = cx * dd1(q + UX * fs, 1);
-    e[2] = cy * dd1(q + UY * fs, sy);
+    e[1] = C.cx * dd1(q + UX * fs, 1);
+    e[2] = C.cy * dd1(q + UY * fs, sy);
     n[5] = e[1] + e[2];
   };
-  auto slot = [](int p, int m) { const int r = p % m; return r < 0 ? r + m : r; };
-
-  if (live) {
-    for (int p = k0 - NG; p < k0 + NG; ++p) {
+  const long long n2 = (long long)L.nx * L.ny, n3 = n2 * L.nz;
+  double cur[NSRC], ax_[NAUX];
+  if (i < L.nx) {
+    // this layer's sources (a layer above the top is a neighbour's source
+    // only), and one of the six planes beyond the block's layers per warp
+    if (k < L.nz + NG) {
+      front(k, cur, ax_);
+#pragma unroll
+      for (int q = 0; q < NSRC; ++q) src[w_ + NG][q][tx] = cur[q];
+    }
+    const int ps = w_ < NG ? w_ : KZ + w_;  // slot of the extra plane (w_ < 2 NG)
+    if (w_ < 2 * NG && k0 - NG + ps < L.nz + NG) {
       double n[NSRC], e[NAUX];
-      front(p, n, e);
-      const int s = slot(p, RS), s3 = slot(p, RA);
+      front(k0 - NG + ps, n, e);
 #pragma unroll
-      for (int q = 0; q < NSRC; ++q) ring[(s * NSRC + q) * NT] = n[q];
-      if (p >= k0) {
-#pragma unroll
-        for (int q = 0; q < NAUX; ++q) aux[(s3 * NAUX + q) * NT] = e[q];
-      }
+      for (int q = 0; q < NSRC; ++q) src[ps][q][tx] = n[q];
     }
   }
-  const long long n2 = (long long)L.nx * L.ny, n3 = n2 * L.nz;
-  for (int k = k0; k < k1; ++k) {
+  {
     const double* f = a.fin + L.at(0, k, j, i);
-    double mz[NSRC], cur[NSRC], ax_[NAUX];
-    if (live) {
-      double n[NSRC], e[NAUX];
-      front(k + NG, n, e);
-      const int s0 = slot(k, RS), s1 = slot(k + 1, RS), s2 = slot(k + 2, RS), s3 = slot(k + 3, RS),
-                t2 = slot(k - 2, RS), t1 = slot(k - 1, RS), s = slot(k, RA);
-#pragma unroll
-      for (int q = 0; q < NSRC; ++q) {
-        mz[q] = comb1(ring[(s1 * NSRC + q) * NT], ring[(t1 * NSRC + q) * NT], ring[(s2 * NSRC + q) * NT],
-                      ring[(t2 * NSRC + q) * NT], n[q], ring[(s3 * NSRC + q) * NT]);
-        cur[q] = ring[(s0 * NSRC + q) * NT];
-        ring[(s3 * NSRC + q) * NT] = n[q];
-      }
-#pragma unroll
-      for (int q = 0; q < NAUX; ++q) {
-        ax_[q] = aux[(s * NAUX + q) * NT];
-        aux[(s * NAUX + q) * NT] = e[q];
-      }
-    }
-    // y differences of A_y, A_x, u_y, u_x of the rows, with the x halo
+    double* scr = &scr_all[w_][0][0];
+    // y differences of A_y, A_x, u_y, u_x of the row, with the x halo
     double dyAx = 0.0, yyAx = 0.0, dyUx = 0.0, yyUx = 0.0;
     if (near) {
       const double ca = __ldg(f + AX * fs), cu = __ldg(f + UX * fs);
       dyAx = dd12(f + AX * fs, sy, ca, yyAx);
       dyUx = dd12(f + UX * fs, sy, cu, yyUx);
-      double* sc = scr + ty * SW + tx + NG;
-      sc[1 * TY * SW] = dyAx;
-      sc[3 * TY * SW] = dyUx;
-      if (live) {
-        sc[0] = ax_[0];
-        sc[2 * TY * SW] = ax_[2];
-      } else {
-        sc[0] = dd1(f + AY * fs, sy);
-        sc[2 * TY * SW] = cy * dd1(f + UY * fs, sy);
-      }
+      double* sc = scr + tx + NG;
+      sc[1 * SW] = dyAx;
+      sc[3 * SW] = dyUx;
+      sc[0] = live ? ax_[0] : dd1(f + AY * fs, sy);
+      sc[2 * SW] = live ? ax_[2] : C.cy * dd1(f + UY * fs, sy);
     }
-    if (hlive) {
-      const double v = dd1(a.fin + L.at(hfield, k, y0 + hr, x0 + hc), sy);
-      *hdst = hf == 2 ? cy * v : v;
+    if (tx < NSC * 2 * NG && k < L.nz) {
+      const int hf = tx / (2 * NG), hq = tx - hf * 2 * NG, hc = hq < NG ? hq - NG : TX + hq - NG;
+      if (x0 + hc < L.nx + NG) {
+        const int fld = hf == 0 ? AY : (hf == 1 ? AX : (hf == 2 ? UY : UX));
+        const double v = dd1(a.fin + L.at(fld, k, j, x0 + hc), sy);
+        scr[hf * SW + hc + NG] = hf == 2 ? C.cy * v : v;
+      }
     }
     __syncthreads();
     if (live) {
-      const double* sc = scr + ty * SW + tx + NG;
-      const double m1 = zg ? a.bg.zm1[k] : ph.idz, r21 = zg ? a.bg.zr21[k] : 0.0;
-      const double cz = m1 * (1.0 / 60.0), ez = (zg ? m1 * m1 : ph.idz2) * (1.0 / 90.0);
+      double mz[NSRC];
+#pragma unroll
+      for (int q = 0; q < NSRC; ++q)
+        mz[q] = comb1(src[w_ + 4][q][tx], src[w_ + 2][q][tx], src[w_ + 5][q][tx], src[w_ + 1][q][tx],
+                      src[w_ + 6][q][tx], src[w_][q][tx]);
+      const double* sc = scr + tx + NG;
+      double cz = C.cz, ez = C.ez, cxz = C.cxz, cyz = C.cyz, v1ez = C.v1ez, v4ez = C.v4ez, v3cxz = C.v3cxz,
+             v3cyz = C.v3cyz, v3cz = C.v3cz, r21 = 0.0;
+      if constexpr (ZG) {
+        const double m1 = a.bg.zm1[k], m2 = m1 * m1;  // the host's entries are those of unit spacing
+        r21 = a.bg.zr21[k];
+        cz *= m1; cxz *= m1; cyz *= m1; v3cxz *= m1; v3cyz *= m1; v3cz *= m1;
+        ez *= m2; v1ez *= m2; v4ez *= m2;
+      }
       const double w = a.wtab[k], wp = a.wptab[k];
       const bool swamp = !ADJ && (w != 0.0 || wp != 0.0);
       // ---- A: B = curl A + B_ext, J = grad div A - lap A (the own-axis
@@ -233,32 +219,32 @@ __global__ void __launch_bounds__(NT, 4) rk64_kernel(const __grid_constant__ Arg
         const double A2 = __ldg(pc);
         double zz;
         double dzA = dd12(pa, sz, A0, zz);
-        B[1] = fma(cz, dzA, fma(-cx, cur[0], ph.bext[1]));
-        J[0] = fma(cx * cy, ds1(sc), fma(cx * cz, mz[0], fma(-ey, yyAx, -ez * zz)));
-        if (zg) J[0] = fma(-r21 * cz, dzA, J[0]);
+        B[1] = fma(cz, dzA, fma(-C.cx, cur[0], ph.bext[1]));
+        J[0] = fma(C.cxy, ds1(sc), fma(cxz, mz[0], fma(-C.ey, yyAx, -ez * zz)));
+        if constexpr (ZG) J[0] = fma(-r21 * cz, dzA, J[0]);
         double l0 = 0.0, l1 = 0.0, l2 = 0.0, dv = 0.0;
         if (swamp) {
-          l0 = fma(ex, dd2(pa, 1, A0), fma(ey, yyAx, ez * zz));
-          if (zg) l0 = fma(r21 * cz, dzA, l0);
+          l0 = fma(C.ex, dd2(pa, 1, A0), fma(C.ey, yyAx, ez * zz));
+          if constexpr (ZG) l0 = fma(r21 * cz, dzA, l0);
         }
         double xx;
         const double dxA = dd12(pb, 1, A1, xx);
         dzA = dd12(pb, sz, A1, zz);
-        B[0] = fma(-cz, dzA, fma(cy, cur[1], ph.bext[0]));
-        B[2] = fma(cx, dxA, fma(-cy, dyAx, ph.bext[2]));
-        J[1] = fma(cx * cy, ds1(sc + 1 * TY * SW), fma(cy * cz, mz[1], fma(-ex, xx, -ez * zz)));
-        if (zg) J[1] = fma(-r21 * cz, dzA, J[1]);
+        B[0] = fma(-cz, dzA, fma(C.cy, cur[1], ph.bext[0]));
+        B[2] = fma(C.cx, dxA, fma(-C.cy, dyAx, ph.bext[2]));
+        J[1] = fma(C.cxy, ds1(sc + 1 * SW), fma(cyz, mz[1], fma(-C.ex, xx, -ez * zz)));
+        if constexpr (ZG) J[1] = fma(-r21 * cz, dzA, J[1]);
         if (swamp) {
-          l1 = fma(ex, xx, fma(ey, dd2(pb, sy, A1), ez * zz));
-          if (zg) l1 = fma(r21 * cz, dzA, l1);
+          l1 = fma(C.ex, xx, fma(C.ey, dd2(pb, sy, A1), ez * zz));
+          if constexpr (ZG) l1 = fma(r21 * cz, dzA, l1);
         }
         xx = dd2(pc, 1, A2);
         const double yy = dd2(pc, sy, A2);
-        J[2] = fma(cz, mz[2], fma(-ex, xx, -ey * yy));
+        J[2] = fma(cz, mz[2], fma(-C.ex, xx, -C.ey * yy));
         if (swamp) {
           dzA = dd12(pc, sz, A2, zz);
-          l2 = fma(ex, xx, fma(ey, yy, ez * zz));
-          if (zg) l2 = fma(r21 * cz, dzA, l2);
+          l2 = fma(C.ex, xx, fma(C.ey, yy, ez * zz));
+          if constexpr (ZG) l2 = fma(r21 * cz, dzA, l2);
           dv = fma(cz, dzA, cur[2]);
           const double ews = ph.eta_s * w;
           if (a.bg.bB && k >= a.bg.ksw) {
@@ -290,35 +276,31 @@ __global__ void __launch_bounds__(NT, 4) rk64_kernel(const __grid_constant__ Arg
         u[1] = __ldg(pb);
         u[2] = __ldg(pc);
         dU[0][0] = ax_[1];
-        dU[0][1] = cy * dyUx;
+        dU[0][1] = C.cy * dyUx;
         dU[1][1] = ax_[2];
-        dU[2][0] = cx * cur[3];
-        dU[2][1] = cy * cur[4];
+        dU[2][0] = C.cx * cur[3];
+        dU[2][1] = C.cy * cur[4];
         if constexpr (ADJ) {
           dU[0][2] = cz * dd1(pa, sz);
-          dU[1][0] = cx * dd1(pb, 1);
+          dU[1][0] = C.cx * dd1(pb, 1);
           dU[1][2] = cz * dd1(pb, sz);
           dU[2][2] = cz * dd1(pc, sz);
         } else {
-          const double n1 = ph.nu, n13 = ph.nu * (1.0 / 3.0), n43 = ph.nu * (4.0 / 3.0);
           double xx, zz;
           dU[0][2] = cz * dd12(pa, sz, u[0], zz);
           // the scratch holds D1y u_y already scaled (field 2), d_y u_x not (field 3)
-          vis[0] = fma(n43 * ex, dd2(pa, 1, u[0]),
-                       fma(n1 * ey, yyUx,
-                           fma(n1 * ez, zz, fma(n13 * cx, ds1(sc + 2 * TY * SW), n13 * cx * cz * mz[3]))));
-          dU[1][0] = cx * dd12(pb, 1, u[1], xx);
+          vis[0] = fma(C.v4ex, dd2(pa, 1, u[0]),
+                       fma(C.v1ey, yyUx, fma(v1ez, zz, fma(C.v3cx, ds1(sc + 2 * SW), v3cxz * mz[3]))));
+          dU[1][0] = C.cx * dd12(pb, 1, u[1], xx);
           dU[1][2] = cz * dd12(pb, sz, u[1], zz);
-          vis[1] = fma(n1 * ex, xx,
-                       fma(n43 * ey, dd2(pb, sy, u[1]),
-                           fma(n1 * ez, zz, fma(n13 * cx * cy, ds1(sc + 3 * TY * SW), n13 * cy * cz * mz[4]))));
+          vis[1] = fma(C.v1ex, xx,
+                       fma(C.v4ey, dd2(pb, sy, u[1]), fma(v1ez, zz, fma(C.v3cxy, ds1(sc + 3 * SW), v3cyz * mz[4]))));
           dU[2][2] = cz * dd12(pc, sz, u[2], zz);
-          vis[2] = fma(n1 * ex, dd2(pc, 1, u[2]),
-                       fma(n1 * ey, dd2(pc, sy, u[2]), fma(n43 * ez, zz, n13 * cz * mz[5])));
-          if (zg) {
-            vis[0] = fma(n1 * r21, dU[0][2], vis[0]);
-            vis[1] = fma(n1 * r21, dU[1][2], vis[1]);
-            vis[2] = fma(n43 * r21, dU[2][2], vis[2]);
+          vis[2] = fma(C.v1ex, dd2(pc, 1, u[2]), fma(C.v1ey, dd2(pc, sy, u[2]), fma(v4ez, zz, v3cz * mz[5])));
+          if constexpr (ZG) {
+            vis[0] = fma(ph.nu * r21, dU[0][2], vis[0]);
+            vis[1] = fma(ph.nu * r21, dU[1][2], vis[1]);
+            vis[2] = fma((4.0 / 3.0) * ph.nu * r21, dU[2][2], vis[2]);
           }
         }
       }
@@ -329,17 +311,17 @@ __global__ void __launch_bounds__(NT, 4) rk64_kernel(const __grid_constant__ Arg
         const double c = __ldg(p);
         lr = a.bg.lbar[k + NG] + c;
         if constexpr (ADJ) {
-          gL[0] = cx * dd1(p, 1);
-          gL[1] = cy * dd1(p, sy);
+          gL[0] = C.cx * dd1(p, 1);
+          gL[1] = C.cy * dd1(p, sy);
           gL[2] = fma(cz, dd1(p, sz), a.bg.dl[k]);
         } else {
           double xx, yy, zz;
-          gL[0] = cx * dd12(p, 1, c, xx);
-          gL[1] = cy * dd12(p, sy, c, yy);
+          gL[0] = C.cx * dd12(p, 1, c, xx);
+          gL[1] = C.cy * dd12(p, sy, c, yy);
           const double dz = dd12(p, sz, c, zz);
           gL[2] = fma(cz, dz, a.bg.dl[k]);
-          lapL = fma(ex, xx, fma(ey, yy, fma(ez, zz, a.bg.d2l[k])));
-          if (zg) lapL = fma(r21 * cz, dz, lapL);
+          lapL = fma(C.ex, xx, fma(C.ey, yy, fma(ez, zz, a.bg.d2l[k])));
+          if constexpr (ZG) lapL = fma(r21 * cz, dz, lapL);
         }
       }
       {
@@ -347,12 +329,12 @@ __global__ void __launch_bounds__(NT, 4) rk64_kernel(const __grid_constant__ Arg
         const double c = __ldg(p);
         th = a.bg.tbar[k + NG] + c;
         double xx, yy, zz;
-        gT[0] = cx * dd12(p, 1, c, xx);
-        gT[1] = cy * dd12(p, sy, c, yy);
+        gT[0] = C.cx * dd12(p, 1, c, xx);
+        gT[1] = C.cy * dd12(p, sy, c, yy);
         const double dz = dd12(p, sz, c, zz);
         gT[2] = fma(cz, dz, a.bg.dt[k]);
-        lapT = fma(ex, xx, fma(ey, yy, fma(ez, zz, a.bg.d2t[k])));
-        if (zg) lapT = fma(r21 * cz, dz, lapT);
+        lapT = fma(C.ex, xx, fma(C.ey, yy, fma(ez, zz, a.bg.d2t[k])));
+        if constexpr (ZG) lapT = fma(r21 * cz, dz, lapT);
       }
 
       if constexpr (ADJ) {
@@ -420,14 +402,18 @@ __global__ void __launch_bounds__(NT, 4) rk64_kernel(const __grid_constant__ Arg
         }
         const double ugL = fma(u[0], gL[0], fma(u[1], gL[1], u[2] * gL[2]));
         const double gLs = fma(gL[0], gL[0], fma(gL[1], gL[1], gL[2] * gL[2]));
-        out[6] = fma(ph.drho, gLs, fma(fma(ph.drho_s, w, ph.drho), lapL, -(ugL + div)));
+        out[6] = fma(ph.drho, gLs + lapL, -(ugL + div));
+        if (swamp) out[6] = fma(ph.drho_s * w, lapL, out[6]);
         const double ugT = fma(u[0], gT[0], fma(u[1], gT[1], u[2] * gT[2]));
         const double gTs = fma(gT[0], gT[0], fma(gT[1], gT[1], gT[2] * gT[2]));
         const double JJ = fma(J[0], J[0], fma(J[1], J[1], J[2] * J[2]));
-        const double heat = ph.gm1 * fma(ph.eta * JJ, rho1, ph.nu * S2) / T;
-        // kappa0 T^{5/2} / rho
-        const double kt = ph.gm1 * ph.kappa0 * (T * T * sqrt(T)) * rho1;
-        out[7] = fma(kt, fma(3.5, gTs, lapT), fma(ph.chi_s * w, lapT, heat - fma(ph.gm1, div, ugT)));
+        // 1 / T and kappa0 T^{5/2} / rho from one reciprocal square root
+        const double rs = rsqrt(T);
+        const double heat = fma(C.heat * JJ, rho1, C.visc * S2) * (rs * rs);
+        const double kt = C.cond * rho1 * (T * T * T * rs);
+        double diff = lapT * kt;
+        if (swamp) diff = fma(ph.chi_s * w, lapT, diff);
+        out[7] = fma(3.5 * kt, gTs, diff) + (heat - fma(ph.gm1, div, ugT));
         if (k < ph.nc_k1) out[LT] += nc_term<double>(ph, a.bg, L.nz, k, lr, th, nullptr, nullptr);
 
         double tgx = 0.0, tgy = 0.0;
@@ -476,36 +462,37 @@ __global__ void __launch_bounds__(NT, 4) rk64_kernel(const __grid_constant__ Arg
         }
       }
     }
-    __syncthreads();  // the scratch is free for the next plane
   }
 }
 
-// z chunk: whole waves of CTAs against the six planes of sources each chunk
-// forms before its first centre (a front costs about a tenth of a centre)
-static int zchunk64(int nz, int tiles, int slots) {
-  int best = nz;
-  double cost = 0.0;
-  for (int kc = 1; kc <= nz; ++kc) {
-    const long long ctas = (long long)tiles * ((nz + kc - 1) / kc);
-    const double c = (double)((ctas + slots - 1) / slots) * (kc + 0.6);
-    if (kc == 1 || c < cost - 1e-9) {
-      cost = c;
-      best = kc;
-    }
-  }
-  return best;
-}
+static dim3 grid64(const Layout& L) { return dim3((L.nx + TX - 1) / TX, L.ny, (L.nz + KZ - 1) / KZ); }
 
-static dim3 grid64(Args& a) {
-  static PerDevice<int> sms;
-  const int n = sms.get([] {
-    cudaFuncSetAttribute(rk64_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
-    cudaFuncSetAttribute(rk64_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
-    return sm_count();
-  });
-  const int ntx = (a.L.nx + TX - 1) / TX, nty = (a.L.ny + TY - 1) / TY;
-  a.kchunk = zchunk64(a.L.nz, ntx * nty, n);
-  return dim3(ntx, nty, (a.L.nz + a.kchunk - 1) / a.kchunk);
+static Coef64 coef64(const Phys<double>& ph, bool zg) {
+  Coef64 c;
+  c.cx = ph.idx / 60.0;
+  c.cy = ph.idy / 60.0;
+  c.cz = (zg ? 1.0 : ph.idz) / 60.0;
+  c.cxy = c.cx * c.cy;
+  c.cxz = c.cx * c.cz;
+  c.cyz = c.cy * c.cz;
+  c.ex = ph.idx2 / 90.0;
+  c.ey = ph.idy2 / 90.0;
+  c.ez = (zg ? 1.0 : ph.idz2) / 90.0;
+  c.v1ex = ph.nu * c.ex;
+  c.v1ey = ph.nu * c.ey;
+  c.v1ez = ph.nu * c.ez;
+  c.v4ex = c.v1ex * 4.0 / 3.0;
+  c.v4ey = c.v1ey * 4.0 / 3.0;
+  c.v4ez = c.v1ez * 4.0 / 3.0;
+  c.v3cx = ph.nu * c.cx / 3.0;
+  c.v3cxy = ph.nu * c.cxy / 3.0;
+  c.v3cxz = ph.nu * c.cxz / 3.0;
+  c.v3cyz = ph.nu * c.cyz / 3.0;
+  c.v3cz = ph.nu * c.cz / 3.0;
+  c.heat = ph.gm1 * ph.eta;
+  c.visc = ph.gm1 * ph.nu;
+  c.cond = ph.gm1 * ph.kappa0;
+  return c;
 }
 
 }  // namespace r64
@@ -528,8 +515,11 @@ void launch_rk64(const Layout& L, const Phys<double>& ph, const Background<doubl
   a.v1 = (const double*)drv.v1;
   a.ss = ss;
   a.sub = sub;
-  const dim3 g = r64::grid64(a);
-  r64::rk64_kernel<false><<<g, dim3(r64::TX, r64::TY), r64::SMEM, st>>>(a);
+  const bool zg = bg.zm1 != nullptr;
+  a.c = r64::coef64(ph, zg);
+  const dim3 g = r64::grid64(L), b(r64::TX, r64::KZ);
+  if (zg) r64::rk64_kernel<false, true><<<g, b, 0, st>>>(a);
+  else r64::rk64_kernel<false, false><<<g, b, 0, st>>>(a);
 }
 
 void launch_adj_point64(const Layout& L, const Phys<double>& ph, const Background<double>& bg, const double* g,
@@ -547,8 +537,8 @@ void launch_adj_point64(const Layout& L, const Phys<double>& ph, const Backgroun
   a.dbar = dbar;
   a.coef = coef;
   a.thbar = thbar;
-  const dim3 gr = r64::grid64(a);
-  r64::rk64_kernel<true><<<gr, dim3(r64::TX, r64::TY), r64::SMEM, st>>>(a);
+  a.c = r64::coef64(ph, false);
+  r64::rk64_kernel<true, false><<<r64::grid64(L), dim3(r64::TX, r64::KZ), 0, st>>>(a);
 }
 
 }  // namespace mhd
