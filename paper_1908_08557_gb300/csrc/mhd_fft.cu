@@ -211,18 +211,14 @@ __global__ void __launch_bounds__(256) cols_kernel(FFTPlan fp, int mode, const S
       // e^(i theta) = (k_x + i k_y) / |k|; times the filter
       // exp(-(2 |k| / k_N)^4).  The mean and the Nyquist modes (whose signed
       // wavenumber has no partner) carry none.
-      const double kxw = fp.ktx[col], kyw = fp.kty[ky];
-      const double k2 = kxw * kxw + kyw * kyw;
-      if (k2 > 0.0 && 2 * col != nx && 2 * ky != ny) {
-        const double2 Fm = spec[(line ^ 1) * ny + ((ny - ky) & (ny - 1))];
-        const double c2 = (kxw * kxw - kyw * kyw) / k2, s2 = 2.0 * kxw * kyw / k2;
-        const double ax = kxw / fp.knx, ay = kyw / fp.kny;
-        const double q4 = 4.0 * (ax * ax + ay * ay);
-        const double w = 0.5 * exp(-q4 * q4);
-        g = make_double2(w * (F.x - (c2 * Fm.x + s2 * Fm.y)), w * (F.y - (s2 * Fm.x - c2 * Fm.y)));
-      } else {
-        g = make_double2(0.0, 0.0);
-      }
+      // (w, w cos 2 theta, w sin 2 theta) from the quarter table: formed
+      // here, the exponential and the divisions took half of the launch
+      const int ka = col <= nx / 2 ? col : nx - col, kb = ky <= ny / 2 ? ky : ny - ky;
+      const double* t = fp.filt + 3 * ((long long)ka * (ny / 2 + 1) + kb);
+      const double w = __ldg(t), wc = __ldg(t + 1), ws0 = __ldg(t + 2);
+      const double ws = (col > nx / 2) != (ky > ny / 2) ? -ws0 : ws0;
+      const double2 Fm = spec[(line ^ 1) * ny + ((ny - ky) & (ny - 1))];
+      g = make_double2(w * F.x - (wc * Fm.x + ws * Fm.y), w * F.y - (ws * Fm.x - wc * Fm.y));
     } else if (mode == 2) {
       // transpose of Eq. 7's inversion: with F = FFT(X + i Y) for real X,
       // Y (the adjoints of A_x, A_y), the spectrum of the B_z adjoint is
@@ -276,10 +272,18 @@ __global__ void __launch_bounds__(256) cols_kernel(FFTPlan fp, int mode, const S
 // mode 2 (adjoint): plane c adds its real part into A_c at the top layer and
 // its imaginary part into A_c at the photosphere (interior x, y only);
 // mode 3: real part into out_re.
+struct RowsAdd {  // mode 5
+  const double* vx;
+  const double* vy;
+  double f_rot;
+  double* part;
+};
+
 template <typename R>
 __global__ void __launch_bounds__(256) rows_inv_kernel(FFTPlan fp, Layout L, R* __restrict__ f, R* out_re,
-                                                       R* out_im, int mode, const StepState* ss, int nb) {
+                                                       R* out_im, int mode, const StepState* ss, int nb, RowsAdd add) {
   extern __shared__ double2 sm[];
+  double energy = 0.0;
   if (ss && halted(ss)) return;
   const int nx = fp.nx, ny = fp.ny;
   const int y0 = blockIdx.x * nb;
@@ -299,6 +303,14 @@ __global__ void __launch_bounds__(256) rows_inv_kernel(FFTPlan fp, Layout L, R* 
   for (int q = threadIdx.x; q < nb * nx; q += blockDim.x) {
     const int line = q / nx, x = q - line * nx, y = y0 + line;
     const double2 v = r[line * nx + x];
+    if (mode == 5) {
+      const long long o = (long long)y * nx + x;
+      const double wx = fma(add.f_rot, v.x * sc, add.vx[o]), wy = fma(add.f_rot, v.y * sc, add.vy[o]);
+      out_re[o] = (R)wx;
+      out_im[o] = (R)wy;
+      energy = fma(wx, wx, fma(wy, wy, energy));
+      continue;
+    }
     const R re = (R)(v.x * sc), im = (R)(v.y * sc);
     if (mode == 1) {
       out_re[(long long)y * nx + x] = re;
@@ -329,6 +341,18 @@ __global__ void __launch_bounds__(256) rows_inv_kernel(FFTPlan fp, Layout L, R* 
         f[L.at(f1, k1, ys[bb], xs[aa])] = re;
         f[L.at(f2, k2, ys[bb], xs[aa])] = im;
       }
+  }
+  if (mode == 5) {
+    // fixed order: warp tree, then the warps in turn
+    __shared__ double sh[8];
+    for (int o2 = 16; o2 > 0; o2 >>= 1) energy += __shfl_down_sync(0xffffffffu, energy, o2);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = energy;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double s = 0.0;
+      for (int q = 0; q < (int)(blockDim.x >> 5); ++q) s += sh[q];
+      add.part[blockIdx.x] = s;
+    }
   }
 }
 
@@ -484,7 +508,7 @@ void launch_pfe(const FFTPlan& fp, const Layout& L, R* f, const StepState* ss, c
                                                                             nullptr, nullptr);
     cols_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 3), l.threads3, l.smem_cols3, st>>>(fp, 0, ss, l.ppb, l.lg);
     rows_inv_kernel<R><<<dim3(fp.ny / ri.nb, 3, 3), ri.threads, ri.smem, st>>>(fp, L, f, nullptr, nullptr, 0, ss,
-                                                                              ri.nb);
+                                                                              ri.nb, RowsAdd{});
     return;
   }
   // one chain (rows, columns, inverse rows) per packed plane, on its own
@@ -501,7 +525,7 @@ void launch_pfe(const FFTPlan& fp, const Layout& L, R* f, const StepState* ss, c
                                                                             nullptr, nullptr);
     cols_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 1), l.threads3, l.smem_cols3, sp>>>(fq, 0, ss, l.ppb, l.lg);
     rows_inv_kernel<R><<<dim3(fp.ny / ri.nb, 1, 3), ri.threads, ri.smem, sp>>>(fq, L, f, nullptr, nullptr, 0, ss,
-                                                                              ri.nb);
+                                                                              ri.nb, RowsAdd{});
   }
   for (int i = 0; i < 2; ++i) {
     cudaEventRecord(ps->join[i], ps->s[i]);
@@ -520,11 +544,11 @@ void launch_atarget(const FFTPlan& fp, const R* bz, R* axt, R* ayt, cudaStream_t
                                                                           nullptr, nullptr);
   cols_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 1), l.threads, l.smem_cols, st>>>(fp, 1, nullptr, l.ppb, 1);
   rows_inv_kernel<R><<<dim3(fp.ny / r1.nb, 1, 1), r1.threads, r1.smem, st>>>(fp, L, nullptr, axt, ayt, 1, nullptr,
-                                                                             r1.nb);
+                                                                             r1.nb, RowsAdd{});
 }
 
-void launch_rotational(const FFTPlan& fp, const double* vx, const double* vy, double* rx, double* ry,
-                       cudaStream_t st) {
+int launch_rotational(const FFTPlan& fp, const double* vx, const double* vy, double* rx, double* ry, bool add,
+                      double f_rot, double* part, cudaStream_t st) {
   set_smem_once();
   Layout L{};
   const FFTLaunch l = fft_launch(fp, 1);
@@ -533,8 +557,9 @@ void launch_rotational(const FFTPlan& fp, const double* vx, const double* vy, do
   rows_fwd_kernel<double><<<dim3(fp.ny / r1.nb, 1), r1.threads, r1.smem, st>>>(fp, L, nullptr, nullptr, 3, nullptr,
                                                                                r1.nb, vx, vy);
   cols_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 1), l.threads, l.smem_cols, st>>>(fp, 4, nullptr, l.ppb, 1);
-  rows_inv_kernel<double><<<dim3(fp.ny / r1.nb, 1, 1), r1.threads, r1.smem, st>>>(fp, L, nullptr, rx, ry, 1,
-                                                                                 nullptr, r1.nb);
+  rows_inv_kernel<double><<<dim3(fp.ny / r1.nb, 1, 1), r1.threads, r1.smem, st>>>(
+      fp, L, nullptr, rx, ry, add ? 5 : 1, nullptr, r1.nb, RowsAdd{vx, vy, f_rot, part});
+  return fp.ny / r1.nb;
 }
 
 // Adjoint of the potential-field ghosts: gbar (adjoint of the ghost-filled
@@ -551,7 +576,7 @@ void launch_pfe_adjoint(const FFTPlan& fp_adj, const Layout& L, R* gbar, const S
                                                                               nullptr, nullptr);
   cols_adj_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 3), l.threads, l.smem_cols, st>>>(fp_adj, ss, l.ppb);
   rows_inv_kernel<R><<<dim3(fp_adj.ny / r3.nb, 3, 1), r3.threads, r3.smem, st>>>(fp_adj, L, gbar, nullptr, nullptr, 2,
-                                                                                ss, r3.nb);
+                                                                                ss, r3.nb, RowsAdd{});
 }
 
 // Transpose of the magnetogram inversion: B_z adjoint (out, [ny][nx]) from
@@ -567,7 +592,7 @@ void launch_atarget_adjoint(const FFTPlan& fp, const double* abx, const double* 
                                                                           abx, aby);
   cols_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 1), l.threads, l.smem_cols, st>>>(fp, 2, nullptr, l.ppb, 1);
   rows_inv_kernel<R><<<dim3(fp.ny / r1.nb, 1, 1), r1.threads, r1.smem, st>>>(fp, L, nullptr, out, nullptr, 3, nullptr,
-                                                                             r1.nb);
+                                                                             r1.nb, RowsAdd{});
 }
 
 template void launch_pfe_adjoint<float>(const FFTPlan&, const Layout&, float*, const StepState*, cudaStream_t);

@@ -4,25 +4,39 @@
 // need no list, compaction or host bookkeeping.
 //
 // Update (the population at time t):
-//   1. expire:  occ = 0 where t - t0 - t_max > t_max (Eq. 2 is back at v_min)
-//   2. seed:    a pixel within r_inner of a live centre is out, the rest
-//               undecided
-//   3. rounds:  join: an undecided pixel with no undecided pixel of smaller
+//   1. seed:    a pixel within r_inner of a live centre is out, the rest
+//               undecided; a granule with t - t0 - t_max > t_max (Eq. 2 is
+//               back at v_min) no longer counts as live
+//   2. rounds:  join: an undecided pixel with no undecided pixel of smaller
 //               (key, index) within r_inner, and no member there, becomes a
 //               member; exclude: an undecided pixel with a member within
 //               r_inner is out.  Repeated until nothing is undecided, this
 //               gives exactly the set the sequential visit in (key, index)
 //               order accepts (the first undecided pixel in that order joins
 //               every round, so the rounds end).
-//   4. birth:   members become granules with the draws at their pixel.
+//   3. birth:   expired granules are cleared, members become granules with
+//               the draws at their pixel.
 // Velocity at time t:
-//   5. amp:     per pixel, Eq. 2 of its granule (0 where none)
-//   6. render:  v_gran(p) = sum over lane offsets o of amp(p - o) w(o), with
+//   4. amp:     per pixel, Eq. 2 of its granule (0 where none)
+//   5. render:  v_gran(p) = sum over lane offsets o of amp(p - o) w(o), with
 //               w(o) = profile(|o|) o / |o| tabulated on the host
-//   7. FFT:     the filtered rotational part (Eq. 3), packed plane v_x + i v_y
-//   8. combine: v_vor = v_gran + f_rot v_rot', with block sums of |v|^2 of
-//               both fields; one block totals them in a fixed order; scale
-//               v_vor to the rms of v_gran (Eq. 4) into the caller's array.
+//   6. FFT:     the filtered rotational part (Eq. 3), packed plane v_x + i v_y;
+//               its last kernel adds it to v_gran (v_vor = v_gran + f_rot
+//               v_rot') and sums |v_vor|^2 per block
+//   7. total, scale: block sums of |v|^2 of both fields totalled in a fixed
+//               order; v_vor scaled to the rms of v_gran (Eq. 4) into the
+//               caller's array.
+//
+// What bounds the pixel kernels.  One pixel in ten carries a granule, but a
+// warp that tests pixel by pixel does FP64 work (2 operations per clock and SM)
+// for every offset at which any of its 32 lanes has one, which is nearly all
+// of them.  So the neighbourhood kernels work on tiles of 32 x 8 pixels whose
+// occupancy, halo included, is a 64-bit mask per row (one ballot or two per
+// row): a disk test is an AND per row, and the render walks each lane's own
+// hits, so a warp takes as many steps as its busiest lane has granules in
+// reach (about 9) instead of one per offset (68 at 0.23 Mm pixels); amplitudes
+// and births are computed on lists of the occupied pixels of a block.  Disks
+// wider than 16 pixels, or planes narrower than a tile, take the plain kernels.
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -54,36 +68,133 @@ struct GranDev {
   int n_l;
   double* part;  // [2][nblk] block sums
   double* tot;   // [2]: scale, spare
-  int* cnt;
+  int* cnt;      // [BATCH] undecided pixels left after each round of a batch
+};
+
+// rounds launched between two reads of the undecided counts (the rounds after
+// the last needed one return at once)
+constexpr int BATCH = 4;
+
+// disk row by row: offsets (o_x, o_y) of the disk are |o_x| <= lim[|o_y|]
+constexpr int MAXR = 16;
+struct Disk {
+  int rx, ry;                 // largest |o_x|, |o_y|
+  signed char lim[MAXR + 1];  // -1: no offset in that row
 };
 
 __device__ __forceinline__ int wrap(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
 
-__global__ void __launch_bounds__(GT) expire_kernel(GranDev g, double t) {
-  const int p = blockIdx.x * GT + threadIdx.x;
-  if (p >= g.nx * g.ny) return;
-  if (g.occ[p] && t - g.t0[p] - g.tmax[p] > g.tmax[p]) {
-    g.occ[p] = 0;
-    g.t0[p] = g.life[p] = g.vmax[p] = g.tmax[p] = 0.0;
-  }
+// a granule whose amplitude has fallen below v_min after its peak
+__device__ __forceinline__ bool expired(const GranDev& g, int p, double t) {
+  const double tm = g.tmax[p];
+  return t - g.t0[p] - tm > tm;
 }
 
-__global__ void __launch_bounds__(GT) seed_kernel(GranDev g) {
+__global__ void __launch_bounds__(GT) seed_kernel(GranDev g, double t) {
   const int p = blockIdx.x * GT + threadIdx.x;
   if (p >= g.nx * g.ny) return;
   const int y = p / g.nx, x = p - y * g.nx;
-  bool blocked = g.occ[p] != 0;
+  bool blocked = g.occ[p] != 0 && !expired(g, p, t);
   for (int n = 0; n < g.n_in && !blocked; ++n) {
     const int2 o = __ldg(g.off_in + n);
-    blocked = g.occ[wrap(y + o.y, g.ny) * g.nx + wrap(x + o.x, g.nx)] != 0;
+    const int q = wrap(y + o.y, g.ny) * g.nx + wrap(x + o.x, g.nx);
+    blocked = g.occ[q] != 0 && !expired(g, q, t);
   }
   g.mis[p] = blocked ? OUT : UNDECIDED;
+}
+
+// ---- tiles of 32 x 8 pixels with row masks (nx, ny powers of two) ----------
+constexpr int TW = 32, TH = 8;
+constexpr int TROWS = TH + 2 * MAXR;
+
+// masks[r]: bit c set where flag(pixel) holds at halo column x0 - rx + c of
+// halo row y0 - ry + r (periodic)
+template <typename F>
+__device__ __forceinline__ void row_masks(const GranDev& g, int x0, int y0, int rx, int ry,
+                                          unsigned long long* masks, F flag) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int r = w; r < TH + 2 * ry; r += GT / 32) {
+    const int row = ((y0 - ry + r) & (g.ny - 1)) * g.nx;
+    const bool f0 = flag(row + ((x0 - rx + lane) & (g.nx - 1)));
+    const bool f1 = lane < 2 * rx && flag(row + ((x0 - rx + 32 + lane) & (g.nx - 1)));
+    const unsigned lo = __ballot_sync(0xffffffffu, f0), hi = __ballot_sync(0xffffffffu, f1);
+    if (lane == 0) masks[r] = (unsigned long long)hi << 32 | lo;
+  }
+}
+// the bits of a row mask within the disk's row o_y of the pixel at tile column
+// tx: bit lim + o_x of the result
+__device__ __forceinline__ unsigned long long disk_bits(unsigned long long m, int tx, int rx, int lim) {
+  return lim < 0 ? 0ull : (m >> (tx + rx - lim)) & ((1ull << (2 * lim + 1)) - 1ull);
+}
+__device__ __forceinline__ bool disk_any(const unsigned long long* masks, const Disk& d, int tx, int ty) {
+  unsigned long long any = 0;
+  for (int oy = -d.ry; oy <= d.ry; ++oy)
+    any |= disk_bits(masks[ty + d.ry + oy], tx, d.rx, d.lim[oy < 0 ? -oy : oy]);
+  return any != 0;
+}
+
+__global__ void __launch_bounds__(GT) seed_tile_kernel(GranDev g, Disk d, double t) {
+  __shared__ unsigned long long live[TROWS];
+  const int x0 = blockIdx.x * TW, y0 = blockIdx.y * TH, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  row_masks(g, x0, y0, d.rx, d.ry, live, [&](int p) { return g.occ[p] != 0 && !expired(g, p, t); });
+  __syncthreads();
+  g.mis[(y0 + ty) * g.nx + x0 + tx] = disk_any(live, d, tx, ty) ? OUT : UNDECIDED;
+}
+
+// As join_kernel below: a snapshot of the neighbours' states, taken while
+// other tiles may be joining, gives the same decision either way.
+__global__ void __launch_bounds__(GT) join_tile_kernel(GranDev g, Disk d, const unsigned* __restrict__ keys,
+                                                       int round) {
+  if (round > 0 && g.cnt[round - 1] == 0) return;
+  const int x0 = blockIdx.x * TW, y0 = blockIdx.y * TH, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int p = (y0 + ty) * g.nx + x0 + tx;
+  const bool open = g.mis[p] == UNDECIDED;
+  if (!__syncthreads_or(open)) return;
+  __shared__ unsigned long long mem[TROWS], und[TROWS];
+  const volatile int* mis = g.mis;
+  row_masks(g, x0, y0, d.rx, d.ry, mem, [&](int q) { return mis[q] == MEMBER; });
+  // every neighbour that is not out: one that joins while this tile reads is
+  // still compared by its key, which precedes p's
+  row_masks(g, x0, y0, d.rx, d.ry, und, [&](int q) { return mis[q] != OUT; });
+  __syncthreads();
+  if (!open || disk_any(mem, d, tx, ty)) return;
+  const unsigned kp = keys[p];
+  for (int oy = -d.ry; oy <= d.ry; ++oy) {
+    const int lim = d.lim[oy < 0 ? -oy : oy];
+    unsigned long long b = disk_bits(und[ty + d.ry + oy], tx, d.rx, lim);
+    if (oy == 0) b &= ~(1ull << lim);  // the pixel itself
+    const int row = ((y0 + ty + oy) & (g.ny - 1)) * g.nx;
+    while (b) {
+      const int c = __ffsll((long long)b) - 1;
+      b &= b - 1;
+      const int q = row + ((x0 + tx + c - lim) & (g.nx - 1));
+      const unsigned kq = keys[q];
+      if (kq < kp || (kq == kp && q < p)) return;
+    }
+  }
+  g.mis[p] = MEMBER;
+}
+
+__global__ void __launch_bounds__(GT) exclude_tile_kernel(GranDev g, Disk d, int round) {
+  if (round > 0 && g.cnt[round - 1] == 0) return;
+  const int x0 = blockIdx.x * TW, y0 = blockIdx.y * TH, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int p = (y0 + ty) * g.nx + x0 + tx;
+  const bool open = g.mis[p] == UNDECIDED;
+  if (!__syncthreads_or(open)) return;
+  __shared__ unsigned long long mem[TROWS];
+  row_masks(g, x0, y0, d.rx, d.ry, mem, [&](int q) { return g.mis[q] == MEMBER; });
+  __syncthreads();
+  const bool hit = open && disk_any(mem, d, tx, ty);
+  if (hit) g.mis[p] = OUT;
+  const int c = __syncthreads_count(open && !hit);
+  if (threadIdx.x == 0 && c) atomicAdd(g.cnt + round, c);
 }
 
 // Reads of neighbours race with their writes in the same launch; either
 // value gives the same decision (a neighbour that joins now precedes p, so
 // p does not join whether it reads UNDECIDED or MEMBER).
-__global__ void __launch_bounds__(GT) join_kernel(GranDev g, const unsigned* __restrict__ keys) {
+__global__ void __launch_bounds__(GT) join_kernel(GranDev g, const unsigned* __restrict__ keys, int round) {
+  if (round > 0 && g.cnt[round - 1] == 0) return;
   const int p = blockIdx.x * GT + threadIdx.x;
   if (p >= g.nx * g.ny) return;
   if (g.mis[p] != UNDECIDED) return;
@@ -102,7 +213,8 @@ __global__ void __launch_bounds__(GT) join_kernel(GranDev g, const unsigned* __r
   g.mis[p] = MEMBER;
 }
 
-__global__ void __launch_bounds__(GT) exclude_kernel(GranDev g) {
+__global__ void __launch_bounds__(GT) exclude_kernel(GranDev g, int round) {
+  if (round > 0 && g.cnt[round - 1] == 0) return;
   const int p = blockIdx.x * GT + threadIdx.x;
   int undecided = 0;
   if (p < g.nx * g.ny && g.mis[p] == UNDECIDED) {
@@ -116,34 +228,68 @@ __global__ void __launch_bounds__(GT) exclude_kernel(GranDev g) {
     else undecided = 1;
   }
   const int c = __syncthreads_count(undecided);
-  if (threadIdx.x == 0 && c) atomicAdd(g.cnt, c);
+  if (threadIdx.x == 0 && c) atomicAdd(g.cnt + round, c);
+}
+
+// The occupied (or chosen) pixels of a block's LP * GT pixels as a list in
+// shared memory, so that the FP64 work on them runs in full warps; returns
+// their number.  The order within the list does not matter.
+constexpr int LP = 8;
+template <typename F>
+__device__ __forceinline__ int block_list(int N, int* list, int* count, F take) {
+  if (threadIdx.x == 0) *count = 0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  for (int u = 0; u < LP; ++u) {
+    const int p = (blockIdx.x * LP + u) * GT + threadIdx.x;
+    const bool in = p < N && take(p);
+    const unsigned m = __ballot_sync(0xffffffffu, in);
+    int base = 0;
+    if (lane == 0 && m) base = atomicAdd(count, __popc(m));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (in) list[base + __popc(m & ((1u << lane) - 1))] = p;
+  }
+  __syncthreads();
+  return *count;
 }
 
 __global__ void __launch_bounds__(GT) birth_kernel(GranDev g, mhd_gran_params gp, double t,
                                                    const double* __restrict__ c_life,
                                                    const double* __restrict__ c_amp) {
-  const int p = blockIdx.x * GT + threadIdx.x;
-  if (p >= g.nx * g.ny || g.mis[p] != MEMBER) return;
-  const double cl = fmin(1.0, fmax(-1.0, c_life[p]));
-  const double ca = fmin(1.0, fmax(-1.0, c_amp[p]));
-  const double T = gp.lifetime * (1.0 + gp.lifetime_spread * cl);
-  const double vm = gp.v0 * (1.0 + gp.amp_spread * ca);
-  g.occ[p] = 1;
-  g.t0[p] = t;
-  g.life[p] = T;
-  g.vmax[p] = vm;
-  g.tmax[p] = T * sqrt(fabs(log(gp.vmin_frac * gp.v0 / vm)));  // Eq. 1
+  __shared__ int list[LP * GT], count;
+  const int n = block_list(g.nx * g.ny, list, &count, [&](int p) {
+    if (g.occ[p] && expired(g, p, t)) {
+      g.occ[p] = 0;
+      g.t0[p] = g.life[p] = g.vmax[p] = g.tmax[p] = 0.0;
+    }
+    return g.mis[p] == MEMBER;
+  });
+  for (int i = threadIdx.x; i < n; i += GT) {
+    const int p = list[i];
+    const double cl = fmin(1.0, fmax(-1.0, c_life[p]));
+    const double ca = fmin(1.0, fmax(-1.0, c_amp[p]));
+    const double T = gp.lifetime * (1.0 + gp.lifetime_spread * cl);
+    const double vm = gp.v0 * (1.0 + gp.amp_spread * ca);
+    g.occ[p] = 1;
+    g.t0[p] = t;
+    g.life[p] = T;
+    g.vmax[p] = vm;
+    g.tmax[p] = T * sqrt(fabs(log(gp.vmin_frac * gp.v0 / vm)));  // Eq. 1
+  }
 }
 
 __global__ void __launch_bounds__(GT) amp_kernel(GranDev g, double t) {
-  const int p = blockIdx.x * GT + threadIdx.x;
-  if (p >= g.nx * g.ny) return;
-  double a = 0.0;
-  if (g.occ[p]) {
+  __shared__ int list[LP * GT], count;
+  const int n = block_list(g.nx * g.ny, list, &count, [&](int p) {
+    const bool in = g.occ[p] != 0;
+    if (!in) g.amp[p] = 0.0;
+    return in;
+  });
+  for (int i = threadIdx.x; i < n; i += GT) {
+    const int p = list[i];
     const double s = (t - g.t0[p] - g.tmax[p]) / g.life[p];
-    a = g.vmax[p] * exp(-s * s);  // Eq. 2
+    g.amp[p] = g.vmax[p] * exp(-s * s);  // Eq. 2
   }
-  g.amp[p] = a;
 }
 
 __device__ __forceinline__ double block_sum(double v, double* sh) {
@@ -184,31 +330,88 @@ __global__ void __launch_bounds__(GT) render_kernel(GranDev g) {
   if (threadIdx.x == 0) g.part[blockIdx.x] = s;
 }
 
-// v_vor = v_gran + f_rot v_rot' into vr; block sums of |v_vor|^2 into part[1][block]
-__global__ void __launch_bounds__(GT) combine_kernel(GranDev g, double f_rot, int nblk) {
+// The same sum over a tile: each lane walks the granules within its own disk,
+// in the order of the offset list, so the result equals render_kernel's.
+__global__ void __launch_bounds__(GT) render_tile_kernel(GranDev g, Disk d) {
+  extern __shared__ double2 dyn[];
+  __shared__ unsigned long long occ[TROWS];
   __shared__ double sh[GT / 32];
-  const int N = g.nx * g.ny;
-  const int p = blockIdx.x * GT + threadIdx.x;
-  double e = 0.0;
-  if (p < N) {
-    const double wx = g.vg[p] + f_rot * g.vr[p];
-    const double wy = g.vg[N + p] + f_rot * g.vr[N + p];
-    g.vr[p] = wx;
-    g.vr[N + p] = wy;
-    e = wx * wx + wy * wy;
+  const int wr = 2 * d.rx + 1, ww = TW + 2 * d.rx, hh = TH + 2 * d.ry;
+  double2* wt = dyn;                                      // [2 ry + 1][2 rx + 1] weights
+  double* am = reinterpret_cast<double*>(dyn + wr * (2 * d.ry + 1));  // [hh][ww] amplitudes
+  const int x0 = blockIdx.x * TW, y0 = blockIdx.y * TH, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (int n = threadIdx.x; n < g.n_l; n += GT) {
+    const int2 o = __ldg(g.off_l + n);
+    wt[(o.y + d.ry) * wr + o.x + d.rx] = __ldg(g.w_l + n);
   }
-  const double s = block_sum(e, sh);
-  if (threadIdx.x == 0) g.part[nblk + blockIdx.x] = s;
+  for (int r = ty; r < hh; r += GT / 32) {
+    const int row = ((y0 - d.ry + r) & (g.ny - 1)) * g.nx;
+    const double a0 = __ldg(g.amp + row + ((x0 - d.rx + tx) & (g.nx - 1)));
+    const double a1 = tx < 2 * d.rx ? __ldg(g.amp + row + ((x0 - d.rx + 32 + tx) & (g.nx - 1))) : 0.0;
+    am[r * ww + tx] = a0;
+    if (tx < 2 * d.rx) am[r * ww + 32 + tx] = a1;
+    const unsigned lo = __ballot_sync(0xffffffffu, a0 != 0.0), hi = __ballot_sync(0xffffffffu, a1 != 0.0);
+    if (tx == 0) occ[r] = (unsigned long long)hi << 32 | lo;
+  }
+  __syncthreads();
+  double vx = 0.0, vy = 0.0;
+  int oy = -d.ry - 1, lim = 0;
+  unsigned long long bits = 0;
+  for (;;) {
+    // next granule of this lane: rows by ascending o_y, and within a row the
+    // columns by descending x (ascending o_x; the centre sits at p - o)
+    while (!bits && oy < d.ry) {
+      ++oy;
+      lim = d.lim[oy < 0 ? -oy : oy];
+      bits = disk_bits(occ[ty + d.ry - oy], tx, d.rx, lim);
+      if (oy == 0) bits &= ~(1ull << lim);
+    }
+    if (!__any_sync(0xffffffffu, bits != 0)) break;
+    if (bits) {
+      const int c = 63 - __clzll((long long)bits);
+      bits &= ~(1ull << c);
+      const double a = am[(ty + d.ry - oy) * ww + tx + d.rx - lim + c];
+      const double2 w = wt[(oy + d.ry) * wr + d.rx + lim - c];
+      vx = fma(a, w.x, vx);
+      vy = fma(a, w.y, vy);
+    }
+  }
+  const int N = g.nx * g.ny, p = (y0 + ty) * g.nx + x0 + tx;
+  g.vg[p] = vx;
+  g.vg[N + p] = vy;
+  const double s = block_sum(vx * vx + vy * vy, sh);
+  if (threadIdx.x == 0) g.part[blockIdx.y * gridDim.x + blockIdx.x] = s;
+}
+
+// the filter of Eq. 3 on a quarter of the spectrum (it is even in k_x and k_y
+// but for the sign of sin 2 theta): w = exp(-(2 |k| / k_N)^4) / 2 and w cos, w
+// sin of twice the angle of k; zero on the mean and the Nyquist modes
+__global__ void __launch_bounds__(GT) filter_kernel(FFTPlan fp, double* __restrict__ tab) {
+  const int hx = fp.nx / 2 + 1, hy = fp.ny / 2 + 1;
+  const int q = blockIdx.x * GT + threadIdx.x;
+  if (q >= hx * hy) return;
+  const int a = q / hy, b = q - a * hy;
+  const double kx = fabs(fp.ktx[a]), ky = fabs(fp.kty[b]);
+  const double k2 = kx * kx + ky * ky;
+  double w = 0.0, wc = 0.0, ws = 0.0;
+  if (k2 > 0.0 && 2 * a != fp.nx && 2 * b != fp.ny) {
+    const double ax = kx / fp.knx, ay = ky / fp.kny;
+    const double q4 = 4.0 * (ax * ax + ay * ay);
+    w = 0.5 * exp(-q4 * q4);
+    wc = w * ((kx * kx - ky * ky) / k2);
+    ws = w * (2.0 * kx * ky / k2);
+  }
+  tab[3 * (size_t)q] = w;
+  tab[3 * (size_t)q + 1] = wc;
+  tab[3 * (size_t)q + 2] = ws;
 }
 
 // one block: totals of both block-sum rows in a fixed order, the Eq. 4 scale
-__global__ void __launch_bounds__(GT) total_kernel(GranDev g, int nblk) {
+__global__ void __launch_bounds__(GT) total_kernel(GranDev g, int nblk, int nvor) {
   __shared__ double sh[GT / 32];
   double sv = 0.0, sw = 0.0;
-  for (int i = threadIdx.x; i < nblk; i += GT) {
-    sv += g.part[i];
-    sw += g.part[nblk + i];
-  }
+  for (int i = threadIdx.x; i < nblk; i += GT) sv += g.part[i];
+  for (int i = threadIdx.x; i < nvor; i += GT) sw += g.part[nblk + i];
   const double tv = block_sum(sv, sh);
   __syncthreads();
   const double tw = block_sum(sw, sh);
@@ -232,6 +435,24 @@ int lg2(int n) {
   int l = 0;
   while ((1 << l) < n) ++l;
   return l;
+}
+
+// the same disk by rows (lim is symmetric and falls with |o_y|); false if it is
+// wider than the tile kernels take
+bool disk_rows(double r, double dx, double dy, Disk* d) {
+  d->rx = d->ry = 0;
+  for (int q = 0; q <= MAXR; ++q) d->lim[q] = -1;
+  const int mx = (int)std::ceil(r / dx), my = (int)std::ceil(r / dy);
+  for (int oy = 0; oy <= my; ++oy)
+    for (int ox = 0; ox <= mx; ++ox) {
+      const double ex = ox * dx, ey = oy * dy;
+      if (!(ex * ex + ey * ey < r * r)) continue;
+      if (ox > MAXR || oy > MAXR) return false;
+      d->lim[oy] = (signed char)ox;
+      if (ox > d->rx) d->rx = ox;
+      if (oy > d->ry) d->ry = oy;
+    }
+  return true;
 }
 
 // disk offsets (o != 0) with |o| < r, |o| = sqrt((o_x dx)^2 + (o_y dy)^2)
@@ -277,7 +498,7 @@ struct Carve {
 };
 
 struct Layout2 {
-  size_t occ, par, mis, amp, vg, vr, keys, cl, ca, twx, twy, ktx, kty, P, Q, off_in, off_l, w_l, part, tot, cnt;
+  size_t occ, par, mis, amp, vg, vr, keys, cl, ca, twx, twy, ktx, kty, P, Q, off_in, off_l, w_l, part, tot, cnt, filt;
   size_t total;
   int n_in, n_l, nblk;
 };
@@ -307,9 +528,11 @@ Layout2 carve(int nx, int ny, double dx, double dy, const mhd_gran_params* gp) {
   o.off_in = c.take((size_t)(o.n_in > 0 ? o.n_in : 1) * 8);
   o.off_l = c.take((size_t)o.n_l * 8);
   o.w_l = c.take((size_t)o.n_l * 16);
-  o.part = c.take((size_t)2 * o.nblk * 8);
+  // block sums of the render, then of the last FFT kernel (at most one per row)
+  o.part = c.take((size_t)(o.nblk + (o.nblk > ny ? o.nblk : ny)) * 8);
   o.tot = c.take(2 * 8);
-  o.cnt = c.take(8);
+  o.cnt = c.take(BATCH * 4);
+  o.filt = c.take((size_t)3 * (nx / 2 + 1) * (ny / 2 + 1) * 8);
   o.total = c.off;
   return o;
 }
@@ -328,6 +551,9 @@ struct mhd_gran_ctx {
   GranDev g;
   FFTPlan fp;
   cudaStream_t st;
+  bool tiles;       // the tile kernels serve this plane and these radii
+  Disk din, dl;     // r_inner, r_lane
+  size_t smem_l;    // dynamic shared memory of the tiled render
   long long launches = 0;
   char err[512] = "no error";
 };
@@ -405,6 +631,7 @@ extern "C" int mhd_gran_create(int nx, int ny, double dx, double dy, const mhd_g
   fp.kty = (const double*)(g->ws + o.kty);
   fp.P = (double2*)(g->ws + o.P);
   fp.Q = (double2*)(g->ws + o.Q);
+  fp.filt = (const double*)(g->ws + o.filt);
   fp.p0 = 0;
   fp.knx = M_PI / dx;
   fp.kny = M_PI / dy;
@@ -453,6 +680,15 @@ extern "C" int mhd_gran_create(int nx, int ny, double dx, double dy, const mhd_g
     rc = gcheck(g, cudaMemsetAsync(g->ws + o.par, 0, 4 * N * 8, g->st), "clear granules");
   if (rc == MHD_OK)
     rc = gcheck(g, cudaMemsetAsync(g->ws + o.vg, 0, 4 * N * 8, g->st), "clear fields");
+  if (rc == MHD_OK) {
+    const bool in = disk_rows(gp->r_inner, dx, dy, &g->din), lane = disk_rows(gp->r_lane, dx, dy, &g->dl);
+    g->tiles = in && lane && nx >= TW;
+    g->smem_l = sizeof(double2) * (2 * g->dl.rx + 1) * (2 * g->dl.ry + 1) +
+                sizeof(double) * (TW + 2 * g->dl.rx) * (TH + 2 * g->dl.ry);
+    const int nq = (nx / 2 + 1) * (ny / 2 + 1);
+    filter_kernel<<<(nq + GT - 1) / GT, GT, 0, g->st>>>(fp, (double*)(g->ws + o.filt));
+    rc = gcheck(g, cudaGetLastError(), "filter table");
+  }
   if (rc == MHD_OK) rc = gcheck(g, cudaStreamSynchronize(g->st), "create");
   if (rc != MHD_OK) {
     set_global_error("%s", g->err);
@@ -481,26 +717,39 @@ extern "C" int mhd_gran_update(mhd_gran_handle g, double t, const unsigned int* 
   const double* cl = rc ? nullptr : (const double*)stage(g, c_life, g->o.cl, N * 8, mem, &rc);
   const double* ca = rc ? nullptr : (const double*)stage(g, c_amp, g->o.ca, N * 8, mem, &rc);
   if (rc) return rc;
-  const int nb = g->o.nblk;
-  expire_kernel<<<nb, GT, 0, g->st>>>(g->g, t);
-  seed_kernel<<<nb, GT, 0, g->st>>>(g->g);
-  g->launches += 2;
+  const int nb = g->o.nblk, nl = (int)((N + (size_t)LP * GT - 1) / ((size_t)LP * GT));
+  const dim3 tiles(g->nx / TW, g->ny / TH);
+  if (g->tiles) seed_tile_kernel<<<tiles, GT, 0, g->st>>>(g->g, g->din, t);
+  else seed_kernel<<<nb, GT, 0, g->st>>>(g->g, t);
+  g->launches += 1;
   // each round the first undecided pixel in (key, index) order joins, so
-  // N + 1 rounds always suffice
+  // N + 1 rounds always suffice.  The host reads the undecided counts once per
+  // batch of rounds (a steady update takes about three rounds).
   int r = 0, left = 1;
   while (left > 0) {
     if (r > (int)N) return gfail(g, MHD_ERR_TIMEOUT, "placement did not settle in %d rounds", r);
-    rc = gcheck(g, cudaMemsetAsync(g->g.cnt, 0, 4, g->st), "clear count");
+    rc = gcheck(g, cudaMemsetAsync(g->g.cnt, 0, BATCH * 4, g->st), "clear count");
     if (rc) return rc;
-    join_kernel<<<nb, GT, 0, g->st>>>(g->g, k);
-    exclude_kernel<<<nb, GT, 0, g->st>>>(g->g);
-    g->launches += 2;
-    rc = gcheck(g, cudaMemcpyAsync(&left, g->g.cnt, 4, cudaMemcpyDeviceToHost, g->st), "read count");
+    for (int b = 0; b < BATCH; ++b) {
+      if (g->tiles) {
+        join_tile_kernel<<<tiles, GT, 0, g->st>>>(g->g, g->din, k, b);
+        exclude_tile_kernel<<<tiles, GT, 0, g->st>>>(g->g, g->din, b);
+      } else {
+        join_kernel<<<nb, GT, 0, g->st>>>(g->g, k, b);
+        exclude_kernel<<<nb, GT, 0, g->st>>>(g->g, b);
+      }
+    }
+    g->launches += 2 * BATCH;
+    int cnt[BATCH];
+    rc = gcheck(g, cudaMemcpyAsync(cnt, g->g.cnt, sizeof cnt, cudaMemcpyDeviceToHost, g->st), "read count");
     if (rc == MHD_OK) rc = gcheck(g, cudaStreamSynchronize(g->st), "placement round");
     if (rc) return rc;
-    ++r;
+    for (int b = 0; b < BATCH && left > 0; ++b) {
+      left = cnt[b];
+      ++r;
+    }
   }
-  birth_kernel<<<nb, GT, 0, g->st>>>(g->g, g->gp, t, cl, ca);
+  birth_kernel<<<nl, GT, 0, g->st>>>(g->g, g->gp, t, cl, ca);
   g->launches += 1;
   if (rounds) *rounds = r;
   rc = gcheck(g, cudaGetLastError(), "update");
@@ -517,12 +766,12 @@ extern "C" int mhd_gran_velocity(mhd_gran_handle g, double t, int precision, voi
   const size_t N = (size_t)g->nx * g->ny;
   const int nb = g->o.nblk;
   const GranDev& d = g->g;
-  amp_kernel<<<nb, GT, 0, g->st>>>(d, t);
-  render_kernel<<<nb, GT, 0, g->st>>>(d);
-  launch_rotational(g->fp, d.vg, d.vg + N, d.vr, d.vr + N, g->st);
-  combine_kernel<<<nb, GT, 0, g->st>>>(d, g->gp.f_rot, nb);
-  total_kernel<<<1, GT, 0, g->st>>>(d, nb);
-  g->launches += 7;
+  amp_kernel<<<(int)((N + (size_t)LP * GT - 1) / ((size_t)LP * GT)), GT, 0, g->st>>>(d, t);
+  if (g->tiles) render_tile_kernel<<<dim3(g->nx / TW, g->ny / TH), GT, g->smem_l, g->st>>>(d, g->dl);
+  else render_kernel<<<nb, GT, 0, g->st>>>(d);
+  const int nvor = launch_rotational(g->fp, d.vg, d.vg + N, d.vr, d.vr + N, true, g->gp.f_rot, d.part + nb, g->st);
+  total_kernel<<<1, GT, 0, g->st>>>(d, nb, nvor);
+  g->launches += 6;
   // device output straight into v; host output through the FFT's row
   // spectra (2N doubles), free once the column pass has read them
   void* dst = mem == MHD_MEM_DEVICE ? v : (void*)(g->ws + g->o.P);
@@ -562,11 +811,11 @@ extern "C" int mhd_gran_read_field(mhd_gran_handle g, int which, double* dst, in
   if (mem != MHD_MEM_DEVICE && mem != MHD_MEM_HOST) return gfail(g, MHD_ERR_ARG, "bad mem flag");
   const size_t N = (size_t)g->nx * g->ny;
   if (which == 0) return copy_out(g, dst, g->g.vg, 2 * N * 8, mem);
-  // v_rot' is not kept (combine_kernel overwrites it with v_vor): recompute
+  // v_rot' is not kept (the FFT's last kernel adds it to v_gran): recompute
   // it from v_gran into the FFT's row spectra, free once the column pass has
   // read them
-  launch_rotational(g->fp, g->g.vg, g->g.vg + N, (double*)(g->ws + g->o.P), (double*)(g->ws + g->o.P) + N,
-                    g->st);
+  launch_rotational(g->fp, g->g.vg, g->g.vg + N, (double*)(g->ws + g->o.P), (double*)(g->ws + g->o.P) + N, false, 0.0,
+                    nullptr, g->st);
   g->launches += 3;
   int rc = gcheck(g, cudaGetLastError(), "rotational part");
   if (rc) return rc;
