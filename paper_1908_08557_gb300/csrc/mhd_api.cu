@@ -700,8 +700,10 @@ static int upload_fft_tables(mhd_ctx* h, const Offsets& o) {
   for (int axis = 0; axis < 2; ++axis) {
     int n = axis == 0 ? nx : ny;
     for (int r = 0; r < n; ++r) {
-      tw[2 * r] = cos(2.0 * M_PI * r / n);
-      tw[2 * r + 1] = -sin(2.0 * M_PI * r / n);
+      const double2 w = twiddle_pair(cos(2.0 * M_PI * r / n), -sin(2.0 * M_PI * r / n), r,
+                                     axis == 0 ? fp.lognx : fp.logny);
+      tw[2 * r] = w.x;
+      tw[2 * r + 1] = w.y;
     }
     rc = cuda_check(h, cudaMemcpy((void*)(axis == 0 ? fp.twx : fp.twy), tw.data(), (size_t)n * 16,
                                   cudaMemcpyHostToDevice), "upload twiddles");

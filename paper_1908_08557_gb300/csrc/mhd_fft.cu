@@ -29,13 +29,39 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
   return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
+// One radix-2 butterfly with its twiddle, (b0 + w b1, b0 - w b1), in six FP64
+// multiply-adds (four for the product and four for the sums otherwise; the
+// transforms are bound by the FP64 pipe): with w = m (1 + i t) the product is
+// m (u, v), u = x - t y, v = y + t x, and the factor m rides on the sums.
+// Where |Im w| > |Re w| the same with w = i m (1 + i t), i.e. for (-y, x), so
+// that |t| <= 1 and nothing is lost (twiddle_pair, mhd_internal.h).  inv:
+// conjugate twiddle.
+// Signs and swaps go by integer operations (a negated copy can cost an FP64
+// one).
+__device__ __forceinline__ double flip(double x, int sign) {
+  return __hiloint2double(__double2hiint(x) ^ sign, __double2loint(x));
+}
+__device__ __forceinline__ void bfly(double2 b0, double2 b1, double2 w, bool swap, bool inv, double2& s, double2& d) {
+  constexpr int S = (int)0x80000000;
+  const double ny = flip(b1.y, S);
+  const double p = __hiloint2double(swap ? __double2hiint(ny) : __double2hiint(b1.x),
+                                    swap ? __double2loint(ny) : __double2loint(b1.x));
+  const double q = __hiloint2double(swap ? __double2hiint(b1.x) : __double2hiint(b1.y),
+                                    swap ? __double2loint(b1.x) : __double2loint(b1.y));
+  const double t = flip(w.y, inv ? S : 0), m = flip(w.x, inv && swap ? S : 0);
+  const double u = fma(-t, q, p), v = fma(t, p, q);
+  s = make_double2(fma(m, u, b0.x), fma(m, v, b0.y));
+  d = make_double2(fma(-m, u, b0.x), fma(-m, v, b0.y));
+}
+
 // nb lines of n = 2^logn complex points in a (b is scratch of equal size).
 // Stockham autosort, radix 4, with one radix-2 stage first when logn is odd.
 // With p the length of the sub-transforms done so far, radix-4 butterfly
 // i in [0, n/4) has k = i mod p, j = i div p; it takes x[i + m n/4]
 // (m = 0..3) times w^(m k), w = exp(-+2 pi i / (4p)), and writes their
-// 4-point DFT c_q to y[4 j p + k + q p] = y[4i - 3k + q p].  At p = 1 every
-// k is 0 and the twiddles drop out; the radix-2 stage (p = 1) writes
+// 4-point DFT c_q to y[4 j p + k + q p] = y[4i - 3k + q p]; the twiddles
+// enter as two levels of radix-2 butterflies, w^(2k) then w^k.  At p = 1
+// every k is 0 and the twiddles drop out; the radix-2 stage (p = 1) writes
 // x[i] +- x[i + n/2] to y[2i], y[2i + 1].  Returns the buffer holding the
 // (unnormalised) transform.
 __device__ double2* fft_lines(double2* a, double2* b, int n, int logn, int nb, const double2* __restrict__ tw,
@@ -60,6 +86,7 @@ __device__ double2* fft_lines(double2* a, double2* b, int n, int logn, int nb, c
   }
   const int quarter = n >> 2;
   const int total = nb * quarter;
+  const int rs = inverse ? (int)0x80000000 : 0;
   for (; p < n; p <<= 2, lp += 2) {
     const int tws = logn - 2 - lp;  // twiddle index m k n / (4p) = (m k) << tws
     for (int q = threadIdx.x; q < total; q += blockDim.x) {
@@ -67,26 +94,30 @@ __device__ double2* fft_lines(double2* a, double2* b, int n, int logn, int nb, c
       const int i = q & (quarter - 1);
       const int k = i & (p - 1);
       const double2* x = a + line * n + i;
-      double2 b0 = x[0], b1 = x[quarter], b2 = x[2 * quarter], b3 = x[3 * quarter];
-      if (p > 1) {
-        double2 w1 = __ldg(tw + (k << tws)), w2 = __ldg(tw + ((2 * k) << tws)), w3 = __ldg(tw + ((3 * k) << tws));
-        if (inverse) {
-          w1.y = -w1.y;
-          w2.y = -w2.y;
-          w3.y = -w3.y;
-        }
-        b1 = cmul(w1, b1);
-        b2 = cmul(w2, b2);
-        b3 = cmul(w3, b3);
-      }
-      const double2 t0 = cadd(b0, b2), t1 = csub(b0, b2), t2 = cadd(b1, b3), t3 = csub(b1, b3);
-      // -i t3 for the forward transform, +i t3 for the inverse
-      const double2 r3 = inverse ? make_double2(-t3.y, t3.x) : make_double2(t3.y, -t3.x);
+      const double2 b0 = x[0], b1 = x[quarter], b2 = x[2 * quarter], b3 = x[3 * quarter];
       double2* y = b + line * n + 4 * i - 3 * k;
-      y[0] = cadd(t0, t2);
-      y[p] = cadd(t1, r3);
-      y[2 * p] = csub(t0, t2);
-      y[3 * p] = csub(t1, r3);
+      if (p > 1) {
+        const int r1 = k << tws, r2 = (2 * k) << tws;
+        const double2 w1 = __ldg(tw + r1), w2 = __ldg(tw + r2);
+        const bool s1 = twiddle_swap(r1, logn), s2 = twiddle_swap(r2, logn);
+        double2 t0, t1, t2, t3, y0, y1, y2, y3;
+        bfly(b0, b2, w2, s2, inverse, t0, t1);
+        bfly(b1, b3, w2, s2, inverse, t2, t3);
+        bfly(t0, t2, w1, s1, inverse, y0, y2);
+        // -i t3 for the forward transform, +i t3 for the inverse
+        bfly(t1, make_double2(flip(t3.y, rs), flip(t3.x, ~rs & (int)0x80000000)), w1, s1, inverse, y1, y3);
+        y[0] = y0;
+        y[p] = y1;
+        y[2 * p] = y2;
+        y[3 * p] = y3;
+      } else {
+        const double2 t0 = cadd(b0, b2), t1 = csub(b0, b2), t2 = cadd(b1, b3), t3 = csub(b1, b3);
+        const double2 r3 = inverse ? make_double2(-t3.y, t3.x) : make_double2(t3.y, -t3.x);
+        y[0] = cadd(t0, t2);
+        y[p] = cadd(t1, r3);
+        y[2 * p] = csub(t0, t2);
+        y[3 * p] = csub(t1, r3);
+      }
     }
     __syncthreads();
     double2* t = a;
@@ -297,7 +328,7 @@ __global__ void __launch_bounds__(256) rows_inv_kernel(FFTPlan fp, Layout L, R* 
   }
   __syncthreads();
   double2* r = fft_lines(a, b, nx, fp.lognx, nb, fp.twx, true);
-  const double sc = 1.0 / ((double)nx * (double)ny);
+  const double sc = 1.0 / ((double)nx * (double)ny), frs = add.f_rot * sc;
   const int m = o + 1;
   const int ktop = L.nz - 1 + m, kbot = -m;
   for (int q = threadIdx.x; q < nb * nx; q += blockDim.x) {
@@ -305,7 +336,7 @@ __global__ void __launch_bounds__(256) rows_inv_kernel(FFTPlan fp, Layout L, R* 
     const double2 v = r[line * nx + x];
     if (mode == 5) {
       const long long o = (long long)y * nx + x;
-      const double wx = fma(add.f_rot, v.x * sc, add.vx[o]), wy = fma(add.f_rot, v.y * sc, add.vy[o]);
+      const double wx = fma(frs, v.x, add.vx[o]), wy = fma(frs, v.y, add.vy[o]);
       out_re[o] = (R)wx;
       out_im[o] = (R)wy;
       energy = fma(wx, wx, fma(wy, wy, energy));

@@ -644,8 +644,10 @@ extern "C" int mhd_gran_create(int nx, int ny, double dx, double dy, const mhd_g
     const double L = n * (axis == 0 ? dx : dy);
     std::vector<double> tw((size_t)2 * n), k((size_t)n);
     for (int r = 0; r < n; ++r) {
-      tw[2 * r] = cos(2.0 * M_PI * r / n);
-      tw[2 * r + 1] = -sin(2.0 * M_PI * r / n);
+      const double2 w = twiddle_pair(cos(2.0 * M_PI * r / n), -sin(2.0 * M_PI * r / n), r,
+                                     axis == 0 ? fp.lognx : fp.logny);
+      tw[2 * r] = w.x;
+      tw[2 * r + 1] = w.y;
       k[r] = 2.0 * M_PI * (2 * r > n ? r - n : r) / L;
     }
     rc = gcheck(g, cudaMemcpy((void*)(axis == 0 ? fp.twx : fp.twy), tw.data(), (size_t)n * 16,

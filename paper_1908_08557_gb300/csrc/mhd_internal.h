@@ -12,11 +12,19 @@
 
 namespace mhd {
 
+// Twiddle w = c + i s = exp(-2 pi i r / n) as (m, t) with |t| <= 1: w = m (1 + i t)
+// in the octants next to the real axis, w = i m (1 + i t) in the others
+// (twiddle_swap; n = 2^logn >= 8).
+__host__ __device__ __forceinline__ bool twiddle_swap(int r, int logn) { return (((8 * r) >> logn) + 1) & 2; }
+__host__ __device__ __forceinline__ double2 twiddle_pair(double c, double s, int r, int logn) {
+  return twiddle_swap(r, logn) ? make_double2(s, -c / s) : make_double2(c, s / c);
+}
+
 // Potential-field FFT plan: all arrays live in the caller's workspace.
 struct FFTPlan {
   int nx, ny, lognx, logny;
-  const double2* twx;  // exp(-2 pi i r / nx), r < nx
-  const double2* twy;  // exp(-2 pi i r / ny), r < ny
+  const double2* twx;  // twiddles exp(-2 pi i r / nx), r < nx, as twiddle_pair gives them
+  const double2* twy;  // the same for ny
   const double* et;    // [3][kx][ky] exp(-|k| d_m), ghost layer m above the top (Eq. 17)
   const double* eb;    // [3][kx][ky] exp(+f_b |k| d'_m), ghost layer m below the photosphere (Sect. 2.4)
   const double* ktx;   // modified first-derivative wavenumbers, [nx]

@@ -85,7 +85,7 @@ __global__ void static_tables_kernel(unsigned char* base, int nx, int ny, double
       if (r >= n) continue;
       double s, c;
       sincospi(2.0 * (double)r / (double)n, &s, &c);
-      (axis == 0 ? twx : twy)[r] = make_double2(c, -s);
+      (axis == 0 ? twx : twy)[r] = twiddle_pair(c, -s, r, 31 - __clz(n));
       double kt = 0.0;
       if (r != 0 && 2 * r != n) {
         const double a = 2.0 * (double)(2 * r > n ? r - n : r) / (double)n;  // theta / pi
