@@ -38,6 +38,7 @@ struct AdjPointArgs {
   const R* wptab;
   const StepState* ss;
   int sub;
+  bool compact;  // CLA holds the swamp's part alone (for the z-march gather)
 };
 
 template <typename R>
@@ -107,6 +108,7 @@ __global__ void __launch_bounds__(128) adj_point_kernel(AdjPointArgs<R> a) {
   adjoint_cell<R>(c, ph, a.wtab[k], a.wptab[k], wo, dt, k, L.nz, a.dbar + L.at(UX, 0, j, i),
                   a.dbar + L.at(UY, 0, j, i), L.sz(), a.thbar, q2, n2, a.ss, a.sub, cf);
   if (k < ph.nc_k1) nc_adjoint<R>(ph, a.bg, L.nz, k, c.L, c.Th, wo[LT], cf);
+  if (a.compact) coef_swamp_part<R>(ph, a.wtab[k], wo, cf);
   const long long n3 = n2 * L.nz, cq = (long long)k * n2 + q2;
   for (int q = 0; q < NCOEF; ++q) a.coef[q * n3 + cq] = cf[q];
 }
@@ -377,10 +379,11 @@ void launch_d2r(const double* in, R* out, long long n, cudaStream_t st) {
 // ---------------------------------------------------------------------------
 template <typename R>
 void launch_adj_point(const Layout& L, const Phys<R>& ph, const Background<R>& bg, const R* g, const R* dbar, R* coef,
-                      double* thbar, const R* wtab, const R* wptab, const StepState* ss, int sub, cudaStream_t st) {
+                      double* thbar, const R* wtab, const R* wptab, const StepState* ss, int sub, bool compact,
+                      cudaStream_t st) {
   AdjPointArgs<R> a;
   a.L = L; a.ph = ph; a.bg = bg; a.g = g; a.dbar = dbar; a.coef = coef; a.thbar = thbar;
-  a.wtab = wtab; a.wptab = wptab; a.ss = ss; a.sub = sub;
+  a.wtab = wtab; a.wptab = wptab; a.ss = ss; a.sub = sub; a.compact = compact;
   dim3 blk(32, 4, 1), grd((L.nx + 31) / 32, (L.ny + 3) / 4, L.nz);
   adj_point_kernel<R><<<grd, blk, 0, st>>>(a);
 }
@@ -417,7 +420,7 @@ void launch_bz_plane(int nx, int ny, int nz, int k, double dx, double dy, const 
 
 #define INST(R)                                                                                                    \
   template void launch_adj_point<R>(const Layout&, const Phys<R>&, const Background<R>&, const R*, const R*, R*,     \
-                                    double*, const R*, const R*, const StepState*, int, cudaStream_t);             \
+                                    double*, const R*, const R*, const StepState*, int, bool, cudaStream_t);       \
   template void launch_adj_gather<R>(const Layout&, const Phys<R>&, const R*, const R*, R*, const StepState*,       \
                                      cudaStream_t);                                                               \
   template void launch_adj_bc<R>(const Layout&, const Phys<R>&, const Background<R>&, const R*, R*, R,             \

@@ -172,6 +172,24 @@ __device__ __forceinline__ void rhs_point_adjoint(const Cell<R>& c, const Phys<R
   cf[CGL + 0] += bgL0; cf[CGL + 1] += bgL1; cf[CGL + 2] += bgL2;
 }
 
+// What the z-march gathers read.  Many of the 40 coefficients repeat one
+// another: A enters the right-hand side through B = curl A and J = grad div A -
+// lap A, so away from the swamp layers its nine first-derivative coefficients
+// are +-bB and zero, and its Laplacian ones are -bJ.  Those gathers read bB
+// (slots CDA + 7, CDA + 2, CDA + 3), bJ (CGA), and, on the swamp layers alone,
+// the swamp's own Laplacian coefficients eta_s w (dt D_A) (in CLA) and bdivA
+// (CDA): 31 fields instead of 40.
+__host__ __device__ constexpr bool coef_always(int q) {
+  return q < CDA || q == CDA + 2 || q == CDA + 3 || q == CDA + 7 || (q >= CDU && q < CLA) || q >= CLU;
+}
+__host__ __device__ constexpr bool coef_swamp(int q) { return q == CDA || (q >= CLA && q < CLU); }
+// CLA from the full Laplacian coefficients to the swamp's part of them
+template <typename R>
+__device__ __forceinline__ void coef_swamp_part(const Phys<R>& ph, R w_, const R wo[NF], R (&cf)[NCOEF]) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) cf[CLA + c] = ph.eta_s * w_ * wo[c];
+}
+
 // Adjoint of one interior cell's right-hand-side row in substep `sub`.  wo
 // holds dt * D at the cell on entry (D: adjoint of the RK accumulator); rows
 // the boundary overwrites carry no dependence and are masked; the nudging

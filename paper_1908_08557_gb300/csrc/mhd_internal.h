@@ -128,7 +128,7 @@ void launch_rk_tiled(const CUtensorMap* tm, const Layout& L, const Phys<float>& 
 void launch_adj_point_tiled(const CUtensorMap* tm, const Layout& L, const Phys<float>& ph,
                             const Background<float>& bg, const float* dbar, float* coef, double* thbar,
                             const float* wtab, const float* wptab, StepState* ss, int sub, double dx, double dy,
-                            double dz, cudaStream_t st);
+                            double dz, bool compact, cudaStream_t st);
 // tensor map of one padded FP32 state set (dims mx, my, mz, 8 fields) whose box is
 // one plane (box_x x box_y x 1; default a 32 x 8 tile with its halo, 40 x 14)
 // of box_fields consecutive fields
@@ -162,7 +162,7 @@ void launch_adj_point_pair(const CUtensorMap* tm, const CUtensorMap* tmd, const 
 constexpr int NCOEF_ADJ = 40;
 template <typename R> void launch_adj_point(const Layout& L, const Phys<R>& ph, const Background<R>& bg, const R* g,
                                             const R* dbar, R* coef, double* thbar, const R* wtab, const R* wptab,
-                                            const StepState* ss, int sub, cudaStream_t st);
+                                            const StepState* ss, int sub, bool compact, cudaStream_t st);
 template <typename R> void launch_adj_gather(const Layout& L, const Phys<R>& ph, const R* coef, const R* dbar,
                                              R* gbar, const StepState* ss, cudaStream_t st);
 // tiled gather (needs adj_gather_tiled_ok): folds the in-plane grad-div terms into the
@@ -172,12 +172,16 @@ bool adj_gather_tiled_ok(const Layout& L);
 template <typename R> void launch_adj_gather_tiled(const Layout& L, const Phys<R>& ph, R* coef, R* dbar, R* gbar,
                                                    R* fbar, double alpha, double beta, int klo, int khi,
                                                    const StepState* ss, cudaStream_t st);
-// the same contract as a z-march over coefficient planes (coef is not modified): a
-// CTA stages one output group's 20 coefficient fields plane by plane and
-// scatters the z stencils into a register ring (needs adj_gather_tiled_ok)
-template <typename R> void launch_adj_gather_zm(const Layout& L, const Phys<R>& ph, const R* coef, R* dbar, R* gbar,
-                                                R* fbar, double alpha, double beta, int klo, int khi, StepState* ss,
-                                                cudaStream_t st);
+// the same contract from the 31 coefficients of coef_always (and, on layers k >=
+// ksw, those of coef_swamp): FP32 as a z-march over coefficient planes, FP64 a
+// warp per output layer (coef is not modified; needs adj_gather_tiled_ok and
+// nx, ny powers of two)
+void launch_adj_gather_zm(const Layout& L, const Phys<float>& ph, const float* coef, float* dbar, float* gbar,
+                          float* fbar, double alpha, double beta, int klo, int khi, int ksw, StepState* ss,
+                          cudaStream_t st);
+void launch_adj_gather64(const Layout& L, const Phys<double>& ph, const double* coef, double* dbar, double* gbar,
+                         double* fbar, double alpha, double beta, int klo, int khi, int ksw, const StepState* ss,
+                         cudaStream_t st);
 template <typename R> void launch_adj_bc(const Layout& L, const Phys<R>& ph, const Background<R>& bg, const R* g,
                                          R* gbar, R dz, const StepState* ss, cudaStream_t st);
 // adjoint elementwise update F += G, D = alpha D + beta F,

@@ -368,9 +368,11 @@ __global__ void __launch_bounds__(NT, 2) rk64_kernel(const __grid_constant__ Arg
         adjoint_cell<double>(c, ph, w, wp, wo, dt, k, L.nz, a.dbar + L.at(UX, 0, j, i), a.dbar + L.at(UY, 0, j, i),
                              L.sz(), a.thbar, q2, n2, a.ss, sub, cf);
         if (k < ph.nc_k1) nc_adjoint<double>(ph, a.bg, L.nz, k, lr, th, wo[LT], cf);
+        coef_swamp_part<double>(ph, w, wo, cf);
         double* co = a.coef + (long long)k * n2 + q2;
 #pragma unroll
-        for (int q = 0; q < NCOEF; ++q) co[q * n3] = cf[q];
+        for (int q = 0; q < NCOEF; ++q)
+          if (coef_always(q) || (coef_swamp(q) && k >= a.bg.ksw)) co[q * n3] = cf[q];
       } else {
         const double T = exp(th), rho1 = exp(-lr);
         double out[NF];

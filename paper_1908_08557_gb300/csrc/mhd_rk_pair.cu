@@ -261,8 +261,16 @@ __device__ __forceinline__ void adjoint_centre(const Args& a, const float* Pk, c
       cf[CV + LR] += wo[LT] * P2(make_float2(dL0, dL1));
     }
     float* co = a.coef + (long long)k * n2 + (long long)j * L.nx + i;
+    // the 31 coefficients the gather reads, four more on the swamp layers
 #pragma unroll
-    for (int q = 0; q < NCOEF; ++q) *reinterpret_cast<f2*>(co + q * n3) = cf[q].v;
+    for (int q = 0; q < NCOEF; ++q)
+      if (coef_always(q)) *reinterpret_cast<f2*>(co + q * n3) = cf[q].v;
+    if (k >= a.bg.ksw) {
+      coef_swamp_part<P2>(pp, P2(wk), wo, cf);
+#pragma unroll
+      for (int q = 0; q < NCOEF; ++q)
+        if (coef_swamp(q)) *reinterpret_cast<f2*>(co + q * n3) = cf[q].v;
+    }
     return;
   }
   // photosphere: one cell at a time (nudging rows, FP64 driver adjoints)
@@ -298,9 +306,11 @@ __device__ __forceinline__ void adjoint_centre(const Args& a, const float* Pk, c
     adjoint_cell<float>(cl, a.ph, wk, wpk, wo, dt, k, L.nz, a.dbar + cu, a.dbar + cu + L.fs, L.sz(), a.thbar, q2,
                         n2, a.ss, sub, cf);
     if (k < a.ph.nc_k1) nc_adjoint<float>(a.ph, a.bg, L.nz, k, cl.L, cl.Th, wo[LT], cf);
+    coef_swamp_part<float>(a.ph, wk, wo, cf);
     float* co = a.coef + (long long)k * n2 + q2;
 #pragma unroll
-    for (int q = 0; q < NCOEF; ++q) co[q * n3] = cf[q];
+    for (int q = 0; q < NCOEF; ++q)
+      if (coef_always(q) || (coef_swamp(q) && k >= a.bg.ksw)) co[q * n3] = cf[q];
   }
 }
 

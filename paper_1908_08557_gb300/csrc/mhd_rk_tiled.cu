@@ -69,6 +69,7 @@ struct Args {
   // NCOEF coefficient fields ([NCOEF][nz][ny][nx]) and the driver adjoints out
   const float* dbar;
   float* coef;
+  bool compact;  // CLA holds the swamp's part alone (for the z-march gather)
   double* thbar;
   float c1x, c2x, c3x, c1y, c2y, c3y, c1z, c2z, c3z;   // D1 weights / spacing
   float e0x, e1x, e2x, e3x, e0y, e1y, e2y, e3y, e0z, e1z, e2z, e3z;  // D2 weights / spacing^2
@@ -294,6 +295,7 @@ __global__ void __launch_bounds__(TILE, 1) rk_tiled_kernel(const __grid_constant
           adjoint_cell<float>(c, a.ph, a.wtab[k], a.wptab[k], wo, dt, k, L.nz, a.dbar + cu, a.dbar + cu + L.fs,
                               L.sz(), a.thbar, q2, n2, a.ss, sub, cf);
           if (k < a.ph.nc_k1) nc_adjoint<float>(a.ph, a.bg, L.nz, k, c.L, c.Th, wo[LT], cf);
+          if (a.compact) coef_swamp_part<float>(a.ph, a.wtab[k], wo, cf);
           float* co = a.coef + (long long)k * n2 + q2;
           const long long n3 = n2 * L.nz;
 #pragma unroll
@@ -453,10 +455,11 @@ void launch_rk_tiled(const CUtensorMap* tm, const Layout& L, const Phys<float>& 
 void launch_adj_point_tiled(const CUtensorMap* tm, const Layout& L, const Phys<float>& ph,
                             const Background<float>& bg, const float* dbar, float* coef, double* thbar,
                             const float* wtab, const float* wptab, StepState* ss, int sub, double dx, double dy,
-                            double dz, cudaStream_t st) {
+                            double dz, bool compact, cudaStream_t st) {
   Args a = tiled_args(L, ph, bg, wtab, wptab, ss, sub, dx, dy, dz);
   a.dbar = dbar;
   a.coef = coef;
+  a.compact = compact;
   a.thbar = thbar;
   tiled::rk_tiled_kernel<true><<<tiled_grid(a), dim3(tiled::TX, tiled::TY), tiled::SMEM_BYTES, st>>>(*tm, a);
 }
