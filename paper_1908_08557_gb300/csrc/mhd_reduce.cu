@@ -9,6 +9,14 @@
 
 namespace mhd {
 
+__device__ __forceinline__ long long warp_max_bits(long long v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long u = __shfl_xor_sync(0xffffffffu, v, o);
+    v = u > v ? u : v;
+  }
+  return v;
+}
 __device__ __forceinline__ double warp_max(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -155,6 +163,84 @@ __global__ void __launch_bounds__(256) cfl_partial_kernel(Layout L, Phys<R> ph, 
   }
 }
 
+// The FP64 state: one cell per thread, rows of 32 in blocks of four.  Bound by
+// the FP64 pipe, so what counts is the number of FP64 operations (about 95 a
+// cell; 123 in the pair form above) and, in small boxes, their spread: the six
+// end layers of a 32^3 box took 23 us on 24 blocks of 256 threads.  The
+// conduction term grows with 2.5 ln T - ln rho at a fixed layer, so its maximum
+// takes one exponential per block, and maxima are compared as integers (the
+// bits of non-negative doubles order like integers; ordered_bits extends that
+// to either sign).
+__device__ __forceinline__ long long ordered_bits(double x) {
+  const long long b = __double_as_longlong(x);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double from_ordered(long long b) {
+  return __longlong_as_double(b ^ ((b >> 63) & 0x7fffffffffffffffll));
+}
+constexpr int C64Y = 4;
+__global__ void __launch_bounds__(32 * C64Y) cfl64_kernel(Layout L, Phys<double> ph, Background<double> bg,
+                                                          const double* __restrict__ f,
+                                                          const double* __restrict__ wtab, double* partial,
+                                                          StepState* ss, double sqinv2, int k0, int nlo, int kgap) {
+  __shared__ long long sa[C64Y], sd[C64Y];
+  const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * C64Y + threadIdx.y;
+  const int k = k0 + (int)blockIdx.z + ((int)blockIdx.z >= nlo ? kgap : 0);
+  if (halted(ss)) return;
+  const bool zg = bg.zm1 != nullptr;
+  const double idzk = zg ? bg.zm1[k] : ph.idz;
+  long long mar = 0, mq = ordered_bits(-1e300);
+  if (i < L.nx && j < L.ny) {
+    const int sy = L.mx, sz = L.mx * L.my;
+    const double* px = f + L.at(AX, k, j, i);
+    const double *py = px + L.fs, *pz = py + L.fs;
+    // 60 h D1
+    auto d = [](const double* p, int s) {
+      return fma(45.0, __ldg(p + s) - __ldg(p - s),
+                 fma(-9.0, __ldg(p + 2 * s) - __ldg(p - 2 * s), __ldg(p + 3 * s) - __ldg(p - 3 * s)));
+    };
+    const double cx = ph.idx * (1.0 / 60.0), cy = ph.idy * (1.0 / 60.0), cz = idzk * (1.0 / 60.0);
+    double B0 = fma(cy, d(pz, sy), fma(-cz, d(py, sz), ph.bext[0]));
+    double B1 = fma(cz, d(px, sz), fma(-cx, d(pz, 1), ph.bext[1]));
+    double B2 = fma(cx, d(py, 1), fma(-cy, d(px, sy), ph.bext[2]));
+    if (bg.bB) {
+      // A stored about a background: its curl per cell
+      const long long n2 = (long long)L.nx * L.ny, n3 = n2 * L.nz, q3 = (long long)k * n2 + (long long)j * L.nx + i;
+      B0 += bg.bB[q3];
+      B1 += bg.bB[n3 + q3];
+      B2 += bg.bB[2 * n3 + q3];
+    }
+    const double* pu = pz + L.fs;
+    const double lr = bg.lbar[k + NG] + __ldg(pu + 3 * L.fs), lt = bg.tbar[k + NG] + __ldg(pu + 4 * L.fs);
+    const double b2 = fma(B0, B0, fma(B1, B1, B2 * B2));
+    const double c2 = fma(b2, exp(-lr), ph.gamma * exp(lt));
+    const double sqk = zg ? sqrt(ph.idx2 + ph.idy2 + idzk * idzk) : sqinv2;
+    const double adv = fma(sqrt(c2), sqk, fma(fabs(__ldg(pu)), ph.idx, fma(fabs(__ldg(pu + L.fs)), ph.idy,
+                                                                           fabs(__ldg(pu + 2 * L.fs)) * idzk)));
+    const double q = fma(2.5, lt, -lr);
+    if (!isfinite(adv) || !isfinite(q)) atomicOr(&ss->nonfinite, 1);
+    mar = __double_as_longlong(adv);
+    mq = ordered_bits(q);
+  }
+  mar = warp_max_bits(mar);
+  mq = warp_max_bits(mq);
+  if (threadIdx.x == 0) { sa[threadIdx.y] = mar; sd[threadIdx.y] = mq; }
+  __syncthreads();
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
+    for (int w = 1; w < C64Y; ++w) {
+      mar = sa[w] > mar ? sa[w] : mar;
+      mq = sd[w] > mq ? sd[w] : mq;
+    }
+    const double w = wtab[k], kt = ph.gm1 * ph.kappa0 * exp(from_ordered(mq));
+    double dm = fmax(fmax(ph.nu, ph.eta + ph.eta_s * w), fmax(ph.drho + ph.drho_s * w, ph.chi_s * w + kt));
+    if (zg) dm *= ph.idx2 + ph.idy2 + idzk * idzk;
+    if (!isfinite(dm)) atomicOr(&ss->nonfinite, 1);
+    const int b = ((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) & (CFL_SLOTS - 1);
+    atomicMax((unsigned long long*)&partial[2 * b], (unsigned long long)mar);
+    atomicMax((unsigned long long*)&partial[2 * b + 1], (unsigned long long)__double_as_longlong(dm));
+  }
+}
+
 template <typename R>
 int launch_cfl_partial(const Layout& L, const Phys<R>& ph, const Background<R>& bg, const R* f, const R* wtab,
                        double* partial, StepState* ss, CflPlanes planes, bool zero, cudaStream_t st) {
@@ -170,6 +256,10 @@ int launch_cfl_partial(const Layout& L, const Phys<R>& ph, const Background<R>& 
   const int nk = planes == CflPlanes::ends ? 2 * NG : nlo;
   if (nk > 0) {
     R s2 = (R)sqrt((double)ph.idx2 + (double)ph.idy2 + (double)ph.idz2);
+    if constexpr (sizeof(R) == 8)
+      cfl64_kernel<<<dim3((L.nx + 31) / 32, (L.ny + C64Y - 1) / C64Y, nk), dim3(32, C64Y), 0, st>>>(
+          L, ph, bg, f, wtab, partial, ss, s2, k0, nlo, kgap);
+    else
     cfl_partial_kernel<R><<<dim3((L.nx + 63) / 64, (L.ny + 7) / 8, nk), dim3(32, 8), 0, st>>>(
         L, ph, bg, f, wtab, partial, ss, s2, k0, nlo, kgap);
   }
@@ -179,45 +269,63 @@ int launch_cfl_partial(const Layout& L, const Phys<R>& ph, const Background<R>& 
 // dt = min(C_adv / max adv, C_diff / max(D_max) / sum 1/dx_i^2) (or dt_fixed);
 // then the substep times t + c_s dt with their ramp r and driver weight s
 // (Sect. 2.3: linear switch-on, linear interpolation between snapshots).
+// Bound by latency (one block, dependent FP64 divisions): the maxima are taken
+// as integers, and each substep's time and weights by a thread of its own.
 __global__ void cfl_finalize_kernel(const double* partial, int nblk, StepState* ss, double c_adv,
                                     double c_diff, double dt_fixed, double inv2sum, double t0, double t1,
                                     double t_ramp, int probe) {
-  __shared__ double sa[32], sd[32];
-  double ma = 0.0, md = 0.0;
+  __shared__ long long sa[32], sd[32];
+  __shared__ double s_dt;
+  __shared__ int s_stop;
+  const long long* bits = (const long long*)partial;  // non-negative doubles
+  long long ma = 0, md = 0;
   for (int b = threadIdx.x; b < nblk; b += blockDim.x) {
-    ma = fmax(ma, partial[2 * b]);
-    md = fmax(md, partial[2 * b + 1]);
+    const long long va = bits[2 * b], vd = bits[2 * b + 1];
+    ma = va > ma ? va : ma;
+    md = vd > md ? vd : md;
   }
-  ma = warp_max(ma);
-  md = warp_max(md);
+  ma = warp_max_bits(ma);
+  md = warp_max_bits(md);
   if ((threadIdx.x & 31) == 0) { sa[threadIdx.x >> 5] = ma; sd[threadIdx.x >> 5] = md; }
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  for (int w = 1; w < (int)(blockDim.x >> 5); ++w) { ma = fmax(ma, sa[w]); md = fmax(md, sd[w]); }
-  double dt;
-  if (dt_fixed > 0.0) {
-    dt = dt_fixed;
-  } else {
-    const double d1 = ma > 0.0 ? c_adv / ma : INFINITY;
-    const double d2 = md > 0.0 ? c_diff / (md * inv2sum) : INFINITY;
-    dt = d1 < d2 ? d1 : d2;
-  }
-  if (!(dt > 0.0) || !isfinite(dt)) ss->nonfinite = 1;
-  if (probe) { ss->probe_dt = dt; return; }
-  if (ss->nonfinite) return;
   const double t = ss->t;
-  ss->dt = dt;
-  for (int s = 0; s < 3; ++s) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
+      ma = sa[w] > ma ? sa[w] : ma;
+      md = sd[w] > md ? sd[w] : md;
+    }
+    const double a = __longlong_as_double(ma), d = __longlong_as_double(md);
+    double dt;
+    if (dt_fixed > 0.0) {
+      dt = dt_fixed;
+    } else {
+      const double d1 = a > 0.0 ? c_adv / a : INFINITY;
+      const double d2 = d > 0.0 ? c_diff / (d * inv2sum) : INFINITY;
+      dt = d1 < d2 ? d1 : d2;
+    }
+    if (!(dt > 0.0) || !isfinite(dt)) ss->nonfinite = 1;
+    if (probe) ss->probe_dt = dt;
+    s_dt = dt;
+    s_stop = probe || ss->nonfinite;
+  }
+  __syncthreads();
+  if (s_stop) return;
+  const double dt = s_dt;
+  if (threadIdx.x == 0) {
+    ss->dt = dt;
+    ss->t = t + dt;
+    ss->step += 1;
+  }
+  if (threadIdx.x % 32 == 0 && threadIdx.x / 32 < 3) {  // one warp per substep
+    const int s = threadIdx.x / 32;
     const double ts = t + rk_c(s) * dt;
     ss->tsub[s] = ts;
     double r = 1.0;
     if (t_ramp > 0.0) r = fmin(fmax(ts / t_ramp, 0.0), 1.0);
-    double q = t1 > t0 ? (ts - t0) / (t1 - t0) : 0.0;
+    const double q = t1 > t0 ? (ts - t0) / (t1 - t0) : 0.0;
     ss->r[s] = r;
     ss->s[s] = fmin(fmax(q, 0.0), 1.0);
   }
-  ss->t = t + dt;
-  ss->step += 1;
 }
 
 void launch_cfl_finalize(const double* partial, int nblk, StepState* ss, double c_adv, double c_diff,
