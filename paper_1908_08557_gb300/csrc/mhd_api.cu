@@ -499,16 +499,25 @@ static int upload_background(mhd_ctx* h, const double* lnrho0, const double* lnT
 }
 
 // ---- launch sequence ----------------------------------------------------------
+// whether the boundary chain of this handle is a row of kernels on its stream
+// alone, each of which may be launched behind its predecessor (not while
+// events are recorded between them)
+static bool one_chain(const mhd_ctx* h) {
+  return !h->prof && (h->p.bc_z == 1 || pfe_one_chain(h->p.nx, h->p.ny));
+}
+
+// chained: a kernel was launched on the handle's stream right before
 template <typename R>
-static void ghost_fill(mhd_ctx* h, R* f) {
+static void ghost_fill(mhd_ctx* h, R* f, bool chained = false) {
   Phys<R> ph = make_phys<R>(&h->p);
+  const bool one = one_chain(h);
   {
     ClassTimer ct(h, MHD_KC_GHOST, 1);
-    launch_bc<R>(h->L, ph, bgr<R>(h), f, h->ss, h->st);
+    launch_bc<R>(h->L, ph, bgr<R>(h), f, h->ss, h->st, chained && one);
   }
   if (h->p.bc_z == 0) {
     ClassTimer ct(h, MHD_KC_PFE, 3);
-    launch_pfe<R>(h->fp, h->L, f, h->ss, h->st, h->serial ? nullptr : &h->ps);
+    launch_pfe<R>(h->fp, h->L, f, h->ss, h->st, h->serial ? nullptr : &h->ps, one);
   }
 }
 
@@ -565,7 +574,8 @@ static Driver kernel_driver(const mhd_ctx* h) {
 // tmin: the tensor map of fin when fin is not one of the handle's two state
 // sets (a tape of substep states)
 template <typename R>
-static void launch_rk_any(mhd_ctx* h, const R* fin, R* fout, int sub, const CUtensorMap* tmin = nullptr) {
+static void launch_rk_any(mhd_ctx* h, const R* fin, R* fout, int sub, const CUtensorMap* tmin = nullptr,
+                          bool chained = false) {
   Phys<R> ph = make_phys<R>(&h->p);
   Driver drv = kernel_driver(h);
   if (sizeof(R) == 4 && h->pair) {
@@ -574,7 +584,7 @@ static void launch_rk_any(mhd_ctx* h, const R* fin, R* fout, int sub, const CUte
     // (unit spacing) and the kernel applies the metric per layer
     launch_rk_pair(tmin ? tmin : &h->tm[which], &h->tmdf, h->L, *(const Phys<float>*)&ph, h->bgf, (float*)fout, (float*)h->df,
                    (const float*)h->wtab, (const float*)h->wptab, drv, h->ss, sub, h->p.dx, h->p.dy,
-                   h->p.z ? 1.0 : h->p.dz, h->st, h->dbg_skip_plane, h->dbg_wait_limit);
+                   h->p.z ? 1.0 : h->p.dz, h->st, h->dbg_skip_plane, h->dbg_wait_limit, chained);
     h->dbg_skip_plane = INT_MIN;  // one launch only
     return;
   }
@@ -594,7 +604,7 @@ static void launch_rk_any(mhd_ctx* h, const R* fin, R* fout, int sub, const CUte
   }
   if (sizeof(R) == 8 && h->rk64) {
     launch_rk64(h->L, *(const Phys<double>*)&ph, h->bgd, (const double*)fin, (double*)fout, (double*)h->df,
-                (const double*)h->wtab, (const double*)h->wptab, drv, h->ss, sub, h->st);
+                (const double*)h->wtab, (const double*)h->wptab, drv, h->ss, sub, h->st, chained);
     return;
   }
   launch_rk<R>(h->L, ph, bgr<R>(h), fin, fout, (R*)h->df, (const R*)h->wtab, (const R*)h->wptab, drv, h->ss, sub,
@@ -652,7 +662,7 @@ static void run_step(mhd_ctx* h, bool stats) {
       launch_cfl_finalize(h->cfl, nb, h->ss, h->p.c_adv, h->p.c_diff, h->p.dt_fixed, inv2sum(&h->p), h->t0,
                           h->t1, h->p.t_ramp, 0, h->st);
     } else {
-      ghost_fill<R>(h, fin);
+      ghost_fill<R>(h, fin, sub > 0);
       if (sub == 0) {
         if (stats) run_stats<R>(h, fin);
         const bool zmarch = adaptive && sizeof(R) == 4 && h->pair && h->L.nz > 2 * NG;
@@ -672,7 +682,7 @@ static void run_step(mhd_ctx* h, bool stats) {
     }
     {
       ClassTimer ct(h, MHD_KC_RK, 1);
-      launch_rk_any<R>(h, fin, fout, sub);
+      launch_rk_any<R>(h, fin, fout, sub, nullptr, one_chain(h));
     }
     h->cur = 1 - h->cur;
   }

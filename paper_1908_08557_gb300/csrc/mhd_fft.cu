@@ -134,11 +134,11 @@ __device__ double2* fft_lines(double2* a, double2* b, int n, int logn, int nb, c
 // the ghost adjoints of A_c at the top layer nz-1+m (real) and at -m
 // (imaginary); mode 3: the complex plane dre + i dim (FP64 inputs).
 template <typename R>
-__global__ void __launch_bounds__(256) rows_fwd_kernel(FFTPlan fp, Layout L, const R* __restrict__ f,
-                                                       const R* __restrict__ src2d, int mode,
-                                                       const StepState* ss, int nb, const double* __restrict__ dre,
-                                                       const double* __restrict__ dim) {
+__global__ void __launch_bounds__(256) rows_fwd_kernel(FFTPlan fp, Layout L, const R* f, const R* src2d, int mode,
+                                                       const StepState* ss, int nb, const double* dre,
+                                                       const double* dim) {
   extern __shared__ double2 sm[];
+  chain_enter();
   if (ss && halted(ss)) return;
   const int nx = fp.nx, ny = fp.ny;
   const int y0 = blockIdx.x * nb;
@@ -193,6 +193,7 @@ __global__ void __launch_bounds__(256) rows_fwd_kernel(FFTPlan fp, Layout L, con
 // three (the spectrum is kept).
 __global__ void __launch_bounds__(256) cols_kernel(FFTPlan fp, int mode, const StepState* ss, int ppb, int lg) {
   extern __shared__ double2 sm[];
+  chain_enter();
   if (ss && halted(ss)) return;
   const int nx = fp.nx, ny = fp.ny;
   const int npairs = nx / 2 + 1;
@@ -311,9 +312,10 @@ struct RowsAdd {  // mode 5
 };
 
 template <typename R>
-__global__ void __launch_bounds__(256) rows_inv_kernel(FFTPlan fp, Layout L, R* __restrict__ f, R* out_re,
+__global__ void __launch_bounds__(256) rows_inv_kernel(FFTPlan fp, Layout L, R* f, R* out_re,
                                                        R* out_im, int mode, const StepState* ss, int nb, RowsAdd add) {
   extern __shared__ double2 sm[];
+  chain_enter();
   double energy = 0.0;
   if (ss && halted(ss)) return;
   const int nx = fp.nx, ny = fp.ny;
@@ -393,6 +395,7 @@ __global__ void __launch_bounds__(256) rows_inv_kernel(FFTPlan fp, Layout L, R* 
 // fp.P, output plane c in fp.Q.
 __global__ void __launch_bounds__(256) cols_adj_kernel(FFTPlan fp, const StepState* ss, int ppb) {
   extern __shared__ double2 sm[];
+  chain_enter();
   if (ss && halted(ss)) return;
   const int nx = fp.nx, ny = fp.ny;
   const int npairs = nx / 2 + 1;
@@ -524,22 +527,30 @@ static RowsCfg rows_cfg(const FFTPlan& fp, int planes) {
   return c;
 }
 
+bool pfe_one_chain(int nx, int ny) { return nx * ny <= 8192; }
+
 template <typename R>
 void launch_pfe(const FFTPlan& fp, const Layout& L, R* f, const StepState* ss, cudaStream_t st,
-                const PlaneStreams* ps) {
+                const PlaneStreams* ps, bool chained) {
   set_smem_once();
   const int npairs = fp.nx / 2 + 1;
   const FFTLaunch l = fft_launch(fp, 3);
   // small planes are bound by launches and latency, not by the FP64 pipe: the
   // three planes go as one chain (64 x 64, ten steps: 2.06 -> 1.95 ms; at
   // 128 x 128 three chains are 2 % faster, at 256 x 256 5 %)
-  if (!ps || fp.nx * fp.ny <= 8192) {
+  if (!ps || pfe_one_chain(fp.nx, fp.ny)) {
     const RowsCfg rf = rows_cfg(fp, 3), ri = rows_cfg(fp, 9);
-    rows_fwd_kernel<R><<<dim3(fp.ny / rf.nb, 3), rf.threads, rf.smem, st>>>(fp, L, f, nullptr, 0, ss, rf.nb,
-                                                                            nullptr, nullptr);
-    cols_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 3), l.threads3, l.smem_cols3, st>>>(fp, 0, ss, l.ppb, l.lg);
-    rows_inv_kernel<R><<<dim3(fp.ny / ri.nb, 3, 3), ri.threads, ri.smem, st>>>(fp, L, f, nullptr, nullptr, 0, ss,
-                                                                              ri.nb, RowsAdd{});
+    const double* none = nullptr;
+    R* nout = nullptr;
+    launch_chained(chained, rows_fwd_kernel<R>, dim3(fp.ny / rf.nb, 3), rf.threads, rf.smem, st, fp, L, f, nout, 0, ss,
+                   rf.nb, none, none);
+    // (at 128 x 128 and above the waiting blocks of the successors cost more
+    // than the launches they hide: 17 -> 23 us a kernel)
+    const bool small = pfe_one_chain(fp.nx, fp.ny);
+    launch_chained(small, cols_kernel, dim3((npairs + l.ppb - 1) / l.ppb, 3), l.threads3, l.smem_cols3, st, fp, 0, ss,
+                   l.ppb, l.lg);
+    launch_chained(small, rows_inv_kernel<R>, dim3(fp.ny / ri.nb, 3, 3), ri.threads, ri.smem, st, fp, L, f, nout, nout,
+                   0, ss, ri.nb, RowsAdd{});
     return;
   }
   // one chain (rows, columns, inverse rows) per packed plane, on its own
@@ -631,9 +642,9 @@ template void launch_pfe_adjoint<double>(const FFTPlan&, const Layout&, double*,
 template void launch_atarget_adjoint<float>(const FFTPlan&, const double*, const double*, float*, cudaStream_t);
 template void launch_atarget_adjoint<double>(const FFTPlan&, const double*, const double*, double*, cudaStream_t);
 template void launch_pfe<float>(const FFTPlan&, const Layout&, float*, const StepState*, cudaStream_t,
-                                const PlaneStreams*);
+                                const PlaneStreams*, bool);
 template void launch_pfe<double>(const FFTPlan&, const Layout&, double*, const StepState*, cudaStream_t,
-                                 const PlaneStreams*);
+                                 const PlaneStreams*, bool);
 template void launch_atarget<float>(const FFTPlan&, const float*, float*, float*, cudaStream_t);
 template void launch_atarget<double>(const FFTPlan&, const double*, double*, double*, cudaStream_t);
 

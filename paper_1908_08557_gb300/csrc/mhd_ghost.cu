@@ -28,8 +28,8 @@ namespace mhd {
 // threads with both ends in a thread took 19 us on 6 SMs).
 constexpr int BC_TH = 64;
 template <typename R>
-__global__ void __launch_bounds__(BC_TH) bc_kernel(Layout L, Phys<R> ph, Background<R> bg, R* __restrict__ f,
-                                                   const StepState* ss) {
+__global__ void __launch_bounds__(BC_TH) bc_kernel(Layout L, Phys<R> ph, Background<R> bg, R* f, const StepState* ss) {
+  chain_enter();
   const int pw = L.nx + 2 * NG, phh = L.ny + 2 * NG;
   const int q = blockIdx.x * BC_TH + threadIdx.x;
   if (q >= pw * phh) return;
@@ -84,9 +84,9 @@ __global__ void __launch_bounds__(BC_TH) bc_kernel(Layout L, Phys<R> ph, Backgro
 
 template <typename R>
 void launch_bc(const Layout& L, const Phys<R>& ph, const Background<R>& bg, R* f, const StepState* ss,
-               cudaStream_t st) {
+               cudaStream_t st, bool chained) {
   int n = (L.nx + 2 * NG) * (L.ny + 2 * NG);
-  bc_kernel<R><<<dim3((n + BC_TH - 1) / BC_TH, 2), BC_TH, 0, st>>>(L, ph, bg, f, ss);
+  launch_chained(chained, bc_kernel<R>, dim3((n + BC_TH - 1) / BC_TH, 2), BC_TH, 0, st, L, ph, bg, f, ss);
 }
 
 // interior [field][nz][ny][nx] <-> padded; the background is added on the
@@ -353,7 +353,7 @@ void launch_layer_mean(const Layout& L, const R* in, int field, double* out, cud
 
 #define INST(R)                                                                               \
   template void launch_bc<R>(const Layout&, const Phys<R>&, const Background<R>&, R*,          \
-                             const StepState*, cudaStream_t);                                  \
+                             const StepState*, cudaStream_t, bool);                            \
   template void launch_pack<R>(const Layout&, const Background<R>&, const R*, R*, int, cudaStream_t); \
   template void launch_adj_pack<R>(const Layout&, int, const R*, R*, cudaStream_t);           \
   template void launch_adj_unpack<R>(const Layout&, const R*, R*, R*, double, cudaStream_t);  \

@@ -87,17 +87,53 @@ inline int sm_count() {
   return n;
 }
 
+// Launch of a kernel that may be scheduled before its predecessor in the stream
+// has finished (programmatic dependent launch); it begins with chain_enter(),
+// which waits for the predecessor's end and memory.  The boundary chain of a
+// small box is a row of short kernels, and this hides their launch latency.
+// Only where the predecessor is a kernel launched right before on the same
+// stream; other work in between (events, copies) takes a plain launch.
+template <typename... P, typename... A>
+inline void launch_chained(bool chained, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                           const A&... a) {
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &at;
+  c.numAttrs = chained ? 1 : 0;
+  cudaLaunchKernelEx(&c, k, P(a)...);
+}
+#ifdef __CUDACC__
+// Wait for the predecessor of a chained launch, then let the successor's blocks
+// be scheduled.  A successor's blocks so start when all of this grid's blocks
+// have passed here, hence after everything before this grid has ended: at most
+// two neighbours of a chain are ever in flight together.  (Kernels that use it
+// take their array pointers without __restrict__ and do not read arrays a
+// predecessor writes by non-coherent loads, which could be moved above it.)
+__device__ __forceinline__ void chain_enter() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
+
 constexpr int FFT_PTS = 2048;          // complex points per shared buffer
 constexpr int RED_BLOCKS_MAX = 4096;   // partial-reduction slots
 constexpr int CFL_SLOTS = 256;         // CFL maxima slot pairs (after the partials)
 
 // ghost fill
 template <typename R> void launch_bc(const Layout& L, const Phys<R>& ph, const Background<R>& bg, R* f,
-                                     const StepState* ss, cudaStream_t st);
+                                     const StepState* ss, cudaStream_t st, bool chained = false);
 // potential-field ghosts of A (three FFT kernels)
 // (ps: run the three planes on three streams; nullptr: one stream)
 template <typename R> void launch_pfe(const FFTPlan& fp, const Layout& L, R* f, const StepState* ss,
-                                      cudaStream_t st, const PlaneStreams* ps = nullptr);
+                                      cudaStream_t st, const PlaneStreams* ps = nullptr, bool chained = false);
+// planes small enough to go as one chain of kernels whatever ps says
+bool pfe_one_chain(int nx, int ny);
 // vector potential of the target magnetogram into axt, ayt
 template <typename R> void launch_atarget(const FFTPlan& fp, const R* bz, R* axt, R* ayt, cudaStream_t st);
 // filtered rotational part (Eq. 3) of the plane field (vx, vy) into (rx, ry),
@@ -115,7 +151,7 @@ template <typename R> void launch_rk(const Layout& L, const Phys<R>& ph, const B
 // mixed ones (mhd_rk64.cu), and the FP64 pointwise adjoint on it
 void launch_rk64(const Layout& L, const Phys<double>& ph, const Background<double>& bg, const double* fin,
                  double* fout, double* df, const double* wtab, const double* wptab, const Driver& drv,
-                 const StepState* ss, int sub, cudaStream_t st);
+                 const StepState* ss, int sub, cudaStream_t st, bool chained = false);
 void launch_adj_point64(const Layout& L, const Phys<double>& ph, const Background<double>& bg, const double* g,
                         const double* dbar, double* coef, double* thbar, const double* wtab, const double* wptab,
                         const StepState* ss, int sub, cudaStream_t st);
@@ -151,7 +187,7 @@ bool rk_pair_supported(const Layout& L);
 void launch_rk_pair(const CUtensorMap* tm, const CUtensorMap* tmd, const Layout& L, const Phys<float>& ph, const Background<float>& bg,
                     float* fout, float* df, const float* wtab, const float* wptab, const Driver& drv, StepState* ss,
                     int sub, double dx, double dy, double dz, cudaStream_t st, int skip_plane = INT_MIN,
-                    int wait_limit = 0);
+                    int wait_limit = 0, bool chained = false);
 // pointwise adjoint of substep sub on the same z-march (tm: the ghost-filled
 // substep state, tmd: D, the adjoint of the RK accumulator, 32 x 8 tiles)
 void launch_adj_point_pair(const CUtensorMap* tm, const CUtensorMap* tmd, const Layout& L, const Phys<float>& ph,

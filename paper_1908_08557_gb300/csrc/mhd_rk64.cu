@@ -80,26 +80,26 @@ __device__ __forceinline__ double comb2(double c, double a1, double b1, double a
 }
 // first difference along stride s; first and second
 template <typename I>
-__device__ __forceinline__ double dd1(const double* __restrict__ p, I s) {
-  return comb1(__ldg(p + s), __ldg(p - s), __ldg(p + 2 * s), __ldg(p - 2 * s), __ldg(p + 3 * s), __ldg(p - 3 * s));
+__device__ __forceinline__ double dd1(const double* p, I s) {
+  return comb1(p[s], p[-s], p[2 * s], p[-2 * s], p[3 * s], p[-3 * s]);
 }
 template <typename I>
-__device__ __forceinline__ double dd12(const double* __restrict__ p, I s, double c, double& d2) {
-  const double a1 = __ldg(p + s), b1 = __ldg(p - s), a2 = __ldg(p + 2 * s), b2 = __ldg(p - 2 * s),
-               a3 = __ldg(p + 3 * s), b3 = __ldg(p - 3 * s);
+__device__ __forceinline__ double dd12(const double* p, I s, double c, double& d2) {
+  const double a1 = p[s], b1 = p[-s], a2 = p[2 * s], b2 = p[-2 * s],
+               a3 = p[3 * s], b3 = p[-3 * s];
   d2 = comb2(c, a1, b1, a2, b2, a3, b3);
   return comb1(a1, b1, a2, b2, a3, b3);
 }
 template <typename I>
-__device__ __forceinline__ double dd2(const double* __restrict__ p, I s, double c) {
-  return comb2(c, __ldg(p + s), __ldg(p - s), __ldg(p + 2 * s), __ldg(p - 2 * s), __ldg(p + 3 * s),
-               __ldg(p - 3 * s));
+__device__ __forceinline__ double dd2(const double* p, I s, double c) {
+  return comb2(c, p[s], p[-s], p[2 * s], p[-2 * s], p[3 * s],
+               p[-3 * s]);
 }
 __device__ __forceinline__ double ds1(const double* p) {
   return comb1(p[1], p[-1], p[2], p[-2], p[3], p[-3]);
 }
 
-__device__ __forceinline__ void put_images(const Layout& L, double* __restrict__ f, int fl, int k, int j, int i,
+__device__ __forceinline__ void put_images(const Layout& L, double* f, int fl, int k, int j, int i,
                                            double v) {
   int xs[3], ys[3], nxs = 1, nys = 1;
   xs[0] = i;
@@ -119,6 +119,7 @@ template <bool ADJ, bool ZG>
 __global__ void __launch_bounds__(NT, 2) rk64_kernel(const __grid_constant__ Args a) {
   __shared__ double src[KZ + 2 * NG][NSRC][TX];
   __shared__ double scr_all[KZ][NSC][SW];
+  chain_enter();
   if (halted(a.ss)) return;
   const Layout& L = a.L;
   const Phys<double>& ph = a.ph;
@@ -174,7 +175,7 @@ __global__ void __launch_bounds__(NT, 2) rk64_kernel(const __grid_constant__ Arg
     // y differences of A_y, A_x, u_y, u_x of the row, with the x halo
     double dyAx = 0.0, yyAx = 0.0, dyUx = 0.0, yyUx = 0.0;
     if (near) {
-      const double ca = __ldg(f + AX * fs), cu = __ldg(f + UX * fs);
+      const double ca = f[AX * fs], cu = f[UX * fs];
       dyAx = dd12(f + AX * fs, sy, ca, yyAx);
       dyUx = dd12(f + UX * fs, sy, cu, yyUx);
       double* sc = scr + tx + NG;
@@ -214,9 +215,9 @@ __global__ void __launch_bounds__(NT, 2) rk64_kernel(const __grid_constant__ Arg
       double A0, A1, B[3], J[3], sw[3] = {0.0, 0.0, 0.0};
       {
         const double *pa = f + AX * fs, *pb = f + AY * fs, *pc = f + AZ * fs;
-        A0 = __ldg(pa);
-        A1 = __ldg(pb);
-        const double A2 = __ldg(pc);
+        A0 = *pa;
+        A1 = *pb;
+        const double A2 = *pc;
         double zz;
         double dzA = dd12(pa, sz, A0, zz);
         B[1] = fma(cz, dzA, fma(-C.cx, cur[0], ph.bext[1]));
@@ -272,9 +273,9 @@ __global__ void __launch_bounds__(NT, 2) rk64_kernel(const __grid_constant__ Arg
       double u[3], dU[3][3], vis[3] = {0.0, 0.0, 0.0};
       {
         const double *pa = f + UX * fs, *pb = f + UY * fs, *pc = f + UZ * fs;
-        u[0] = __ldg(pa);
-        u[1] = __ldg(pb);
-        u[2] = __ldg(pc);
+        u[0] = *pa;
+        u[1] = *pb;
+        u[2] = *pc;
         dU[0][0] = ax_[1];
         dU[0][1] = C.cy * dyUx;
         dU[1][1] = ax_[2];
@@ -308,7 +309,7 @@ __global__ void __launch_bounds__(NT, 2) rk64_kernel(const __grid_constant__ Arg
       double lr, th, gL[3], gT[3], lapL = 0.0, lapT;
       {
         const double* p = f + LR * fs;
-        const double c = __ldg(p);
+        const double c = *p;
         lr = a.bg.lbar[k + NG] + c;
         if constexpr (ADJ) {
           gL[0] = C.cx * dd1(p, 1);
@@ -326,7 +327,7 @@ __global__ void __launch_bounds__(NT, 2) rk64_kernel(const __grid_constant__ Arg
       }
       {
         const double* p = f + LT * fs;
-        const double c = __ldg(p);
+        const double c = *p;
         th = a.bg.tbar[k + NG] + c;
         double xx, yy, zz;
         gT[0] = C.cx * dd12(p, 1, c, xx);
@@ -443,7 +444,7 @@ __global__ void __launch_bounds__(NT, 2) rk64_kernel(const __grid_constant__ Arg
           const double dfn = sub > 0 ? fma(alpha, a.df[q], dt * out[fl]) : dt * out[fl];
           if (sub < 2) a.df[q] = dfn;
           if (!eval) {
-            const double v = fma(beta, dfn, __ldg(f + fl * fs));
+            const double v = fma(beta, dfn, f[fl * fs]);
             if (edge) put_images(L, a.fout, fl, k, j, i, v);
             else a.fout[q] = v;
           }
@@ -501,7 +502,7 @@ static Coef64 coef64(const Phys<double>& ph, bool zg) {
 
 void launch_rk64(const Layout& L, const Phys<double>& ph, const Background<double>& bg, const double* fin,
                  double* fout, double* df, const double* wtab, const double* wptab, const Driver& drv,
-                 const StepState* ss, int sub, cudaStream_t st) {
+                 const StepState* ss, int sub, cudaStream_t st, bool chained) {
   r64::Args a{};
   a.L = L;
   a.ph = ph;
@@ -520,8 +521,8 @@ void launch_rk64(const Layout& L, const Phys<double>& ph, const Background<doubl
   const bool zg = bg.zm1 != nullptr;
   a.c = r64::coef64(ph, zg);
   const dim3 g = r64::grid64(L), b(r64::TX, r64::KZ);
-  if (zg) r64::rk64_kernel<false, true><<<g, b, 0, st>>>(a);
-  else r64::rk64_kernel<false, false><<<g, b, 0, st>>>(a);
+  if (zg) launch_chained(chained, r64::rk64_kernel<false, true>, g, b, 0, st, a);
+  else launch_chained(chained, r64::rk64_kernel<false, false>, g, b, 0, st, a);
 }
 
 void launch_adj_point64(const Layout& L, const Phys<double>& ph, const Background<double>& bg, const double* g,

@@ -340,6 +340,7 @@ __global__ void __launch_bounds__(NT, 2) rk_pair_kernel(const __grid_constant__ 
 
   const Layout& L = a.L;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, warp = tid >> 5;
+  chain_enter();
   if (halted(a.ss)) return;
   if (tid == 0) {
     for (int s = 0; s < NR; ++s) zm::mbar_init(&mbar[s]);
@@ -915,7 +916,7 @@ static pair::Args pair_args(const Layout& L, const Phys<float>& ph, const Backgr
 void launch_rk_pair(const CUtensorMap* tm, const CUtensorMap* tmd, const Layout& L, const Phys<float>& ph,
                     const Background<float>& bg, float* fout, float* df, const float* wtab, const float* wptab,
                     const Driver& drv, StepState* ss, int sub, double dx, double dy, double dz, cudaStream_t st,
-                    int skip_plane, int wait_limit) {
+                    int skip_plane, int wait_limit, bool chained) {
   pair::Args a = pair_args(L, ph, bg, wtab, wptab, ss, sub, dx, dy, dz);
   if (skip_plane != INT_MIN) {
     a.skip_plane = skip_plane;
@@ -938,15 +939,19 @@ void launch_rk_pair(const CUtensorMap* tm, const CUtensorMap* tmd, const Layout&
   const int opt = (ph.nc_k1 > 0 ? 1 : 0) | (bg.bB != nullptr ? 2 : 0) | (bg.zm1 != nullptr ? 4 : 0);
   const dim3 g(grid), b(pair::NT);
   if (a.dyn) cudaMemsetAsync(&ss->items, 0, sizeof(int), st);
+  chained = chained && !a.dyn;
+  auto go = [&](void (*k)(const CUtensorMap, const CUtensorMap, const pair::Args)) {
+    launch_chained(chained, k, g, b, pair::SMEM_BYTES, st, *tm, *tmd, a);
+  };
   switch (opt) {
-    case 0: pair::rk_pair_kernel<false, false, false, false><<<g, b, pair::SMEM_BYTES, st>>>(*tm, *tmd, a); break;
-    case 1: pair::rk_pair_kernel<false, true, false, false><<<g, b, pair::SMEM_BYTES, st>>>(*tm, *tmd, a); break;
-    case 2: pair::rk_pair_kernel<false, false, true, false><<<g, b, pair::SMEM_BYTES, st>>>(*tm, *tmd, a); break;
-    case 3: pair::rk_pair_kernel<false, true, true, false><<<g, b, pair::SMEM_BYTES, st>>>(*tm, *tmd, a); break;
-    case 4: pair::rk_pair_kernel<false, false, false, true><<<g, b, pair::SMEM_BYTES, st>>>(*tm, *tmd, a); break;
-    case 5: pair::rk_pair_kernel<false, true, false, true><<<g, b, pair::SMEM_BYTES, st>>>(*tm, *tmd, a); break;
-    case 6: pair::rk_pair_kernel<false, false, true, true><<<g, b, pair::SMEM_BYTES, st>>>(*tm, *tmd, a); break;
-    default: pair::rk_pair_kernel<false, true, true, true><<<g, b, pair::SMEM_BYTES, st>>>(*tm, *tmd, a); break;
+    case 0: go(pair::rk_pair_kernel<false, false, false, false>); break;
+    case 1: go(pair::rk_pair_kernel<false, true, false, false>); break;
+    case 2: go(pair::rk_pair_kernel<false, false, true, false>); break;
+    case 3: go(pair::rk_pair_kernel<false, true, true, false>); break;
+    case 4: go(pair::rk_pair_kernel<false, false, false, true>); break;
+    case 5: go(pair::rk_pair_kernel<false, true, false, true>); break;
+    case 6: go(pair::rk_pair_kernel<false, false, true, true>); break;
+    default: go(pair::rk_pair_kernel<false, true, true, true>); break;
   }
 }
 
