@@ -64,11 +64,11 @@ __device__ __forceinline__ void gather(const Args& a, double (*tz)[3][TX], doubl
   }
   auto P = [&](int q, int p) { return a.coef + q * n3 + (long long)p * n2 + (long long)j * nx + ic; };
   auto d1 = [&](const double* p, const int (&o)[7]) {
-    return comb1(__ldg(p + o[4]), __ldg(p + o[2]), __ldg(p + o[5]), __ldg(p + o[1]), __ldg(p + o[6]), __ldg(p + o[0]));
+    return comb1(p[o[4]], p[o[2]], p[o[5]], p[o[1]], p[o[6]], p[o[0]]);
   };
   auto d2 = [&](const double* p, const int (&o)[7]) {
-    return comb2(__ldg(p), __ldg(p + o[4]), __ldg(p + o[2]), __ldg(p + o[5]), __ldg(p + o[1]), __ldg(p + o[6]),
-                 __ldg(p + o[0]));
+    return comb2(p[0], p[o[4]], p[o[2]], p[o[5]], p[o[1]], p[o[6]],
+                 p[o[0]]);
   };
   constexpr int QX = GRP == 0 ? CGA : CLU, QY = QX + 1, QZ = QX + 2;  // bJ, or the Laplacian coefficients of u
   constexpr double g = GRP == 0 ? 1.0 : 1.0 / 3.0;
@@ -77,13 +77,13 @@ __device__ __forceinline__ void gather(const Args& a, double (*tz)[3][TX], doubl
     yQ = d1(P(QY, p), yo);
     const double xq = d1(P(QZ, p), xo), yq = d1(P(QZ, p), yo), dv = fma(a.cx, d1(P(QX, p), xo), a.cy * yQ);
     if (GRP == 0) {
-      t[0] = fma(-a.cx, xq, __ldg(P(CDA + 2, p)));
-      t[1] = -fma(a.cy, yq, __ldg(P(CDA + 7, p)));
-      t[2] = p >= a.ksw ? __ldg(P(CDA, p)) - dv : -dv;
+      t[0] = fma(-a.cx, xq, *P(CDA + 2, p));
+      t[1] = -fma(a.cy, yq, *P(CDA + 7, p));
+      t[2] = p >= a.ksw ? *P(CDA, p) - dv : -dv;
     } else {
-      t[0] = fma(-g * a.cx, xq, __ldg(P(CDU + 2, p)));
-      t[1] = fma(-g * a.cy, yq, __ldg(P(CDU + 5, p)));
-      t[2] = fma(-g, dv, __ldg(P(CDU + 8, p)));
+      t[0] = fma(-g * a.cx, xq, *P(CDU + 2, p));
+      t[1] = fma(-g * a.cy, yq, *P(CDU + 5, p));
+      t[2] = fma(-g, dv, *P(CDU + 8, p));
     }
   };
   double yQ = 0.0;
@@ -123,7 +123,7 @@ __device__ __forceinline__ void gather(const Args& a, double (*tz)[3][TX], doubl
                          tz[w][c][tx]);
   auto zcol = [&](int q, int m) {  // coefficient q at plane k + m, zero outside
     const int p = k + m;
-    return p >= 0 && p < nz ? __ldg(P(q, p)) : 0.0;
+    return p >= 0 && p < nz ? *P(q, p) : 0.0;
   };
   auto zz = [&](int q) {
     return comb2(zcol(q, 0), zcol(q, 1), zcol(q, -1), zcol(q, 2), zcol(q, -2), zcol(q, 3), zcol(q, -3));
@@ -140,7 +140,7 @@ __device__ __forceinline__ void gather(const Args& a, double (*tz)[3][TX], doubl
       for (int c = 0; c < 3; ++c) {
         auto sc = [&](int m) {
           const int p = k + m;
-          return p >= a.ksw && p < nz ? __ldg(P(CLA + c, p)) : 0.0;
+          return p >= a.ksw && p < nz ? *P(CLA + c, p) : 0.0;
         };
         v[c] = fma(a.ez, comb2(sc(0), sc(1), sc(-1), sc(2), sc(-2), sc(3), sc(-3)), v[c]);
       }
@@ -173,13 +173,13 @@ __device__ __forceinline__ void gather(const Args& a, double (*tz)[3][TX], doubl
         const double wx = c == 0 ? f43 * a.ex : a.ex, wy = c == 1 ? f43 * a.ey : a.ey;
         v[c] += fma(wx, d2(P(QX + c, k), xo), fma(wy, d2(P(QX + c, k), yo),
                 fma(-a.cx, d1(P(CDU + 3 * c, k), xo), fma(-a.cy, d1(P(CDU + 3 * c + 1, k), yo),
-                                                          __ldg(P(CV + UX + c, k))))));
+                                                          *P(CV + UX + c, k)))));
       }
       v[0] = fma(g * a.cxy, xyY, v[0]);
       v[1] = fma(g * a.cxy, xyX, v[1]);
     }
     v[3] += fma(a.ex, d2(P(QL, k), xo), fma(a.ey, d2(P(QL, k), yo),
-            fma(-a.cx, d1(P(QG, k), xo), fma(-a.cy, d1(P(QG + 1, k), yo), __ldg(P(QV, k))))));
+            fma(-a.cx, d1(P(QG, k), xo), fma(-a.cy, d1(P(QG + 1, k), yo), *P(QV, k)))));
   }
   // the substep's update, or G with the nudging's value adjoints
   const bool fz = k >= a.klo && k < a.khi;
@@ -205,6 +205,7 @@ __device__ __forceinline__ void gather(const Args& a, double (*tz)[3][TX], doubl
 __global__ void __launch_bounds__(NT, 2) gather64_kernel(const __grid_constant__ Args a) {
   __shared__ double tz[KZ + 2 * NG][3][TX];
   __shared__ double scr[KZ][2][SW];
+  chain_enter();
   if (halted(a.ss)) return;
   const int k0 = (int)(blockIdx.z >> 1) * KZ - NG;
   if (blockIdx.z & 1) gather<1>(a, tz, scr[threadIdx.y], k0);
@@ -215,7 +216,7 @@ __global__ void __launch_bounds__(NT, 2) gather64_kernel(const __grid_constant__
 
 void launch_adj_gather64(const Layout& L, const Phys<double>& ph, const double* coef, double* dbar, double* gbar,
                          double* fbar, double alpha, double beta, int klo, int khi, int ksw, const StepState* ss,
-                         cudaStream_t st) {
+                         cudaStream_t st, bool chained) {
   g64::Args a;
   a.L = L;
   a.coef = coef;
@@ -239,7 +240,7 @@ void launch_adj_gather64(const Layout& L, const Phys<double>& ph, const double* 
   a.ez = ph.idz2 / 90.0;
   a.ss = ss;
   const dim3 grid((L.nx + g64::TX - 1) / g64::TX, L.ny, 2 * ((L.nz + 2 * NG + g64::KZ - 1) / g64::KZ));
-  g64::gather64_kernel<<<grid, dim3(g64::TX, g64::KZ), 0, st>>>(a);
+  launch_chained(chained, g64::gather64_kernel, grid, dim3(g64::TX, g64::KZ), 0, st, a);
 }
 
 }  // namespace mhd

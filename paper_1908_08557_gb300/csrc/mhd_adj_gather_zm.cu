@@ -138,7 +138,7 @@ __device__ __noinline__ void swamp_pair(const Args& a, int p, int j, int i, f2 (
   const int nx = a.L.nx, ny = a.L.ny;
   const long long n2 = (long long)nx * ny, n3 = n2 * a.L.nz;
   const float* base = a.coef + (long long)p * n2;
-  auto at = [&](int q, int jj, int ii) { return __ldg(base + q * n3 + (long long)(jj & (ny - 1)) * nx + (ii & (nx - 1))); };
+  auto at = [&](int q, int jj, int ii) { return base[q * n3 + (long long)(jj & (ny - 1)) * nx + (ii & (nx - 1))]; };
   const float c1[4] = {0.f, W<float>::c1, W<float>::c2, W<float>::c3};
   const float e[4] = {W<float>::e0, W<float>::e1, W<float>::e2, W<float>::e3};
   float r[3][2], v[3][2], d[2];
@@ -366,6 +366,7 @@ __global__ void __launch_bounds__(NT, 2) gather_pair_kernel(const __grid_constan
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* buf = reinterpret_cast<float*>(smem_raw);
   float* scr = buf + NB * PL;
+  chain_enter();
   if (halted(a.ss)) return;
   const int nzo = a.L.nz + 2 * NG;
   const int tiles = a.ntx * a.nty;
@@ -410,7 +411,7 @@ __global__ void __launch_bounds__(NT, 2) gather_pair_kernel(const __grid_constan
 
 void launch_adj_gather_zm(const Layout& L, const Phys<float>& ph, const float* coef, float* dbar, float* gbar,
                           float* fbar, double alpha, double beta, int klo, int khi, int ksw, StepState* ss,
-                          cudaStream_t st) {
+                          cudaStream_t st, bool chained) {
   // persistent CTAs on the current device (shared-memory limit set there)
   static PerDevice<int> per_dev;
   const int ctas = per_dev.get([] {
@@ -452,7 +453,7 @@ void launch_adj_gather_zm(const Layout& L, const Phys<float>& ph, const float* c
   const int grid = nitems < ctas ? nitems : ctas;
   a.dyn = nitems >= 4 * grid;
   if (a.dyn) cudaMemsetAsync(&ss->items, 0, sizeof(int), st);
-  gzm::gather_pair_kernel<<<grid, gzm::NT, gzm::SMEM, st>>>(a);
+  launch_chained(chained && !a.dyn, gzm::gather_pair_kernel, grid, gzm::NT, gzm::SMEM, st, a);
 }
 
 }  // namespace mhd

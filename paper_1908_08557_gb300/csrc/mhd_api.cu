@@ -1479,6 +1479,7 @@ static void adjoint_reverse(mhd_ctx* h, R* const (&S)[3], const CUtensorMap* con
   // tiled gather: it applies the update itself on the layers no ghost rule
   // feeds back into (the ghost-rule transposes touch k < 4 and k >= nz - 4)
   const bool tg = h->adj_tiled && adj_gather_tiled_ok(h->L);
+  const bool one = one_chain(h);
   const bool compact = tg && h->adj_zm;  // point kernel and gather exchange the reduced coefficient set
   int klo = 0, khi = 0;
   if (tg && h->p.nz - NG - 1 > NG + 1) {
@@ -1491,34 +1492,36 @@ static void adjoint_reverse(mhd_ctx* h, R* const (&S)[3], const CUtensorMap* con
   // mhd_adjoint_init starts from D = beta_2 lam).
   for (int s = 2; s >= 0; --s) {
     const double alpha = rk_alpha(s), beta = rk_beta(s > 0 ? s - 1 : 2);
+    const bool behind = one && s < 2;  // the update of the last substep was launched right before
     if (sizeof(R) == 4 && h->adj_pair && compact)
       launch_adj_point_pair(tms[s], &h->tmdbar, h->L, *(const Phys<float>*)&ph, h->bgf, (const float*)h->dbar,
                             (float*)h->coef, h->thbar, (const float*)h->wtab, (const float*)h->wptab, h->ss, s,
-                            h->p.dx, h->p.dy, h->p.dz, h->st);
+                            h->p.dx, h->p.dy, h->p.dz, h->st, behind);
     else if (sizeof(R) == 4 && h->tiled && h->adj_tiled)
       launch_adj_point_tiled(tms[s], h->L, *(const Phys<float>*)&ph, h->bgf, (const float*)h->dbar,
                              (float*)h->coef, h->thbar, (const float*)h->wtab, (const float*)h->wptab, h->ss, s,
                              h->p.dx, h->p.dy, h->p.dz, compact, h->st);
     else if (sizeof(R) == 8 && compact)
       launch_adj_point64(h->L, *(const Phys<double>*)&ph, h->bgd, (const double*)S[s], (const double*)h->dbar,
-                         (double*)h->coef, h->thbar, (const double*)h->wtab, (const double*)h->wptab, h->ss, s, h->st);
+                         (double*)h->coef, h->thbar, (const double*)h->wtab, (const double*)h->wptab, h->ss, s, h->st,
+                         behind);
     else
       launch_adj_point<R>(h->L, ph, bg, S[s], (const R*)h->dbar, (R*)h->coef, h->thbar, (const R*)h->wtab,
                           (const R*)h->wptab, h->ss, s, compact, h->st);
     if (compact && sizeof(R) == 8)
       launch_adj_gather64(h->L, *(const Phys<double>*)&ph, (const double*)h->coef, (double*)h->dbar, (double*)h->gbar,
-                          (double*)h->fbar, alpha, beta, klo, khi, h->ksw, h->ss, h->st);
+                          (double*)h->fbar, alpha, beta, klo, khi, h->ksw, h->ss, h->st, one);
     else if (compact)
       launch_adj_gather_zm(h->L, *(const Phys<float>*)&ph, (const float*)h->coef, (float*)h->dbar, (float*)h->gbar,
-                           (float*)h->fbar, alpha, beta, klo, khi, h->ksw, h->ss, h->st);
+                           (float*)h->fbar, alpha, beta, klo, khi, h->ksw, h->ss, h->st, one);
     else if (tg)
       launch_adj_gather_tiled<R>(h->L, ph, (R*)h->coef, (R*)h->dbar, (R*)h->gbar, (R*)h->fbar, alpha, beta, klo, khi,
                                  h->ss, h->st);
     else
       launch_adj_gather<R>(h->L, ph, (const R*)h->coef, (const R*)h->dbar, (R*)h->gbar, h->ss, h->st);
-    launch_adj_bc<R>(h->L, ph, bg, S[s], (R*)h->gbar, (R)h->p.dz, h->ss, h->st);
-    launch_pfe_adjoint<R>(fpa, h->L, (R*)h->gbar, h->ss, h->st);
-    launch_adj_update<R>(h->L, (R*)h->fbar, (R*)h->dbar, (const R*)h->gbar, alpha, beta, klo, khi, h->ss, h->st);
+    launch_adj_bc<R>(h->L, ph, bg, S[s], (R*)h->gbar, (R)h->p.dz, h->ss, h->st, one);
+    launch_pfe_adjoint<R>(fpa, h->L, (R*)h->gbar, h->ss, h->st, one);
+    launch_adj_update<R>(h->L, (R*)h->fbar, (R*)h->dbar, (const R*)h->gbar, alpha, beta, klo, khi, h->ss, h->st, one);
     h->nlaunch += (tg && !h->adj_zm) ? 8 : 7;  // point, [fold], gather, bc, 3 FFT, update
   }
 }

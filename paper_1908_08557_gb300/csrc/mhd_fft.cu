@@ -392,8 +392,10 @@ __global__ void __launch_bounds__(256) rows_inv_kernel(FFTPlan fp, Layout L, R* 
 // Adjoint columns: for component c, sum over the three ghost layers m of the
 // extrapolated spectra of the packed ghost adjoints (top real, bottom
 // imaginary), then one inverse FFT along y.  Input planes 3c + m - 1 in
-// fp.P, output plane c in fp.Q.
-__global__ void __launch_bounds__(256) cols_adj_kernel(FFTPlan fp, const StepState* ss, int ppb) {
+// fp.P, output plane c in fp.Q.  lg = 3: the layers' forward transforms as one
+// batch of lines (two buffers of three layers); lg = 1: one after the other
+// (two buffers of a layer and the sum).
+__global__ void __launch_bounds__(256) cols_adj_kernel(FFTPlan fp, const StepState* ss, int ppb, int lg) {
   extern __shared__ double2 sm[];
   chain_enter();
   if (ss && halted(ss)) return;
@@ -401,46 +403,54 @@ __global__ void __launch_bounds__(256) cols_adj_kernel(FFTPlan fp, const StepSta
   const int npairs = nx / 2 + 1;
   const int pair0 = blockIdx.x * ppb;
   const int np = min(ppb, npairs - pair0);
-  const int nl = 2 * np;
+  const int nl = 2 * np, npts = nl * ny;
   const int c = blockIdx.y;
-  const int buf = 2 * ppb * ny;
+  const int buf = lg * 2 * ppb * ny;
   double2* X = sm;
   double2* Y = sm + buf;
-  double2* acc = sm + 2 * buf;
-  for (int q = threadIdx.x; q < nl * ny; q += blockDim.x) acc[q] = make_double2(0.0, 0.0);
-  for (int m = 1; m <= 3; ++m) {
-    const int p = 3 * c + m - 1;
+  double2* acc = sm + 2 * buf;  // lg = 1
+  double2* T = X;
+  for (int m0 = 0; m0 < 3; m0 += lg) {
     __syncthreads();
-    for (int q = threadIdx.x; q < nl * ny; q += blockDim.x) {
-      const int line = q / ny, y = q - line * ny;
+    for (int q = threadIdx.x; q < lg * npts; q += blockDim.x) {
+      const int m = q / npts, qq = q - m * npts;
+      const int line = qq / ny, y = qq - line * ny;
       const int kx = pair0 + (line >> 1);
       const int col = (line & 1) ? ((nx - kx) & (nx - 1)) : kx;
-      X[line * ny + y] = fp.P[((long long)p * nx + col) * ny + y];
+      X[q] = fp.P[((long long)(3 * c + m0 + m) * nx + col) * ny + y];
     }
     __syncthreads();
-    double2* spec = fft_lines(X, Y, ny, fp.logny, nl, fp.twy, false);
-    for (int q = threadIdx.x; q < nl * ny; q += blockDim.x) {
+    double2* spec = fft_lines(X, Y, ny, fp.logny, lg * nl, fp.twy, false);
+    if (lg == 3) {
+      acc = spec == X ? Y : X;  // free once transformed
+      T = spec;
+    }
+    for (int q = threadIdx.x; q < npts; q += blockDim.x) {
       const int line = q / ny, ky = q - line * ny;
       const int kx = pair0 + (line >> 1);
       const int col = (line & 1) ? ((nx - kx) & (nx - 1)) : kx;
-      const long long e = (long long)(m - 1) * nx * ny + (long long)col * ny + ky;
-      const double mt = fp.et[e], mb = fp.eb[e];
-      const double2 F = spec[line * ny + ky];
-      const double2 Fm = spec[(line ^ 1) * ny + ((ny - ky) & (ny - 1))];
-      const double ca = 0.5 * (mt + mb), cb = 0.5 * (mt - mb);
-      acc[q].x += ca * F.x + cb * Fm.x;
-      acc[q].y += ca * F.y - cb * Fm.y;
+      const int mir = (line ^ 1) * ny + ((ny - ky) & (ny - 1));
+      double2 s = lg == 3 || m0 == 0 ? make_double2(0.0, 0.0) : acc[q];
+      for (int m = 0; m < lg; ++m) {
+        const long long e = (long long)(m0 + m) * nx * ny + (long long)col * ny + ky;
+        const double mt = fp.et[e], mb = fp.eb[e];
+        const double2 F = spec[m * npts + q], Fm = spec[m * npts + mir];
+        const double ca = 0.5 * (mt + mb), cb = 0.5 * (mt - mb);
+        s.x += ca * F.x + cb * Fm.x;
+        s.y += ca * F.y - cb * Fm.y;
+      }
+      acc[q] = s;
     }
   }
   __syncthreads();
-  double2* r = fft_lines(acc, X, ny, fp.logny, nl, fp.twy, true);
-  for (int q = threadIdx.x; q < nl * ny; q += blockDim.x) {
+  double2* r = fft_lines(acc, T, ny, fp.logny, nl, fp.twy, true);
+  for (int q = threadIdx.x; q < npts; q += blockDim.x) {
     const int line = q / ny, y = q - line * ny;
     const int kx = pair0 + (line >> 1);
     const bool self = (kx == 0 || 2 * kx == nx);
     if ((line & 1) && self) continue;
     const int col = (line & 1) ? ((nx - kx) & (nx - 1)) : kx;
-    fp.Q[((long long)c * nx + col) * ny + y] = r[line * ny + y];
+    fp.Q[((long long)c * nx + col) * ny + y] = r[q];
   }
 }
 
@@ -454,7 +464,7 @@ static void set_smem_once() {
     cudaFuncSetAttribute(rows_inv_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * FFT_PTS * 16);
     cudaFuncSetAttribute(rows_inv_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * FFT_PTS * 16);
     cudaFuncSetAttribute(cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 6 * FFT_PTS * 16);
-    cudaFuncSetAttribute(cols_adj_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * FFT_PTS * 16);
+    cudaFuncSetAttribute(cols_adj_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 6 * FFT_PTS * 16);
     return true;
   });
 }
@@ -609,16 +619,20 @@ int launch_rotational(const FFTPlan& fp, const double* vx, const double* vy, dou
 // the photosphere.  `fp_adj` is the plan with the 9-plane buffer as P and the
 // 3-plane buffer as Q.
 template <typename R>
-void launch_pfe_adjoint(const FFTPlan& fp_adj, const Layout& L, R* gbar, const StepState* ss, cudaStream_t st) {
+void launch_pfe_adjoint(const FFTPlan& fp_adj, const Layout& L, R* gbar, const StepState* ss, cudaStream_t st,
+                        bool chained) {
   set_smem_once();
   const FFTLaunch l = fft_launch(fp_adj, 3);
   const int npairs = fp_adj.nx / 2 + 1;
   const RowsCfg r9 = rows_cfg(fp_adj, 9), r3 = rows_cfg(fp_adj, 3);
-  rows_fwd_kernel<R><<<dim3(fp_adj.ny / r9.nb, 9), r9.threads, r9.smem, st>>>(fp_adj, L, gbar, nullptr, 2, ss, r9.nb,
-                                                                              nullptr, nullptr);
-  cols_adj_kernel<<<dim3((npairs + l.ppb - 1) / l.ppb, 3), l.threads, l.smem_cols, st>>>(fp_adj, ss, l.ppb);
-  rows_inv_kernel<R><<<dim3(fp_adj.ny / r3.nb, 3, 1), r3.threads, r3.smem, st>>>(fp_adj, L, gbar, nullptr, nullptr, 2,
-                                                                                ss, r3.nb, RowsAdd{});
+  const double* none = nullptr;
+  R* nout = nullptr;
+  launch_chained(chained, rows_fwd_kernel<R>, dim3(fp_adj.ny / r9.nb, 9), r9.threads, r9.smem, st, fp_adj, L, gbar, nout,
+                 2, ss, r9.nb, none, none);
+  launch_chained(chained, cols_adj_kernel, dim3((npairs + l.ppb - 1) / l.ppb, 3), l.threads3, l.smem_cols3, st, fp_adj,
+                 ss, l.ppb, l.lg);
+  launch_chained(chained, rows_inv_kernel<R>, dim3(fp_adj.ny / r3.nb, 3, 1), r3.threads, r3.smem, st, fp_adj, L, gbar,
+                 nout, nout, 2, ss, r3.nb, RowsAdd{});
 }
 
 // Transpose of the magnetogram inversion: B_z adjoint (out, [ny][nx]) from
@@ -637,8 +651,9 @@ void launch_atarget_adjoint(const FFTPlan& fp, const double* abx, const double* 
                                                                              r1.nb, RowsAdd{});
 }
 
-template void launch_pfe_adjoint<float>(const FFTPlan&, const Layout&, float*, const StepState*, cudaStream_t);
-template void launch_pfe_adjoint<double>(const FFTPlan&, const Layout&, double*, const StepState*, cudaStream_t);
+template void launch_pfe_adjoint<float>(const FFTPlan&, const Layout&, float*, const StepState*, cudaStream_t, bool);
+template void launch_pfe_adjoint<double>(const FFTPlan&, const Layout&, double*, const StepState*, cudaStream_t,
+                                         bool);
 template void launch_atarget_adjoint<float>(const FFTPlan&, const double*, const double*, float*, cudaStream_t);
 template void launch_atarget_adjoint<double>(const FFTPlan&, const double*, const double*, double*, cudaStream_t);
 template void launch_pfe<float>(const FFTPlan&, const Layout&, float*, const StepState*, cudaStream_t,

@@ -154,7 +154,7 @@ void launch_rk64(const Layout& L, const Phys<double>& ph, const Background<doubl
                  const StepState* ss, int sub, cudaStream_t st, bool chained = false);
 void launch_adj_point64(const Layout& L, const Phys<double>& ph, const Background<double>& bg, const double* g,
                         const double* dbar, double* coef, double* thbar, const double* wtab, const double* wptab,
-                        const StepState* ss, int sub, cudaStream_t st);
+                        const StepState* ss, int sub, cudaStream_t st, bool chained = false);
 // FP32 TMA-fed variant of launch_rk (tensor map of the input state set)
 void launch_rk_tiled(const CUtensorMap* tm, const Layout& L, const Phys<float>& ph, const Background<float>& bg,
                      float* fout, float* df, const float* wtab, const float* wptab, const Driver& drv,
@@ -193,7 +193,7 @@ void launch_rk_pair(const CUtensorMap* tm, const CUtensorMap* tmd, const Layout&
 void launch_adj_point_pair(const CUtensorMap* tm, const CUtensorMap* tmd, const Layout& L, const Phys<float>& ph,
                            const Background<float>& bg, const float* dbar, float* coef, double* thbar,
                            const float* wtab, const float* wptab, StepState* ss, int sub, double dx, double dy,
-                           double dz, cudaStream_t st);
+                           double dz, cudaStream_t st, bool chained = false);
 // adjoint (transposed linearisation of one substep)
 constexpr int NCOEF_ADJ = 40;
 template <typename R> void launch_adj_point(const Layout& L, const Phys<R>& ph, const Background<R>& bg, const R* g,
@@ -214,17 +214,18 @@ template <typename R> void launch_adj_gather_tiled(const Layout& L, const Phys<R
 // nx, ny powers of two)
 void launch_adj_gather_zm(const Layout& L, const Phys<float>& ph, const float* coef, float* dbar, float* gbar,
                           float* fbar, double alpha, double beta, int klo, int khi, int ksw, StepState* ss,
-                          cudaStream_t st);
+                          cudaStream_t st, bool chained = false);
 void launch_adj_gather64(const Layout& L, const Phys<double>& ph, const double* coef, double* dbar, double* gbar,
                          double* fbar, double alpha, double beta, int klo, int khi, int ksw, const StepState* ss,
-                         cudaStream_t st);
+                         cudaStream_t st, bool chained = false);
 template <typename R> void launch_adj_bc(const Layout& L, const Phys<R>& ph, const Background<R>& bg, const R* g,
-                                         R* gbar, R dz, const StepState* ss, cudaStream_t st);
+                                         R* gbar, R dz, const StepState* ss, cudaStream_t st, bool chained = false);
 // adjoint elementwise update F += G, D = alpha D + beta F,
 // skipping interior layers klo <= k < khi; nx must be a multiple of 4 and
 // NF * (nz + 6) * ny * nx / 4 < 2^31
 template <typename R> void launch_adj_update(const Layout& L, R* fbar, R* dbar, const R* gbar, double alpha,
-                                             double beta, int klo, int khi, const StepState* ss, cudaStream_t st);
+                                             double beta, int klo, int khi, const StepState* ss, cudaStream_t st,
+                                             bool chained = false);
 template <typename R> void launch_bz_plane(int nx, int ny, int nz, int k, double dx, double dy, const R* st_in,
                                            R* out, int adjoint, const R* bbar, R* lam, cudaStream_t st);
 // adjoint state <-> interior layout (no background: these are adjoints); on
@@ -236,7 +237,7 @@ template <typename R> void launch_adj_unpack(const Layout& L, const R* in, R* fb
                                              cudaStream_t st);
 template <typename R> void launch_d2r(const double* in, R* out, long long n, cudaStream_t st);
 template <typename R> void launch_pfe_adjoint(const FFTPlan& fp_adj, const Layout& L, R* gbar, const StepState* ss,
-                                              cudaStream_t st);
+                                              cudaStream_t st, bool chained = false);
 template <typename R> void launch_atarget_adjoint(const FFTPlan& fp, const double* abx, const double* aby, R* out,
                                                   cudaStream_t st);
 // A stored about a fixed background (params a_background): FP64 packed

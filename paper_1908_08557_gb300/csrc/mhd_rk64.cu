@@ -527,7 +527,7 @@ void launch_rk64(const Layout& L, const Phys<double>& ph, const Background<doubl
 
 void launch_adj_point64(const Layout& L, const Phys<double>& ph, const Background<double>& bg, const double* g,
                         const double* dbar, double* coef, double* thbar, const double* wtab, const double* wptab,
-                        const StepState* ss, int sub, cudaStream_t st) {
+                        const StepState* ss, int sub, cudaStream_t st, bool chained) {
   r64::Args a{};
   a.L = L;
   a.ph = ph;
@@ -541,7 +541,7 @@ void launch_adj_point64(const Layout& L, const Phys<double>& ph, const Backgroun
   a.coef = coef;
   a.thbar = thbar;
   a.c = r64::coef64(ph, false);
-  r64::rk64_kernel<true, false><<<r64::grid64(L), dim3(r64::TX, r64::KZ), 0, st>>>(a);
+  launch_chained(chained, r64::rk64_kernel<true, false>, r64::grid64(L), dim3(r64::TX, r64::KZ), 0, st, a);
 }
 
 }  // namespace mhd

@@ -958,7 +958,7 @@ void launch_rk_pair(const CUtensorMap* tm, const CUtensorMap* tmd, const Layout&
 void launch_adj_point_pair(const CUtensorMap* tm, const CUtensorMap* tmd, const Layout& L, const Phys<float>& ph,
                            const Background<float>& bg, const float* dbar, float* coef, double* thbar,
                            const float* wtab, const float* wptab, StepState* ss, int sub, double dx, double dy,
-                           double dz, cudaStream_t st) {
+                           double dz, cudaStream_t st, bool chained) {
   pair::Args a = pair_args(L, ph, bg, wtab, wptab, ss, sub, dx, dy, dz);
   a.dbar = dbar;
   a.coef = coef;
@@ -967,7 +967,8 @@ void launch_adj_point_pair(const CUtensorMap* tm, const CUtensorMap* tmd, const 
   const int grid = nitems < pair_ctas() ? nitems : pair_ctas();
   a.dyn = nitems >= 12 * grid;
   if (a.dyn) cudaMemsetAsync(&ss->items, 0, sizeof(int), st);
-  pair::rk_pair_kernel<true, false, false, false><<<grid, pair::NT, pair::SMEM_BYTES, st>>>(*tm, *tmd, a);
+  launch_chained(chained && !a.dyn, pair::rk_pair_kernel<true, false, false, false>, grid, pair::NT, pair::SMEM_BYTES, st,
+                 *tm, *tmd, a);
 }
 
 }  // namespace mhd
