@@ -200,33 +200,47 @@ __global__ void __launch_bounds__(CTH) unpack_kernel(Layout L, Background<R> bg,
     const R* src = in + ((long long)fl * L.nz + (layer ? k : 0)) * n2;
     const long long base = L.at(fl, kg, -NG, -XOFF);
     Vec<R, P> v[CPT];
+    if constexpr (E == P) {
+      // whole vectors throughout, the periodic images too (a vector that holds
+      // one may carry a further cell into the row padding), so that no warp
+      // splits at the row ends; all loads go out before the first is used
+      int off[CPT];
+      bool take[CPT];
 #pragma unroll
-    for (int u = 0; u < CPT; ++u) {
-      const int x = blockIdx.x * (CTH * CPT) + u * CTH + threadIdx.x;
-      if (x >= total) continue;
-      const int r = x / nv, i0 = (x - r * nv) * P - XOFF;
-      int j = r - NG;
-      const bool inrow = j >= 0 && j < L.ny;
-      if (j < 0) j += L.ny;
-      else if (j >= L.ny) j -= L.ny;
-      if (!layer || (ADJ && !inrow)) {
+      for (int u = 0; u < CPT; ++u) {
+        const int x = min((int)blockIdx.x * (CTH * CPT) + u * CTH + (int)threadIdx.x, total - 1);
+        const int r = x / nv, i0 = (x - r * nv) * P - XOFF;
+        int j = r - NG;
+        const bool rim = j < 0 || j >= L.ny;
+        j = j < 0 ? j + L.ny : (j >= L.ny ? j - L.ny : j);
+        take[u] = layer && (ADJ ? !rim && i0 >= 0 && i0 < L.nx : i0 + P > -NG && i0 < L.nx + NG);
+        off[u] = take[u] ? j * L.nx + (i0 < 0 ? i0 + L.nx : (i0 >= L.nx ? i0 - L.nx : i0)) : 0;
+      }
 #pragma unroll
-        for (int e = 0; e < P; ++e) v[u].v[e] = R(0);
-      } else if (E == P && i0 >= 0 && i0 + P <= L.nx) {
-        v[u] = Vec<R, P>::ld(src + (long long)j * L.nx + i0);
-        if (ab) {
-          const Vec<R, P> b = Vec<R, P>::ld(bg.abg + L.at(fl, k, j, i0));
+      for (int u = 0; u < CPT; ++u) v[u] = Vec<R, P>::ld(src + off[u]);
+      if (ab) {
+#pragma unroll
+        for (int u = 0; u < CPT; ++u) {
+          const int j = off[u] / L.nx;
+          const Vec<R, P> b = Vec<R, P>::ld(bg.abg + L.at(fl, k, j, off[u] - j * L.nx));
 #pragma unroll
           for (int e = 0; e < P; ++e) v[u].v[e] -= b.v[e];
-        } else if (!ADJ) {
-#pragma unroll
-          for (int e = 0; e < P; ++e) v[u].v[e] -= sub;
         }
-      } else {
+      }
 #pragma unroll
+      for (int u = 0; u < CPT; ++u)
+#pragma unroll
+        for (int e = 0; e < P; ++e) v[u].v[e] = take[u] ? (ADJ || ab ? v[u].v[e] : v[u].v[e] - sub) : R(0);
+    } else {
+      for (int u = 0; u < CPT; ++u) {
+        const int x = min((int)blockIdx.x * (CTH * CPT) + u * CTH + (int)threadIdx.x, total - 1);
+        const int r = x / nv, i0 = (x - r * nv) * P - XOFF;
+        int j = r - NG;
+        const bool rim = j < 0 || j >= L.ny;
+        j = j < 0 ? j + L.ny : (j >= L.ny ? j - L.ny : j);
         for (int e = 0; e < P; ++e) {
           int i = i0 + e;
-          const bool cell = ADJ ? (i >= 0 && i < L.nx) : (i >= -NG && i < L.nx + NG);
+          const bool cell = layer && (ADJ ? !rim && i >= 0 && i < L.nx : i >= -NG && i < L.nx + NG);
           if (i < 0) i += L.nx;
           else if (i >= L.nx) i -= L.nx;
           R t = R(0);

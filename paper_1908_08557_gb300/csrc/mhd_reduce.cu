@@ -344,22 +344,51 @@ void launch_cfl_finalize(const double* partial, int nblk, StepState* ss, double 
 // the second pass finds every neighbour of its divergence stencil stored,
 // the periodic images being computed from the state's images, bit for bit
 // equal to the interior values they copy.
+// Two x-adjacent cells per thread (pairs from x = -4 on, whole sectors), as in
+// the reductions: one cell per thread was bound by instructions and L1
+// (184 us at 256^3 in FP32 against a floor of 60).
 template <typename R>
 __global__ void __launch_bounds__(256) curl_a_kernel(Layout L, Phys<R> ph, Background<R> bg, const R* __restrict__ f,
                                                      R* __restrict__ bsc) {
-  const int i = (int)(blockIdx.x * 32 + threadIdx.x) - NG, j = (int)(blockIdx.y * 8 + threadIdx.y) - NG;
+  const int i = 2 * (int)(blockIdx.x * 32 + threadIdx.x) - 4, j = (int)(blockIdx.y * 8 + threadIdx.y) - NG;
   const int k = (int)blockIdx.z - NG;
   if (i >= L.nx + NG || j >= L.ny + NG) return;
-  const bool ix = i >= 0 && i < L.nx, jy = j >= 0 && j < L.ny, kz = k >= 0 && k < L.nz;
-  const long long sy = L.sy(), sz = L.sz();
-  const R* ax = f + L.at(AX, k, j, i);
-  const R* ay = f + L.at(AY, k, j, i);
-  const R* az = f + L.at(AZ, k, j, i);
+  const bool jy = j >= 0 && j < L.ny, kz = k >= 0 && k < L.nz;
+  const bool ix = i + 1 >= 0 && i < L.nx;  // a cell of the pair is interior
+  const bool i0 = i >= 0, i1 = i + 1 < L.nx;
+  const int sy = L.mx, sz = (int)L.sz();
   const long long c = L.at(0, k, j, i);
+  const R *ax = f + c, *ay = ax + L.fs, *az = ay + L.fs;
   const R idzk = (kz && bg.zm1) ? bg.zm1[k] : ph.idz;  // dxi/dz of the layer on a non-uniform grid
-  if (ix && jy) bsc[c + 2 * L.fs] = d1(ay, (long long)1, ph.idx) - d1(ax, sy, ph.idy);
-  if (jy && kz) bsc[c] = d1(az, sy, ph.idy) - d1(ay, sz, idzk);
-  if (ix && kz) bsc[c + L.fs] = d1(ax, sz, idzk) - d1(az, (long long)1, ph.idx);
+  auto put = [&](long long o, R v0, R v1, bool w0, bool w1) {
+    using T = typename Pair2<R>::T;
+    if (w0 && w1) {
+      T t;
+      t.x = v0;
+      t.y = v1;
+      *reinterpret_cast<T*>(bsc + o) = t;
+    } else if (w0) {
+      bsc[o] = v0;
+    } else if (w1) {
+      bsc[o + 1] = v1;
+    }
+  };
+  R p0, p1, q0, q1;
+  if (ix && jy) {
+    d1x_pair(ay, ph.idx, p0, p1);
+    d1s_pair(ax, sy, ph.idy, q0, q1);
+    put(c + 2 * L.fs, p0 - q0, p1 - q1, i0, i1);
+  }
+  if (jy && kz) {
+    d1s_pair(az, sy, ph.idy, p0, p1);
+    d1s_pair(ay, sz, idzk, q0, q1);
+    put(c, p0 - q0, p1 - q1, i >= -NG, i + 1 < L.nx + NG);
+  }
+  if (ix && kz) {
+    d1s_pair(ax, sz, idzk, p0, p1);
+    d1x_pair(az, ph.idx, q0, q1);
+    put(c + L.fs, p0 - q0, p1 - q1, i0, i1);
+  }
 }
 
 // Second pass: per block 7 values (sums of rho u^2/2, B^2/2, rho T/(gamma-1),
@@ -368,7 +397,7 @@ __global__ void __launch_bounds__(256) curl_a_kernel(Layout L, Phys<R> ph, Backg
 // sixth-order divergence of the stored curl A, so it measures how far the
 // discrete operators fail to commute; B_ext drops out of it.
 template <typename R>
-__global__ void __launch_bounds__(256) stats_partial_kernel(Layout L, Phys<R> ph, Background<R> bg,
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 0) stats_partial_kernel(Layout L, Phys<R> ph, Background<R> bg,
                                                             const R* __restrict__ f,
                                                             const R* __restrict__ bsc,
                                                             double* partial, int kchunk) {
@@ -458,7 +487,7 @@ __global__ void __launch_bounds__(256) stats_partial_kernel(Layout L, Phys<R> ph
 template <typename R>
 int launch_stats_partial(const Layout& L, const Phys<R>& ph, const Background<R>& bg, const R* f, R* bsc,
                          double* partial, cudaStream_t st) {
-  dim3 gc((L.nx + 2 * NG + 31) / 32, (L.ny + 2 * NG + 7) / 8, L.nz + 2 * NG);
+  dim3 gc((L.nx + NG + 4 + 63) / 64, (L.ny + 2 * NG + 7) / 8, L.nz + 2 * NG);
   curl_a_kernel<R><<<gc, dim3(32, 8), 0, st>>>(L, ph, bg, f, bsc);
   int kchunk;
   dim3 g = red_grid(L, &kchunk);
