@@ -11,17 +11,25 @@
 //  front (plane k + 3): each thread copies its two cells of the 8 fields into
 //    TMEM (ring of 8 planes) and forms the sources of the xz / yz mixed
 //    derivatives -- D1x X_z, D1y X_z, D1x X_x + D1y X_y for X = A, u -- also
-//    into a TMEM ring of 8 planes;
+//    into a TMEM ring of 8 planes, and beside them the horizontal Laplacians
+//    of A_z and u_z, so that the centre reads these two fields' x and y
+//    derivatives back instead of forming them from shared memory again;
 //  centre (plane k): D1z and D2z of the fields and D1z of the mixed sources
-//    from TMEM (tcgen05.ld), x and y derivatives from the shared ring, the xy
-//    mixed derivatives D1x(D1y X_y), D1x(D1y X_x) through a small shared
-//    scratch with an x halo (the tensor-product operator D1x D1y equals
+//    from TMEM (tcgen05.ld), the other x and y derivatives from the shared
+//    ring, the xy mixed derivatives D1x(D1y X_y), D1x(D1y X_x) through a small
+//    shared scratch with an x halo (the tensor-product operator D1x D1y equals
 //    D1y D1x), the pointwise physics, nudging and boundary rows, the
 //    low-storage RK update and the stores (with periodic images).
 //
+// What bounds it: issue and latency at 8 warps per SM (TMEM and shared memory
+// are full), so the count of instructions per cell pair and plane matters, and
+// of shared-memory reads: differences in units of their smallest weight
+// (mhd_pair.cuh), scales and signs folded into multiply-adds.
+//
 // TMEM: each CTA allocates 256 columns; thread t owns lane t.  Columns
 // [0, 128): values, 16 per plane slot (field f, cell c at 2f + c); columns
-// [128, 256): mixed sources, 16 per plane slot (source q, cell c at 2q + c).
+// [128, 256): mixed sources and the two Laplacians, 16 per plane slot (entry
+// q, cell c at 2q + c).
 // The shared ring (> 76 KB per CTA) admits at most two CTAs per SM, so the
 // two allocations never exceed the SM's 512 columns and tcgen05.alloc never
 // waits.  Every exit path deallocates.
@@ -66,7 +74,15 @@ struct Args {
   StepState* ss;
   int sub;
   int ntx, nty, nch, kchunk;
-  Coef cx, cy, cz;
+  // scales of the differences, as pairs: D1 = s* d with s = 1 / 60 h, D2 = e* dd
+  // with e = 1 / 90 h^2, their products and signs, and (v*) nu times 1, 1/3 or
+  // 4/3 of them.  On a non-uniform vertical grid the z scales are those of unit
+  // spacing and the metric is applied per layer.
+  f2 sx, sy, sz, nsx, nsy, nsz, sxy, sxz, syz;
+  f2 ex, ey, ez, nex, ney, nez;
+  f2 v1ex, v1ey, v1ez, v4ex, v4ey, v4ez, v3xy, v3xz, v3yz, v3z;
+  f2 neta, nu, gm1, heat, visc, cond, drho;
+  f2 bext[3];
   // adjoint mode: D (adjoint of the RK accumulator, padded layout; the
   // accumulator tiles then carry D), the NCOEF coefficient fields
   // ([NCOEF][nz][ny][nx]) and the driver adjoints out
@@ -143,62 +159,59 @@ template <> __device__ __forceinline__ pair::P2 rexp<pair::P2>(pair::P2 x) {
 namespace pair {
 
 // ---- adjoint mode: the derivatives the pointwise adjoint reads, then the
-// per-cell transpose (adjoint_cell) of each of the pair's two cells --------
+// per-cell transpose (adjoint_cell) of each of the pair's two cells.  s0: the
+// sources of plane k; d1z, d2z, mz: unscaled z differences --------------------
 __device__ __forceinline__ void adjoint_centre(const Args& a, const float* Pk, const float* Praw, float* scr,
                                                const float* dtile, uint64_t* dbar_mb, uint32_t& dphase,
                                                uint32_t& dpending, int k, int k0, int x0, int y0,
                                                const f2 (&vz)[NF], const f2 (&d1z)[NF], const f2 (&d2z)[NF],
-                                               const f2 (&mz)[6], float wk, float wpk, float lbk, float tbk,
-                                               float dlk, float dtk, float d2tk, float dt, int sub) {
+                                               const f2 (&mz)[6], const V16& s0, float wk, float wpk, float lbk,
+                                               float tbk, float dlk, float dtk, float d2tk, float dt, int sub) {
   const Layout& L = a.L;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, warp = tid >> 5;
   const int e = 2 * tx + 4;
-  // y derivatives of A_y, A_x (also the sources of the xy-mixed terms of
-  // grad div A) and of u_y, u_x; the scratch holds D1y A_y, D1y A_x on the
-  // tile plus an x halo (fields 0, 1; warps 0, 1 compute the halo items)
-  f2 dyAy, yyAy, dyAx, yyAx, dyUy, dyUx;
-  ds_pair(Pk + AY * FP, BX, a.cy, dyAy, &yyAy);
-  ds_pair(Pk + AX * FP, BX, a.cy, dyAx, &yyAx);
-  ds_pair(Pk + UY * FP, BX, a.cy, dyUy, nullptr);
-  ds_pair(Pk + UX * FP, BX, a.cy, dyUx, nullptr);
+  // y differences of A_y, A_x (the sources of the xy-mixed terms of grad div
+  // A); the scratch holds them on the tile plus an x halo (fields 0, 1; warps
+  // 0, 1 compute the halo items)
+  f2 dyAx, yyAx;
+  const f2 dyAy = us1(Pk + AY * FP, BX);
+  us_pair<true, true>(Pk + AX * FP, BX, dyAx, yyAx);
+  const f2 dyUy = us1(Pk + UY * FP, BX), dyUx = us1(Pk + UX * FP, BX);
   {
     float* sc = scr + ty * BX + e;
     *reinterpret_cast<f2*>(sc + 0 * SCF) = dyAy;
     *reinterpret_cast<f2*>(sc + 1 * SCF) = dyAx;
     if (warp < 2) {
       const int hr = (tid & 31) >> 2, hx = ((tid & 3) < 2) ? 2 * (tid & 3) : 32 + 2 * (tid & 3);
-      f2 h;
-      ds_pair(Praw + (warp == 0 ? AY : AX) * FP + (hr + 3) * BX + hx, BX, a.cy, h, nullptr);
-      *reinterpret_cast<f2*>(scr + warp * SCF + hr * BX + hx) = h;
+      *reinterpret_cast<f2*>(scr + warp * SCF + hr * BX + hx) =
+          us1(Praw + (warp == 0 ? AY : AX) * FP + (hr + 3) * BX + hx, BX);
     }
   }
   __syncthreads();
-  f2 m0, m1;
-  dx_pair(scr + 0 * SCF + ty * BX + e, a.cx, m0, nullptr);
-  dx_pair(scr + 1 * SCF + ty * BX + e, a.cx, m1, nullptr);
-  // A: off-diagonal first derivatives, Laplacians, grad div
-  f2 dxAy, xxAy, dxAz, xxAz, dyAz, yyAz, dxAx, xxAx;
-  dx_pair(Pk + AX * FP, a.cx, dxAx, &xxAx);
-  dx_pair(Pk + AY * FP, a.cx, dxAy, &xxAy);
-  dx_pair(Pk + AZ * FP, a.cx, dxAz, &xxAz);
-  ds_pair(Pk + AZ * FP, BX, a.cy, dyAz, &yyAz);
-  const f2 lapA0 = add(add(xxAx, yyAx), d2z[AX]);
-  const f2 lapA1 = add(add(xxAy, yyAy), d2z[AY]);
-  const f2 lapA2 = add(add(xxAz, yyAz), d2z[AZ]);
-  const f2 gdA0 = add(add(xxAx, m0), mz[0]);
-  const f2 gdA1 = add(add(m1, yyAy), mz[1]);
-  const f2 gdA2 = add(mz[2], d2z[AZ]);
+  const f2 m0 = ux1(scr + 0 * SCF + ty * BX + e), m1 = ux1(scr + 1 * SCF + ty * BX + e);
+  // A: curl and J = grad div A - lap A (the own-axis second derivatives cancel)
+  f2 dxAy, xxAy;
+  ux_pair<true, true>(Pk + AY * FP, dxAy, xxAy);
+  const f2 C0 = fma2(a.sy, s0.get(1), mul(a.nsz, d1z[AY]));
+  const f2 C1 = fma2(a.sz, d1z[AX], mul(a.nsx, s0.get(0)));
+  const f2 C2 = fma2(a.sx, dxAy, mul(a.nsy, dyAx));
+  const f2 J0 = fma2(a.sxy, m0, fma2(a.sxz, mz[0], fma2(a.ney, yyAx, mul(a.nez, d2z[AX]))));
+  const f2 J1 = fma2(a.sxy, m1, fma2(a.syz, mz[1], fma2(a.nex, xxAy, mul(a.nez, d2z[AY]))));
+  const f2 J2 = fma2(a.sz, mz[2], s0.get(6));
   // u: first derivatives; ln rho, ln T: gradients, Laplacian of ln T
-  f2 U00, U10, U20, U21, gL0, gL1, gT0, gT1, xxT, yyT;
-  dx_pair(Pk + UX * FP, a.cx, U00, nullptr);
-  dx_pair(Pk + UY * FP, a.cx, U10, nullptr);
-  dx_pair(Pk + UZ * FP, a.cx, U20, nullptr);
-  ds_pair(Pk + UZ * FP, BX, a.cy, U21, nullptr);
-  dx_pair(Pk + LR * FP, a.cx, gL0, nullptr);
-  ds_pair(Pk + LR * FP, BX, a.cy, gL1, nullptr);
-  dx_pair(Pk + LT * FP, a.cx, gT0, &xxT);
-  ds_pair(Pk + LT * FP, BX, a.cy, gT1, &yyT);
-  const f2 lapT = add(add(add(xxT, yyT), d2z[LT]), F2(d2tk));
+  const f2 U00 = mul(a.sx, ux1(Pk + UX * FP)), U10 = mul(a.sx, ux1(Pk + UY * FP));
+  const f2 U01 = mul(a.sy, dyUx), U11 = mul(a.sy, dyUy);
+  const f2 U20 = mul(a.sx, s0.get(3)), U21 = mul(a.sy, s0.get(4));
+  const f2 U02 = mul(a.sz, d1z[UX]), U12 = mul(a.sz, d1z[UY]), U22 = mul(a.sz, d1z[UZ]);
+  const f2 gL0 = mul(a.sx, ux1(Pk + LR * FP)), gL1 = mul(a.sy, us1(Pk + LR * FP, BX));
+  const f2 gL2 = fma2(a.sz, d1z[LR], F2(dlk));
+  f2 gT0, gT1, xxT, yyT;
+  ux_pair<true, true>(Pk + LT * FP, gT0, xxT);
+  us_pair<true, true>(Pk + LT * FP, BX, gT1, yyT);
+  gT0 = mul(a.sx, gT0);
+  gT1 = mul(a.sy, gT1);
+  const f2 gT2 = fma2(a.sz, d1z[LT], F2(dtk));
+  const f2 lapT = fma2(a.ex, xxT, fma2(a.ey, yyT, fma2(a.ez, d2z[LT], F2(d2tk))));
   // D of the pair (bounded wait; a time-out is recorded and the CTA goes on)
   const int sl = (k - k0) & 1;
   if (!zm::mbar_wait(dbar_mb, (dphase >> sl) & 1u)) atomicOr(&a.ss->nonfinite, 2);
@@ -230,20 +243,22 @@ __device__ __forceinline__ void adjoint_centre(const Args& a, const float* Pk, c
     cl.U[0] = P2(vz[UX]); cl.U[1] = P2(vz[UY]); cl.U[2] = P2(vz[UZ]);
     cl.L = P2(add(F2(lbk), vz[LR]));
     cl.Th = P2(add(F2(tbk), vz[LT]));
-    cl.dA[0][0] = P2(dxAx); cl.dA[0][1] = P2(dyAx); cl.dA[0][2] = P2(d1z[AX]);
-    cl.dA[1][0] = P2(dxAy); cl.dA[1][1] = P2(dyAy); cl.dA[1][2] = P2(d1z[AY]);
-    cl.dA[2][0] = P2(dxAz); cl.dA[2][1] = P2(dyAz); cl.dA[2][2] = P2(d1z[AZ]);
-    cl.dU[0][0] = P2(U00); cl.dU[0][1] = P2(dyUx); cl.dU[0][2] = P2(d1z[UX]);
-    cl.dU[1][0] = P2(U10); cl.dU[1][1] = P2(dyUy); cl.dU[1][2] = P2(d1z[UY]);
-    cl.dU[2][0] = P2(U20); cl.dU[2][1] = P2(U21); cl.dU[2][2] = P2(d1z[UZ]);
-    cl.lapA[0] = P2(lapA0); cl.lapA[1] = P2(lapA1); cl.lapA[2] = P2(lapA2);
-    cl.gdA[0] = P2(gdA0); cl.gdA[1] = P2(gdA1); cl.gdA[2] = P2(gdA2);
-    // the adjoint reads no second derivative of u and no Laplacian of ln rho
+    // the curl as one entry of each antisymmetric pair, J as grad div A (only
+    // the differences enter); no second derivative of u, no Laplacian of ln rho
+    cl.dA[0][0] = cl.dA[1][1] = cl.dA[2][2] = P2(0.f);
+    cl.dA[2][1] = P2(C0); cl.dA[1][2] = P2(0.f);
+    cl.dA[0][2] = P2(C1); cl.dA[2][0] = P2(0.f);
+    cl.dA[1][0] = P2(C2); cl.dA[0][1] = P2(0.f);
+    cl.dU[0][0] = P2(U00); cl.dU[0][1] = P2(U01); cl.dU[0][2] = P2(U02);
+    cl.dU[1][0] = P2(U10); cl.dU[1][1] = P2(U11); cl.dU[1][2] = P2(U12);
+    cl.dU[2][0] = P2(U20); cl.dU[2][1] = P2(U21); cl.dU[2][2] = P2(U22);
+    cl.lapA[0] = cl.lapA[1] = cl.lapA[2] = P2(0.f);
+    cl.gdA[0] = P2(J0); cl.gdA[1] = P2(J1); cl.gdA[2] = P2(J2);
     cl.lapU[0] = cl.lapU[1] = cl.lapU[2] = P2(0.f);
     cl.gdU[0] = cl.gdU[1] = cl.gdU[2] = P2(0.f);
     cl.lapL = P2(0.f);
-    cl.gL[0] = P2(gL0); cl.gL[1] = P2(gL1); cl.gL[2] = P2(add(d1z[LR], F2(dlk)));
-    cl.gT[0] = P2(gT0); cl.gT[1] = P2(gT1); cl.gT[2] = P2(add(d1z[LT], F2(dtk)));
+    cl.gL[0] = P2(gL0); cl.gL[1] = P2(gL1); cl.gL[2] = P2(gL2);
+    cl.gT[0] = P2(gT0); cl.gT[1] = P2(gT1); cl.gT[2] = P2(gT2);
     cl.lapT = P2(lapT);
     P2 wo[NF];
 #pragma unroll
@@ -282,20 +297,22 @@ __device__ __forceinline__ void adjoint_centre(const Args& a, const float* Pk, c
     cl.U[0] = P(vz[UX]); cl.U[1] = P(vz[UY]); cl.U[2] = P(vz[UZ]);
     cl.L = lbk + P(vz[LR]);
     cl.Th = tbk + P(vz[LT]);
-    cl.dA[0][0] = P(dxAx); cl.dA[0][1] = P(dyAx); cl.dA[0][2] = P(d1z[AX]);
-    cl.dA[1][0] = P(dxAy); cl.dA[1][1] = P(dyAy); cl.dA[1][2] = P(d1z[AY]);
-    cl.dA[2][0] = P(dxAz); cl.dA[2][1] = P(dyAz); cl.dA[2][2] = P(d1z[AZ]);
-    cl.dU[0][0] = P(U00); cl.dU[0][1] = P(dyUx); cl.dU[0][2] = P(d1z[UX]);
-    cl.dU[1][0] = P(U10); cl.dU[1][1] = P(dyUy); cl.dU[1][2] = P(d1z[UY]);
-    cl.dU[2][0] = P(U20); cl.dU[2][1] = P(U21); cl.dU[2][2] = P(d1z[UZ]);
-    cl.lapA[0] = P(lapA0); cl.lapA[1] = P(lapA1); cl.lapA[2] = P(lapA2);
-    cl.gdA[0] = P(gdA0); cl.gdA[1] = P(gdA1); cl.gdA[2] = P(gdA2);
-    // the adjoint reads no second derivative of u and no Laplacian of ln rho
+    // the curl as one entry of each antisymmetric pair, J as grad div A (only
+    // the differences enter); no second derivative of u, no Laplacian of ln rho
+    cl.dA[0][0] = cl.dA[1][1] = cl.dA[2][2] = 0.f;
+    cl.dA[2][1] = P(C0); cl.dA[1][2] = 0.f;
+    cl.dA[0][2] = P(C1); cl.dA[2][0] = 0.f;
+    cl.dA[1][0] = P(C2); cl.dA[0][1] = 0.f;
+    cl.dU[0][0] = P(U00); cl.dU[0][1] = P(U01); cl.dU[0][2] = P(U02);
+    cl.dU[1][0] = P(U10); cl.dU[1][1] = P(U11); cl.dU[1][2] = P(U12);
+    cl.dU[2][0] = P(U20); cl.dU[2][1] = P(U21); cl.dU[2][2] = P(U22);
+    cl.lapA[0] = cl.lapA[1] = cl.lapA[2] = 0.f;
+    cl.gdA[0] = P(J0); cl.gdA[1] = P(J1); cl.gdA[2] = P(J2);
     cl.lapU[0] = cl.lapU[1] = cl.lapU[2] = 0.f;
     cl.gdU[0] = cl.gdU[1] = cl.gdU[2] = 0.f;
     cl.lapL = 0.f;
-    cl.gL[0] = P(gL0); cl.gL[1] = P(gL1); cl.gL[2] = P(d1z[LR]) + dlk;
-    cl.gT[0] = P(gT0); cl.gT[1] = P(gT1); cl.gT[2] = P(d1z[LT]) + dtk;
+    cl.gL[0] = P(gL0); cl.gL[1] = P(gL1); cl.gL[2] = P(gL2);
+    cl.gT[0] = P(gT0); cl.gT[1] = P(gT1); cl.gT[2] = P(gT2);
     cl.lapT = P(lapT);
     float wo[NF];
 #pragma unroll
@@ -414,16 +431,19 @@ __global__ void __launch_bounds__(NT, 2) rk_pair_kernel(const __grid_constant__ 
     for (int g = 0; g < 2; ++g) {
       const int X = g == 0 ? AX : UX;
       f2 zx, zy, xx, yy;
-      dx_pair(P + (X + 2) * FP, a.cx, zx, nullptr);
-      ds_pair(P + (X + 2) * FP, BX, a.cy, zy, nullptr);
-      dx_pair(P + X * FP, a.cx, xx, nullptr);
-      ds_pair(P + (X + 1) * FP, BX, a.cy, yy, nullptr);
+      if (ADJ && g == 1) {
+        zx = ux1(P + (X + 2) * FP);
+        zy = us1(P + (X + 2) * FP, BX);
+        s.set(7, F2(0.f));  // no second derivative of u in the adjoint
+      } else {
+        ux_pair<true, true>(P + (X + 2) * FP, zx, xx);
+        us_pair<true, true>(P + (X + 2) * FP, BX, zy, yy);
+        s.set(6 + g, g == 0 ? fma2(a.nex, xx, mul(a.ney, yy)) : fma2(a.v1ex, xx, mul(a.v1ey, yy)));
+      }
       s.set(3 * g + 0, zx);
       s.set(3 * g + 1, zy);
-      s.set(3 * g + 2, add(xx, yy));
+      s.set(3 * g + 2, fma2(a.sx, ux1(P + X * FP), mul(a.sy, us1(P + (X + 1) * FP, BX))));
     }
-    s.set(6, F2(0.f));
-    s.set(7, F2(0.f));
     tm_st(tlane + VCOL + (uint32_t)(p & 7) * 16, v);
     tm_st(tlane + SCOL + (uint32_t)(p & 7) * 16, s);
   };
@@ -506,39 +526,39 @@ __global__ void __launch_bounds__(NT, 2) rk_pair_kernel(const __grid_constant__ 
       tm_wait_st();
 
       const float* Pk = raw + sk * PLANE + cen;
-      // ---- z derivatives from the TMEM rings --------------------------------
+      // ---- z differences from the TMEM rings --------------------------------
       f2 vz[NF], d1z[NF], d2z[NF], mz[6];
+      V16 s0;  // sources of plane k itself
 #pragma unroll
-      for (int f = 0; f < NF; ++f) {
-        vz[f] = ld2(Pk + f * FP);
-        d1z[f] = F2(0.f);
-        d2z[f] = mul(a.cz.e0, vz[f]);
-      }
-#pragma unroll
-      for (int q = 0; q < 6; ++q) mz[q] = F2(0.f);
+      for (int f = 0; f < NF; ++f) vz[f] = ld2(Pk + f * FP);
 #pragma unroll
       for (int m = 3; m >= 1; --m) {
-        const f2 cm = m == 1 ? a.cz.c1 : (m == 2 ? a.cz.c2 : a.cz.c3);
-        const f2 em = m == 1 ? a.cz.e1 : (m == 2 ? a.cz.e2 : a.cz.e3);
+        const f2 cm = F2(m == 1 ? 45.f : -9.f), em = F2(m == 1 ? 135.f : -13.5f);
         V16 vp, vm, sp, sm;
         tm_ld(tlane + VCOL + (uint32_t)((k + m) & 7) * 16, vp);
         tm_ld(tlane + VCOL + (uint32_t)((k - m) & 7) * 16, vm);
         tm_ld(tlane + SCOL + (uint32_t)((k + m) & 7) * 16, sp);
         tm_ld(tlane + SCOL + (uint32_t)((k - m) & 7) * 16, sm);
+        if (m == 1) tm_ld(tlane + SCOL + (uint32_t)(k & 7) * 16, s0);
         tm_wait_ld();
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
-          d1z[f] = fma2(cm, dif(vp.get(f), vm.get(f)), d1z[f]);
-          d2z[f] = fma2(em, add(vp.get(f), vm.get(f)), d2z[f]);
+          const f2 d = dif(vp.get(f), vm.get(f)), c = add(vp.get(f), vm.get(f));
+          d1z[f] = m == 3 ? d : fma2(cm, d, d1z[f]);
+          d2z[f] = m == 3 ? fma2(F2(-245.f), vz[f], c) : fma2(em, c, d2z[f]);
         }
 #pragma unroll
-        for (int q = 0; q < 6; ++q) mz[q] = fma2(cm, dif(sp.get(q), sm.get(q)), mz[q]);
+        for (int q = 0; q < 6; ++q) {
+          const f2 d = dif(sp.get(q), sm.get(q));
+          mz[q] = m == 3 ? d : fma2(cm, d, mz[q]);
+        }
       }
       if constexpr (ZG) {
+        // d -> m1 d, dd -> m1^2 dd + r21 m1 d (in the units of d and dd)
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
           d1z[f] = mul(F2(zm1k), d1z[f]);
-          d2z[f] = fma2(F2(zr21k), d1z[f], mul(F2(zm1k * zm1k), d2z[f]));
+          d2z[f] = fma2(F2(1.5f * zr21k), d1z[f], mul(F2(zm1k * zm1k), d2z[f]));
         }
 #pragma unroll
         for (int q = 0; q < 6; ++q) mz[q] = mul(F2(zm1k), mz[q]);
@@ -562,67 +582,54 @@ __global__ void __launch_bounds__(NT, 2) rk_pair_kernel(const __grid_constant__ 
 
       if constexpr (ADJ) {
         adjoint_centre(a, Pk, raw + sk * PLANE, scr, dfs + ((k - k0) & 1) * DFT, &mbd[(k - k0) & 1], dphase,
-                       dpending, k, k0, x0, y0, vz, d1z, d2z, mz, wk, wpk, lbk, tbk, dlk, dtk, d2tk, dt, sub);
+                       dpending, k, k0, x0, y0, vz, d1z, d2z, mz, s0, wk, wpk, lbk, tbk, dlk, dtk, d2tk, dt, sub);
         continue;
       }
       // ---- x, y derivatives from the shared ring, folded as they come -------
       // (the own-axis second derivatives D2x A_x, D2y A_y cancel in J outside
       // the swamp layers)
       const bool swamp = wk != 0.f || wpk != 0.f;
-      // y derivatives of A_y, A_x, u_y, u_x: also the sources of the xy-mixed
+      // y differences of A_y, A_x, u_y, u_x: also the sources of the xy-mixed
       // terms D1x(D1y .), through the scratch with an x halo
-      f2 dyAy, dyAx, yyAx, dyUy, yyUy, dyUx, yyUx, yyAy = F2(0.f);
-      if (swamp)
-        ds_pair(Pk + AY * FP, BX, a.cy, dyAy, &yyAy);
-      else
-        ds_pair(Pk + AY * FP, BX, a.cy, dyAy, nullptr);
-      ds_pair(Pk + AX * FP, BX, a.cy, dyAx, &yyAx);
-      ds_pair(Pk + UY * FP, BX, a.cy, dyUy, &yyUy);
-      ds_pair(Pk + UX * FP, BX, a.cy, dyUx, &yyUx);
+      f2 dyAx, yyAx, dyUy, yyUy, dyUx, yyUx;
+      us_pair<true, true>(Pk + AX * FP, BX, dyAx, yyAx);
+      us_pair<true, true>(Pk + UY * FP, BX, dyUy, yyUy);
+      us_pair<true, true>(Pk + UX * FP, BX, dyUx, yyUx);
       {
         float* sc = scr + ty * BX + e;
-        *reinterpret_cast<f2*>(sc + 0 * SCF) = dyAy;
+        *reinterpret_cast<f2*>(sc + 0 * SCF) = us1(Pk + AY * FP, BX);
         *reinterpret_cast<f2*>(sc + 1 * SCF) = dyAx;
         *reinterpret_cast<f2*>(sc + 2 * SCF) = dyUy;
         *reinterpret_cast<f2*>(sc + 3 * SCF) = dyUx;
-        f2 h;
-        ds_pair(raw + sk * PLANE + hfield * FP + (hr + 3) * BX + hx, BX, a.cy, h, nullptr);
-        *reinterpret_cast<f2*>(scr + hq * SCF + hr * BX + hx) = h;
+        *reinterpret_cast<f2*>(scr + hq * SCF + hr * BX + hx) =
+            us1(raw + sk * PLANE + hfield * FP + (hr + 3) * BX + hx, BX);
       }
       __syncthreads();
       f2 mxy[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) dx_pair(scr + q * SCF + ty * BX + e, a.cx, mxy[q], nullptr);
+      for (int q = 0; q < 4; ++q) mxy[q] = ux1(scr + q * SCF + ty * BX + e);
 
       const Phys<float>& ph = a.ph;
-      const f2 w = F2(wk), wp = F2(wpk);
       // A: B = curl A + B_ext, J = grad div A - lap A, swamp terms of the
       // induction equation
       f2 B0, B1, B2, J0, J1, J2, sw0 = F2(0.f), sw1 = F2(0.f), sw2 = F2(0.f);
       {
-        f2 dxAy, xxAy, dxAz, xxAz, dyAz, yyAz;
-        dx_pair(Pk + AY * FP, a.cx, dxAy, &xxAy);
-        dx_pair(Pk + AZ * FP, a.cx, dxAz, &xxAz);
-        ds_pair(Pk + AZ * FP, BX, a.cy, dyAz, &yyAz);
-        B0 = add(dif(dyAz, d1z[AY]), F2(ph.bext[0]));
-        B1 = add(dif(d1z[AX], dxAz), F2(ph.bext[1]));
-        B2 = add(dif(dxAy, dyAx), F2(ph.bext[2]));
-        if (!swamp) {
-          J0 = dif(dif(add(mxy[0], mz[0]), yyAx), d2z[AX]);
-          J1 = dif(dif(add(mxy[1], mz[1]), xxAy), d2z[AY]);
-          J2 = dif(dif(mz[2], xxAz), yyAz);
-        } else {
-          f2 dxAx, xxAx;
-          dx_pair(Pk + AX * FP, a.cx, dxAx, &xxAx);
-          const f2 lap0 = add(add(xxAx, yyAx), d2z[AX]);
-          const f2 lap1 = add(add(xxAy, yyAy), d2z[AY]);
-          const f2 lap2 = add(add(xxAz, yyAz), d2z[AZ]);
-          J0 = dif(add(add(xxAx, mxy[0]), mz[0]), lap0);
-          J1 = dif(add(add(mxy[1], yyAy), mz[1]), lap1);
-          J2 = dif(add(mz[2], d2z[AZ]), lap2);
-          const f2 ews = mul(F2(ph.eta_s), w);
-          f2 divA = add(add(dxAx, dyAy), d1z[AZ]);
-          f2 l0 = lap0, l1 = lap1, l2 = lap2;
+        f2 dxAy, xxAy;
+        ux_pair<true, true>(Pk + AY * FP, dxAy, xxAy);
+        B0 = fma2(a.sy, s0.get(1), fma2(a.nsz, d1z[AY], a.bext[0]));
+        B1 = fma2(a.sz, d1z[AX], fma2(a.nsx, s0.get(0), a.bext[1]));
+        B2 = fma2(a.sx, dxAy, fma2(a.nsy, dyAx, a.bext[2]));
+        J0 = fma2(a.sxy, mxy[0], fma2(a.sxz, mz[0], fma2(a.ney, yyAx, mul(a.nez, d2z[AX]))));
+        J1 = fma2(a.sxy, mxy[1], fma2(a.syz, mz[1], fma2(a.nex, xxAy, mul(a.nez, d2z[AY]))));
+        J2 = fma2(a.sz, mz[2], s0.get(6));
+        if (swamp) {
+          f2 xxAx, yyAy, none;
+          ux_pair<false, true>(Pk + AX * FP, none, xxAx);
+          us_pair<false, true>(Pk + AY * FP, BX, none, yyAy);
+          f2 l0 = fma2(a.ex, xxAx, fma2(a.ey, yyAx, mul(a.ez, d2z[AX])));
+          f2 l1 = fma2(a.ex, xxAy, fma2(a.ey, yyAy, mul(a.ez, d2z[AY])));
+          f2 l2 = dif(mul(a.ez, d2z[AZ]), s0.get(6));
+          f2 divA = fma2(a.sz, d1z[AZ], s0.get(2));
           if constexpr (BG) {
             // the background's lap A and div A on the swamp layers
             if (live && k >= a.bg.ksw) {
@@ -633,9 +640,10 @@ __global__ void __launch_bounds__(NT, 2) rk_pair_kernel(const __grid_constant__ 
               divA = add(divA, __ldg(reinterpret_cast<const float2*>(a.bg.bL + 3 * ns + qs)));
             }
           }
+          const f2 ews = F2(ph.eta_s * wk);
           sw0 = mul(ews, l0);
           sw1 = mul(ews, l1);
-          sw2 = fma2(mul(F2(ph.eta_s), wp), divA, mul(ews, l2));
+          sw2 = fma2(F2(ph.eta_s * wpk), divA, mul(ews, l2));
         }
         if constexpr (BG) {
           B0 = add(B0, gB[0]);
@@ -646,37 +654,38 @@ __global__ void __launch_bounds__(NT, 2) rk_pair_kernel(const __grid_constant__ 
           J2 = add(J2, gJ[2]);
         }
       }
-      // u: dU[c][a] = d_a u_c, lap u, grad div u
-      f2 U00, U10, U20, U21, lapU0, lapU1, lapU2, gdU0, gdU1, gdU2;
+      // u: dU[c][a] = d_a u_c, and nu (lap u + grad div u / 3)
+      f2 U00, U10, v0, v1, v2;
       {
-        f2 xxUx, xxUy, xxUz, yyUz;
-        dx_pair(Pk + UX * FP, a.cx, U00, &xxUx);
-        dx_pair(Pk + UY * FP, a.cx, U10, &xxUy);
-        dx_pair(Pk + UZ * FP, a.cx, U20, &xxUz);
-        ds_pair(Pk + UZ * FP, BX, a.cy, U21, &yyUz);
-        lapU0 = add(add(xxUx, yyUx), d2z[UX]);
-        lapU1 = add(add(xxUy, yyUy), d2z[UY]);
-        lapU2 = add(add(xxUz, yyUz), d2z[UZ]);
-        gdU0 = add(add(xxUx, mxy[2]), mz[3]);
-        gdU1 = add(add(mxy[3], yyUy), mz[4]);
-        gdU2 = add(mz[5], d2z[UZ]);
+        f2 xx;
+        ux_pair<true, true>(Pk + UX * FP, U00, xx);
+        v0 = fma2(a.v4ex, xx, fma2(a.v1ey, yyUx, fma2(a.v1ez, d2z[UX], fma2(a.v3xy, mxy[2], mul(a.v3xz, mz[3])))));
+        ux_pair<true, true>(Pk + UY * FP, U10, xx);
+        v1 = fma2(a.v1ex, xx, fma2(a.v4ey, yyUy, fma2(a.v1ez, d2z[UY], fma2(a.v3xy, mxy[3], mul(a.v3yz, mz[4])))));
+        v2 = fma2(a.v4ez, d2z[UZ], fma2(a.v3z, mz[5], s0.get(7)));
+        U00 = mul(a.sx, U00);
+        U10 = mul(a.sx, U10);
       }
-      const f2 U01 = dyUx, U02 = d1z[UX];
-      const f2 U11 = dyUy, U12 = d1z[UY];
-      const f2 U22 = d1z[UZ];
+      const f2 U01 = mul(a.sy, dyUx), U11 = mul(a.sy, dyUy);
+      const f2 U20 = mul(a.sx, s0.get(3)), U21 = mul(a.sy, s0.get(4));
+      const f2 U02 = mul(a.sz, d1z[UX]), U12 = mul(a.sz, d1z[UY]), U22 = mul(a.sz, d1z[UZ]);
       // ln rho, ln T (perturbations about the background profiles)
       f2 gL0, gL1, lapL, gT0, gT1, lapT;
       {
         f2 xx, yy;
-        dx_pair(Pk + LR * FP, a.cx, gL0, &xx);
-        ds_pair(Pk + LR * FP, BX, a.cy, gL1, &yy);
-        lapL = add(add(add(xx, yy), d2z[LR]), F2(d2lk));
-        dx_pair(Pk + LT * FP, a.cx, gT0, &xx);
-        ds_pair(Pk + LT * FP, BX, a.cy, gT1, &yy);
-        lapT = add(add(add(xx, yy), d2z[LT]), F2(d2tk));
+        ux_pair<true, true>(Pk + LR * FP, gL0, xx);
+        us_pair<true, true>(Pk + LR * FP, BX, gL1, yy);
+        lapL = fma2(a.ex, xx, fma2(a.ey, yy, fma2(a.ez, d2z[LR], F2(d2lk))));
+        ux_pair<true, true>(Pk + LT * FP, gT0, xx);
+        us_pair<true, true>(Pk + LT * FP, BX, gT1, yy);
+        lapT = fma2(a.ex, xx, fma2(a.ey, yy, fma2(a.ez, d2z[LT], F2(d2tk))));
+        gL0 = mul(a.sx, gL0);
+        gL1 = mul(a.sy, gL1);
+        gT0 = mul(a.sx, gT0);
+        gT1 = mul(a.sy, gT1);
       }
-      const f2 gL2 = add(d1z[LR], F2(dlk));
-      const f2 gT2 = add(d1z[LT], F2(dtk));
+      const f2 gL2 = fma2(a.sz, d1z[LR], F2(dlk));
+      const f2 gT2 = fma2(a.sz, d1z[LT], F2(dtk));
       // RK accumulator of the pair (bounded wait; a time-out is recorded and
       // the step continues, so the CTA stays convergent)
       f2 dfo[NF];
@@ -707,51 +716,54 @@ __global__ void __launch_bounds__(NT, 2) rk_pair_kernel(const __grid_constant__ 
         // box, against the 1e-4 of the FP32 path
         const f2 T = make_float2(__expf(Th.x), __expf(Th.y));
         const f2 rho1 = make_float2(__expf(-Lr.x), __expf(-Lr.y));
-        const f2 eta = F2(ph.eta), nu = F2(ph.nu), gm1 = F2(ph.gm1);
+        const f2 m = F2(-1.f), two = F2(2.f);
+        const f2 n0 = mul(m, u0), n1 = mul(m, u1), n2_ = mul(m, u2);  // -u
+        const f2 nB0 = mul(m, B0), nB1 = mul(m, B1), nB2 = mul(m, B2);
         f2 out[NF];
-        // induction
-        out[AX] = add(dif(dif(mul(u1, B2), mul(u2, B1)), mul(eta, J0)), sw0);
-        out[AY] = add(dif(dif(mul(u2, B0), mul(u0, B2)), mul(eta, J1)), sw1);
-        out[AZ] = add(dif(dif(mul(u0, B1), mul(u1, B0)), mul(eta, J2)), sw2);
-        // traceless rate of strain
-        const f2 third = F2(1.f / 3.f), half = F2(0.5f), two = F2(2.f);
-        const f2 s00 = dif(U00, mul(third, divU)), s11 = dif(U11, mul(third, divU)), s22 = dif(U22, mul(third, divU));
-        const f2 s01 = mul(half, add(U01, U10));
-        const f2 s02 = mul(half, add(U02, U20));
-        const f2 s12 = mul(half, add(U12, U21));
-        const f2 S2 = fma2(two, fma2(s01, s01, fma2(s02, s02, mul(s12, s12))),
-                           fma2(s00, s00, fma2(s11, s11, mul(s22, s22))));
-        const f2 SgL0 = fma2(s00, gL0, fma2(s01, gL1, mul(s02, gL2)));
-        const f2 SgL1 = fma2(s01, gL0, fma2(s11, gL1, mul(s12, gL2)));
-        const f2 SgL2 = fma2(s02, gL0, fma2(s12, gL1, mul(s22, gL2)));
-        // Lorentz force
-        const f2 F0 = dif(mul(J1, B2), mul(J2, B1));
-        const f2 F1 = dif(mul(J2, B0), mul(J0, B2));
-        const f2 Fz = dif(mul(J0, B1), mul(J1, B0));
-        const f2 adv0 = fma2(u0, U00, fma2(u1, U01, mul(u2, U02)));
-        const f2 adv1 = fma2(u0, U10, fma2(u1, U11, mul(u2, U12)));
-        const f2 adv2 = fma2(u0, U20, fma2(u1, U21, mul(u2, U22)));
-        out[UX] = add(dif(mul(F0, rho1), add(adv0, mul(T, add(gL0, gT0)))),
-                      mul(nu, fma2(two, SgL0, fma2(third, gdU0, lapU0))));
-        out[UY] = add(dif(mul(F1, rho1), add(adv1, mul(T, add(gL1, gT1)))),
-                      mul(nu, fma2(two, SgL1, fma2(third, gdU1, lapU1))));
-        out[UZ] = add(add(dif(mul(Fz, rho1), add(adv2, mul(T, add(gL2, gT2)))),
-                          mul(nu, fma2(two, SgL2, fma2(third, gdU2, lapU2)))),
-                      F2(ph.gz));
+        // induction: u x B - eta J + swamp
+        out[AX] = fma2(u1, B2, fma2(u2, nB1, fma2(a.neta, J0, sw0)));
+        out[AY] = fma2(u2, B0, fma2(u0, nB2, fma2(a.neta, J1, sw1)));
+        out[AZ] = fma2(u0, B1, fma2(u1, nB0, fma2(a.neta, J2, sw2)));
+        // traceless rate of strain, off-diagonal entries doubled (t_ab = 2 S_ab)
+        const f2 d3 = mul(F2(-1.f / 3.f), divU);
+        const f2 s00 = add(U00, d3), s11 = add(U11, d3), s22 = add(U22, d3);
+        const f2 t01 = add(U01, U10), t02 = add(U02, U20), t12 = add(U12, U21);
+        // 2 S:S
+        const f2 S2 = fma2(t01, t01, fma2(t02, t02, fma2(t12, t12,
+                      mul(two, fma2(s00, s00, fma2(s11, s11, mul(s22, s22)))))));
+        // 2 nu S . grad ln rho
+        const f2 g0 = mul(a.nu, gL0), g1 = mul(a.nu, gL1), g2 = mul(a.nu, gL2);
+        const f2 h0 = add(g0, g0), h1 = add(g1, g1), h2 = add(g2, g2);
+        v0 = fma2(s00, h0, fma2(t01, g1, fma2(t02, g2, v0)));
+        v1 = fma2(s11, h1, fma2(t01, g0, fma2(t12, g2, v1)));
+        v2 = fma2(s22, h2, fma2(t02, g0, fma2(t12, g1, v2)));
+        // Lorentz force J x B
+        const f2 F0 = fma2(J1, B2, mul(J2, nB1));
+        const f2 F1 = fma2(J2, B0, mul(J0, nB2));
+        const f2 Fz = fma2(J0, B1, mul(J1, nB0));
+        // advection, pressure and gravity (whose difference in hydrostatic
+        // balance is formed before the smaller terms join it), force / rho
+        const f2 nT = mul(m, T);
+        out[UX] = fma2(F0, rho1, fma2(n0, U00, fma2(n1, U01, fma2(n2_, U02, fma2(nT, add(gL0, gT0), v0)))));
+        out[UY] = fma2(F1, rho1, fma2(n0, U10, fma2(n1, U11, fma2(n2_, U12, fma2(nT, add(gL1, gT1), v1)))));
+        out[UZ] = fma2(Fz, rho1, fma2(n0, U20, fma2(n1, U21, fma2(n2_, U22,
+                  add(fma2(nT, add(gL2, gT2), F2(ph.gz)), v2)))));
         // continuity
-        const f2 ugL = fma2(u0, gL0, fma2(u1, gL1, mul(u2, gL2)));
         const f2 gLs = fma2(gL0, gL0, fma2(gL1, gL1, mul(gL2, gL2)));
-        out[LR] = add(dif(mul(F2(ph.drho), add(lapL, gLs)), add(ugL, divU)), mul(mul(F2(ph.drho_s), w), lapL));
+        out[LR] = fma2(a.drho, add(lapL, gLs), fma2(n0, gL0, fma2(n1, gL1, fma2(n2_, gL2, mul(m, divU)))));
         // energy (ln T)
-        const f2 ugT = fma2(u0, gT0, fma2(u1, gT1, mul(u2, gT2)));
         const f2 gTs = fma2(gT0, gT0, fma2(gT1, gT1, mul(gT2, gT2)));
         const f2 JJ = fma2(J0, J0, fma2(J1, J1, mul(J2, J2)));
         const f2 T1 = make_float2(__fdividef(1.f, T.x), __fdividef(1.f, T.y));
-        const f2 heat = mul(mul(gm1, fma2(mul(eta, JJ), rho1, mul(two, mul(nu, S2)))), T1);
+        const f2 heat = fma2(mul(a.heat, JJ), rho1, mul(a.visc, S2));
         const f2 ka = dif(mul(F2(2.5f), Th), Lr);
-        const f2 kt = mul(F2(ph.gm1 * ph.kappa0), make_float2(__expf(ka.x), __expf(ka.y)));
-        out[LT] = add(add(dif(heat, fma2(gm1, divU, ugT)), mul(kt, fma2(F2(3.5f), gTs, lapT))),
-                      mul(mul(F2(ph.chi_s), w), lapT));
+        const f2 kt = mul(a.cond, make_float2(__expf(ka.x), __expf(ka.y)));
+        out[LT] = fma2(heat, T1, fma2(kt, fma2(F2(3.5f), gTs, lapT),
+                  fma2(n0, gT0, fma2(n1, gT1, fma2(n2_, gT2, mul(a.gm1, mul(m, divU)))))));
+        if (swamp) {
+          out[LR] = fma2(F2(ph.drho_s * wk), lapL, out[LR]);
+          out[LT] = fma2(F2(ph.chi_s * wk), lapT, out[LT]);
+        }
         if constexpr (NC) {
           if (k < ph.nc_k1)  // Newtonian cooling, one cell at a time
             out[LT] = add(out[LT], make_float2(nc_term<float>(ph, a.bg, L.nz, k, Lr.x, Th.x, nullptr, nullptr),
@@ -891,22 +903,21 @@ static pair::Args pair_args(const Layout& L, const Phys<float>& ph, const Backgr
   a.sub = sub;
   a.ntx = (L.nx + pair::TX - 1) / pair::TX;
   a.nty = (L.ny + pair::TY - 1) / pair::TY;
-  const double W1[4] = {0.0, 45.0 / 60.0, -9.0 / 60.0, 1.0 / 60.0};
-  const double W2[4] = {-490.0 / 180.0, 270.0 / 180.0, -27.0 / 180.0, 2.0 / 180.0};
-  auto coef = [&](double h) {
-    pair::Coef c;
-    c.c1 = make_float2((float)(W1[1] / h), (float)(W1[1] / h));
-    c.c2 = make_float2((float)(W1[2] / h), (float)(W1[2] / h));
-    c.c3 = make_float2((float)(W1[3] / h), (float)(W1[3] / h));
-    c.e0 = make_float2((float)(W2[0] / (h * h)), (float)(W2[0] / (h * h)));
-    c.e1 = make_float2((float)(W2[1] / (h * h)), (float)(W2[1] / (h * h)));
-    c.e2 = make_float2((float)(W2[2] / (h * h)), (float)(W2[2] / (h * h)));
-    c.e3 = make_float2((float)(W2[3] / (h * h)), (float)(W2[3] / (h * h)));
-    return c;
-  };
-  a.cx = coef(dx);
-  a.cy = coef(dy);
-  a.cz = coef(dz);
+  auto P = [](double v) { return make_float2((float)v, (float)v); };
+  const double sx = 1.0 / (60.0 * dx), sy = 1.0 / (60.0 * dy), sz = 1.0 / (60.0 * dz);
+  const double ex = 1.0 / (90.0 * dx * dx), ey = 1.0 / (90.0 * dy * dy), ez = 1.0 / (90.0 * dz * dz);
+  const double nu = ph.nu, nu3 = nu / 3.0, nu43 = 4.0 * nu / 3.0;
+  a.sx = P(sx); a.sy = P(sy); a.sz = P(sz);
+  a.nsx = P(-sx); a.nsy = P(-sy); a.nsz = P(-sz);
+  a.sxy = P(sx * sy); a.sxz = P(sx * sz); a.syz = P(sy * sz);
+  a.ex = P(ex); a.ey = P(ey); a.ez = P(ez);
+  a.nex = P(-ex); a.ney = P(-ey); a.nez = P(-ez);
+  a.v1ex = P(nu * ex); a.v1ey = P(nu * ey); a.v1ez = P(nu * ez);
+  a.v4ex = P(nu43 * ex); a.v4ey = P(nu43 * ey); a.v4ez = P(nu43 * ez);
+  a.v3xy = P(nu3 * sx * sy); a.v3xz = P(nu3 * sx * sz); a.v3yz = P(nu3 * sy * sz); a.v3z = P(nu3 * sz);
+  a.neta = P(-ph.eta); a.nu = P(nu); a.gm1 = P(ph.gm1); a.drho = P(ph.drho);
+  a.heat = P((double)ph.gm1 * ph.eta); a.visc = P((double)ph.gm1 * nu); a.cond = P((double)ph.gm1 * ph.kappa0);
+  for (int c = 0; c < 3; ++c) a.bext[c] = P(ph.bext[c]);
   const int tiles = a.ntx * a.nty;
   a.kchunk = zm::zchunk(L.nz, tiles, ctas);
   a.nch = (L.nz + a.kchunk - 1) / a.kchunk;
