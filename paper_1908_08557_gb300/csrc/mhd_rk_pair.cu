@@ -175,7 +175,7 @@ __device__ __forceinline__ void adjoint_centre(const Args& a, const float* Pk, c
   // 0, 1 compute the halo items)
   f2 dyAx, yyAx;
   const f2 dyAy = us1(Pk + AY * FP, BX);
-  us_pair<true, true>(Pk + AX * FP, BX, dyAx, yyAx);
+  us_pair<true, true>(Pk + AX * FP, BX, vz[AX], dyAx, yyAx);
   const f2 dyUy = us1(Pk + UY * FP, BX), dyUx = us1(Pk + UX * FP, BX);
   {
     float* sc = scr + ty * BX + e;
@@ -188,10 +188,10 @@ __device__ __forceinline__ void adjoint_centre(const Args& a, const float* Pk, c
     }
   }
   __syncthreads();
-  const f2 m0 = ux1(scr + 0 * SCF + ty * BX + e), m1 = ux1(scr + 1 * SCF + ty * BX + e);
+  const f2 m0 = ux1(scr + ty * BX + e, dyAy), m1 = ux1(scr + SCF + ty * BX + e, dyAx);
   // A: curl and J = grad div A - lap A (the own-axis second derivatives cancel)
   f2 dxAy, xxAy;
-  ux_pair<true, true>(Pk + AY * FP, dxAy, xxAy);
+  ux_pair<true, true>(Pk + AY * FP, vz[AY], dxAy, xxAy);
   const f2 C0 = fma2(a.sy, s0.get(1), mul(a.nsz, d1z[AY]));
   const f2 C1 = fma2(a.sz, d1z[AX], mul(a.nsx, s0.get(0)));
   const f2 C2 = fma2(a.sx, dxAy, mul(a.nsy, dyAx));
@@ -199,15 +199,15 @@ __device__ __forceinline__ void adjoint_centre(const Args& a, const float* Pk, c
   const f2 J1 = fma2(a.sxy, m1, fma2(a.syz, mz[1], fma2(a.nex, xxAy, mul(a.nez, d2z[AY]))));
   const f2 J2 = fma2(a.sz, mz[2], s0.get(6));
   // u: first derivatives; ln rho, ln T: gradients, Laplacian of ln T
-  const f2 U00 = mul(a.sx, ux1(Pk + UX * FP)), U10 = mul(a.sx, ux1(Pk + UY * FP));
+  const f2 U00 = mul(a.sx, ux1(Pk + UX * FP, vz[UX])), U10 = mul(a.sx, ux1(Pk + UY * FP, vz[UY]));
   const f2 U01 = mul(a.sy, dyUx), U11 = mul(a.sy, dyUy);
   const f2 U20 = mul(a.sx, s0.get(3)), U21 = mul(a.sy, s0.get(4));
   const f2 U02 = mul(a.sz, d1z[UX]), U12 = mul(a.sz, d1z[UY]), U22 = mul(a.sz, d1z[UZ]);
-  const f2 gL0 = mul(a.sx, ux1(Pk + LR * FP)), gL1 = mul(a.sy, us1(Pk + LR * FP, BX));
+  const f2 gL0 = mul(a.sx, ux1(Pk + LR * FP, vz[LR])), gL1 = mul(a.sy, us1(Pk + LR * FP, BX));
   const f2 gL2 = fma2(a.sz, d1z[LR], F2(dlk));
   f2 gT0, gT1, xxT, yyT;
-  ux_pair<true, true>(Pk + LT * FP, gT0, xxT);
-  us_pair<true, true>(Pk + LT * FP, BX, gT1, yyT);
+  ux_pair<true, true>(Pk + LT * FP, vz[LT], gT0, xxT);
+  us_pair<true, true>(Pk + LT * FP, BX, vz[LT], gT1, yyT);
   gT0 = mul(a.sx, gT0);
   gT1 = mul(a.sy, gT1);
   const f2 gT2 = fma2(a.sz, d1z[LT], F2(dtk));
@@ -432,17 +432,17 @@ __global__ void __launch_bounds__(NT, 2) rk_pair_kernel(const __grid_constant__ 
       const int X = g == 0 ? AX : UX;
       f2 zx, zy, xx, yy;
       if (ADJ && g == 1) {
-        zx = ux1(P + (X + 2) * FP);
+        zx = ux1(P + (X + 2) * FP, v.get(X + 2));
         zy = us1(P + (X + 2) * FP, BX);
         s.set(7, F2(0.f));  // no second derivative of u in the adjoint
       } else {
-        ux_pair<true, true>(P + (X + 2) * FP, zx, xx);
-        us_pair<true, true>(P + (X + 2) * FP, BX, zy, yy);
+        ux_pair<true, true>(P + (X + 2) * FP, v.get(X + 2), zx, xx);
+        us_pair<true, true>(P + (X + 2) * FP, BX, v.get(X + 2), zy, yy);
         s.set(6 + g, g == 0 ? fma2(a.nex, xx, mul(a.ney, yy)) : fma2(a.v1ex, xx, mul(a.v1ey, yy)));
       }
       s.set(3 * g + 0, zx);
       s.set(3 * g + 1, zy);
-      s.set(3 * g + 2, fma2(a.sx, ux1(P + X * FP), mul(a.sy, us1(P + (X + 1) * FP, BX))));
+      s.set(3 * g + 2, fma2(a.sx, ux1(P + X * FP, v.get(X)), mul(a.sy, us1(P + (X + 1) * FP, BX))));
     }
     tm_st(tlane + VCOL + (uint32_t)(p & 7) * 16, v);
     tm_st(tlane + SCOL + (uint32_t)(p & 7) * 16, s);
@@ -528,9 +528,7 @@ __global__ void __launch_bounds__(NT, 2) rk_pair_kernel(const __grid_constant__ 
       const float* Pk = raw + sk * PLANE + cen;
       // ---- z differences from the TMEM rings --------------------------------
       f2 vz[NF], d1z[NF], d2z[NF], mz[6];
-      V16 s0;  // sources of plane k itself
-#pragma unroll
-      for (int f = 0; f < NF; ++f) vz[f] = ld2(Pk + f * FP);
+      V16 s0, v0_;  // sources and values of plane k itself
 #pragma unroll
       for (int m = 3; m >= 1; --m) {
         const f2 cm = F2(m == 1 ? 45.f : -9.f), em = F2(m == 1 ? 135.f : -13.5f);
@@ -540,7 +538,12 @@ __global__ void __launch_bounds__(NT, 2) rk_pair_kernel(const __grid_constant__ 
         tm_ld(tlane + SCOL + (uint32_t)((k + m) & 7) * 16, sp);
         tm_ld(tlane + SCOL + (uint32_t)((k - m) & 7) * 16, sm);
         if (m == 1) tm_ld(tlane + SCOL + (uint32_t)(k & 7) * 16, s0);
+        if (m == 3) tm_ld(tlane + VCOL + (uint32_t)(k & 7) * 16, v0_);
         tm_wait_ld();
+        if (m == 3) {
+#pragma unroll
+          for (int f = 0; f < NF; ++f) vz[f] = v0_.get(f);
+        }
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
           const f2 d = dif(vp.get(f), vm.get(f)), c = add(vp.get(f), vm.get(f));
@@ -591,13 +594,14 @@ __global__ void __launch_bounds__(NT, 2) rk_pair_kernel(const __grid_constant__ 
       const bool swamp = wk != 0.f || wpk != 0.f;
       // y differences of A_y, A_x, u_y, u_x: also the sources of the xy-mixed
       // terms D1x(D1y .), through the scratch with an x halo
+      const f2 dyAy = us1(Pk + AY * FP, BX);
       f2 dyAx, yyAx, dyUy, yyUy, dyUx, yyUx;
-      us_pair<true, true>(Pk + AX * FP, BX, dyAx, yyAx);
-      us_pair<true, true>(Pk + UY * FP, BX, dyUy, yyUy);
-      us_pair<true, true>(Pk + UX * FP, BX, dyUx, yyUx);
+      us_pair<true, true>(Pk + AX * FP, BX, vz[AX], dyAx, yyAx);
+      us_pair<true, true>(Pk + UY * FP, BX, vz[UY], dyUy, yyUy);
+      us_pair<true, true>(Pk + UX * FP, BX, vz[UX], dyUx, yyUx);
       {
         float* sc = scr + ty * BX + e;
-        *reinterpret_cast<f2*>(sc + 0 * SCF) = us1(Pk + AY * FP, BX);
+        *reinterpret_cast<f2*>(sc + 0 * SCF) = dyAy;
         *reinterpret_cast<f2*>(sc + 1 * SCF) = dyAx;
         *reinterpret_cast<f2*>(sc + 2 * SCF) = dyUy;
         *reinterpret_cast<f2*>(sc + 3 * SCF) = dyUx;
@@ -605,9 +609,8 @@ __global__ void __launch_bounds__(NT, 2) rk_pair_kernel(const __grid_constant__ 
             us1(raw + sk * PLANE + hfield * FP + (hr + 3) * BX + hx, BX);
       }
       __syncthreads();
-      f2 mxy[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) mxy[q] = ux1(scr + q * SCF + ty * BX + e);
+      const float* sr = scr + ty * BX + e;
+      const f2 mxy[4] = {ux1(sr, dyAy), ux1(sr + SCF, dyAx), ux1(sr + 2 * SCF, dyUy), ux1(sr + 3 * SCF, dyUx)};
 
       const Phys<float>& ph = a.ph;
       // A: B = curl A + B_ext, J = grad div A - lap A, swamp terms of the
@@ -615,7 +618,7 @@ __global__ void __launch_bounds__(NT, 2) rk_pair_kernel(const __grid_constant__ 
       f2 B0, B1, B2, J0, J1, J2, sw0 = F2(0.f), sw1 = F2(0.f), sw2 = F2(0.f);
       {
         f2 dxAy, xxAy;
-        ux_pair<true, true>(Pk + AY * FP, dxAy, xxAy);
+        ux_pair<true, true>(Pk + AY * FP, vz[AY], dxAy, xxAy);
         B0 = fma2(a.sy, s0.get(1), fma2(a.nsz, d1z[AY], a.bext[0]));
         B1 = fma2(a.sz, d1z[AX], fma2(a.nsx, s0.get(0), a.bext[1]));
         B2 = fma2(a.sx, dxAy, fma2(a.nsy, dyAx, a.bext[2]));
@@ -624,8 +627,8 @@ __global__ void __launch_bounds__(NT, 2) rk_pair_kernel(const __grid_constant__ 
         J2 = fma2(a.sz, mz[2], s0.get(6));
         if (swamp) {
           f2 xxAx, yyAy, none;
-          ux_pair<false, true>(Pk + AX * FP, none, xxAx);
-          us_pair<false, true>(Pk + AY * FP, BX, none, yyAy);
+          ux_pair<false, true>(Pk + AX * FP, vz[AX], none, xxAx);
+          us_pair<false, true>(Pk + AY * FP, BX, vz[AY], none, yyAy);
           f2 l0 = fma2(a.ex, xxAx, fma2(a.ey, yyAx, mul(a.ez, d2z[AX])));
           f2 l1 = fma2(a.ex, xxAy, fma2(a.ey, yyAy, mul(a.ez, d2z[AY])));
           f2 l2 = dif(mul(a.ez, d2z[AZ]), s0.get(6));
@@ -658,9 +661,9 @@ __global__ void __launch_bounds__(NT, 2) rk_pair_kernel(const __grid_constant__ 
       f2 U00, U10, v0, v1, v2;
       {
         f2 xx;
-        ux_pair<true, true>(Pk + UX * FP, U00, xx);
+        ux_pair<true, true>(Pk + UX * FP, vz[UX], U00, xx);
         v0 = fma2(a.v4ex, xx, fma2(a.v1ey, yyUx, fma2(a.v1ez, d2z[UX], fma2(a.v3xy, mxy[2], mul(a.v3xz, mz[3])))));
-        ux_pair<true, true>(Pk + UY * FP, U10, xx);
+        ux_pair<true, true>(Pk + UY * FP, vz[UY], U10, xx);
         v1 = fma2(a.v1ex, xx, fma2(a.v4ey, yyUy, fma2(a.v1ez, d2z[UY], fma2(a.v3xy, mxy[3], mul(a.v3yz, mz[4])))));
         v2 = fma2(a.v4ez, d2z[UZ], fma2(a.v3z, mz[5], s0.get(7)));
         U00 = mul(a.sx, U00);
@@ -673,11 +676,11 @@ __global__ void __launch_bounds__(NT, 2) rk_pair_kernel(const __grid_constant__ 
       f2 gL0, gL1, lapL, gT0, gT1, lapT;
       {
         f2 xx, yy;
-        ux_pair<true, true>(Pk + LR * FP, gL0, xx);
-        us_pair<true, true>(Pk + LR * FP, BX, gL1, yy);
+        ux_pair<true, true>(Pk + LR * FP, vz[LR], gL0, xx);
+        us_pair<true, true>(Pk + LR * FP, BX, vz[LR], gL1, yy);
         lapL = fma2(a.ex, xx, fma2(a.ey, yy, fma2(a.ez, d2z[LR], F2(d2lk))));
-        ux_pair<true, true>(Pk + LT * FP, gT0, xx);
-        us_pair<true, true>(Pk + LT * FP, BX, gT1, yy);
+        ux_pair<true, true>(Pk + LT * FP, vz[LT], gT0, xx);
+        us_pair<true, true>(Pk + LT * FP, BX, vz[LT], gT1, yy);
         lapT = fma2(a.ex, xx, fma2(a.ey, yy, fma2(a.ez, d2z[LT], F2(d2tk))));
         gL0 = mul(a.sx, gL0);
         gL1 = mul(a.sy, gL1);
