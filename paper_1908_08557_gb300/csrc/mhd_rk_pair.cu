@@ -892,7 +892,7 @@ static int pair_ctas() {
 }
 
 static pair::Args pair_args(const Layout& L, const Phys<float>& ph, const Background<float>& bg, const float* wtab,
-                            const float* wptab, StepState* ss, int sub, double dx, double dy, double dz) {
+                            const float* wptab, StepState* ss, int sub, double dx, double dy, double dz, bool adj) {
   const int ctas = pair_ctas();
   pair::Args a{};
   a.wait_limit = zm::WAIT_LIMIT;
@@ -921,9 +921,21 @@ static pair::Args pair_args(const Layout& L, const Phys<float>& ph, const Backgr
   a.neta = P(-ph.eta); a.nu = P(nu); a.gm1 = P(ph.gm1); a.drho = P(ph.drho);
   a.heat = P((double)ph.gm1 * ph.eta); a.visc = P((double)ph.gm1 * nu); a.cond = P((double)ph.gm1 * ph.kappa0);
   for (int c = 0; c < 3; ++c) a.bext[c] = P(ph.bext[c]);
+  // Where a CTA has some fifty planes of work or more, it claims its items and
+  // the chunks are short enough that the launch ends evenly (a chunk's prologue
+  // then costs about 1.35 centre planes, fitted to launches at 1024 x 1024 x
+  // 128 with chunks of 16 to 128 layers; 512 x 256 x 97: 545 us by grid stride
+  // with whole columns, 479 claimed in chunks of 20; 256^3: 526 -> 517; 1024 x
+  // 1024 x 128 about a background: 4534 -> 4404).  Smaller launches are bound
+  // by the latency of a chunk's chain, where every prologue plane counts, and
+  // take whole waves by grid stride.
+  // (The adjoint point kernel, bound by its writes, claims from a dozen items
+  // per CTA on: at 256^3 claimed short chunks cost it 4 %.)
   const int tiles = a.ntx * a.nty;
-  a.kchunk = zm::zchunk(L.nz, tiles, ctas);
+  a.dyn = !adj && (long long)tiles * L.nz >= 48LL * ctas;
+  a.kchunk = a.dyn ? zm::zchunk_claimed(L.nz, tiles, ctas, 1.35) : zm::zchunk(L.nz, tiles, ctas);
   a.nch = (L.nz + a.kchunk - 1) / a.kchunk;
+  a.dyn = adj ? tiles * a.nch >= 12 * ctas : a.dyn && tiles * a.nch > ctas;
   return a;
 }
 
@@ -931,7 +943,7 @@ void launch_rk_pair(const CUtensorMap* tm, const CUtensorMap* tmd, const Layout&
                     const Background<float>& bg, float* fout, float* df, const float* wtab, const float* wptab,
                     const Driver& drv, StepState* ss, int sub, double dx, double dy, double dz, cudaStream_t st,
                     int skip_plane, int wait_limit, bool chained) {
-  pair::Args a = pair_args(L, ph, bg, wtab, wptab, ss, sub, dx, dy, dz);
+  pair::Args a = pair_args(L, ph, bg, wtab, wptab, ss, sub, dx, dy, dz, false);
   if (skip_plane != INT_MIN) {
     a.skip_plane = skip_plane;
     a.wait_limit = wait_limit;
@@ -944,10 +956,6 @@ void launch_rk_pair(const CUtensorMap* tm, const CUtensorMap* tmd, const Layout&
   a.v1 = (const float*)drv.v1;
   const int nitems = a.ntx * a.nty * a.nch;
   const int grid = nitems < pair_ctas() ? nitems : pair_ctas();
-  // claimed work items where a CTA has a dozen or more: there the grid
-  // stride's imbalance outweighs the claims (1024 x 1024 x 256: step 4 %
-  // faster; at 256^3, six items per CTA, the stride is 2 % faster)
-  a.dyn = nitems >= 12 * grid;
   // the instantiation for the options in use (cooling, A about a
   // background, non-uniform vertical grid)
   const int opt = (ph.nc_k1 > 0 ? 1 : 0) | (bg.bB != nullptr ? 2 : 0) | (bg.zm1 != nullptr ? 4 : 0);
@@ -973,13 +981,12 @@ void launch_adj_point_pair(const CUtensorMap* tm, const CUtensorMap* tmd, const 
                            const Background<float>& bg, const float* dbar, float* coef, double* thbar,
                            const float* wtab, const float* wptab, StepState* ss, int sub, double dx, double dy,
                            double dz, cudaStream_t st, bool chained) {
-  pair::Args a = pair_args(L, ph, bg, wtab, wptab, ss, sub, dx, dy, dz);
+  pair::Args a = pair_args(L, ph, bg, wtab, wptab, ss, sub, dx, dy, dz, true);
   a.dbar = dbar;
   a.coef = coef;
   a.thbar = thbar;
   const int nitems = a.ntx * a.nty * a.nch;
   const int grid = nitems < pair_ctas() ? nitems : pair_ctas();
-  a.dyn = nitems >= 12 * grid;
   if (a.dyn) cudaMemsetAsync(&ss->items, 0, sizeof(int), st);
   launch_chained(chained && !a.dyn, pair::rk_pair_kernel<true, false, false, false>, grid, pair::NT, pair::SMEM_BYTES, st,
                  *tm, *tmd, a);

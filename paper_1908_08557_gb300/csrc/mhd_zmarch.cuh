@@ -133,5 +133,22 @@ inline int zchunk(int nz, int tiles, int ctas) {
   return (nz + best - 1) / best;
 }
 
+// The same for work items that CTAs claim as they finish one: the launch takes
+// the work of a CTA (its planes, and `lead` centre planes' worth of prologue
+// per chunk) and, at the end, half an item more.  Returns the chunk length.
+inline int zchunk_claimed(int nz, int tiles, int ctas, double lead) {
+  int best = nz;
+  double cost = 0.0;
+  for (int nch = 1; nch <= nz; ++nch) {
+    const int kc = (nz + nch - 1) / nch;
+    const double c = (double)tiles * nz / ctas * (1.0 + lead / kc) + 0.5 * (kc + lead);
+    if (nch == 1 || c < cost) {
+      cost = c;
+      best = kc;
+    }
+  }
+  return best;
+}
+
 }  // namespace zm
 }  // namespace mhd
