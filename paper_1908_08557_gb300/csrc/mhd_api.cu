@@ -511,14 +511,27 @@ template <typename R>
 static void ghost_fill(mhd_ctx* h, R* f, bool chained = false) {
   Phys<R> ph = make_phys<R>(&h->p);
   const bool one = one_chain(h);
-  {
+  auto rules = [&](bool behind) {
     ClassTimer ct(h, MHD_KC_GHOST, 1);
-    launch_bc<R>(h->L, ph, bgr<R>(h), f, h->ss, h->st, chained && one);
+    launch_bc<R>(h->L, ph, bgr<R>(h), f, h->ss, h->st, behind);
+  };
+  if (h->p.bc_z != 0 || h->serial || pfe_one_chain(h->p.nx, h->p.ny)) {
+    rules(chained && one);
+    if (h->p.bc_z == 0) {
+      ClassTimer ct(h, MHD_KC_PFE, 3);
+      launch_pfe<R>(h->fp, h->L, f, h->ss, h->st, nullptr, one);
+    }
+    return;
   }
-  if (h->p.bc_z == 0) {
+  // three chains of FFT kernels: the ghost rules follow the first one on the
+  // handle's stream, beside the tails of the other two (they touch no plane
+  // the transforms read or write)
+  {
     ClassTimer ct(h, MHD_KC_PFE, 3);
-    launch_pfe<R>(h->fp, h->L, f, h->ss, h->st, h->serial ? nullptr : &h->ps, one);
+    launch_pfe<R>(h->fp, h->L, f, h->ss, h->st, &h->ps);
   }
+  rules(false);
+  pfe_join(h->ps, h->st);
 }
 
 static void release_side(mhd_ctx* h) {
@@ -644,6 +657,7 @@ static void run_step(mhd_ctx* h, bool stats) {
       {
         ClassTimer ct(h, MHD_KC_PFE, 3, h->side);
         launch_pfe<R>(h->fp, h->L, fin, h->ss, h->side, &h->ps);
+        if (!pfe_one_chain(h->p.nx, h->p.ny)) pfe_join(h->ps, h->side);
       }
       cudaEventRecord(h->evj, h->side);
       {
@@ -725,6 +739,9 @@ static int upload_fft_tables(mhd_ctx* h, const Offsets& o) {
   // photosphere, d'_m = z_0 - z_{-m} (m dz on the uniform grid)
   double lx = nx * p->dx, ly = ny * p->dy;
   const size_t n2 = (size_t)nx * ny;
+  // with the normalisation 1 / (nx ny) of the inverse transform, an exact power
+  // of two
+  const double norm = 1.0 / ((double)nx * ny);
   std::vector<double> et(3 * n2), eb(3 * n2);
   const int kt = p->nz - 1;
   for (int m = 1; m <= NG; ++m) {
@@ -736,8 +753,8 @@ static int upload_fft_tables(mhd_ctx* h, const Offsets& o) {
         int mb = 2 * b > ny ? b - ny : b;
         double ky = 2.0 * M_PI * mb / ly;
         double kk = sqrt(kx * kx + ky * ky);
-        et[(size_t)(m - 1) * n2 + (size_t)a * ny + b] = exp(-kk * dt);
-        eb[(size_t)(m - 1) * n2 + (size_t)a * ny + b] = exp(p->f_pfe_bottom * kk * db);
+        et[(size_t)(m - 1) * n2 + (size_t)a * ny + b] = norm * exp(-kk * dt);
+        eb[(size_t)(m - 1) * n2 + (size_t)a * ny + b] = norm * exp(p->f_pfe_bottom * kk * db);
       }
     }
   }

@@ -299,8 +299,8 @@ __global__ void __launch_bounds__(256) cols_kernel(FFTPlan fp, int mode, const S
 }
 
 // ---------------------------------------------------------------------------
-// 3. inverse rows: normalise by 1/(nx ny); mode 0 writes ghost layers of the
-// state, mode 1 the compact planes out_re, out_im ([ny][nx]).
+// 3. inverse rows, normalised by 1/(nx ny) (modes 0 and 2: through the
+// multipliers); mode 0 writes ghost layers of the state, mode 1 the compact planes out_re, out_im ([ny][nx]).
 // mode 2 (adjoint): plane c adds its real part into A_c at the top layer and
 // its imaginary part into A_c at the photosphere (interior x, y only);
 // mode 3: real part into out_re.
@@ -344,7 +344,9 @@ __global__ void __launch_bounds__(256) rows_inv_kernel(FFTPlan fp, Layout L, R* 
       energy = fma(wx, wx, fma(wy, wy, energy));
       continue;
     }
-    const R re = (R)(v.x * sc), im = (R)(v.y * sc);
+    // (modes 0 and 2: the multipliers carry the normalisation)
+    const bool scaled = mode == 0 || mode == 2;
+    const R re = (R)(scaled ? v.x : v.x * sc), im = (R)(scaled ? v.y : v.y * sc);
     if (mode == 1) {
       out_re[(long long)y * nx + x] = re;
       out_im[(long long)y * nx + x] = im;
@@ -579,10 +581,11 @@ void launch_pfe(const FFTPlan& fp, const Layout& L, R* f, const StepState* ss, c
     rows_inv_kernel<R><<<dim3(fp.ny / ri.nb, 1, 3), ri.threads, ri.smem, sp>>>(fq, L, f, nullptr, nullptr, 0, ss,
                                                                               ri.nb, RowsAdd{});
   }
-  for (int i = 0; i < 2; ++i) {
-    cudaEventRecord(ps->join[i], ps->s[i]);
-    cudaStreamWaitEvent(st, ps->join[i], 0);
-  }
+  for (int i = 0; i < 2; ++i) cudaEventRecord(ps->join[i], ps->s[i]);
+}
+
+void pfe_join(const PlaneStreams& ps, cudaStream_t st) {
+  for (int i = 0; i < 2; ++i) cudaStreamWaitEvent(st, ps.join[i], 0);
 }
 
 template <typename R>

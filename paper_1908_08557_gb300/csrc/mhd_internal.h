@@ -25,8 +25,8 @@ struct FFTPlan {
   int nx, ny, lognx, logny;
   const double2* twx;  // twiddles exp(-2 pi i r / nx), r < nx, as twiddle_pair gives them
   const double2* twy;  // the same for ny
-  const double* et;    // [3][kx][ky] exp(-|k| d_m), ghost layer m above the top (Eq. 17)
-  const double* eb;    // [3][kx][ky] exp(+f_b |k| d'_m), ghost layer m below the photosphere (Sect. 2.4)
+  const double* et;    // [3][kx][ky] exp(-|k| d_m) / (nx ny), ghost layer m above the top (Eq. 17)
+  const double* eb;    // [3][kx][ky] exp(+f_b |k| d'_m) / (nx ny), ghost layer m below the photosphere (Sect. 2.4)
   const double* ktx;   // modified first-derivative wavenumbers, [nx]
   const double* kty;   // [ny]
   double2* P;          // [3][nx][ny] row spectra, transposed
@@ -128,12 +128,14 @@ constexpr int CFL_SLOTS = 256;         // CFL maxima slot pairs (after the parti
 // ghost fill
 template <typename R> void launch_bc(const Layout& L, const Phys<R>& ph, const Background<R>& bg, R* f,
                                      const StepState* ss, cudaStream_t st, bool chained = false);
-// potential-field ghosts of A (three FFT kernels)
-// (ps: run the three planes on three streams; nullptr: one stream)
+// potential-field ghosts of A (three FFT kernels); ps: planes above the size of
+// pfe_one_chain run on three streams, joined back by pfe_join; nullptr: one
+// stream
 template <typename R> void launch_pfe(const FFTPlan& fp, const Layout& L, R* f, const StepState* ss,
                                       cudaStream_t st, const PlaneStreams* ps = nullptr, bool chained = false);
 // planes small enough to go as one chain of kernels whatever ps says
 bool pfe_one_chain(int nx, int ny);
+void pfe_join(const PlaneStreams& ps, cudaStream_t st);
 // vector potential of the target magnetogram into axt, ayt
 template <typename R> void launch_atarget(const FFTPlan& fp, const R* bz, R* axt, R* ayt, cudaStream_t st);
 // filtered rotational part (Eq. 3) of the plane field (vx, vy) into (rx, ry),
