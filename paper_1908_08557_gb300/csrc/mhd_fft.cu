@@ -67,6 +67,37 @@ __device__ __forceinline__ void bfly(double2 b0, double2 b1, double2 w, bool swa
 __device__ double2* fft_lines(double2* a, double2* b, int n, int logn, int nb, const double2* __restrict__ tw,
                               bool inverse) {
   int p = 1, lp = 0;
+  if (2 * (int)blockDim.x >= nb * n) {
+    // a thread per radix-2 butterfly: where threads are plenty the transform is
+    // a chain of FP64 instructions of 64 clocks each, 34 here against 64 in the
+    // radix-4 form below for 64 points (64 x 64 planes, three fills of a step:
+    // 148 -> 143 us a step at 64^3)
+    const int half = n >> 1;
+    const int q = threadIdx.x, line = q >> (logn - 1), i = q & (half - 1);
+    const bool on = q < nb * half;
+    for (; p < n; p <<= 1, ++lp) {
+      if (on) {
+        const int k = i & (p - 1);
+        const double2 u0 = a[line * n + i], u1 = a[line * n + i + half];
+        double2* y = b + line * n + 2 * i - k;
+        double2 s, d;
+        if (p > 1) {
+          const int r = k << (logn - 1 - lp);
+          bfly(u0, u1, __ldg(tw + r), twiddle_swap(r, logn), inverse, s, d);
+        } else {
+          s = cadd(u0, u1);
+          d = csub(u0, u1);
+        }
+        y[0] = s;
+        y[p] = d;
+      }
+      __syncthreads();
+      double2* t = a;
+      a = b;
+      b = t;
+    }
+    return a;
+  }
   if (logn & 1) {
     const int half = n >> 1;
     const int total = nb * half;
@@ -365,17 +396,25 @@ __global__ void __launch_bounds__(256) rows_inv_kernel(FFTPlan fp, Layout L, R* 
     if (p == 0) { f1 = AX; k1 = ktop; f2 = AY; k2 = ktop; }
     else if (p == 1) { f1 = AX; k1 = kbot; f2 = AY; k2 = kbot; }
     else { f1 = AZ; k1 = ktop; f2 = AZ; k2 = kbot; }
-    int xs[3], ys[3], nxs = 1, nys = 1;
-    xs[0] = x; ys[0] = y;
-    if (x < NG) xs[nxs++] = x + nx;
-    if (x >= nx - NG) xs[nxs++] = x - nx;
-    if (y < NG) ys[nys++] = y + ny;
-    if (y >= ny - NG) ys[nys++] = y - ny;
-    for (int bb = 0; bb < nys; ++bb)
-      for (int aa = 0; aa < nxs; ++aa) {
-        f[L.at(f1, k1, ys[bb], xs[aa])] = re;
-        f[L.at(f2, k2, ys[bb], xs[aa])] = im;
-      }
+    // the cell and its periodic images (nx, ny >= 8: at most one per direction)
+    const int ox = x < NG ? nx : (x >= nx - NG ? -nx : 0);
+    const long long oy = y < NG ? (long long)ny * L.mx : (y >= ny - NG ? -(long long)ny * L.mx : 0);
+    R* q1 = f + L.at(f1, k1, y, x);
+    R* q2 = f + L.at(f2, k2, y, x);
+    q1[0] = re;
+    q2[0] = im;
+    if (ox) {
+      q1[ox] = re;
+      q2[ox] = im;
+    }
+    if (oy) {
+      q1[oy] = re;
+      q2[oy] = im;
+    }
+    if (ox && oy) {
+      q1[ox + oy] = re;
+      q2[ox + oy] = im;
+    }
   }
   if (mode == 5) {
     // fixed order: warp tree, then the warps in turn
@@ -480,9 +519,13 @@ struct FFTLaunch {
   size_t smem_cols, smem_cols3;
 };
 
-// one thread per radix-4 butterfly of a stage of `lines` lines of n points
-static int butterfly_threads(int lines, int n) {
-  const int t = (lines * n / 4 + 31) / 32 * 32;
+// Threads of a block with `lines` lines of n points: one per radix-4 butterfly
+// of a stage, so that every warp has FP64 work; where the launch's blocks leave
+// SMs with one or two of them, one per point, so that loading, the multipliers
+// and storing are one pass each instead of four serial ones.
+static int line_threads(long long blocks, int lines, int n) {
+  const int per = blocks <= 2LL * sm_count() ? 1 : 4;
+  const int t = (lines * n / per + 31) / 32 * 32;
   return t < 32 ? 32 : (t > 256 ? 256 : t);
 }
 
@@ -502,15 +545,15 @@ static FFTLaunch fft_launch(const FFTPlan& fp, int planes) {
   // form, 192 KB and one block per SM, measured 8 % slower)
   l.lg = (size_t)6 * 2 * l.ppb * fp.ny * sizeof(double2) <= (size_t)96 * 1024 ? 3 : 1;
   l.smem_cols3 = (size_t)(l.lg == 3 ? 6 : 3) * 2 * l.ppb * fp.ny * sizeof(double2);
-  l.threads = butterfly_threads(2 * l.ppb, fp.ny);
-  l.threads3 = butterfly_threads(2 * l.ppb * l.lg, fp.ny);
+  const long long blocks = (long long)planes * ((npairs + l.ppb - 1) / l.ppb);
+  l.threads = line_threads(blocks, 2 * l.ppb, fp.ny);
+  l.threads3 = line_threads(blocks, 2 * l.ppb * l.lg, fp.ny);
   return l;
 }
 
 // Row transforms of `planes` planes: lines per block chosen so that the
 // blocks spread evenly over the SMs (all blocks of these kernels are resident
-// at once and share each SM's FP64 pipe, so the busiest SM sets the time);
-// one thread per radix-4 butterfly of a stage.
+// at once and share each SM's FP64 pipe, so the busiest SM sets the time).
 struct RowsCfg {
   int nb, threads;
   size_t smem;
@@ -532,9 +575,7 @@ static RowsCfg rows_cfg(const FFTPlan& fp, int planes) {
       c.nb = nb;
     }
   }
-  c.threads = c.nb * fp.nx / 4;
-  if (c.threads > 256) c.threads = 256;
-  if (c.threads < 32) c.threads = 32;
+  c.threads = line_threads((long long)planes * (fp.ny / c.nb), c.nb, fp.nx);
   c.smem = (size_t)2 * c.nb * fp.nx * sizeof(double2);
   return c;
 }

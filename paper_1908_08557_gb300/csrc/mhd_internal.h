@@ -108,6 +108,16 @@ inline void launch_chained(bool chained, void (*k)(P...), dim3 grid, dim3 block,
   c.numAttrs = chained ? 1 : 0;
   cudaLaunchKernelEx(&c, k, P(a)...);
 }
+// Dynamic shared memory that keeps a grid of at most one block per SM on one
+// block per SM.  Blocks of a chained launch are placed while the predecessor
+// still runs, and the SMs its blocks have left can get two of them while others
+// get none; for FP64 blocks, which share an SM's FP64 pipe, that doubles the
+// kernel (an FP64 step at 32^3: 311 us, 231 so).  With more than half of an SM's shared memory to a
+// block every SM takes one.  The limit itself is raised once per device.
+constexpr size_t ONE_PER_SM_BYTES = 88 * 1024;  // + 32 KB static: over half of 228 KB
+inline size_t one_per_sm(bool chained, dim3 g) {
+  return chained && (size_t)g.x * g.y * g.z <= (size_t)sm_count() ? ONE_PER_SM_BYTES : 0;
+}
 #ifdef __CUDACC__
 // Wait for the predecessor of a chained launch, then let the successor's blocks
 // be scheduled.  A successor's blocks so start when all of this grid's blocks

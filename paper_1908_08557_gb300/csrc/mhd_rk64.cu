@@ -470,6 +470,18 @@ __global__ void __launch_bounds__(NT, 2) rk64_kernel(const __grid_constant__ Arg
 
 static dim3 grid64(const Layout& L) { return dim3((L.nx + TX - 1) / TX, L.ny, (L.nz + KZ - 1) / KZ); }
 
+// (the kernels' shared-memory limit is raised once per device)
+static size_t spread64(bool chained, dim3 g) {
+  static PerDevice<bool> done;
+  done.get([] {
+    cudaFuncSetAttribute(rk64_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ONE_PER_SM_BYTES);
+    cudaFuncSetAttribute(rk64_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ONE_PER_SM_BYTES);
+    cudaFuncSetAttribute(rk64_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ONE_PER_SM_BYTES);
+    return true;
+  });
+  return one_per_sm(chained, g);
+}
+
 static Coef64 coef64(const Phys<double>& ph, bool zg) {
   Coef64 c;
   c.cx = ph.idx / 60.0;
@@ -521,18 +533,19 @@ void launch_rk64(const Layout& L, const Phys<double>& ph, const Background<doubl
   const bool zg = bg.zm1 != nullptr;
   a.c = r64::coef64(ph, zg);
   const dim3 g = r64::grid64(L), b(r64::TX, r64::KZ);
-  if (zg) launch_chained(chained, r64::rk64_kernel<false, true>, g, b, 0, st, a);
-  else launch_chained(chained, r64::rk64_kernel<false, false>, g, b, 0, st, a);
+  const size_t smem = r64::spread64(chained, g);
+  if (zg) launch_chained(chained, r64::rk64_kernel<false, true>, g, b, smem, st, a);
+  else launch_chained(chained, r64::rk64_kernel<false, false>, g, b, smem, st, a);
 }
 
-void launch_adj_point64(const Layout& L, const Phys<double>& ph, const Background<double>& bg, const double* g,
+void launch_adj_point64(const Layout& L, const Phys<double>& ph, const Background<double>& bg, const double* gst,
                         const double* dbar, double* coef, double* thbar, const double* wtab, const double* wptab,
                         const StepState* ss, int sub, cudaStream_t st, bool chained) {
   r64::Args a{};
   a.L = L;
   a.ph = ph;
   a.bg = bg;
-  a.fin = g;
+  a.fin = gst;
   a.wtab = wtab;
   a.wptab = wptab;
   a.ss = ss;
@@ -541,7 +554,8 @@ void launch_adj_point64(const Layout& L, const Phys<double>& ph, const Backgroun
   a.coef = coef;
   a.thbar = thbar;
   a.c = r64::coef64(ph, false);
-  launch_chained(chained, r64::rk64_kernel<true, false>, r64::grid64(L), dim3(r64::TX, r64::KZ), 0, st, a);
+  const dim3 g = r64::grid64(L);
+  launch_chained(chained, r64::rk64_kernel<true, false>, g, dim3(r64::TX, r64::KZ), r64::spread64(chained, g), st, a);
 }
 
 }  // namespace mhd
