@@ -515,11 +515,17 @@ static void ghost_fill(mhd_ctx* h, R* f, bool chained = false) {
     ClassTimer ct(h, MHD_KC_GHOST, 1);
     launch_bc<R>(h->L, ph, bgr<R>(h), f, h->ss, h->st, behind);
   };
+  if (one && h->p.bc_z == 0) {
+    ClassTimer ct(h, MHD_KC_PFE, 3);
+    const GhostRules<R> gr{ph, bgr<R>(h)};
+    launch_pfe<R>(h->fp, h->L, f, h->ss, h->st, nullptr, chained, &gr);
+    return;
+  }
   if (h->p.bc_z != 0 || h->serial || pfe_one_chain(h->p.nx, h->p.ny)) {
     rules(chained && one);
     if (h->p.bc_z == 0) {
       ClassTimer ct(h, MHD_KC_PFE, 3);
-      launch_pfe<R>(h->fp, h->L, f, h->ss, h->st, nullptr, one);
+      launch_pfe<R>(h->fp, h->L, f, h->ss, h->st);
     }
     return;
   }

@@ -19,6 +19,7 @@
 //                M_b = exp(+f_b |k| j dz)), inverse FFT along y
 //   3. rows_inv: inverse FFT along x, write real/imaginary parts into the
 //                ghost layers (with their periodic x,y images)
+#include "mhd_bc.cuh"
 #include "mhd_internal.h"
 
 namespace mhd {
@@ -219,25 +220,22 @@ __global__ void __launch_bounds__(256) rows_fwd_kernel(FFTPlan fp, Layout L, con
 // transpose; mode 4: the filtered rotational part of the granulation field
 // (Sect. 2.3, Eq. 3).  The spectra of lg output layers at a time are formed and
 // inverted as one batch of lines, so each stage of the inverse transform has
-// lg times the butterflies between two barriers; lg = nout needs two buffers
-// of lg layers (the forward spectrum's buffer becomes the scratch), lg < nout
-// three (the spectrum is kept).
-__global__ void __launch_bounds__(256) cols_kernel(FFTPlan fp, int mode, const StepState* ss, int ppb, int lg) {
+// lg times the butterflies between two barriers; with all of the layers o_first
+// .. o_end - 1 in one batch two buffers of lg layers do (the forward spectrum's
+// buffer becomes the scratch), otherwise three (the spectrum is kept).
+__device__ __forceinline__ void cols_block(const FFTPlan& fp, int mode, int ppb, int lg, int o_first, int o_end) {
   extern __shared__ double2 sm[];
-  chain_enter();
-  if (ss && halted(ss)) return;
   const int nx = fp.nx, ny = fp.ny;
   const int npairs = nx / 2 + 1;
   const int pair0 = blockIdx.x * ppb;  // ppb column pairs per block
   const int np = min(ppb, npairs - pair0);
   const int nl = 2 * np;
   const int p = fp.p0 + blockIdx.y;
-  const int nout = mode == 0 ? 3 : 1;
   const int npts = nl * ny;            // points of one layer
   const int bsz = lg * 2 * ppb * ny;   // points of one buffer
   double2* A = sm;
   double2* B = sm + bsz;
-  double2* Z = sm + 2 * bsz;           // used when lg < nout
+  double2* Z = sm + 2 * bsz;           // more than one batch
   // columns of line l: pair (l >> 1), mirror if odd
   for (int q = threadIdx.x; q < npts; q += blockDim.x) {
     const int line = q / ny, y = q - line * ny;
@@ -248,9 +246,9 @@ __global__ void __launch_bounds__(256) cols_kernel(FFTPlan fp, int mode, const S
   __syncthreads();
   double2* spec = fft_lines(A, B, ny, fp.logny, nl, fp.twy, false);
   double2* G = (spec == A) ? B : A;  // layer o0 + o's lines at G + o npts
-  double2* T = lg == nout ? spec : Z;
+  double2* T = lg == o_end - o_first ? spec : Z;
   const int nplanes = mode == 0 ? 3 : 1;
-  for (int o0 = 0; o0 < nout; o0 += lg) {
+  for (int o0 = o_first; o0 < o_end; o0 += lg) {
   for (int q = threadIdx.x; q < lg * npts; q += blockDim.x) {
     const int o = o0 + q / npts, qq = q - (o - o0) * npts;
     const int line = qq / ny, ky = qq - line * ny;
@@ -327,6 +325,40 @@ __global__ void __launch_bounds__(256) cols_kernel(FFTPlan fp, int mode, const S
   }
   __syncthreads();
   }
+}
+
+// gridDim.z = 3: one ghost layer per block, the forward transform repeated in
+// each.  While that leaves at most two blocks per SM the repetition costs no
+// time and the inverse has a third of the serial FP64 instructions.
+__global__ void __launch_bounds__(256) cols_kernel(FFTPlan fp, int mode, const StepState* ss, int ppb, int lg) {
+  chain_enter();
+  if (ss && halted(ss)) return;
+  const int o = gridDim.z > 1 ? (int)blockIdx.z : 0, n = mode == 0 && gridDim.z == 1 ? 3 : 1;
+  cols_block(fp, mode, ppb, lg, o, o + n);
+}
+
+// The columns of the potential-field ghosts with the pointwise ghost rules in
+// the same launch, on planes whose boundary chain is a row of short kernels:
+// the rules touch no plane of the transforms, and the blocks from x = ncol on
+// take them, both ends of all columns, beside the transforms (ghost
+// fill 64 x 64 31 -> 23 us, 32 x 32 21 -> 17: the rules' launch is gone from the
+// chain, and their time is hidden).
+template <typename R>
+__global__ void __launch_bounds__(256) cols_rules_kernel(FFTPlan fp, const StepState* ss, int ppb, int lg, int ncol,
+                                                         Layout L, Phys<R> ph, Background<R> bg, R* f) {
+  chain_enter();
+  if (halted(ss)) return;
+  if ((int)blockIdx.x < ncol) {
+    const int o = gridDim.z > 1 ? (int)blockIdx.z : 0;
+    cols_block(fp, 0, ppb, lg, o, gridDim.z > 1 ? o + 1 : 3);
+    return;
+  }
+  const int pw = L.nx + 2 * NG, n = pw * (L.ny + 2 * NG);
+  const int blk = ((int)(blockIdx.x - ncol) * gridDim.y + blockIdx.y) * gridDim.z + blockIdx.z;
+  const int q = blk * blockDim.x + threadIdx.x;
+  if (q >= 2 * n) return;
+  const int c = q < n ? q : q - n;
+  ghost_rules<R>(L, ph, bg, f, c % pw - NG, c / pw - NG, q >= n);
 }
 
 // ---------------------------------------------------------------------------
@@ -505,6 +537,8 @@ static void set_smem_once() {
     cudaFuncSetAttribute(rows_inv_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * FFT_PTS * 16);
     cudaFuncSetAttribute(rows_inv_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * FFT_PTS * 16);
     cudaFuncSetAttribute(cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 6 * FFT_PTS * 16);
+    cudaFuncSetAttribute(cols_rules_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 6 * FFT_PTS * 16);
+    cudaFuncSetAttribute(cols_rules_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 6 * FFT_PTS * 16);
     cudaFuncSetAttribute(cols_adj_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 6 * FFT_PTS * 16);
     return true;
   });
@@ -517,6 +551,9 @@ struct FFTLaunch {
   int ppb, lg;                   // lg: ghost layers per inverse batch in cols
   int threads, threads3;         // cols: one output layer, three
   size_t smem_cols, smem_cols3;
+  int layers;                    // cols of all planes in one launch: blocks per column batch (gridDim.z) ...
+  int lgz, threadsz;             // ... and theirs
+  size_t smemz;
 };
 
 // Threads of a block with `lines` lines of n points: one per radix-4 butterfly
@@ -548,6 +585,13 @@ static FFTLaunch fft_launch(const FFTPlan& fp, int planes) {
   const long long blocks = (long long)planes * ((npairs + l.ppb - 1) / l.ppb);
   l.threads = line_threads(blocks, 2 * l.ppb, fp.ny);
   l.threads3 = line_threads(blocks, 2 * l.ppb * l.lg, fp.ny);
+  // one ghost layer per block while that leaves at most two blocks per SM
+  // (FP32 step at 32^3
+  // 98.3 -> 97.6 us, FP64 at 64 x 32 x 45 477.8 -> 475.3)
+  l.layers = 3 * blocks <= 2LL * sm_count() ? 3 : 1;
+  l.lgz = l.layers == 3 ? 1 : l.lg;
+  l.threadsz = l.layers == 3 ? line_threads(3 * blocks, 2 * l.ppb, fp.ny) : l.threads3;
+  l.smemz = l.layers == 3 ? (size_t)2 * 2 * l.ppb * fp.ny * sizeof(double2) : l.smem_cols3;
   return l;
 }
 
@@ -584,7 +628,7 @@ bool pfe_one_chain(int nx, int ny) { return nx * ny <= 8192; }
 
 template <typename R>
 void launch_pfe(const FFTPlan& fp, const Layout& L, R* f, const StepState* ss, cudaStream_t st,
-                const PlaneStreams* ps, bool chained) {
+                const PlaneStreams* ps, bool chained, const GhostRules<R>* rules) {
   set_smem_once();
   const int npairs = fp.nx / 2 + 1;
   const FFTLaunch l = fft_launch(fp, 3);
@@ -600,8 +644,14 @@ void launch_pfe(const FFTPlan& fp, const Layout& L, R* f, const StepState* ss, c
     // (at 128 x 128 and above the waiting blocks of the successors cost more
     // than the launches they hide: 17 -> 23 us a kernel)
     const bool small = pfe_one_chain(fp.nx, fp.ny);
-    launch_chained(small, cols_kernel, dim3((npairs + l.ppb - 1) / l.ppb, 3), l.threads3, l.smem_cols3, st, fp, 0, ss,
-                   l.ppb, l.lg);
+    const int ncol = (npairs + l.ppb - 1) / l.ppb;
+    if (rules) {
+      const int n2 = 2 * (L.nx + 2 * NG) * (L.ny + 2 * NG), per = 3 * l.layers * l.threadsz;
+      launch_chained(small, cols_rules_kernel<R>, dim3(ncol + (n2 + per - 1) / per, 3, l.layers), l.threadsz, l.smemz, st,
+                     fp, ss, l.ppb, l.lgz, ncol, L, rules->ph, rules->bg, f);
+    } else {
+      launch_chained(small, cols_kernel, dim3(ncol, 3, l.layers), l.threadsz, l.smemz, st, fp, 0, ss, l.ppb, l.lgz);
+    }
     launch_chained(small, rows_inv_kernel<R>, dim3(fp.ny / ri.nb, 3, 3), ri.threads, ri.smem, st, fp, L, f, nout, nout,
                    0, ss, ri.nb, RowsAdd{});
     return;
@@ -701,9 +751,9 @@ template void launch_pfe_adjoint<double>(const FFTPlan&, const Layout&, double*,
 template void launch_atarget_adjoint<float>(const FFTPlan&, const double*, const double*, float*, cudaStream_t);
 template void launch_atarget_adjoint<double>(const FFTPlan&, const double*, const double*, double*, cudaStream_t);
 template void launch_pfe<float>(const FFTPlan&, const Layout&, float*, const StepState*, cudaStream_t,
-                                const PlaneStreams*, bool);
+                                const PlaneStreams*, bool, const GhostRules<float>*);
 template void launch_pfe<double>(const FFTPlan&, const Layout&, double*, const StepState*, cudaStream_t,
-                                 const PlaneStreams*, bool);
+                                 const PlaneStreams*, bool, const GhostRules<double>*);
 template void launch_atarget<float>(const FFTPlan&, const float*, float*, float*, cudaStream_t);
 template void launch_atarget<double>(const FFTPlan&, const double*, double*, double*, cudaStream_t);
 

@@ -1,32 +1,19 @@
 // mhd_ghost.cu -- ghost-zone kernels: the pointwise bottom/top atmospheric
 // rules and periodic-z copies; and the copies between interior and padded
 // arrays (which fill the periodic x,y rims).
+#include "mhd_bc.cuh"
 #include "mhd_internal.h"
 
 namespace mhd {
 
-// Pointwise ghost rules over whole padded planes (rims included, so no rim
-// pass is needed afterwards).  In full variables:
-//  bottom: ln rho fixed to the initial profile ('fg', Sect. 2.5);
-//          ln T from hydrostatic equilibrium downward (Eq. 8 with p = rho T):
-//          lnT_j = lnT_{j+1} + lnrho_{j+1} - lnrho_j - dz g_z / T_{j+1};
-//          u_z antisymmetric (closed, u_z = 0 at z = 0).
-//  top:    ln T symmetric (Eq. 11); ln rho hydrostatic with the boundary
-//          temperature (Eq. 13, signed g_z): lnrho_{nz-1+m} = lnrho_{nz-1-m}
-//          + 2 m dz g_z / T_{nz-1}; u_z antisymmetric, u_x, u_y symmetric.
-//  bc_z = 1: periodic copies in z of all fields (test geometry; the
-//          background is zero there).
-// ln rho and ln T are stored as perturbations about the background; the
-// background differences enter through the constants cb, ctT, ctL (FP64 on
-// the host), and the background ghost values of ln rho equal the fixed
-// profile, so their perturbation is zero.
+// The ghost rules (mhd_bc.cuh) of both ends; bc_z = 1: periodic copies in z of
+// all fields (test geometry; the background is zero there).
 //
 // Bound by latency: each column is a chain of exponentials and divisions (in
 // FP64 some hundred dependent operations), and there are few columns.  The
 // two ends are separate threads and blocks hold 64 of them, so that the
 // chains run side by side over all SMs (32^2 columns in FP64: blocks of 256
 // threads with both ends in a thread took 19 us on 6 SMs).
-constexpr int BC_TH = 64;
 template <typename R>
 __global__ void __launch_bounds__(BC_TH) bc_kernel(Layout L, Phys<R> ph, Background<R> bg, R* f, const StepState* ss) {
   chain_enter();
@@ -45,41 +32,7 @@ __global__ void __launch_bounds__(BC_TH) bc_kernel(Layout L, Phys<R> ph, Backgro
       }
     return;
   }
-  // (layer distances from the vertical grid: bg.dzb[m] = z_{1-m} - z_{-m},
-  // bg.dzt[m] = z_{nz-1+m} - z_{nz-1-m}; dz and 2 m dz on the uniform grid)
-  if (!top) {
-    R th1 = f[L.at(LT, 0, j, i)];
-    R l1 = f[L.at(LR, 0, j, i)];
-    R uz[NG];
-#pragma unroll
-    for (int m = 1; m <= NG; ++m) uz[m - 1] = f[L.at(UZ, m, j, i)];
-#pragma unroll
-    for (int m = 1; m <= NG; ++m) {
-      const R T1 = rexp<R>(bg.tbar[NG - m + 1] + th1);
-      const R l0 = R(0);
-      const R th0 = th1 + l1 - l0 + bg.cb[m] - bg.dzb[m] * ph.gz / T1;
-      f[L.at(LR, -m, j, i)] = l0;
-      f[L.at(LT, -m, j, i)] = th0;
-      f[L.at(UZ, -m, j, i)] = -uz[m - 1];
-      th1 = th0;
-      l1 = l0;
-    }
-    return;
-  }
-  R v[NG][5];
-#pragma unroll
-  for (int m = 1; m <= NG; ++m)
-#pragma unroll
-    for (int c = 0; c < 5; ++c) v[m - 1][c] = f[L.at(UX + c, kt - m, j, i)];
-  const R Ttop = rexp<R>(bg.tbar[NG + kt] + f[L.at(LT, kt, j, i)]);
-#pragma unroll
-  for (int m = 1; m <= NG; ++m) {
-    f[L.at(LT, kt + m, j, i)] = v[m - 1][LT - UX] + bg.ctT[m];
-    f[L.at(LR, kt + m, j, i)] = v[m - 1][LR - UX] + bg.ctL[m] + bg.dzt[m] * ph.gz / Ttop;
-    f[L.at(UZ, kt + m, j, i)] = -v[m - 1][UZ - UX];
-    f[L.at(UX, kt + m, j, i)] = v[m - 1][0];
-    f[L.at(UY, kt + m, j, i)] = v[m - 1][1];
-  }
+  ghost_rules<R>(L, ph, bg, f, i, j, top);
 }
 
 template <typename R>

@@ -140,9 +140,15 @@ template <typename R> void launch_bc(const Layout& L, const Phys<R>& ph, const B
                                      const StepState* ss, cudaStream_t st, bool chained = false);
 // potential-field ghosts of A (three FFT kernels); ps: planes above the size of
 // pfe_one_chain run on three streams, joined back by pfe_join; nullptr: one
-// stream
+// stream; rules: the pointwise ghost rules ride with the column transforms
+// (one stream only)
+template <typename R> struct GhostRules {
+  Phys<R> ph;
+  Background<R> bg;
+};
 template <typename R> void launch_pfe(const FFTPlan& fp, const Layout& L, R* f, const StepState* ss,
-                                      cudaStream_t st, const PlaneStreams* ps = nullptr, bool chained = false);
+                                      cudaStream_t st, const PlaneStreams* ps = nullptr, bool chained = false,
+                                      const GhostRules<R>* rules = nullptr);
 // planes small enough to go as one chain of kernels whatever ps says
 bool pfe_one_chain(int nx, int ny);
 void pfe_join(const PlaneStreams& ps, cudaStream_t st);
