@@ -16,10 +16,11 @@
 //     (D1_a D1_b)^T = D1_a D1_b, periodic in x and y) applied to the
 //     coefficient fields, at interior points and z ghost layers, plus the
 //     nudging value adjoints of A and of the u ghost rows;
-//  3. adj_bc_kernel: the transpose of the pointwise ghost rules (Eqs. 8, 11,
+//  3. adj_ghost_rules (mhd_bc.cuh): the transpose of the pointwise ghost rules (Eqs. 8, 11,
 //     13, closed u_z, symmetric u_hor), routing ghost adjoints into the
-//     interior; the potential-field ghosts are transposed by the FFT kernels
-//     (the Eq. 17 multiplier is real and even, so it is its own transpose).
+//     interior, in the launch of the potential-field transposes' columns; the
+//     potential-field ghosts are transposed by the FFT kernels (the Eq. 17
+//     multiplier is real and even, so it is its own transpose).
 #include "mhd_adjoint_point.cuh"
 #include "mhd_internal.h"
 
@@ -224,72 +225,6 @@ __global__ void __launch_bounds__(128) adj_gather_kernel(AdjGatherArgs<R> a) {
   }
 }
 
-// ---------------------------------------------------------------------------
-// Transpose of the pointwise ghost rules (per column, interior x,y): ghost
-// adjoints are routed into the layers they were computed from.  Bound by
-// latency, as the rules themselves: the two ends of a column are separate
-// threads in blocks of 64, and each loads all it needs before it computes (at
-// 64^2 columns 14.6 us with both ends in a thread of 32 blocks).  nz >= 7, so
-// the layers the two ends write (k <= 3 and k >= nz - 4) are disjoint but for
-// the middle one of seven, whose u_z both touch: that box takes one thread for
-// both ends.
-constexpr int ABC_TH = 64;
-template <typename R>
-__global__ void __launch_bounds__(ABC_TH) adj_bc_kernel(Layout L, Phys<R> ph, Background<R> bg, const R* g, R* gbar,
-                                                        R dz, const StepState* ss) {
-  chain_enter();
-  const int q = blockIdx.x * ABC_TH + threadIdx.x;
-  if (q >= L.nx * L.ny) return;
-  if (halted(ss)) return;
-  const int i = q % L.nx, j = q / L.nx;
-  const int kt = L.nz - 1;
-  const R dzg = dz * ph.gz;
-  // bottom: ln T recursion (ln rho ghosts are constants)
-  if (blockIdx.y == 0) {
-    R th[NG], at[NG + 1], uz[NG], gz[NG];
-#pragma unroll
-    for (int m = 0; m < NG; ++m) {
-      th[m] = bg.tbar[NG - m] + g[L.at(LT, -m, j, i)];
-      uz[m] = gbar[L.at(UZ, m + 1, j, i)];
-      gz[m] = gbar[L.at(UZ, -m - 1, j, i)];
-    }
-#pragma unroll
-    for (int m = 0; m <= NG; ++m) at[m] = gbar[L.at(LT, -m, j, i)];
-    const R al = gbar[L.at(LR, 0, j, i)];
-    const R a2 = at[2] + at[3] * (R(1) + dzg * rexp<R>(-th[2]));
-    const R a1 = at[1] + a2 * (R(1) + dzg * rexp<R>(-th[1]));
-    gbar[L.at(LT, 0, j, i)] = at[0] + a1 * (R(1) + dzg * rexp<R>(-th[0]));
-    gbar[L.at(LR, 0, j, i)] = al + a1;
-#pragma unroll
-    for (int m = 0; m < NG; ++m) gbar[L.at(UZ, m + 1, j, i)] = uz[m] - gz[m];
-  }
-  // top
-  if (blockIdx.y == gridDim.y - 1) {
-    R in[NG][5], gh[NG][5];
-#pragma unroll
-    for (int m = 1; m <= NG; ++m)
-#pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        in[m - 1][c] = gbar[L.at(UX + c, kt - m, j, i)];
-        gh[m - 1][c] = gbar[L.at(UX + c, kt + m, j, i)];
-      }
-    const R at = gbar[L.at(LT, kt, j, i)];
-    const R Ttop = rexp<R>(bg.tbar[NG + kt] + g[L.at(LT, kt, j, i)]);
-    R bth = R(0);
-#pragma unroll
-    for (int m = 1; m <= NG; ++m) {
-      const R bl = gh[m - 1][LR - UX];
-      gbar[L.at(LT, kt - m, j, i)] = in[m - 1][LT - UX] + gh[m - 1][LT - UX];
-      gbar[L.at(LR, kt - m, j, i)] = in[m - 1][LR - UX] + bl;
-      bth -= bl * (R(2 * m) * dz) * ph.gz / Ttop;
-      gbar[L.at(UZ, kt - m, j, i)] = in[m - 1][UZ - UX] - gh[m - 1][UZ - UX];
-      gbar[L.at(UX, kt - m, j, i)] = in[m - 1][0] + gh[m - 1][0];
-      gbar[L.at(UY, kt - m, j, i)] = in[m - 1][1] + gh[m - 1][1];
-    }
-    gbar[L.at(LT, kt, j, i)] = at + bth;
-  }
-}
-
 // Elementwise adjoint updates over the cells that carry state (interior, and
 // the u_x, u_y ghost layers below the photosphere), 16 bytes per thread and
 // row-contiguous (nx is a multiple of 4):
@@ -423,14 +358,6 @@ void launch_adj_gather(const Layout& L, const Phys<R>& ph, const R* coef, const 
 }
 
 template <typename R>
-void launch_adj_bc(const Layout& L, const Phys<R>& ph, const Background<R>& bg, const R* g, R* gbar, R dz,
-                   const StepState* ss, cudaStream_t st, bool chained) {
-  const int n = L.nx * L.ny;
-  launch_chained(chained, adj_bc_kernel<R>, dim3((n + ABC_TH - 1) / ABC_TH, L.nz > 2 * NG + 1 ? 2 : 1), ABC_TH, 0, st, L,
-                 ph, bg, g, gbar, dz, ss);
-}
-
-template <typename R>
 void launch_adj_update(const Layout& L, R* fbar, R* dbar, const R* gbar, double alpha, double beta,
                        int klo, int khi, const StepState* ss, cudaStream_t st, bool chained) {
   launch_chained(chained, adj_update_kernel<R>, 152 * 8, 256, 0, st, L, fbar, dbar, gbar, (R)alpha, (R)beta, klo, khi, ss);
@@ -449,8 +376,6 @@ void launch_bz_plane(int nx, int ny, int nz, int k, double dx, double dy, const 
                                     double*, const R*, const R*, const StepState*, int, bool, cudaStream_t);       \
   template void launch_adj_gather<R>(const Layout&, const Phys<R>&, const R*, const R*, R*, const StepState*,       \
                                      cudaStream_t);                                                               \
-  template void launch_adj_bc<R>(const Layout&, const Phys<R>&, const Background<R>&, const R*, R*, R,             \
-                                 const StepState*, cudaStream_t, bool);                                                \
   template void launch_adj_update<R>(const Layout&, R*, R*, const R*, double, double, int, int,              \
                                      const StepState*, cudaStream_t, bool);                                             \
   template void launch_bz_plane<R>(int, int, int, int, double, double, const R*, R*, int, const R*, R*,             \

@@ -680,7 +680,7 @@ static void run_step(mhd_ctx* h, bool stats) {
       int nb = launch_cfl_partial<R>(h->L, ph, bgr<R>(h), fin, (const R*)h->wtab, h->cfl, h->ss, CflPlanes::ends,
                                      false, h->st);
       launch_cfl_finalize(h->cfl, nb, h->ss, h->p.c_adv, h->p.c_diff, h->p.dt_fixed, inv2sum(&h->p), h->t0,
-                          h->t1, h->p.t_ramp, 0, h->st);
+                          h->t1, h->p.t_ramp, 0, h->st, one_chain(h));
     } else {
       ghost_fill<R>(h, fin, sub > 0);
       if (sub == 0) {
@@ -697,7 +697,7 @@ static void run_step(mhd_ctx* h, bool stats) {
                                      true, h->st);
         }
         launch_cfl_finalize(h->cfl, nb, h->ss, h->p.c_adv, h->p.c_diff, h->p.dt_fixed, inv2sum(&h->p), h->t0,
-                            h->t1, h->p.t_ramp, 0, h->st);
+                            h->t1, h->p.t_ramp, 0, h->st, one_chain(h) && !stats);
       }
     }
     {
@@ -1477,13 +1477,14 @@ template <typename R>
 static void adjoint_step_impl(mhd_ctx* h) {
   R* S[3] = {(R*)h->f[h->cur], (R*)h->f[1 - h->cur], (R*)h->s2};
   // forward recompute of the substep states (ghost-filled)
+  const bool one = one_chain(h);
   ghost_fill<R>(h, S[0]);
   launch_cfl_finalize(h->cfl, 0, h->ss, h->p.c_adv, h->p.c_diff, h->p.dt_fixed, inv2sum(&h->p), h->t0, h->t1,
-                      h->p.t_ramp, 0, h->st);
-  launch_rk_any<R>(h, S[0], S[1], 0);
-  ghost_fill<R>(h, S[1]);
-  launch_rk_any<R>(h, S[1], S[2], 1);
-  ghost_fill<R>(h, S[2]);
+                      h->p.t_ramp, 0, h->st, one);
+  launch_rk_any<R>(h, S[0], S[1], 0, nullptr, one);
+  ghost_fill<R>(h, S[1], one);
+  launch_rk_any<R>(h, S[1], S[2], 1, nullptr, one);
+  ghost_fill<R>(h, S[2], one);
   h->nlaunch += 3;  // cfl finalize and the two RK substeps (ghost_fill counts its own)
   const CUtensorMap* tms[3] = {&h->tm[h->cur], &h->tm[1 - h->cur], &h->tm[2]};
   adjoint_reverse<R>(h, S, tms);
@@ -1542,10 +1543,9 @@ static void adjoint_reverse(mhd_ctx* h, R* const (&S)[3], const CUtensorMap* con
                                  h->ss, h->st);
     else
       launch_adj_gather<R>(h->L, ph, (const R*)h->coef, (const R*)h->dbar, (R*)h->gbar, h->ss, h->st);
-    launch_adj_bc<R>(h->L, ph, bg, S[s], (R*)h->gbar, (R)h->p.dz, h->ss, h->st, one);
-    launch_pfe_adjoint<R>(fpa, h->L, (R*)h->gbar, h->ss, h->st, one);
+    launch_pfe_adjoint<R>(fpa, h->L, GhostRules<R>{ph, bg}, S[s], (R*)h->gbar, (R)h->p.dz, h->ss, h->st, one);
     launch_adj_update<R>(h->L, (R*)h->fbar, (R*)h->dbar, (const R*)h->gbar, alpha, beta, klo, khi, h->ss, h->st, one);
-    h->nlaunch += (tg && !h->adj_zm) ? 8 : 7;  // point, [fold], gather, bc, 3 FFT, update
+    h->nlaunch += (tg && !h->adj_zm) ? 7 : 6;  // point, [fold], gather, 3 FFT, update
   }
 }
 
@@ -1586,7 +1586,7 @@ static void run_step_taped(mhd_ctx* h, char* tape, const CUtensorMap* maps, bool
   Phys<R> ph = make_phys<R>(&h->p);
   R* S0 = (R*)h->f[h->cur];
   R* T[3] = {(R*)tape, (R*)(tape + set), (R*)(tape + 2 * set)};
-  const bool adaptive = !(h->p.dt_fixed > 0.0);
+  const bool adaptive = !(h->p.dt_fixed > 0.0), one = one_chain(h);
   ghost_fill<R>(h, S0);
   if (stats) run_stats<R>(h, S0);
   {
@@ -1596,7 +1596,7 @@ static void run_step_taped(mhd_ctx* h, char* tape, const CUtensorMap* maps, bool
       nb = launch_cfl_partial<R>(h->L, ph, bgr<R>(h), S0, (const R*)h->wtab, h->cfl, h->ss, CflPlanes::all, true,
                                  h->st);
     launch_cfl_finalize(h->cfl, nb, h->ss, h->p.c_adv, h->p.c_diff, h->p.dt_fixed, inv2sum(&h->p), h->t0, h->t1,
-                        h->p.t_ramp, 0, h->st);
+                        h->p.t_ramp, 0, h->st, one && !stats);
   }
   // the ghost-filled substep inputs go to the tape: S0 by a copy, S1 and S2
   // as the RK kernel's outputs (filled in place there)
@@ -1605,15 +1605,15 @@ static void run_step_taped(mhd_ctx* h, char* tape, const CUtensorMap* maps, bool
     ClassTimer ct(h, MHD_KC_RK, 1);
     launch_rk_any<R>(h, S0, T[1], 0);
   }
-  ghost_fill<R>(h, T[1]);
+  ghost_fill<R>(h, T[1], one);
   {
     ClassTimer ct(h, MHD_KC_RK, 1);
-    launch_rk_any<R>(h, T[1], T[2], 1, maps ? &maps[1] : nullptr);
+    launch_rk_any<R>(h, T[1], T[2], 1, maps ? &maps[1] : nullptr, one);
   }
-  ghost_fill<R>(h, T[2]);
+  ghost_fill<R>(h, T[2], one);
   {
     ClassTimer ct(h, MHD_KC_RK, 1);
-    launch_rk_any<R>(h, T[2], (R*)h->f[1 - h->cur], 2, maps ? &maps[2] : nullptr);
+    launch_rk_any<R>(h, T[2], (R*)h->f[1 - h->cur], 2, maps ? &maps[2] : nullptr, one);
   }
   h->cur = 1 - h->cur;
 }

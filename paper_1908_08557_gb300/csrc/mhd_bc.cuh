@@ -63,4 +63,61 @@ __device__ __forceinline__ void ghost_rules(const Layout& L, const Phys<R>& ph, 
   }
 }
 
+// Transpose of the rules (one column, interior x, y): ghost adjoints are routed
+// into the layers they were computed from.  Bound by latency, as the rules
+// themselves: the two ends of a column are separate threads, and each loads all
+// it needs before it computes.  nz >= 7, so the layers the two ends write
+// (k <= 3 and k >= nz - 4) are disjoint but for the middle one of seven, whose
+// u_z both touch: that box takes one thread for both ends.
+template <typename R>
+__device__ __forceinline__ void adj_ghost_rules(const Layout& L, const Phys<R>& ph, const Background<R>& bg, const R* g,
+                                                R* gbar, R dz, int i, int j, bool bottom, bool top) {
+  const int kt = L.nz - 1;
+  const R dzg = dz * ph.gz;
+  // bottom: ln T recursion (ln rho ghosts are constants)
+  if (bottom) {
+    R th[NG], at[NG + 1], uz[NG], gz[NG];
+#pragma unroll
+    for (int m = 0; m < NG; ++m) {
+      th[m] = bg.tbar[NG - m] + g[L.at(LT, -m, j, i)];
+      uz[m] = gbar[L.at(UZ, m + 1, j, i)];
+      gz[m] = gbar[L.at(UZ, -m - 1, j, i)];
+    }
+#pragma unroll
+    for (int m = 0; m <= NG; ++m) at[m] = gbar[L.at(LT, -m, j, i)];
+    const R al = gbar[L.at(LR, 0, j, i)];
+    const R a2 = at[2] + at[3] * (R(1) + dzg * rexp<R>(-th[2]));
+    const R a1 = at[1] + a2 * (R(1) + dzg * rexp<R>(-th[1]));
+    gbar[L.at(LT, 0, j, i)] = at[0] + a1 * (R(1) + dzg * rexp<R>(-th[0]));
+    gbar[L.at(LR, 0, j, i)] = al + a1;
+#pragma unroll
+    for (int m = 0; m < NG; ++m) gbar[L.at(UZ, m + 1, j, i)] = uz[m] - gz[m];
+  }
+  // top
+  if (top) {
+    R in[NG][5], gh[NG][5];
+#pragma unroll
+    for (int m = 1; m <= NG; ++m)
+#pragma unroll
+      for (int c = 0; c < 5; ++c) {
+        in[m - 1][c] = gbar[L.at(UX + c, kt - m, j, i)];
+        gh[m - 1][c] = gbar[L.at(UX + c, kt + m, j, i)];
+      }
+    const R at = gbar[L.at(LT, kt, j, i)];
+    const R Ttop = rexp<R>(bg.tbar[NG + kt] + g[L.at(LT, kt, j, i)]);
+    R bth = R(0);
+#pragma unroll
+    for (int m = 1; m <= NG; ++m) {
+      const R bl = gh[m - 1][LR - UX];
+      gbar[L.at(LT, kt - m, j, i)] = in[m - 1][LT - UX] + gh[m - 1][LT - UX];
+      gbar[L.at(LR, kt - m, j, i)] = in[m - 1][LR - UX] + bl;
+      bth -= bl * (R(2 * m) * dz) * ph.gz / Ttop;
+      gbar[L.at(UZ, kt - m, j, i)] = in[m - 1][UZ - UX] - gh[m - 1][UZ - UX];
+      gbar[L.at(UX, kt - m, j, i)] = in[m - 1][0] + gh[m - 1][0];
+      gbar[L.at(UY, kt - m, j, i)] = in[m - 1][1] + gh[m - 1][1];
+    }
+    gbar[L.at(LT, kt, j, i)] = at + bth;
+  }
+}
+
 }  // namespace mhd

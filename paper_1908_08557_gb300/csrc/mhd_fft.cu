@@ -468,10 +468,24 @@ __global__ void __launch_bounds__(256) rows_inv_kernel(FFTPlan fp, Layout L, R* 
 // fp.P, output plane c in fp.Q.  lg = 3: the layers' forward transforms as one
 // batch of lines (two buffers of three layers); lg = 1: one after the other
 // (two buffers of a layer and the sum).
-__global__ void __launch_bounds__(256) cols_adj_kernel(FFTPlan fp, const StepState* ss, int ppb, int lg) {
+// Blocks ncol .. of x take the transpose of the pointwise ghost rules, which
+// touches no plane of the transforms (as in cols_rules_kernel; a taped adjoint
+// step at 64 x 32 x 45 in FP64 767 -> 754 us against a launch of its own).
+template <typename R>
+__global__ void __launch_bounds__(256) cols_adj_kernel(FFTPlan fp, const StepState* ss, int ppb, int lg, int ncol,
+                                                       Layout L, Phys<R> ph, Background<R> bg, const R* g, R* gbar,
+                                                       R dz) {
   extern __shared__ double2 sm[];
   chain_enter();
   if (ss && halted(ss)) return;
+  if ((int)blockIdx.x >= ncol) {
+    const int n = fp.nx * fp.ny, q = (((int)blockIdx.x - ncol) * 3 + (int)blockIdx.y) * (int)blockDim.x + (int)threadIdx.x;
+    const bool both = L.nz == 2 * NG + 1;
+    if (q >= (both ? n : 2 * n)) return;
+    const int c = q < n ? q : q - n;
+    adj_ghost_rules<R>(L, ph, bg, g, gbar, dz, c % fp.nx, c / fp.nx, q < n, both || q >= n);
+    return;
+  }
   const int nx = fp.nx, ny = fp.ny;
   const int npairs = nx / 2 + 1;
   const int pair0 = blockIdx.x * ppb;
@@ -539,7 +553,8 @@ static void set_smem_once() {
     cudaFuncSetAttribute(cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 6 * FFT_PTS * 16);
     cudaFuncSetAttribute(cols_rules_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 6 * FFT_PTS * 16);
     cudaFuncSetAttribute(cols_rules_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 6 * FFT_PTS * 16);
-    cudaFuncSetAttribute(cols_adj_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 6 * FFT_PTS * 16);
+    cudaFuncSetAttribute(cols_adj_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 6 * FFT_PTS * 16);
+    cudaFuncSetAttribute(cols_adj_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 6 * FFT_PTS * 16);
     return true;
   });
 }
@@ -710,11 +725,12 @@ int launch_rotational(const FFTPlan& fp, const double* vx, const double* vy, dou
 
 // Adjoint of the potential-field ghosts: gbar (adjoint of the ghost-filled
 // state) has its A ghost-layer entries mapped back onto the top layer and
-// the photosphere.  `fp_adj` is the plan with the 9-plane buffer as P and the
+// the photosphere; with them the transpose of the pointwise rules (g: the
+// ghost-filled forward state).  `fp_adj` is the plan with the 9-plane buffer as P and the
 // 3-plane buffer as Q.
 template <typename R>
-void launch_pfe_adjoint(const FFTPlan& fp_adj, const Layout& L, R* gbar, const StepState* ss, cudaStream_t st,
-                        bool chained) {
+void launch_pfe_adjoint(const FFTPlan& fp_adj, const Layout& L, const GhostRules<R>& rules, const R* g, R* gbar, R dz,
+                        const StepState* ss, cudaStream_t st, bool chained) {
   set_smem_once();
   const FFTLaunch l = fft_launch(fp_adj, 3);
   const int npairs = fp_adj.nx / 2 + 1;
@@ -723,8 +739,11 @@ void launch_pfe_adjoint(const FFTPlan& fp_adj, const Layout& L, R* gbar, const S
   R* nout = nullptr;
   launch_chained(chained, rows_fwd_kernel<R>, dim3(fp_adj.ny / r9.nb, 9), r9.threads, r9.smem, st, fp_adj, L, gbar, nout,
                  2, ss, r9.nb, none, none);
-  launch_chained(chained, cols_adj_kernel, dim3((npairs + l.ppb - 1) / l.ppb, 3), l.threads3, l.smem_cols3, st, fp_adj,
-                 ss, l.ppb, l.lg);
+  // both ends of a column, or one thread for both (nz = 7)
+  const int ncol = (npairs + l.ppb - 1) / l.ppb, per = 3 * l.threads3;
+  const int ends = (L.nz == 2 * NG + 1 ? 1 : 2) * fp_adj.nx * fp_adj.ny;
+  launch_chained(chained, cols_adj_kernel<R>, dim3(ncol + (ends + per - 1) / per, 3), l.threads3, l.smem_cols3, st,
+                 fp_adj, ss, l.ppb, l.lg, ncol, L, rules.ph, rules.bg, g, gbar, dz);
   launch_chained(chained, rows_inv_kernel<R>, dim3(fp_adj.ny / r3.nb, 3, 1), r3.threads, r3.smem, st, fp_adj, L, gbar,
                  nout, nout, 2, ss, r3.nb, RowsAdd{});
 }
@@ -745,9 +764,10 @@ void launch_atarget_adjoint(const FFTPlan& fp, const double* abx, const double* 
                                                                              r1.nb, RowsAdd{});
 }
 
-template void launch_pfe_adjoint<float>(const FFTPlan&, const Layout&, float*, const StepState*, cudaStream_t, bool);
-template void launch_pfe_adjoint<double>(const FFTPlan&, const Layout&, double*, const StepState*, cudaStream_t,
-                                         bool);
+template void launch_pfe_adjoint<float>(const FFTPlan&, const Layout&, const GhostRules<float>&, const float*, float*,
+                                        float, const StepState*, cudaStream_t, bool);
+template void launch_pfe_adjoint<double>(const FFTPlan&, const Layout&, const GhostRules<double>&, const double*,
+                                         double*, double, const StepState*, cudaStream_t, bool);
 template void launch_atarget_adjoint<float>(const FFTPlan&, const double*, const double*, float*, cudaStream_t);
 template void launch_atarget_adjoint<double>(const FFTPlan&, const double*, const double*, double*, cudaStream_t);
 template void launch_pfe<float>(const FFTPlan&, const Layout&, float*, const StepState*, cudaStream_t,

@@ -236,8 +236,6 @@ void launch_adj_gather_zm(const Layout& L, const Phys<float>& ph, const float* c
 void launch_adj_gather64(const Layout& L, const Phys<double>& ph, const double* coef, double* dbar, double* gbar,
                          double* fbar, double alpha, double beta, int klo, int khi, int ksw, const StepState* ss,
                          cudaStream_t st, bool chained = false);
-template <typename R> void launch_adj_bc(const Layout& L, const Phys<R>& ph, const Background<R>& bg, const R* g,
-                                         R* gbar, R dz, const StepState* ss, cudaStream_t st, bool chained = false);
 // adjoint elementwise update F += G, D = alpha D + beta F,
 // skipping interior layers klo <= k < khi; nx must be a multiple of 4 and
 // NF * (nz + 6) * ny * nx / 4 < 2^31
@@ -254,8 +252,9 @@ template <typename R> void launch_adj_pack(const Layout& L, int bcz, const R* fb
 template <typename R> void launch_adj_unpack(const Layout& L, const R* in, R* fbar, R* dbar, double beta,
                                              cudaStream_t st);
 template <typename R> void launch_d2r(const double* in, R* out, long long n, cudaStream_t st);
-template <typename R> void launch_pfe_adjoint(const FFTPlan& fp_adj, const Layout& L, R* gbar, const StepState* ss,
-                                              cudaStream_t st, bool chained = false);
+template <typename R> void launch_pfe_adjoint(const FFTPlan& fp_adj, const Layout& L, const GhostRules<R>& rules,
+                                              const R* g, R* gbar, R dz, const StepState* ss, cudaStream_t st,
+                                              bool chained = false);
 template <typename R> void launch_atarget_adjoint(const FFTPlan& fp, const double* abx, const double* aby, R* out,
                                                   cudaStream_t st);
 // A stored about a fixed background (params a_background): FP64 packed
@@ -304,7 +303,7 @@ int launch_cfl_inner_zm(const CUtensorMap* tma, const Layout& L, const Phys<floa
                         cudaStream_t st);
 void launch_cfl_finalize(const double* partial, int nblk, StepState* ss, double c_adv, double c_diff,
                          double dt_fixed, double inv2sum, double t0, double t1, double t_ramp, int probe,
-                         cudaStream_t st);
+                         cudaStream_t st, bool chained = false);
 // diagnostics partials; bsc = three scratch fields in the state layout
 // (overwritten), e.g. the RK accumulator between steps
 template <typename R> int launch_stats_partial(const Layout& L, const Phys<R>& ph, const Background<R>& bg,
