@@ -481,7 +481,7 @@ int mhd_gran_create(int nx, int ny, double dx, double dy,
  * closer than r_inner (nearest periodic image).  The result equals that
  * sequential visit exactly; the GPU reaches it in parallel rounds (a pixel
  * joins once no undecided pixel within r_inner precedes it), and the call
- * synchronises the stream once per round.
+ * synchronises the stream once per batch of four rounds.
  *   keys [ny][nx] uint32, c_life, c_amp [ny][nx] double: the random draws
  *   (uniform keys, standard normals); mem: MHD_MEM_DEVICE or MHD_MEM_HOST.
  *   rounds (may be NULL): the parallel rounds taken.

@@ -222,7 +222,9 @@ __global__ void __launch_bounds__(256) rows_fwd_kernel(FFTPlan fp, Layout L, con
 // inverted as one batch of lines, so each stage of the inverse transform has
 // lg times the butterflies between two barriers; with all of the layers o_first
 // .. o_end - 1 in one batch two buffers of lg layers do (the forward spectrum's
-// buffer becomes the scratch), otherwise three (the spectrum is kept).
+// buffer becomes the scratch), otherwise three (the spectrum is kept).  A block
+// reads and writes its own columns only, so with one output plane P and Q may be
+// the same.
 __device__ __forceinline__ void cols_block(const FFTPlan& fp, int mode, int ppb, int lg, int o_first, int o_end) {
   extern __shared__ double2 sm[];
   const int nx = fp.nx, ny = fp.ny;
@@ -591,7 +593,7 @@ static FFTLaunch fft_launch(const FFTPlan& fp, int planes) {
   const int spread = npairs * planes / (2 * sm_count());
   if (l.ppb > spread) l.ppb = spread;
   if (l.ppb < 1) l.ppb = 1;
-  l.smem_cols = (size_t)3 * 2 * l.ppb * fp.ny * sizeof(double2);  // also cols_adj_kernel
+  l.smem_cols = (size_t)2 * 2 * l.ppb * fp.ny * sizeof(double2);
   // the three ghost layers in one batch while that keeps two column blocks
   // per SM (at most 96 KB), one at a time otherwise (at 1024^2 the batched
   // form, 192 KB and one block per SM, measured 8 % slower)

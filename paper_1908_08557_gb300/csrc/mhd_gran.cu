@@ -523,8 +523,11 @@ Layout2 carve(int nx, int ny, double dx, double dy, const mhd_gran_params* gp) {
   o.twy = c.take((size_t)ny * 16);
   o.ktx = c.take((size_t)nx * 8);
   o.kty = c.take((size_t)ny * 8);
-  o.P = c.take(N * 16);
-  o.Q = c.take(N * 16);
+  // one complex plane: the column kernel reads and writes the columns its block
+  // owns, so it works in place; the place of a second plane holds the filter
+  // table, 24 (nx / 2 + 1) (ny / 2 + 1) <= 16 N bytes for nx, ny >= 8
+  o.P = o.Q = c.take(N * 16);
+  o.filt = c.take(N * 16);
   o.off_in = c.take((size_t)(o.n_in > 0 ? o.n_in : 1) * 8);
   o.off_l = c.take((size_t)o.n_l * 8);
   o.w_l = c.take((size_t)o.n_l * 16);
@@ -532,7 +535,6 @@ Layout2 carve(int nx, int ny, double dx, double dy, const mhd_gran_params* gp) {
   o.part = c.take((size_t)(o.nblk + (o.nblk > ny ? o.nblk : ny)) * 8);
   o.tot = c.take(2 * 8);
   o.cnt = c.take(BATCH * 4);
-  o.filt = c.take((size_t)3 * (nx / 2 + 1) * (ny / 2 + 1) * 8);
   o.total = c.off;
   return o;
 }
@@ -774,8 +776,8 @@ extern "C" int mhd_gran_velocity(mhd_gran_handle g, double t, int precision, voi
   const int nvor = launch_rotational(g->fp, d.vg, d.vg + N, d.vr, d.vr + N, true, g->gp.f_rot, d.part + nb, g->st);
   total_kernel<<<1, GT, 0, g->st>>>(d, nb, nvor);
   g->launches += 6;
-  // device output straight into v; host output through the FFT's row
-  // spectra (2N doubles), free once the column pass has read them
+  // device output straight into v; host output through the FFT's plane (2N
+  // doubles), free once the inverse rows have read it
   void* dst = mem == MHD_MEM_DEVICE ? v : (void*)(g->ws + g->o.P);
   if (precision == 64) scale_kernel<double><<<nb, GT, 0, g->st>>>(d, (double*)dst);
   else scale_kernel<float><<<nb, GT, 0, g->st>>>(d, (float*)dst);
@@ -813,15 +815,13 @@ extern "C" int mhd_gran_read_field(mhd_gran_handle g, int which, double* dst, in
   if (mem != MHD_MEM_DEVICE && mem != MHD_MEM_HOST) return gfail(g, MHD_ERR_ARG, "bad mem flag");
   const size_t N = (size_t)g->nx * g->ny;
   if (which == 0) return copy_out(g, dst, g->g.vg, 2 * N * 8, mem);
-  // v_rot' is not kept (the FFT's last kernel adds it to v_gran): recompute
-  // it from v_gran into the FFT's row spectra, free once the column pass has
-  // read them
-  launch_rotational(g->fp, g->g.vg, g->g.vg + N, (double*)(g->ws + g->o.P), (double*)(g->ws + g->o.P) + N, false, 0.0,
-                    nullptr, g->st);
+  // v_rot' is not kept (the FFT's last kernel adds it to v_gran): recompute it
+  // from v_gran in the place of v_vor, which the next velocity forms anew
+  launch_rotational(g->fp, g->g.vg, g->g.vg + N, g->g.vr, g->g.vr + N, false, 0.0, nullptr, g->st);
   g->launches += 3;
   int rc = gcheck(g, cudaGetLastError(), "rotational part");
   if (rc) return rc;
-  return copy_out(g, dst, g->ws + g->o.P, 2 * N * 8, mem);
+  return copy_out(g, dst, g->g.vr, 2 * N * 8, mem);
 }
 
 extern "C" long long mhd_gran_launch_count(mhd_gran_handle g) { return g ? g->launches : 0; }

