@@ -30,18 +30,18 @@ METRIC = "MHD cell-updates/s per RK step"
 UNIT = "cell-updates/s"
 WORDS_PER_CELL_STEP = 80  # algorithmic state words moved per cell per RK3 step
 RUNS = 5                  # timed runs of K steps; the median is reported
-# FP64 operations per cell and substep of rk_simple_kernel<double> (2 flops
+# FP64 operations per cell and substep of rk64_kernel (2 flops
 # per DFMA, 1 per DADD / DMUL; each of the three one FP64-pipe instruction),
 # from the ncu instruction counts summarised in
-# profiles/rk_simple_fp64_flops_bipoles20_128x128x128.md
-FP64_FLOPS_PER_CELL_SUBSTEP = 1459.4
-FP64_PIPE_OPS_PER_CELL_SUBSTEP = 1022.3
+# profiles/rk64_fp64_flops_bipoles20_128x128x128.md
+FP64_FLOPS_PER_CELL_SUBSTEP = 820.7
+FP64_PIPE_OPS_PER_CELL_SUBSTEP = 545.0
 # FP32 operations per cell and substep of rk_pair_kernel (f32x2 instructions
 # one operation per cell, FFMA two flops; FFMA, FADD and FMUL one FMA-pipe
 # lane operation each), from the ncu instruction counts in
 # profiles/rk_pair_fp32_flops_bipoles20_128x128x128.md
-FP32_FLOPS_PER_CELL_SUBSTEP = 1021.3
-FP32_PIPE_OPS_PER_CELL_SUBSTEP = 621.3
+FP32_FLOPS_PER_CELL_SUBSTEP = 874.5
+FP32_PIPE_OPS_PER_CELL_SUBSTEP = 521.8
 RK_KERNEL = ("rk_pair_kernel (fused RHS + RK update, TMA z-march, two cells per thread in f32x2, "
              "z histories in TMEM)")
 
@@ -873,7 +873,7 @@ def run_native(args, ws, rank, local):
             # pipe occupancy: DFMA, DADD and DMUL each take one FP64-pipe slot
             ops64 = FP64_PIPE_OPS_PER_CELL_SUBSTEP * cells / (rk64_ms / rk64_n / 1e3) / 1e12
             fp64["roofline"] = {"bound": "alu", "achieved": ach64, "peak": peak64, "unit": "TFLOP/s",
-                                "frac": ach64 / peak64, "kernel": "rk_simple_kernel<double>",
+                                "frac": ach64 / peak64, "kernel": "rk64_kernel",
                                 "flops_per_cell_substep": FP64_FLOPS_PER_CELL_SUBSTEP,
                                 "pipe_ops_per_cell_substep": FP64_PIPE_OPS_PER_CELL_SUBSTEP,
                                 "pipe_frac": ops64 / (peak64 / 2),
