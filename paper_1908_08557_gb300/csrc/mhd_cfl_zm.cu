@@ -105,7 +105,11 @@ __global__ void __launch_bounds__(NT, 6) cfl_zm_kernel(const __grid_constant__ C
       break;
     }
     phase ^= 1u << s;
-    if (tid == 0) pending &= ~(1u << s);
+    if (tid == 0) {
+      pending &= ~(1u << s);
+      // every thread is past plane k - 1: its slot takes plane k - 1 + NS
+      if (k > k0 && k - 1 + NS < k1) load(k - 1 + NS, s == 0 ? NS - 1 : s - 1);
+    }
     if (live) {
       const float* P = ring + s * SLOT + (ty + 3) * BX + 2 * tx + 4;
       auto sp = [](const float* p) { return *reinterpret_cast<const float2*>(p); };
@@ -154,9 +158,6 @@ __global__ void __launch_bounds__(NT, 6) cfl_zm_kernel(const __grid_constant__ C
         mdr = fmaxf(mdr, dm);
       }
     }
-    // every thread is past plane k: its slot takes plane k + NS
-    __syncthreads();
-    if (tid == 0 && k + NS < k1) load(k + NS, s);
     s = s + 1 == NS ? 0 : s + 1;
 #pragma unroll
     for (int m = 0; m < 6; ++m) {
@@ -212,10 +213,17 @@ int launch_cfl_inner_zm(const CUtensorMap* tma, const Layout& L, const Phys<floa
   });
   const int ntx = (L.nx + cflz::TX - 1) / cflz::TX, nty = (L.ny + cflz::TY - 1) / cflz::TY;
   const long long tiles = (long long)ntx * nty;
-  // chunks of 8 .. 64 layers, about four waves of resident CTAs in all
   const int nk = kend - kbeg;
+  // chunks of up to 64 layers, about four waves of resident CTAs (whole waves of
+  // longer chunks finish sooner alone, but beside the transforms of the first
+  // substep they hold the SMs longer: a step at 256^3 1988 -> 1997 us); where
+  // that is less than 8 layers, 8 or what fills half of one wave: a small box is
+  // bound by the serial layers of a chunk (64^3: 8 -> 3 layers, a step 139 -> 135
+  // us; 128 x 128 x 64 with 5 layers 314 -> 317)
+  const long long one = (2 * tiles * nk + res - 1) / res;
   long long kc = tiles * nk / (4LL * res);
-  kc = kc < 8 ? 8 : (kc > 64 ? 64 : kc);
+  const long long lo = one < 8 ? one : 8;
+  kc = kc < lo ? lo : (kc > 64 ? 64 : kc);
   const int kchunk = (int)kc;
   const int nch = (nk + kchunk - 1) / kchunk;
   const float s2 = (float)sqrt((double)ph.idx2 + (double)ph.idy2 + (double)ph.idz2);
