@@ -38,8 +38,12 @@
  *   available from mhd_last_error().  Argument errors are reported before any
  *   launch.  A non-finite value met by the time-step reduction (or a device
  *   wait that exceeded its bound) sets a device flag: from then on every
- *   kernel of the handle returns without work, and the next synchronising
- *   call returns MHD_ERR_NONFINITE (or MHD_ERR_TIMEOUT).
+ *   kernel of the handle that computes returns without work, and the next
+ *   mhd_get_time, mhd_read_stats, mhd_compute_stats, mhd_compute_dt or
+ *   mhd_write_snapshot returns MHD_ERR_NONFINITE (or MHD_ERR_TIMEOUT).  The
+ *   state can still be read and saved: a step that finds a non-finite value
+ *   leaves the state it began from, and so do all further steps of the halted
+ *   handle (after a wait that gave up within a step: what that step left).
  */
 #ifndef MHD_H
 #define MHD_H

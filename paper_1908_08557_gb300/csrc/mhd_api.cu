@@ -3,6 +3,7 @@
 // step.  All device memory comes from the caller's workspace.
 #include <math.h>
 #include <stdarg.h>
+#include <stddef.h>
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
@@ -644,6 +645,11 @@ static void cfl_inner(mhd_ctx* h, const R* fin, bool zero) {
   launch_cfl_partial<R>(h->L, ph, bgr<R>(h), fin, (const R*)h->wtab, h->cfl, h->ss, CflPlanes::inner, zero, h->st);
 }
 
+// the two state sets of a step about to be taken
+static KeepSets keep_sets(const mhd_ctx* h) {
+  return KeepSets{h->f[h->cur], h->f[1 - h->cur], (size_t)NF * h->L.fs * h->esz};
+}
+
 template <typename R>
 static void run_step(mhd_ctx* h, bool stats) {
   Phys<R> ph = make_phys<R>(&h->p);
@@ -680,7 +686,7 @@ static void run_step(mhd_ctx* h, bool stats) {
       int nb = launch_cfl_partial<R>(h->L, ph, bgr<R>(h), fin, (const R*)h->wtab, h->cfl, h->ss, CflPlanes::ends,
                                      false, h->st);
       launch_cfl_finalize(h->cfl, nb, h->ss, h->p.c_adv, h->p.c_diff, h->p.dt_fixed, inv2sum(&h->p), h->t0,
-                          h->t1, h->p.t_ramp, 0, h->st, one_chain(h));
+                          h->t1, h->p.t_ramp, 0, h->st, one_chain(h), keep_sets(h));
     } else {
       ghost_fill<R>(h, fin, sub > 0);
       if (sub == 0) {
@@ -697,7 +703,7 @@ static void run_step(mhd_ctx* h, bool stats) {
                                      true, h->st);
         }
         launch_cfl_finalize(h->cfl, nb, h->ss, h->p.c_adv, h->p.c_diff, h->p.dt_fixed, inv2sum(&h->p), h->t0,
-                            h->t1, h->p.t_ramp, 0, h->st, one_chain(h) && !stats);
+                            h->t1, h->p.t_ramp, 0, h->st, one_chain(h) && !stats, keep_sets(h));
       }
     }
     {
@@ -1005,11 +1011,13 @@ extern "C" int mhd_write(mhd_handle h, const void* src, int mem) {
     if (rc) return rc;
     src = h->df;
   }
-  // a state written afresh may be stepped again: clear the halt flag
-  rc = cuda_check(h, cudaMemsetAsync(&h->ss->nonfinite, 0, sizeof(int), h->st), "clear status");
+  // a state written afresh may be stepped again: clear the halt flag and its
+  // neighbour StepState::held
+  rc = cuda_check(h, cudaMemsetAsync(&h->ss->nonfinite, 0, 2 * sizeof(int), h->st), "clear status");
   if (rc) return rc;
-  // the other state set needs nothing: a substep writes its interior, images
-  // and u ghost rows, and the ghost rules the rest, before anything reads it
+  // the other state set needs nothing: before anything reads it a substep has
+  // written its interior, images and u ghost rows, and the ghost rules the rest;
+  // or, if the first step halts, cfl_finalize_kernel has copied this one
   const bool ug = h->p.bc_z == 0;
   if (h->esz == 8) launch_unpack<double>(L, h->bgd, (const double*)src, (double*)h->f[0], ug, h->st);
   else launch_unpack<float>(L, h->bgf, (const float*)src, (float*)h->f[0], ug, h->st);
@@ -1074,6 +1082,7 @@ extern "C" int mhd_set_a_background(mhd_handle h, const double* a_bg, const void
   // the state's A is now the perturbation: a_pert, or zero
   const size_t abytes = (size_t)3 * L.fs * h->esz;
   rc = cuda_check(h, cudaMemsetAsync(h->f[h->cur], 0, abytes, h->st), "zero A");
+  if (!rc) rc = cuda_check(h, cudaMemsetAsync(&h->ss->held, 0, sizeof(int), h->st), "clear held");
   if (!rc && a_pert) {
     const void* ps = a_pert;
     if (mem == MHD_MEM_HOST) {
@@ -1433,8 +1442,11 @@ extern "C" int mhd_restore(mhd_handle h, const void* src, double t) {
   if (!h || !src) return fail(h, MHD_ERR_ARG, "NULL argument");
   int rc = cuda_check(h, cudaMemcpyAsync(h->f[h->cur], src, mhd_checkpoint_bytes(h), cudaMemcpyDeviceToDevice, h->st),
                       "restore");
-  double tt = t;
-  if (!rc) rc = cuda_check(h, cudaMemcpyAsync(&h->ss->t, &tt, sizeof(double), cudaMemcpyHostToDevice, h->st),
+  // the time, and before it StepState::held: the sets of a halted handle differ again
+  struct { int held; int t[2]; } in = {0, {0, 0}};
+  static_assert(offsetof(StepState, t) == offsetof(StepState, held) + sizeof(int), "one copy");
+  memcpy(in.t, &t, sizeof t);
+  if (!rc) rc = cuda_check(h, cudaMemcpyAsync(&h->ss->held, &in, sizeof in, cudaMemcpyHostToDevice, h->st),
                            "restore t");
   if (!rc) rc = cuda_check(h, cudaStreamSynchronize(h->st), "restore synchronize");
   return rc;
@@ -1596,7 +1608,7 @@ static void run_step_taped(mhd_ctx* h, char* tape, const CUtensorMap* maps, bool
       nb = launch_cfl_partial<R>(h->L, ph, bgr<R>(h), S0, (const R*)h->wtab, h->cfl, h->ss, CflPlanes::all, true,
                                  h->st);
     launch_cfl_finalize(h->cfl, nb, h->ss, h->p.c_adv, h->p.c_diff, h->p.dt_fixed, inv2sum(&h->p), h->t0, h->t1,
-                        h->p.t_ramp, 0, h->st, one && !stats);
+                        h->p.t_ramp, 0, h->st, one && !stats, keep_sets(h));
   }
   // the ghost-filled substep inputs go to the tape: S0 by a copy, S1 and S2
   // as the RK kernel's outputs (filled in place there)

@@ -104,6 +104,8 @@ struct Background {
 
 // Device-resident bookkeeping of the time integration (FP64).
 struct StepState {
+  int nonfinite;     // set by the reductions and the bounded waits: every kernel then returns without work
+  int held;          // halted, and both state sets hold the state the halted step began from
   double t;          // time of the current state
   double dt;         // time step of the current / last step
   double tsub[3];    // substep times t + c_s dt
@@ -114,7 +116,6 @@ struct StepState {
   double eval_r, eval_s;   // driver weights of a single RHS evaluation
   double probe_dt;         // time step computed without advancing time
   long long step;
-  int nonfinite;
   int items;         // work-item counter of the z-march launches (zeroed before each)
 };
 

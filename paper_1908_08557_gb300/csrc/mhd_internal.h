@@ -301,9 +301,17 @@ template <typename R> int launch_cfl_partial(const Layout& L, const Phys<R>& ph,
 int launch_cfl_inner_zm(const CUtensorMap* tma, const Layout& L, const Phys<float>& ph, const Background<float>& bg,
                         const float* f, const float* wtab, double* partial, StepState* ss, bool zero,
                         cudaStream_t st);
+// state sets of a step that swaps them: in a halted step nothing is written, so
+// the finalize kernel copies the one the step began from into the other, which
+// the step leaves current (once; StepState::held)
+struct KeepSets {
+  const void* from;
+  void* to;
+  size_t bytes;
+};
 void launch_cfl_finalize(const double* partial, int nblk, StepState* ss, double c_adv, double c_diff,
                          double dt_fixed, double inv2sum, double t0, double t1, double t_ramp, int probe,
-                         cudaStream_t st, bool chained = false);
+                         cudaStream_t st, bool chained = false, const KeepSets& keep = KeepSets{});
 // diagnostics partials; bsc = three scratch fields in the state layout
 // (overwritten), e.g. the RK accumulator between steps
 template <typename R> int launch_stats_partial(const Layout& L, const Phys<R>& ph, const Background<R>& bg,

@@ -275,7 +275,7 @@ int launch_cfl_partial(const Layout& L, const Phys<R>& ph, const Background<R>& 
 // substeps of a taped step 144 -> 136 us at 64^3 in FP32).
 __global__ void cfl_finalize_kernel(const double* partial, int nblk, StepState* ss, double c_adv,
                                     double c_diff, double dt_fixed, double inv2sum, double t0, double t1,
-                                    double t_ramp, int probe) {
+                                    double t_ramp, int probe, KeepSets keep) {
   __shared__ long long sa[32], sd[32];
   __shared__ double s_dt;
   __shared__ int s_stop;
@@ -312,7 +312,16 @@ __global__ void cfl_finalize_kernel(const double* partial, int nblk, StepState* 
     s_stop = probe || ss->nonfinite;
   }
   __syncthreads();
-  if (s_stop) return;
+  if (s_stop) {
+    if (!probe && keep.to && !ss->held) {
+      const uint4* from = (const uint4*)keep.from;
+      uint4* to = (uint4*)keep.to;
+      for (size_t q = threadIdx.x; q < keep.bytes / 16; q += blockDim.x) to[q] = from[q];
+      __syncthreads();
+      if (threadIdx.x == 0) ss->held = 1;
+    }
+    return;
+  }
   const double dt = s_dt;
   if (threadIdx.x == 0) {
     ss->dt = dt;
@@ -333,9 +342,9 @@ __global__ void cfl_finalize_kernel(const double* partial, int nblk, StepState* 
 
 void launch_cfl_finalize(const double* partial, int nblk, StepState* ss, double c_adv, double c_diff,
                          double dt_fixed, double inv2sum, double t0, double t1, double t_ramp, int probe,
-                         cudaStream_t st, bool chained) {
+                         cudaStream_t st, bool chained, const KeepSets& keep) {
   launch_chained(chained, cfl_finalize_kernel, 1, 256, 0, st, partial, nblk, ss, c_adv, c_diff, dt_fixed, inv2sum, t0, t1,
-                 t_ramp, probe);
+                 t_ramp, probe, keep);
 }
 
 // Diagnostics, first pass: curl A (Eq. 6, without the uniform B_ext) into the
