@@ -21,7 +21,7 @@
  *   velocities are [2][ny][nx] (vx, vy).  z index 0 is the photosphere.
  * - Element type = the handle's precision (float for 32, double for 64).
  * - `mem` selects where a caller array lives: MHD_MEM_DEVICE (device pointer,
- *   copied device-to-device on the handle's stream) or MHD_MEM_HOST (host
+ *   read or written by work queued on the handle's stream) or MHD_MEM_HOST (host
  *   pointer; the call copies and returns when the host buffer may be reused).
  * - The library never allocates device memory: the caller passes one
  *   workspace of mhd_workspace_bytes() bytes (256-byte aligned) and owns it;

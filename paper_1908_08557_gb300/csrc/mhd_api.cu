@@ -40,6 +40,7 @@ struct mhd_ctx {
   cudaEvent_t evf, evj;
   cudaEvent_t evc;     // end of the host-to-device driver copies (mhd_set_driver)
   PlaneStreams ps;     // two more FFT streams (planes 1, 2 of the potential-field boundary)
+  int dev;             // device of the workspace
   size_t esz;          // bytes per state element
   char* ws;
   size_t ws_bytes;
@@ -369,6 +370,18 @@ static void driver_weights(const mhd_ctx* h, double t, double* r, double* s) {
 
 static cudaMemcpyKind kind_in(int mem) { return mem == MHD_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice; }
 static cudaMemcpyKind kind_out(int mem) { return mem == MHD_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice; }
+
+// whether kernels of this handle may use a caller's MHD_MEM_DEVICE array where
+// it lies: memory of the handle's own device.  Any other array a copy takes
+// (another GPU's without peer access, managed memory) is staged.
+static bool in_place(const void* p, int dev) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
 
 static int sync_status(mhd_ctx* h) {
   int rc = cuda_check(h, cudaStreamSynchronize(h->st), "stream synchronize");
@@ -829,6 +842,11 @@ extern "C" int mhd_create(const mhd_params* p, void* workspace, size_t ws_bytes,
   }
   h->L = make_layout(p->nx, p->ny, p->nz);
   h->st = (cudaStream_t)stream;
+  {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, workspace) == cudaSuccess) h->dev = a.device;
+    else cudaGetLastError();
+  }
   h->esz = p->precision == 64 ? 8 : 4;
   h->ws = (char*)workspace;
   h->ws_bytes = ws_bytes;
@@ -1004,10 +1022,10 @@ extern "C" int mhd_write(mhd_handle h, const void* src, int mem) {
   const Layout& L = h->L;
   size_t bytes = (size_t)NF * L.nx * L.ny * L.nz * h->esz;
   int rc = MHD_OK;
-  if (mem == MHD_MEM_HOST) {
-    // a host array is staged in the accumulator buffer; a device array is
-    // read where it lies
-    rc = cuda_check(h, cudaMemcpyAsync(h->df, src, bytes, cudaMemcpyHostToDevice, h->st), "copy state in");
+  if (mem == MHD_MEM_HOST || !in_place(src, h->dev)) {
+    // staged in the accumulator buffer; an array of this device is read where
+    // it lies
+    rc = cuda_check(h, cudaMemcpyAsync(h->df, src, bytes, kind_in(mem), h->st), "copy state in");
     if (rc) return rc;
     src = h->df;
   }
@@ -1465,9 +1483,9 @@ extern "C" int mhd_adjoint_init(mhd_handle h, const void* lam, int mem) {
   if (rc) return rc;
   const size_t n2 = (size_t)h->p.nx * h->p.ny;
   rc = cuda_check(h, cudaMemsetAsync(h->thbar, 0, 6 * n2 * sizeof(double), h->st), "zero thbar");
-  if (!rc && mem == MHD_MEM_HOST) {
+  if (!rc && (mem == MHD_MEM_HOST || !in_place(lam, h->dev))) {
     rc = cuda_check(h, cudaMemcpyAsync(h->gbar, lam, (size_t)NF * h->p.nx * h->p.ny * h->p.nz * h->esz,
-                                       cudaMemcpyHostToDevice, h->st), "copy lam");
+                                       kind_in(mem), h->st), "copy lam");
     lam = h->gbar;
   }
   if (rc) return rc;
@@ -1686,11 +1704,11 @@ extern "C" int mhd_adjoint_read(mhd_handle h, void* lam, void* grad_bz, void* gr
   // results are staged in the coefficient buffer, then copied out
   char* stage = (char*)h->coef;
   if (lam) {
-    // a device array takes the copy directly, a host array through the stage
-    void* to = mem == MHD_MEM_HOST ? (void*)stage : lam;
+    // an array of this device takes the pack directly, others through the stage
+    void* to = mem == MHD_MEM_HOST || !in_place(lam, h->dev) ? (void*)stage : lam;
     if (h->esz == 8) launch_adj_pack<double>(h->L, h->p.bc_z, (const double*)h->fbar, (double*)to, h->st);
     else launch_adj_pack<float>(h->L, h->p.bc_z, (const float*)h->fbar, (float*)to, h->st);
-    if (mem == MHD_MEM_HOST) rc = cuda_check(h, cudaMemcpyAsync(lam, stage, n3b, cudaMemcpyDeviceToHost, h->st), "copy lam");
+    if (to != lam) rc = cuda_check(h, cudaMemcpyAsync(lam, stage, n3b, kind_out(mem), h->st), "copy lam");
     if (rc) return rc;
   }
   char* stage2 = stage + (n3b + 255) / 256 * 256;
