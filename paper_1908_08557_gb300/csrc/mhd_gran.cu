@@ -577,6 +577,14 @@ static int gcheck(mhd_gran_ctx* g, cudaError_t e, const char* what) {
   return MHD_OK;
 }
 
+// A host table to the device, ordered on the generator's stream: cudaMemcpy may
+// return once the table is staged, with its transfer still under way on the
+// legacy stream, which a non-blocking stream does not wait for.  (Pageable
+// memory is staged before the call returns, so the table may go.)
+static int upload(mhd_gran_ctx* g, const void* dst, const void* src, size_t bytes, const char* what) {
+  return gcheck(g, cudaMemcpyAsync((void*)dst, src, bytes, cudaMemcpyHostToDevice, g->st), what);
+}
+
 extern "C" size_t mhd_gran_workspace_bytes(int nx, int ny, double dx, double dy, const mhd_gran_params* gp) {
   if (check(nx, ny, dx, dy, gp)) return 0;
   return carve(nx, ny, dx, dy, gp).total;
@@ -652,11 +660,8 @@ extern "C" int mhd_gran_create(int nx, int ny, double dx, double dy, const mhd_g
       tw[2 * r + 1] = w.y;
       k[r] = 2.0 * M_PI * (2 * r > n ? r - n : r) / L;
     }
-    rc = gcheck(g, cudaMemcpy((void*)(axis == 0 ? fp.twx : fp.twy), tw.data(), (size_t)n * 16,
-                              cudaMemcpyHostToDevice), "upload twiddles");
-    if (rc == MHD_OK)
-      rc = gcheck(g, cudaMemcpy((void*)(axis == 0 ? fp.ktx : fp.kty), k.data(), (size_t)n * 8,
-                                cudaMemcpyHostToDevice), "upload wavenumbers");
+    rc = upload(g, axis == 0 ? fp.twx : fp.twy, tw.data(), (size_t)n * 16, "upload twiddles");
+    if (rc == MHD_OK) rc = upload(g, axis == 0 ? fp.ktx : fp.kty, k.data(), (size_t)n * 8, "upload wavenumbers");
   }
   const std::vector<int2> din = disk(gp->r_inner, dx, dy), dl = disk(gp->r_lane, dx, dy);
   std::vector<double2> wl(dl.size());
@@ -672,12 +677,9 @@ extern "C" int mhd_gran_create(int nx, int ny, double dx, double dy, const mhd_g
     }
     wl[n] = make_double2(f * ex / r, f * ey / r);
   }
-  if (rc == MHD_OK && !din.empty())
-    rc = gcheck(g, cudaMemcpy((void*)d.off_in, din.data(), din.size() * 8, cudaMemcpyHostToDevice), "upload disk");
-  if (rc == MHD_OK)
-    rc = gcheck(g, cudaMemcpy((void*)d.off_l, dl.data(), dl.size() * 8, cudaMemcpyHostToDevice), "upload lane");
-  if (rc == MHD_OK)
-    rc = gcheck(g, cudaMemcpy((void*)d.w_l, wl.data(), wl.size() * 16, cudaMemcpyHostToDevice), "upload weights");
+  if (rc == MHD_OK && !din.empty()) rc = upload(g, d.off_in, din.data(), din.size() * 8, "upload disk");
+  if (rc == MHD_OK) rc = upload(g, d.off_l, dl.data(), dl.size() * 8, "upload lane");
+  if (rc == MHD_OK) rc = upload(g, d.w_l, wl.data(), wl.size() * 16, "upload weights");
   if (rc == MHD_OK)
     rc = gcheck(g, cudaMemsetAsync(g->ws + o.occ, 0, N * 4, g->st), "clear granules");
   if (rc == MHD_OK)

@@ -3,9 +3,12 @@ import ctypes
 
 import pytest
 
-from hostlib import HostLib
+from hostlib import STREAM, HostLib
+from paper_1908_08557_gb300.binding import GranParams
+from paper_1908_08557_gb300.granulation import paper_params
 
 P = ctypes.c_void_p
+D = ctypes.c_double
 
 
 @pytest.fixture(scope="module")
@@ -37,9 +40,34 @@ def test_arrays_of_another_device_travel_by_copy(host, precision):
             else:
                 assert used != far and len(copies) == 1
                 i, o = copies[0]
-                assert o[1] == "3" and int(o[5], 16) == 0x77  # device to device, on the caller's stream
+                assert o[1] == "3" and int(o[5], 16) == STREAM  # device to device, on the caller's stream
                 if kernel == "unpack_kernel":
                     assert i < at[0] and int(o[3], 16) == far and int(o[2], 16) == used
                 else:
                     assert i > at[0] and int(o[2], 16) == far and int(o[3], 16) == used
     host.lib.mhd_destroy(h)
+
+
+def _uploads_on_the_stream(ops):
+    """Every host-to-device copy is queued on the caller's stream, so that the
+    kernels behind it there find the table: one on the legacy stream may still
+    be under way when cudaMemcpy returns."""
+    ups = [o for o in ops if o[0] == "copy" and o[1] == "1"]
+    assert ups
+    for o in ups:
+        assert o[5] != "sync" and int(o[5], 16) == STREAM, o
+
+
+@pytest.mark.parametrize("nx,ny", [(64, 32), (16, 64)])
+def test_generator_tables_are_ordered_before_their_kernels(host, nx, ny):
+    gp = GranParams(**paper_params(mm_per_unit=0.23))
+    n = host.lib.mhd_gran_workspace_bytes(nx, ny, D(1.0), D(1.0), ctypes.byref(gp))
+    assert n
+    g = P()
+    host.clear()
+    host.ok(host.lib.mhd_gran_create(nx, ny, D(1.0), D(1.0), ctypes.byref(gp), P(host.memory(n)), ctypes.c_size_t(n),
+                                     P(STREAM), ctypes.byref(g)), None)
+    ops = host.log()
+    assert any(o[0] == "launch" for o in ops)
+    _uploads_on_the_stream(ops)
+    host.lib.mhd_gran_destroy(g)
