@@ -383,6 +383,14 @@ static bool in_place(const void* p, int dev) {
   return a.type == cudaMemoryTypeDevice && a.device == dev;
 }
 
+// A host table to the device, ordered on the handle's stream: cudaMemcpy may
+// return once the table is staged, with its transfer still under way on the
+// legacy stream, which a non-blocking stream does not wait for.  (Pageable
+// memory is staged before the call returns, so the table may go.)
+static int upload(mhd_ctx* h, const void* dst, const void* src, size_t bytes, const char* what) {
+  return cuda_check(h, cudaMemcpyAsync((void*)dst, src, bytes, cudaMemcpyHostToDevice, h->st), what);
+}
+
 static int sync_status(mhd_ctx* h) {
   int rc = cuda_check(h, cudaStreamSynchronize(h->st), "stream synchronize");
   if (rc) return rc;
@@ -484,10 +492,8 @@ static int upload_background(mhd_ctx* h, const double* lnrho0, const double* lnT
       z64[k] = 1.0 / z1;
       z64[(size_t)nz + k] = -z2 / (z1 * z1);
     }
-    int rz = cuda_check(h, cudaMemcpy(h->ztab, zt.data(), zt.size() * sizeof(R), cudaMemcpyHostToDevice),
-                        "upload vertical grid");
-    if (!rz) rz = cuda_check(h, cudaMemcpy(h->zt64, z64.data(), z64.size() * 8, cudaMemcpyHostToDevice),
-                             "upload vertical grid (FP64)");
+    int rz = upload(h, h->ztab, zt.data(), zt.size() * sizeof(R), "upload vertical grid");
+    if (!rz) rz = upload(h, h->zt64, z64.data(), z64.size() * 8, "upload vertical grid (FP64)");
     if (rz) return rz;
     bg.zm1 = (const R*)h->ztab;
     bg.zr21 = bg.zm1 + nz;
@@ -508,8 +514,7 @@ static int upload_background(mhd_ctx* h, const double* lnrho0, const double* lnT
     bg.ctL[m] = (R)(lb[NG + kt - m] - lb[NG + kt + m]);
   }
   if (sizeof(R) == 8) h->bgd = *(Background<double>*)&bg; else h->bgf = *(Background<float>*)&bg;
-  return cuda_check(h, cudaMemcpy(h->bgtab, tab.data(), tab.size() * sizeof(R), cudaMemcpyHostToDevice),
-                    "upload background");
+  return upload(h, h->bgtab, tab.data(), tab.size() * sizeof(R), "upload background");
 }
 
 // ---- launch sequence ----------------------------------------------------------
@@ -754,8 +759,7 @@ static int upload_fft_tables(mhd_ctx* h, const Offsets& o) {
       tw[2 * r] = w.x;
       tw[2 * r + 1] = w.y;
     }
-    rc = cuda_check(h, cudaMemcpy((void*)(axis == 0 ? fp.twx : fp.twy), tw.data(), (size_t)n * 16,
-                                  cudaMemcpyHostToDevice), "upload twiddles");
+    rc = upload(h, axis == 0 ? fp.twx : fp.twy, tw.data(), (size_t)n * 16, "upload twiddles");
     if (rc) return rc;
   }
   // continuous |k| = 2 pi sqrt((m/Lx)^2 + (n/Ly)^2), signed m, n; tables
@@ -783,9 +787,9 @@ static int upload_fft_tables(mhd_ctx* h, const Offsets& o) {
       }
     }
   }
-  rc = cuda_check(h, cudaMemcpy((void*)fp.et, et.data(), et.size() * 8, cudaMemcpyHostToDevice), "upload et");
+  rc = upload(h, fp.et, et.data(), et.size() * 8, "upload et");
   if (rc) return rc;
-  rc = cuda_check(h, cudaMemcpy((void*)fp.eb, eb.data(), eb.size() * 8, cudaMemcpyHostToDevice), "upload eb");
+  rc = upload(h, fp.eb, eb.data(), eb.size() * 8, "upload eb");
   if (rc) return rc;
   // modified wavenumber of the sixth-order first derivative; zero at m = 0
   // and at the Nyquist mode
@@ -798,8 +802,7 @@ static int upload_fft_tables(mhd_ctx* h, const Offsets& o) {
       double th = 2.0 * M_PI * (2 * m > n ? m - n : m) / n;
       kt[m] = (45.0 * sin(th) - 9.0 * sin(2.0 * th) + sin(3.0 * th)) / (30.0 * hsp);
     }
-    rc = cuda_check(h, cudaMemcpy((void*)(axis == 0 ? fp.ktx : fp.kty), kt.data(), (size_t)n * 8,
-                                  cudaMemcpyHostToDevice), "upload kt");
+    rc = upload(h, axis == 0 ? fp.ktx : fp.kty, kt.data(), (size_t)n * 8, "upload kt");
     if (rc) return rc;
   }
   return MHD_OK;
@@ -924,7 +927,7 @@ extern "C" int mhd_create(const mhd_params* p, void* workspace, size_t ws_bytes,
       double v = lnrho0[m];  // z index m - 3
       if (es == 8) ((double*)buf.data())[m] = v; else ((float*)buf.data())[m] = (float)v;
     }
-    rc = cuda_check(h, cudaMemcpy(h->lnrho0, buf.data(), 8 * es, cudaMemcpyHostToDevice), "upload lnrho0");
+    rc = upload(h, h->lnrho0, buf.data(), 8 * es, "upload lnrho0");
     std::vector<double> w(p->nz), wp(p->nz);
     for (int k = 0; k < p->nz; ++k) swamp_weight(p, zpos(p, k), &w[k], &wp[k]);
     char* wb = buf.data() + 8 * es;
@@ -932,9 +935,8 @@ extern "C" int mhd_create(const mhd_params* p, void* workspace, size_t ws_bytes,
       if (es == 8) { ((double*)wb)[k] = w[k]; ((double*)wb)[p->nz + k] = wp[k]; }
       else { ((float*)wb)[k] = (float)w[k]; ((float*)wb)[p->nz + k] = (float)wp[k]; }
     }
-    if (!rc) rc = cuda_check(h, cudaMemcpy(h->wtab, wb, (size_t)p->nz * es, cudaMemcpyHostToDevice), "upload w");
-    if (!rc) rc = cuda_check(h, cudaMemcpy(h->wptab, wb + (size_t)p->nz * es, (size_t)p->nz * es,
-                                            cudaMemcpyHostToDevice), "upload wp");
+    if (!rc) rc = upload(h, h->wtab, wb, (size_t)p->nz * es, "upload w");
+    if (!rc) rc = upload(h, h->wptab, wb + (size_t)p->nz * es, (size_t)p->nz * es, "upload wp");
   }
   if (!rc && h->have_fft) rc = upload_fft_tables(h, o);
   if (!rc && h->have_fft) {
@@ -968,7 +970,7 @@ extern "C" int mhd_create(const mhd_params* p, void* workspace, size_t ws_bytes,
   if (!rc) {
     StepState s0;
     memset(&s0, 0, sizeof s0);
-    rc = cuda_check(h, cudaMemcpy(h->ss, &s0, sizeof s0, cudaMemcpyHostToDevice), "init step state");
+    rc = upload(h, h->ss, &s0, sizeof s0, "init step state");
   }
   if (!rc) {
     // zero the driver (no nudging target until mhd_set_driver)

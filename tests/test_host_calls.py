@@ -3,6 +3,7 @@ import ctypes
 
 import pytest
 
+import inputs
 from hostlib import STREAM, HostLib
 from paper_1908_08557_gb300.binding import GranParams
 from paper_1908_08557_gb300.granulation import paper_params
@@ -71,3 +72,14 @@ def test_generator_tables_are_ordered_before_their_kernels(host, nx, ny):
     assert any(o[0] == "launch" for o in ops)
     _uploads_on_the_stream(ops)
     host.lib.mhd_gran_destroy(g)
+
+
+@pytest.mark.parametrize("precision", [32, 64])
+@pytest.mark.parametrize("over", [{}, {"z": True}, {"bc_z": 1}])
+def test_handle_tables_are_ordered_before_their_kernels(host, precision, over):
+    if "z" in over:
+        over = dict(z=inputs.stretched_z(12, 0.5, 1.5, 4, 2)[0])
+    host.clear()
+    h = host.handle(16, 8, 12, precision, **over)
+    _uploads_on_the_stream(host.log())
+    host.lib.mhd_destroy(h)
