@@ -554,7 +554,16 @@ static void ghost_fill(mhd_ctx* h, R* f, bool chained = false) {
   {
     ClassTimer ct(h, MHD_KC_PFE, 3);
     launch_pfe<R>(h->fp, h->L, f, h->ss, h->st, &h->ps);
+    if (h->prof) {
+      // the class ends with the last of the chains, not with the one here: its
+      // end is recorded behind all three on another chain's stream
+      cudaEventRecord(h->evj, h->st);
+      cudaStreamWaitEvent(h->ps.s[0], h->evj, 0);
+      cudaStreamWaitEvent(h->ps.s[0], h->ps.join[1], 0);
+      ct.st = h->ps.s[0];
+    }
   }
+  if (h->prof) cudaEventRecord(h->ps.join[0], h->ps.s[0]);
   rules(false);
   pfe_join(h->ps, h->st);
 }

@@ -83,3 +83,50 @@ def test_handle_tables_are_ordered_before_their_kernels(host, precision, over):
     h = host.handle(16, 8, 12, precision, **over)
     _uploads_on_the_stream(host.log())
     host.lib.mhd_destroy(h)
+
+
+def _reaches(ops):
+    """after(i, j): operation j can only run once i has (stream order and events)."""
+    before = [set() for _ in ops]  # direct predecessors
+    last, recorded = {}, {}
+    for n, o in enumerate(ops):
+        stream = o[2] if o[0] in ("launch", "record") else o[1] if o[0] in ("wait", "sync") else o[-1]
+        if stream in last:
+            before[n].add(last[stream])
+        if o[0] == "record":
+            recorded[o[1]] = n
+        elif o[0] == "wait":
+            before[n].add(recorded[o[2]])
+        last[stream] = n
+    anc = [set() for _ in ops]
+    for n in range(len(ops)):
+        for b in before[n]:
+            anc[n] |= anc[b] | {b}
+    return lambda i, j: i in anc[j]
+
+
+@pytest.mark.parametrize("nx,ny,fft_kernels", [(128, 128, 9), (64, 64, 3)])
+def test_profiled_fft_time_ends_with_its_last_chain(host, nx, ny, fft_kernels):
+    """mhd_profile(h, 1): a class's times hold all of its kernels, on whatever
+    stream they run, and none of the step's other work."""
+    h = host.handle(nx, ny, 8, 32, dt_fixed=0.01)
+    host.ok(host.lib.mhd_profile(h, 1), h)
+    host.clear()
+    host.ok(host.lib.mhd_step(h, 1), h)
+    ops = host.log()
+    after = _reaches(ops)
+    fft = [i for i, o in enumerate(ops) if o[0] == "launch" and ("rows_" in o[1] or "cols_" in o[1])]
+    assert len(fft) == 3 * fft_kernels
+    at = {}  # where each event is recorded first; a timer's two events are created together
+    for i, o in enumerate(ops):
+        if o[0] == "record":
+            at.setdefault(int(o[1], 16), i)
+    rules = [i for i, o in enumerate(ops) if o[0] == "launch" and "bc_kernel" in o[1]]
+    assert len(rules) == 3
+    for sub in range(3):
+        ks = fft[sub * fft_kernels:(sub + 1) * fft_kernels]
+        a = max(e for e, i in at.items() if i < ks[0] and e + 0x10 in at and at[e + 0x10] > ks[0])
+        start, end = at[a], at[a + 0x10]
+        assert all(after(start, k) and after(k, end) for k in ks)
+        assert not any(after(start, r) and after(r, end) for r in rules)
+    host.lib.mhd_destroy(h)
