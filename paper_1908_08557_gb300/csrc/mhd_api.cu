@@ -1040,9 +1040,10 @@ extern "C" int mhd_write(mhd_handle h, const void* src, int mem) {
     if (rc) return rc;
     src = h->df;
   }
-  // a state written afresh may be stepped again: clear the halt flag and its
-  // neighbour StepState::held
-  rc = cuda_check(h, cudaMemsetAsync(&h->ss->nonfinite, 0, 2 * sizeof(int), h->st), "clear status");
+  // a state written afresh may be stepped again: clear the halt flag (and behind
+  // it the item counter, which every launch that uses it clears, and `held`)
+  static_assert(offsetof(StepState, held) == offsetof(StepState, nonfinite) + 2 * sizeof(int), "one fill");
+  rc = cuda_check(h, cudaMemsetAsync(&h->ss->nonfinite, 0, 3 * sizeof(int), h->st), "clear status");
   if (rc) return rc;
   // the other state set needs nothing: before anything reads it a substep has
   // written its interior, images and u ghost rows, and the ghost rules the rest;
@@ -1471,12 +1472,11 @@ extern "C" int mhd_restore(mhd_handle h, const void* src, double t) {
   if (!h || !src) return fail(h, MHD_ERR_ARG, "NULL argument");
   int rc = cuda_check(h, cudaMemcpyAsync(h->f[h->cur], src, mhd_checkpoint_bytes(h), cudaMemcpyDeviceToDevice, h->st),
                       "restore");
-  // the time, and before it StepState::held: the sets of a halted handle differ again
-  struct { int held; int t[2]; } in = {0, {0, 0}};
-  static_assert(offsetof(StepState, t) == offsetof(StepState, held) + sizeof(int), "one copy");
-  memcpy(in.t, &t, sizeof t);
-  if (!rc) rc = cuda_check(h, cudaMemcpyAsync(&h->ss->held, &in, sizeof in, cudaMemcpyHostToDevice, h->st),
+  double tt = t;
+  if (!rc) rc = cuda_check(h, cudaMemcpyAsync(&h->ss->t, &tt, sizeof(double), cudaMemcpyHostToDevice, h->st),
                            "restore t");
+  // the sets of a halted handle differ again
+  if (!rc) rc = cuda_check(h, cudaMemsetAsync(&h->ss->held, 0, sizeof(int), h->st), "clear held");
   if (!rc) rc = cuda_check(h, cudaStreamSynchronize(h->st), "restore synchronize");
   return rc;
 }
