@@ -360,7 +360,7 @@ void launch_adj_gather(const Layout& L, const Phys<R>& ph, const R* coef, const 
 template <typename R>
 void launch_adj_update(const Layout& L, R* fbar, R* dbar, const R* gbar, double alpha, double beta,
                        int klo, int khi, const StepState* ss, cudaStream_t st, bool chained) {
-  launch_chained(chained, adj_update_kernel<R>, 152 * 8, 256, 0, st, L, fbar, dbar, gbar, (R)alpha, (R)beta, klo, khi, ss);
+  launch_chained(chained, adj_update_kernel<R>, 8 * sm_count(), 256, 0, st, L, fbar, dbar, gbar, (R)alpha, (R)beta, klo, khi, ss);
 }
 
 template <typename R>

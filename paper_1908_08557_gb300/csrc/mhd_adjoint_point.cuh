@@ -172,7 +172,7 @@ __device__ __forceinline__ void rhs_point_adjoint(const Cell<R>& c, const Phys<R
   cf[CGL + 0] += bgL0; cf[CGL + 1] += bgL1; cf[CGL + 2] += bgL2;
 }
 
-// What the z-march gathers read.  Many of the 40 coefficients repeat one
+// What the default gathers read (FP32 z-march, FP64 warp per layer).  Many of the 40 coefficients repeat one
 // another: A enters the right-hand side through B = curl A and J = grad div A -
 // lap A, so away from the swamp layers its nine first-derivative coefficients
 // are +-bB and zero, and its Laplacian ones are -bJ.  Those gathers read bB

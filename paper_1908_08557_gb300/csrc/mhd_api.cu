@@ -25,12 +25,13 @@ struct mhd_ctx {
   bool tiled;          // FP32: TMA-fed z-march kernels; otherwise the simple kernel
   bool split;          // FP32 forward: split passes (else the fused z-march kernel)
   bool pair;           // FP32 forward: one-pass f32x2 kernel with TMEM z histories
-  bool rk64;           // FP64 forward: z-march with shared first derivatives (else one thread per cell)
+  bool rk64;           // FP64 forward: a warp per layer, first derivatives shared (else one thread per cell)
   void* bj;            // split: [6][nz][ny][nx] B, J of the current substep
   void* sw;            // split: [3][nz - ksw][ny][nx] swamp terms
   int ksw;             // first layer with a nonzero swamp weight or slope (nz if none)
   bool adj_tiled;      // adjoint: tiled gather and (FP32) z-march point kernel, else one thread per point
-  bool adj_zm;         // adjoint gather as a z-march (else 3D tiles after a grad-div fold)
+  bool adj_zm;         // adjoint gather as a z-march (FP32) or a warp per layer (FP64), 31 exchanged
+                       // coefficients (else 3D tiles after a grad-div fold, all 40)
   bool adj_pair;       // FP32 adjoint point kernel on the pair z-march (else the one-cell-per-thread z-march)
   mhd_params p;
   Layout L;
@@ -520,7 +521,11 @@ static int upload_background(mhd_ctx* h, const double* lnrho0, const double* lnT
 // ---- launch sequence ----------------------------------------------------------
 // whether the boundary chain of this handle is a row of kernels on its stream
 // alone, each of which may be launched behind its predecessor (not while
-// events are recorded between them)
+// events are recorded between them).  Planes with the transforms: up to the size
+// of pfe_one_chain, above which the waiting blocks cost more than they hide.
+// Triply periodic boxes at every size, plain over chained launches in time a
+// step: FP32 32^3 81.7 / 64.4 us, 150 x 99 x 70 230.2 / 218.0, 384 x 320 x 100
+// 1402 / 1395; FP64 32^3 201 / 190, 256 x 255 x 150 33085 / 33070.
 static bool one_chain(const mhd_ctx* h) {
   return !h->prof && (h->p.bc_z == 1 || pfe_one_chain(h->p.nx, h->p.ny));
 }

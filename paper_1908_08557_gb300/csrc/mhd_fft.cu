@@ -35,8 +35,9 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 // transforms are bound by the FP64 pipe): with w = m (1 + i t) the product is
 // m (u, v), u = x - t y, v = y + t x, and the factor m rides on the sums.
 // Where |Im w| > |Re w| the same with w = i m (1 + i t), i.e. for (-y, x), so
-// that |t| <= 1 and nothing is lost (twiddle_pair, mhd_internal.h).  inv:
-// conjugate twiddle.
+// that |t| <= 1 and nothing is lost (twiddle_pair, mhd_internal.h); the tangent
+// form of a twiddle for fused multiply-adds is that of Linzer and Feig (1993).
+// inv: conjugate twiddle.
 // Signs and swaps go by integer operations (a negated copy can cost an FP64
 // one).
 __device__ __forceinline__ double flip(double x, int sign) {

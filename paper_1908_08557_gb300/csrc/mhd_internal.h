@@ -112,8 +112,10 @@ inline void launch_chained(bool chained, void (*k)(P...), dim3 grid, dim3 block,
 // block per SM.  Blocks of a chained launch are placed while the predecessor
 // still runs, and the SMs its blocks have left can get two of them while others
 // get none; for FP64 blocks, which share an SM's FP64 pipe, that doubles the
-// kernel (an FP64 step at 32^3: 311 us, 231 so).  With more than half of an SM's shared memory to a
-// block every SM takes one.  The limit itself is raised once per device.
+// kernel.  With more than half of an SM's shared memory to a block every SM takes
+// one.  An FP64 step, without and with it: 32^3 (128 blocks) 297 / 220 us, 64 x
+// 16 x 32 (128) 297 / 221, 32 x 32 x 16 (64) 217 / 218; grids of more blocks than
+// SMs go without.  The limit itself is raised once per device.
 constexpr size_t ONE_PER_SM_BYTES = 88 * 1024;  // + 32 KB static: over half of 228 KB
 inline size_t one_per_sm(bool chained, dim3 g) {
   return chained && (size_t)g.x * g.y * g.z <= (size_t)sm_count() ? ONE_PER_SM_BYTES : 0;
@@ -165,7 +167,7 @@ template <typename R> void launch_rk(const Layout& L, const Phys<R>& ph, const B
                                      const R* fin, R* fout, R* df,
                                      const R* wtab, const R* wptab, const Driver& drv, const StepState* ss,
                                      int sub, cudaStream_t st);
-// the same in FP64 as a z-march that shares the first derivatives between the
+// the same in FP64, a warp per layer, sharing the first derivatives between the
 // mixed ones (mhd_rk64.cu), and the FP64 pointwise adjoint on it
 void launch_rk64(const Layout& L, const Phys<double>& ph, const Background<double>& bg, const double* fin,
                  double* fout, double* df, const double* wtab, const double* wptab, const Driver& drv,
@@ -178,7 +180,7 @@ void launch_rk_tiled(const CUtensorMap* tm, const Layout& L, const Phys<float>& 
                      float* fout, float* df, const float* wtab, const float* wptab, const Driver& drv,
                      StepState* ss, int sub, double dx, double dy, double dz, cudaStream_t st);
 // FP32 pointwise adjoint of substep `sub` on the TMA-fed z-march (tm maps the
-// ghost-filled substep state): 46 coefficient fields and the driver adjoints
+// ghost-filled substep state): 40 coefficient fields and the driver adjoints
 void launch_adj_point_tiled(const CUtensorMap* tm, const Layout& L, const Phys<float>& ph,
                             const Background<float>& bg, const float* dbar, float* coef, double* thbar,
                             const float* wtab, const float* wptab, StepState* ss, int sub, double dx, double dy,

@@ -260,8 +260,8 @@ int launch_cfl_partial(const Layout& L, const Phys<R>& ph, const Background<R>& 
       cfl64_kernel<<<dim3((L.nx + 31) / 32, (L.ny + C64Y - 1) / C64Y, nk), dim3(32, C64Y), 0, st>>>(
           L, ph, bg, f, wtab, partial, ss, s2, k0, nlo, kgap);
     else
-    cfl_partial_kernel<R><<<dim3((L.nx + 63) / 64, (L.ny + 7) / 8, nk), dim3(32, 8), 0, st>>>(
-        L, ph, bg, f, wtab, partial, ss, s2, k0, nlo, kgap);
+      cfl_partial_kernel<R><<<dim3((L.nx + 63) / 64, (L.ny + 7) / 8, nk), dim3(32, 8), 0, st>>>(
+          L, ph, bg, f, wtab, partial, ss, s2, k0, nlo, kgap);
   }
   return CFL_SLOTS;
 }
@@ -271,8 +271,10 @@ int launch_cfl_partial(const Layout& L, const Phys<R>& ph, const Background<R>& 
 // (Sect. 2.3: linear switch-on, linear interpolation between snapshots).
 // Bound by latency (one block, dependent FP64 divisions): the maxima are taken
 // as integers, and each substep's time and weights by a thread of its own; in a
-// boundary chain of short kernels it is chained as they are (with the chained
-// substeps of a taped step 144 -> 136 us at 64^3 in FP32).
+// boundary chain of short kernels it is chained as they are (this, the chained
+// substeps and the ghost-rule transpose beside the columns together: a taped step
+// at 64^3 in FP32 144 -> 134 us).  A halted step copies the state it began from
+// (KeepSets): one block, but once.
 __global__ void cfl_finalize_kernel(const double* partial, int nblk, StepState* ss, double c_adv,
                                     double c_diff, double dt_fixed, double inv2sum, double t0, double t1,
                                     double t_ramp, int probe, KeepSets keep) {

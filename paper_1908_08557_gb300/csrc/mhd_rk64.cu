@@ -30,8 +30,8 @@
 // each instead of 64).  Neighbours come through L1 from the padded state.
 //
 // Measured (GB300, a launch): 256 x 256 x 128 16.5 -> 8.9 ms against the
-// cell-by-cell kernel (mhd_rk.cu), 32^3 93 -> 55 us; the FP64 pipe is busy 86 %
-// of the time.
+// cell-by-cell kernel (mhd_rk.cu), 32^3 93 -> 55 us; the FP64 pipe is active
+// 85 % of the time at 128^3.
 #include "mhd_adjoint_point.cuh"
 #include "mhd_internal.h"
 

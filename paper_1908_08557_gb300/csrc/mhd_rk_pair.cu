@@ -930,7 +930,13 @@ static pair::Args pair_args(const Layout& L, const Phys<float>& ph, const Backgr
   // with whole columns, 479 claimed in chunks of 20; 256^3: 526 -> 517; 1024 x
   // 1024 x 128 about a background: 4534 -> 4404).  Smaller launches are bound
   // by the latency of a chunk's chain, where every prologue plane counts, and
-  // take whole waves by grid stride.
+  // take whole waves by grid stride.  A step with a fixed time step, by grid
+  // stride over claimed, at a CTA's planes: 13 (128 x 128 x 64) 302 / 317 us, 40
+  // (256 x 256 x 48) 698 / 709, 54 (256 x 256 x 64) 797 / 802, 82 (256 x 256 x 97)
+  // 1023 / 971, 108 1250 / 1178, 163 (512 x 256 x 97) 1917 / 1733, 216 (256^3)
+  // 1883 / 1877, 431 (1024 x 512 x 64) 5477 / 5370.  Other leads than 1.35 at
+  // 256^3 (0.7, 1.0, 1.35, 1.8, 2.5): 1930, 1931, 1888, 1938, 1920; 512 x 256 x 97
+  // 1819, 1788, 1753, 1785, 1787; at 1024 x 512 x 128 all within 0.6 %.
   // (The adjoint point kernel, bound by its writes, claims from a dozen items
   // per CTA on: at 256^3 claimed short chunks cost it 4 %.)
   const int tiles = a.ntx * a.nty;
